@@ -187,6 +187,7 @@ wt_status run(wt_ctx* ctx, const char* fn, F&& body) {
             cudaError_t e = cudaSetDevice(ctx->dev);
             if (e != cudaSuccess) fail(WT_ERR_CUDA, std::string("cudaSetDevice: ") + cudaGetErrorString(e));
         }
+        DenseScratch scratch(ctx ? ctx->d_err.p : nullptr);
         body();
         if (ctx) ctx->err.clear();
         return WT_OK;

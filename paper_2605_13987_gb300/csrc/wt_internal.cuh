@@ -113,10 +113,29 @@ struct DBuf {
 };
 
 // ---------------------------------------------------------------- dense FP64
-// Row-major matrices.  op(A) is M x K, op(B) is K x N, C is M x N.
+// Row-major matrices.  op(A) is M x K, op(B) is K x N, C is M x N.  lower_only: entries above the
+// diagonal of C are left as they are.  Large products run on the tensor cores (fp64_cores: never).
 void dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
            const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
-           bool lower_only = false);
+           bool lower_only = false, bool fp64_cores = false);
+// Device workspace of the tensor-core products of one library call: made by the C entry points,
+// found by dgemm through the calling thread, freed when the call returns.  Products of one call
+// run on one stream, so they share it in turn.
+struct DenseScratch {
+    int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
+    explicit DenseScratch(int* err);
+    ~DenseScratch();
+    DenseScratch(const DenseScratch&) = delete;
+    DenseScratch& operator=(const DenseScratch&) = delete;
+    unsigned char* get(size_t bytes);     // NULL when the memory is not to be had
+private:
+    unsigned char* p = nullptr;
+    size_t cap = 0;
+    DenseScratch* outer;
+};
+// dgemm on the tensor cores (k_dgemm_tc.cu); false when it does not take the product.
+bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
+              const double* B, int ldb, double beta, double* C, int ldc, bool lower_only);
 void symmetrize_from_lower(cudaStream_t s, double* A, int n, int lda);
 void symmetrize_avg(cudaStream_t s, const double* F, double* C, int n);   // C = (F + F^T)/2
 void transpose(cudaStream_t s, const double* A, int rows, int cols, double* At);
