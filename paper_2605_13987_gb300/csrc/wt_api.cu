@@ -631,20 +631,22 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     const bool pre = ns >= nt;                    // column-pivoted QR first
     DBuf<double> A, V, sig, Rm;
     DBuf<int> dpiv;
+    int nr = nt;                                  // rows of R that are not negligible
     A.alloc((size_t)nt * ns);
     transpose(s, Q, ns, nt, A.p);                 // rows = time samples (the columns of Q)
     sig.alloc(nt);
+    sig.zero(s);
     if (pre) {
         Rm.alloc((size_t)nt * nt);
         dpiv.alloc(nt);
-        qrcp_r(s, A.p, ns, nt, ns, Rm.p, dpiv.p);
+        nr = qrcp_r(s, A.p, ns, nt, ns, Rm.p, dpiv.p);
         A.release();
     } else {
         V.alloc((size_t)nt * nt);
     }
     clear_err(c);
     double coupling = 0.0;
-    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nt, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling)
+    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nr, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling)
                            : onesided_jacobi_rows(s, A.p, nt, ns, ns, V.p, sig.p, c->d_err.p, 40, &coupling);
     if (read_err(c)) {
         char msg[160];
