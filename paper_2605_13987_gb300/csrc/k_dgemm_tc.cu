@@ -16,7 +16,8 @@
 // What bounds it: at the fit's sizes the bf16 product (15 x 2 M N K flop); for a short K the
 // residue planes of C (15 bytes written and read per output).  Kernels:
 //   scale     largest exponent and sum of squares of every row of op(A) / column of op(B);
-//   residues  a' and its 15 residues as bf16 planes [modulus][row][K], K-major;
+//   residues  a' and its 15 residues as bf16 planes [modulus][row][K], K-major
+//             (convert: both, for both operands, in one launch where K is short);
 //   product   persistent CTAs over (modulus, 128 x 256 tile): TMA loads into four 128-byte
 //             swizzled stages, tcgen05.mma kind::f16 into two 256-column accumulators in tensor
 //             memory (a chunk of 1024 terms each), eight epilogue warps that reduce and sum the
@@ -40,6 +41,7 @@ constexpr int kNormBits = 58;             // log2 of the largest ||a'||, ||b'||
 constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
 constexpr int CHUNK = 1024;               // terms per accumulator: 1024 x 127^2 < 2^24
 constexpr int EPI_WARPS = 8;
+constexpr int kFusedK = 1024;             // longest K whose operands one launch converts
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
 
 // pairwise coprime: 3 5 17, 11 23, 251, 13 19, 241, 239, 233, 229, 227, 223, 7 31, 211, 199, 197, 193
@@ -176,13 +178,44 @@ __device__ __forceinline__ int row_shift(unsigned emax, unsigned long long ss) {
 }
 
 // --------------------------------------------------------------- residues
+// The residues of two neighbouring entries of a row scaled by 2^sh: 12-bit limbs of a' in FP32,
+// whose sums with the centred powers of 2^12 stay below 2^24 (exact), reduced mod p.
+__device__ __forceinline__ void residues_of(const double (&x)[2], int sh, __nv_bfloat162* dst, size_t plane) {
+    constexpr Tables kT = make_tables();
+    float limb[2][5];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const unsigned hi = (unsigned)__double2hiint(x[j]);
+        const int ex = (int)((hi >> 20) & 0x7ff);
+        unsigned long long mant = ((unsigned long long)(hi & 0xfffffu) << 32) | (unsigned)__double2loint(x[j]) |
+                                  (1ull << 52);
+        const int s = ex - 1075 + sh;                          // a' = round(mant 2^s), s <= 58 - 52
+        if (sh >= kZeroRow / 2 || ex == 0 || s < -54) mant = 0;
+        else if (s >= 0) mant <<= s;
+        else mant = (mant + (1ull << (-s - 1))) >> -s;
+        const float sg = (hi >> 31) ? -1.f : 1.f;
+#pragma unroll
+        for (int l = 0; l < 5; ++l) limb[j][l] = sg * (float)(unsigned)((mant >> (12 * l)) & 0xfffu);
+    }
+#pragma unroll
+    for (int m = 0; m < NMOD; ++m) {
+        float v[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float y = limb[j][0];
+#pragma unroll
+            for (int l = 1; l < 5; ++l) y = fmaf(limb[j][l], kT.coef[m][l], y);
+            v[j] = mod_centred(y, kT.p[m], kT.inv[m]);
+        }
+        dst[m * plane] = __floats2bfloat162_rn(v[0], v[1]);
+    }
+}
 // 32 rows x 64 k per block through shared memory; planes out[m][row][Kp].
 template <bool TRANS>
 __global__ void __launch_bounds__(256) residue_kernel(const double* __restrict__ X, int ld, int rows, int k_begin,
                                                       int k_end, int Kp, const unsigned* __restrict__ emax,
                                                       const unsigned long long* __restrict__ ss,
                                                       __nv_bfloat16* __restrict__ out) {
-    constexpr Tables kT = make_tables();
     __shared__ double tile[32][65];
     const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 64;      // k0 relative to k_begin
     const int K = k_end - k_begin;
@@ -199,41 +232,88 @@ __global__ void __launch_bounds__(256) residue_kernel(const double* __restrict__
     for (int i = w; i < 32; i += 8) {
         const int r = r0 + i;
         if (r >= rows) break;
-        const int sh = row_shift(emax[r], ss[r]);
-        const bool live = sh < kZeroRow / 2;
-        float limb[2][5];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const double x = tile[i][2 * lane + j];
-            const unsigned hi = (unsigned)__double2hiint(x);
-            const int ex = (int)((hi >> 20) & 0x7ff);
-            unsigned long long mant = ((unsigned long long)(hi & 0xfffffu) << 32) | (unsigned)__double2loint(x) |
-                                      (1ull << 52);
-            const int s = ex - 1075 + sh;                      // a' = round(mant 2^s), s <= 58 - 52
-            if (!live || ex == 0 || s < -54) mant = 0;
-            else if (s >= 0) mant <<= s;
-            else mant = (mant + (1ull << (-s - 1))) >> -s;
-            const float sg = (hi >> 31) ? -1.f : 1.f;
-#pragma unroll
-            for (int l = 0; l < 5; ++l) limb[j][l] = sg * (float)(unsigned)((mant >> (12 * l)) & 0xfffu);
-        }
         const int k = k0 + 2 * lane;
         if (k < Kp) {
-            __nv_bfloat162* dst = reinterpret_cast<__nv_bfloat162*>(out + (size_t)r * Kp + k);
-            const size_t plane = (size_t)rows * Kp / 2;
-#pragma unroll
-            for (int m = 0; m < NMOD; ++m) {
-                float v[2];
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    float x = limb[j][0];
-#pragma unroll
-                    for (int l = 1; l < 5; ++l) x = fmaf(limb[j][l], kT.coef[m][l], x);
-                    v[j] = mod_centred(x, kT.p[m], kT.inv[m]);
-                }
-                dst[m * plane] = __floats2bfloat162_rn(v[0], v[1]);
-            }
+            const double x[2] = {tile[i][2 * lane], tile[i][2 * lane + 1]};
+            residues_of(x, row_shift(emax[r], ss[r]),
+                        reinterpret_cast<__nv_bfloat162*>(out + (size_t)r * Kp + k), (size_t)rows * Kp / 2);
         }
+    }
+}
+
+// Scale and residues of both operands in one launch, for products whose K a block can go over
+// itself: 32 rows per block, three passes (exponents, squares, residues; the later ones find the
+// operand in L2).  The tall case leaves too few blocks, so it takes the three kernels above.
+struct Operand {
+    const double* X;
+    int ld, rows, blocks;
+    bool trans;
+    unsigned* emax;
+    unsigned long long* ss;
+    __nv_bfloat16* out;
+};
+__global__ void __launch_bounds__(256) convert_kernel(Operand A, Operand B, int K, int Kp) {
+    const bool first = (int)blockIdx.x < A.blocks;
+    const Operand P = first ? A : B;
+    const int r0 = (first ? blockIdx.x : blockIdx.x - A.blocks) * 32;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double tile[32][65];
+    __shared__ unsigned e_sh[32];
+    __shared__ unsigned long long s_sh[32];
+    if (threadIdx.x < 32) { e_sh[threadIdx.x] = 0; s_sh[threadIdx.x] = 0; }
+    __syncthreads();
+    auto at = [&](int r, int k) { return P.trans ? P.X[(size_t)k * P.ld + r0 + r] : P.X[(size_t)(r0 + r) * P.ld + k]; };
+    auto square = [](double x, unsigned em) {                  // (x 2^-(em - 1023))^2 from the top 24 bits
+        const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+        const int ex = (int)(hi >> 20), d = ex - (int)em;
+        const float f = (ex == 0 || d < -60) ? 0.f
+            : __uint_as_float(((unsigned)(127 + d) << 23) | ((hi & 0xfffffu) << 3) | ((unsigned)__double2loint(x) >> 29));
+        return f * f;
+    };
+    if (P.trans) {
+        if (r0 + lane < P.rows) {
+            unsigned e = 0;
+            for (int k = w; k < K; k += 8) e = max(e, ((unsigned)__double2hiint(at(lane, k)) >> 20) & 0x7ffu);
+            atomicMax(&e_sh[lane], e);
+        }
+        __syncthreads();
+        if (r0 + lane < P.rows) {
+            float s = 0.f;
+            for (int k = w; k < K; k += 8) s += square(at(lane, k), e_sh[lane]);
+            atomicAdd(&s_sh[lane], (unsigned long long)ceilf(s * 1048576.0f));
+        }
+    } else {
+        for (int i = w; i < 32 && r0 + i < P.rows; i += 8) {
+            unsigned e = 0;
+            for (int k = lane; k < K; k += 32) e = max(e, ((unsigned)__double2hiint(at(i, k)) >> 20) & 0x7ffu);
+            e = __reduce_max_sync(0xffffffffu, e);
+            float s = 0.f;
+            for (int k = lane; k < K; k += 32) s += square(at(i, k), e);
+            for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) { e_sh[i] = e; s_sh[i] = (unsigned long long)ceilf(s * 1048576.0f); }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 && r0 + (int)threadIdx.x < P.rows) {
+        P.emax[r0 + threadIdx.x] = e_sh[threadIdx.x];
+        P.ss[r0 + threadIdx.x] = s_sh[threadIdx.x];
+    }
+    const size_t plane = (size_t)P.rows * Kp / 2;
+    for (int k0 = 0; k0 < K; k0 += 64) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < 32 * 64; e += 256) {
+            int r, k;
+            if (P.trans) { k = e >> 5; r = e & 31; } else { r = e >> 6; k = e & 63; }
+            tile[r][k] = (r0 + r < P.rows && k0 + k < K) ? at(r, k0 + k) : 0.0;
+        }
+        __syncthreads();
+        const int k = k0 + 2 * lane;
+        if (k < Kp)
+            for (int i = w; i < 32 && r0 + i < P.rows; i += 8) {
+                const double x[2] = {tile[i][2 * lane], tile[i][2 * lane + 1]};
+                residues_of(x, row_shift(e_sh[i], s_sh[i]),
+                            reinterpret_cast<__nv_bfloat162*>(P.out + (size_t)(r0 + i) * Kp + k), plane);
+            }
     }
 }
 
@@ -566,24 +646,39 @@ bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alph
     __nv_bfloat16* ra = reinterpret_cast<__nv_bfloat16*>(p + b_e + b_s);
     __nv_bfloat16* rb = same ? ra : reinterpret_cast<__nv_bfloat16*>(p + b_e + b_s + b_a);
     signed char* T = reinterpret_cast<signed char*>(p + b_e + b_s + b_a + b_b);
-    WT_CUDA(cudaMemsetAsync(p, 0, b_e + b_s, s));
-    scales(s, A, lda, ta, M, K, ea, sa);                       // op(A) rows: k contiguous unless transposed
-    if (!same) scales(s, B, ldb, !tb, N, K, eb, sb);           // op(B) columns: k contiguous when transposed
+    // op(A) rows: k contiguous unless transposed; op(B) columns: k contiguous when transposed.  One
+    // conversion launch up to K = kFusedK (2304 x 2304 x 256: 3 launches, 21 us against 9 and 47 us of
+    // host time); beyond, 32 rows per block leave SMs idle.
+    const bool fused = K <= kFusedK && kc >= K;
+    if (fused) {
+        Operand oa{A, lda, M, (M + 31) / 32, ta, ea, sa, ra}, ob{B, ldb, N, (N + 31) / 32, !tb, eb, sb, rb};
+        convert_kernel<<<oa.blocks + (same ? 0 : ob.blocks), 256, 0, s>>>(oa, ob, K, Kp);
+        WT_LAUNCH("residues");
+    } else {
+        WT_CUDA(cudaMemsetAsync(p, 0, b_e + b_s, s));
+        scales(s, A, lda, ta, M, K, ea, sa);
+        if (!same) scales(s, B, ldb, !tb, N, K, eb, sb);
+    }
     Units U{};
     U.tm = (M + BM - 1) / BM;
     U.tn = (N + BN - 1) / BN;
     U.per_mod = U.tm * U.tn;
     U.n = U.per_mod * NMOD;
     U.lower = lower_only ? 1 : 0;
-    int dev = 0, n_sm = 0;
-    WT_CUDA(cudaGetDevice(&dev));
-    WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     const size_t sh = 1024 + (size_t)STAGES * (A_BYTES + B_BYTES) + sizeof(Smem);
-    allow_dyn_smem(product_kernel, sh);
+    if (!ws->n_sm) {                                           // once per call of the library
+        int dev = 0;
+        WT_CUDA(cudaGetDevice(&dev));
+        WT_CUDA(cudaDeviceGetAttribute(&ws->n_sm, cudaDevAttrMultiProcessorCount, dev));
+        allow_dyn_smem(product_kernel, sh);
+    }
+    const int n_sm = ws->n_sm;
     for (int k0 = 0; k0 < K; k0 += kc) {
         const int k1 = std::min(K, k0 + kc);
-        residues(s, A, lda, ta, M, k0, k1, Kp, ea, sa, ra);
-        if (!same) residues(s, B, ldb, !tb, N, k0, k1, Kp, eb, sb, rb);
+        if (!fused) {
+            residues(s, A, lda, ta, M, k0, k1, Kp, ea, sa, ra);
+            if (!same) residues(s, B, ldb, !tb, N, k0, k1, Kp, eb, sb, rb);
+        }
         CUtensorMap ma, mb;
         encode_planes(&ma, ra, M, k1 - k0, Kp, BM);
         encode_planes(&mb, rb, N, k1 - k0, Kp, BN);

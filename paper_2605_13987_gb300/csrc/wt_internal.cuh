@@ -128,6 +128,7 @@ struct DenseScratch {
     DenseScratch(const DenseScratch&) = delete;
     DenseScratch& operator=(const DenseScratch&) = delete;
     unsigned char* get(size_t bytes);     // NULL when the memory is not to be had
+    int n_sm = 0;                    // SMs of the device (0: not asked yet)
 private:
     unsigned char* p = nullptr;
     size_t cap = 0;
