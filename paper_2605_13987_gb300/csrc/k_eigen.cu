@@ -3,25 +3,24 @@
 //
 //   1. Householder tridiagonalisation Y = Q T Q^T, one reflector per column:
 //      H_k = I - tau_k u_k u_k^T with u_k = [0 (k + 1 entries); v_k],
-//      v_k[0] = 1.  Per step: the reflector (one block), p = tau A22 v (one
-//      warp per row), w = p - (tau p.v / 2) v (one block), and the rank-two
-//      update A22 -= v w^T + w v^T, both products rounded before the sum so
-//      that A stays exactly symmetric.  v_k is kept in row k of A.
+//      v_k[0] = 1.  Per step: the reflector, p = tau A22 v, w = p -
+//      (tau p.v / 2) v, and the rank-two update A22 -= v w^T + w v^T, taken
+//      with the next step's pass over A22.  v_k is kept in row k of A.
 //   2. Divide and conquer on T (Cuppen's splitting): T = diag(T1', T2') +
 //      |rho| s s^T with rho the coupling at the split, s = [e_last; sign(rho)
 //      e_first] and T1', T2' the halves with |rho| taken off the touching
-//      diagonal entries.  Leaves (<= 32 rows) by implicit QL with Wilkinson
+//      diagonal entries.  Leaves (<= 8 rows) by implicit QL with Wilkinson
 //      shifts, one warp each.  A merge turns the halves' eigen-
 //      decompositions into that of D + r z z^T (r = 2|rho|, |z| = 1):
 //      deflation of negligible z entries and of close pairs of D (a Givens
 //      rotation zeroes one z entry), the roots of the secular equation
-//      1 + r sum_i z_i^2 / (d_i - lambda) = 0 (one thread per root, each root
+//      1 + r sum_i z_i^2 / (d_i - lambda) = 0 (one warp per root, each root
 //      held as the offset tau from its nearer pole so that every difference
 //      d_i - lambda is formed without cancellation), the update vector
 //      recomputed from the roots by Loewner's formula (Gu and Eisenstat), so
 //      that the eigenvectors z^_i / (d_i - lambda_j) come out orthogonal to
 //      working precision, and one GEMM per merge for the new eigenvectors.
-//   3. Back-transformation V = H_0 H_1 ... H_{n-3} Z in blocks of 32
+//   3. Back-transformation V = H_0 H_1 ... H_{n-3} Z in blocks of 128
 //      reflectors (compact WY form I - W T W^T, three GEMMs per block).
 #include "wt_internal.cuh"
 
@@ -33,8 +32,10 @@ namespace wt {
 
 namespace {
 
-constexpr int kLeaf = 32;       // largest leaf of the divide-and-conquer tree
-constexpr int kWyBlock = 32;    // reflectors per back-transformation block
+// Largest leaf of the divide-and-conquer tree.  A leaf's QL iteration is a serial chain of about
+// 2 K^2 rotations on one lane (32 rows: 0.9-2.4 ms); two more levels of merges cost less.
+constexpr int kLeaf = 8;
+constexpr int kWyBlock = 128;   // reflectors per back-transformation block (the products' K)
 constexpr double kEps = 2.220446049250313e-16;
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -60,6 +61,168 @@ __device__ double block_sum(double v, double* sh) {
 }
 
 // ------------------------------------------------------ tridiagonalisation
+// 1 / x and 1 / sqrt(x) by Newton's iteration from the FP32 value (24 -> 48 -> FP64's rounding level):
+// short chains where every FP64 operation costs a warp 16 cycles.  x is normalised by its exponent.
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
+    const int e = (ex - 1023) & ~1;
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
+    double y = (double)rsqrtf((float)m);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
+}
+
+// Barrier of the co-resident blocks of a cooperative launch: `round` counts them.  Gives up after two
+// seconds (or when another block has): error word set, every later barrier passes at once, and the
+// caller leaves.
+constexpr unsigned long long kGridWaitNs = 2000000000ull;
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int* err) {
+    __syncthreads();
+    __shared__ int ok_sh;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const unsigned want = round * gridDim.x;
+        volatile unsigned* vb = bar;
+        volatile unsigned* gone = bar + 1;
+        int ok = 1;
+        if (*vb < want) {
+            unsigned long long t0, t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+            while (*vb < want) {
+                if (*gone) { ok = 0; break; }
+                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+                if (t - t0 > kGridWaitNs) {
+                    *gone = 1;
+                    atomicMax(err, (int)DERR_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        ok_sh = ok;
+    }
+    __syncthreads();
+    return ok_sh != 0;
+}
+
+// All columns in one cooperative launch (one block per SM, rows dealt out cyclically, one warp per
+// row).  Step k, with v, w of step k - 1 in shared memory:
+//   every block forms row k of the updated matrix, A[k] - v[k] w - w[k] v, and its reflector (the
+//   same work in every block: 3 m operations, cheaper than a barrier);
+//   a warp takes a row i > k: A[i] -= v[i] w + w[i] v and, on the same pass, p[i] = tau A[i] . vn;
+//   barrier; every block reads p and forms w = p - (tau (p . vn) / 2) vn.
+// One barrier per column and one pass over the trailing block (three FP64 operations per entry: the
+// FP64 units bound it, 2 per clock and SM), where four launches a column took three passes:
+// n = 2304 94 ms before.  p alternates between two buffers, so that a block still reading one is not
+// overtaken.  The reflector of step k is written into row k one step later, when no block reads that
+// row any more.
+constexpr int kTrdThreads = 512;
+__global__ void __launch_bounds__(kTrdThreads, 1)
+    trd_kernel(double* A, int n, double* __restrict__ d, double* __restrict__ e, double* __restrict__ tau_out,
+               double* p, unsigned* bar, int* err) {
+    extern __shared__ double sm[];
+    double* v = sm;
+    double* w = sm + n;
+    double* vn = sm + 2 * (size_t)n;
+    __shared__ double red[33];
+    __shared__ double par[4];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int T = kTrdThreads, NW = T / 32;
+    const int nblk = gridDim.x, blk = blockIdx.x;
+    for (int j = tid; j < n; j += T) { v[j] = 0.0; w[j] = 0.0; }
+    __syncthreads();
+    for (int k = 0; k + 2 < n; ++k) {
+        // row k of the current matrix, and the squares below its subdiagonal entry
+        const double vk = v[k], wk = w[k];
+        double ss = 0.0;
+        for (int j = k + tid; j < n; j += T) {
+            const double x = fma(-wk, v[j], fma(-vk, w[j], __ldcg(A + (size_t)k * n + j)));
+            vn[j] = x;
+            if (j >= k + 2) ss = fma(x, x, ss);
+        }
+        ss = block_sum(ss, red);
+        if (tid == 0) {
+            const double x0 = vn[k + 1];
+            double t = 0.0, beta = x0, scale = 0.0;
+            if (ss > 0.0) {
+                const double q = fma(x0, x0, ss), rq = rsqrt_newton(q), nrm = q * rq;
+                beta = -copysign(nrm, x0);
+                t = fma(fabs(x0), rq, 1.0);                    // (beta - x0) / beta
+                scale = 1.0 / (x0 - beta);
+            }
+            par[0] = t;
+            par[1] = scale;
+            if (blk == 0) {
+                d[k] = vn[k];
+                e[k] = beta;
+                tau_out[k] = t;
+            }
+        }
+        __syncthreads();
+        const double t = par[0], scale = par[1];
+        for (int j = k + 1 + tid; j < n; j += T) vn[j] = j == k + 1 ? 1.0 : vn[j] * scale;
+        if (k > 0 && (k - 1) % nblk == blk)
+            for (int j = k + tid; j < n; j += T) A[(size_t)(k - 1) * n + j] = v[j];
+        __syncthreads();
+        // own rows below k
+        double* pk = p + (size_t)(k & 1) * n;
+        const int first = k + 1 + ((blk - (k + 1)) % nblk + nblk) % nblk;
+        for (int i = first + warp * nblk; i < n; i += NW * nblk) {
+            const double vi = v[i], wi = w[i];
+            double* row = A + (size_t)i * n;
+            double acc = 0.0;
+#pragma unroll 4
+            for (int j = k + 1 + lane; j < n; j += 32) {
+                const double x = fma(-wi, v[j], fma(-vi, w[j], row[j]));
+                row[j] = x;
+                acc = fma(x, vn[j], acc);
+            }
+            acc = warp_sum(acc);
+            if (lane == 0) __stcg(pk + i, t * acc);
+        }
+        if (nblk > 1) {
+            if (!grid_barrier(bar, k + 1, err)) return;
+        } else {
+            __syncthreads();
+        }
+        double sp = 0.0;
+        for (int j = k + 1 + tid; j < n; j += T) {
+            const double x = __ldcg(pk + j);
+            w[j] = x;
+            sp = fma(x, vn[j], sp);
+        }
+        sp = block_sum(sp, red);
+        const double al = 0.5 * t * sp;
+        for (int j = k + 1 + tid; j < n; j += T) w[j] = fma(-al, vn[j], w[j]);
+        double* x = v;
+        v = vn;
+        vn = x;
+        __syncthreads();
+    }
+    // the last 2 x 2 block and the last reflector (its row was read before the last barrier)
+    if (blk == 0) {
+        if (n > 2)
+            for (int j = n - 2 + tid; j < n; j += T) A[(size_t)(n - 3) * n + j] = v[j];
+        if (tid == 0) {
+            const int a = n - 2, b = n - 1;
+            auto at = [&](int i, int j) { return fma(-w[i], v[j], fma(-v[i], w[j], __ldcg(A + (size_t)i * n + j))); };
+            if (n >= 2) {
+                d[a] = at(a, a);
+                e[a] = at(a, b);
+                tau_out[a] = 0.0;
+            }
+            d[b] = at(b, b);
+            e[b] = 0.0;
+            tau_out[b] = 0.0;
+        }
+    }
+}
+
+// The same steps by four launches a column, for matrices whose three vectors do not fit shared memory:
 // Reflector of step k from x = A[k][k+1 ..] (row k equals column k): H x = beta e_0.
 __global__ void __launch_bounds__(1024) trd_house_kernel(double* A, int n, int k, double* vk, double* d, double* e,
                                                         double* tau) {
@@ -235,7 +398,7 @@ __global__ void dc_split_kernel(double* d, const double* e, const int* splits, i
 __global__ void __launch_bounds__(128) dc_leaf_kernel(const double* __restrict__ d, const double* __restrict__ e,
                                                       const int* __restrict__ starts, int n_leaves, int n,
                                                       double* __restrict__ lam, double* __restrict__ Q, int* err) {
-    __shared__ double Zs[4][kLeaf][kLeaf + 1];
+    __shared__ double Zs[4][32][kLeaf + 1];
     __shared__ double dd[4][kLeaf], ee[4][kLeaf], rc[4][kLeaf], rs[4][kLeaf];
     __shared__ int ctl[4][4];
     __shared__ int perm[4][kLeaf];
@@ -364,93 +527,139 @@ struct DcNode {
     int l, mid, r;
 };
 
-// One block per merge node: the rank-one update vector, the merged order, deflation (thread 0,
-// sequential over the sorted entries) and the compaction of the non-deflated poles.
-__global__ void __launch_bounds__(256) dc_prep_kernel(const DcNode* __restrict__ nodes, const double* __restrict__ e,
-                                                      const double* __restrict__ lamA, const double* __restrict__ QA,
-                                                      int n, DcWork W, double* zbuf) {
+// Exclusive prefix sum (or running maximum) over the block's per-thread values; blockDim.x = 1024.
+__device__ __forceinline__ int block_scan(int v, bool maximum, int identity, int* sh) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x = maximum ? max(x, y) : x + y;
+    }
+    __syncthreads();
+    if (lane == 31) sh[w] = x;
+    __syncthreads();
+    int base = identity;
+    for (int q = 0; q < w; ++q) base = maximum ? max(base, sh[q]) : base + sh[q];
+    const int up = __shfl_up_sync(0xffffffffu, x, 1);
+    return lane == 0 ? base : (maximum ? max(base, up) : base + up);
+}
+
+// One block per merge node: the rank-one update vector, the merged order (each entry's rank by a
+// binary search in the other half), deflation and the compaction of the non-deflated poles.  Two
+// non-deflated neighbours are close when |x y (d_p - d_q)| <= tol (x^2 + y^2) (the coupling that the
+// rotation would leave, without its square root); all pairs are looked at together, and only when one
+// is close does thread 0 go through them in order, rotating.
+constexpr int kPrepThreads = 1024;
+__global__ void __launch_bounds__(kPrepThreads) dc_prep_kernel(const DcNode* __restrict__ nodes,
+                                                               const double* __restrict__ e,
+                                                               const double* __restrict__ lamA,
+                                                               const double* __restrict__ QA, int n, DcWork W,
+                                                               double* zbuf) {
+    __shared__ int sh_i[32];
+    __shared__ double sh_d[32];
+    __shared__ int any_close, n_rot;
     const DcNode nd = nodes[blockIdx.x];
-    const int l = nd.l, K = nd.r - nd.l, K1 = nd.mid - nd.l;
+    const int l = nd.l, K = nd.r - nd.l, K1 = nd.mid - nd.l, tid = threadIdx.x;
     const double rho = e[nd.mid - 1];
     const double sg = rho < 0.0 ? -1.0 : 1.0;
     const double inv_sqrt2 = 0.70710678118654752440;
-    double* z = zbuf + l;
-    for (int i = threadIdx.x; i < K; i += blockDim.x)
-        z[i] = inv_sqrt2 * (i < K1 ? QA[(size_t)(nd.mid - 1) * n + l + i] : sg * QA[(size_t)nd.mid * n + l + i]);
-    __syncthreads();
-    if (threadIdx.x) return;
     const double r = 2.0 * fabs(rho);
     int* perm = W.perm + l;
     double* ds = W.ds + l;
-    // merge the two ascending halves
-    {
-        int a = 0, b = K1, q = 0;
-        while (a < K1 || b < K) {
-            const bool ta = b >= K || (a < K1 && lamA[l + a] <= lamA[l + b]);
-            perm[q++] = ta ? a++ : b++;
-        }
-    }
+    double* zs = W.zh + l;                 // update vector in merged order, until the Loewner pass overwrites it
+    int* flag = W.oper + l;                // 1 = deflated (oper is written after the merge)
+    const double* lam = lamA + l;
+    if (tid == 0) { any_close = 0; n_rot = 0; }
     double dmax = 0.0;
-    for (int q = 0; q < K; ++q) {
-        ds[q] = lamA[l + perm[q]];
-        dmax = fmax(dmax, fabs(ds[q]));
-    }
-    const double tol = 8.0 * kEps * fmax(dmax, r);
-    // deflation: zs kept in zbuf at sorted positions from here on (reuse: z is read through perm)
-    double* zs = W.zh + l;                 // scratch until the Loewner pass overwrites it
-    for (int q = 0; q < K; ++q) zs[q] = z[perm[q]];
-    unsigned char* flag = reinterpret_cast<unsigned char*>(W.fcol + l);   // temporary: 1 = deflated
-    for (int q = 0; q < K; ++q) flag[q] = 0;
-    int nrot = 0, p = -1;
-    for (int q = 0; q < K; ++q) {
-        if (r * fabs(zs[q]) <= tol) {
-            flag[q] = 1;
-            continue;
+    for (int i = tid; i < K; i += kPrepThreads) {
+        const double x = lam[i];
+        const bool a = i < K1;
+        int lo = a ? K1 : 0, hi = a ? K : K1;
+        const int base = lo;
+        while (lo < hi) {                  // entries of the other half before x (ties: first half first)
+            const int mid = (lo + hi) / 2;
+            if (a ? lam[mid] < x : lam[mid] <= x) lo = mid + 1; else hi = mid;
         }
+        const int q = (a ? i : i - K1) + (lo - base);
+        perm[q] = i;
+        ds[q] = x;
+        zs[q] = inv_sqrt2 * (a ? QA[(size_t)(nd.mid - 1) * n + l + i] : sg * QA[(size_t)nd.mid * n + l + i]);
+        dmax = fmax(dmax, fabs(x));
+    }
+    for (int o = 16; o; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+    if ((tid & 31) == 0) sh_d[tid >> 5] = dmax;
+    __syncthreads();
+    for (int q = 0; q < kPrepThreads / 32; ++q) dmax = fmax(dmax, sh_d[q]);
+    const double tol = 8.0 * kEps * fmax(dmax, r);
+    // contiguous pieces of the merged order per thread from here on
+    const int per = (K + kPrepThreads - 1) / kPrepThreads, q0 = min(K, tid * per), q1 = min(K, q0 + per);
+    int last = -1;
+    for (int q = q0; q < q1; ++q) {
+        const int f = r * fabs(zs[q]) <= tol;
+        flag[q] = f;
+        if (!f) last = q;
+    }
+    int p = block_scan(last, true, -1, sh_i);       // last non-deflated entry before this piece
+    __syncthreads();
+    for (int q = q0; q < q1; ++q) {
+        if (flag[q]) continue;
         if (p >= 0) {
             const double x = zs[p], y = zs[q];
-            const double t = hypot(x, y);
-            const double c = y / t, s = x / t;
-            const double off = c * s * (ds[p] - ds[q]);
-            if (fabs(off) <= tol) {
-                const double a = ds[p], b = ds[q];
-                ds[p] = c * c * a + s * s * b;
-                ds[q] = s * s * a + c * c * b;
-                zs[p] = 0.0;
-                zs[q] = t;
-                flag[p] = 1;
-                W.rot_p[l + nrot] = p;
-                W.rot_i[l + nrot] = q;
-                W.rot_c[l + nrot] = c;
-                W.rot_s[l + nrot] = s;
-                ++nrot;
-            }
+            if (fabs(x * y * (ds[p] - ds[q])) <= tol * fma(x, x, y * y)) any_close = 1;
         }
         p = q;
     }
+    __syncthreads();
+    if (any_close && tid == 0) {
+        int nrot = 0, pp = -1;
+        for (int q = 0; q < K; ++q) {
+            if (flag[q]) continue;
+            if (pp >= 0) {
+                const double x = zs[pp], y = zs[q], a = ds[pp], b = ds[q];
+                if (fabs(x * y * (a - b)) <= tol * fma(x, x, y * y)) {
+                    const double t = hypot(x, y);
+                    const double c = y / t, s = x / t;
+                    ds[pp] = c * c * a + s * s * b;
+                    ds[q] = s * s * a + c * c * b;
+                    zs[pp] = 0.0;
+                    zs[q] = t;
+                    flag[pp] = 1;
+                    W.rot_p[l + nrot] = pp;
+                    W.rot_i[l + nrot] = q;
+                    W.rot_c[l + nrot] = c;
+                    W.rot_s[l + nrot] = s;
+                    ++nrot;
+                }
+            }
+            pp = q;
+        }
+        n_rot = nrot;
+    }
+    __syncthreads();
     // compaction: non-deflated first (ascending), then deflated
-    int kp = 0;
-    for (int q = 0; q < K; ++q)
-        if (!flag[q]) ++kp;
-    int a = 0, b = kp;
-    double* delta = W.delta + l;
-    double* zeta = W.zeta + l;
-    double* dv = W.defl_val + l;
-    // flag lives in fcol's storage: read it all before fcol is written
-    for (int q = 0; q < K; ++q) {
+    int live = 0;
+    for (int q = q0; q < q1; ++q) live += !flag[q];
+    int a = block_scan(live, false, 0, sh_i);
+    __shared__ int kp_sh;
+    if (tid == kPrepThreads - 1) kp_sh = a + live;
+    __syncthreads();
+    const int kp = kp_sh;
+    for (int q = q0; q < q1; ++q) {
         if (!flag[q]) {
-            delta[a] = ds[q];
-            zeta[a] = zs[q];
-            W.org[l + q] = a++;          // temporary: sorted position -> gathered column
+            W.delta[l + a] = ds[q];
+            W.zeta[l + a] = zs[q];
+            W.fcol[l + q] = a++;
         } else {
-            dv[b - kp] = ds[q];
-            W.org[l + q] = b++;
+            const int b = q - a;           // deflated entries before this one
+            W.defl_val[l + b] = ds[q];
+            W.fcol[l + q] = kp + b;
         }
     }
-    for (int q = 0; q < K; ++q) W.fcol[l + q] = W.org[l + q];
-    W.node_kp[blockIdx.x] = kp;
-    W.node_nrot[blockIdx.x] = nrot;
-    W.node_r[blockIdx.x] = r;
+    if (tid == 0) {
+        W.node_kp[blockIdx.x] = kp;
+        W.node_nrot[blockIdx.x] = n_rot;
+        W.node_r[blockIdx.x] = r;
+    }
 }
 
 // f(tau) = 1 + r sum_i zeta_i^2 / ((delta_i - delta_org) - tau) and its derivative, summed by the
@@ -471,8 +680,30 @@ __device__ __forceinline__ void secular_f(const double* __restrict__ delta, cons
     *fp = r * sp;
 }
 
+// The same in FP32 on differences taken in FP64 (their rounding is relative, so near poles keep their
+// sign and size): two FP64 operations per pole instead of about fifteen.
+__device__ __forceinline__ void secular_f32(const double* __restrict__ delta, const double* __restrict__ zeta, int kp,
+                                            double dorg, double r, float tau, float* f, float* fp) {
+    float s = 0.f, sp = 0.f;
+    const float rf = (float)r;
+    for (int i = threadIdx.x & 31; i < kp; i += 32) {
+        const float q = __fdividef(1.f, (float)(delta[i] - dorg) - tau), z = (float)zeta[i];
+        const float zq = z * z * rf * q;
+        s += zq;
+        sp = fmaf(zq, q, sp);
+    }
+    for (int o = 16; o; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        sp += __shfl_xor_sync(0xffffffffu, sp, o);
+    }
+    *f = 1.f + s;
+    *fp = sp;
+}
+
 // One warp per root (eight per block): bracket between the poles, Newton steps kept inside the
-// bracket, else bisection; stops when the bracket is at the rounding level of tau.
+// bracket, else bisection; stops when the bracket is at the rounding level of tau.  The first steps,
+// to about 1e-5 of tau, run in FP32; they only choose where the FP64 iteration starts, whose bracket
+// and stopping rules are its own.
 __global__ void __launch_bounds__(256) dc_secular_kernel(const DcNode* __restrict__ nodes, DcWork W) {
     const DcNode nd = nodes[blockIdx.y];
     const int l = nd.l, kp = W.node_kp[blockIdx.y];
@@ -499,6 +730,20 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcNode* __restric
     }
     const double dorg = delta[org];
     double t = 0.5 * (lo + hi);
+    {
+        float flo = (float)lo, fhi = (float)hi, x = (float)t;
+        for (int it = 0; it < 24; ++it) {
+            float f, fp;
+            secular_f32(delta, zeta, kp, dorg, r, x, &f, &fp);
+            if (f > 0.f) fhi = x; else flo = x;
+            float xn = x - f / fp;
+            if (!(xn > flo && xn < fhi) || (fabsf(xn - x) > 0.5f * (fhi - flo) && it > 2)) xn = 0.5f * (flo + fhi);
+            const bool close = fabsf(xn - x) <= 1e-5f * fabsf(x);
+            x = xn;
+            if (close || !isfinite(xn)) break;
+        }
+        if (isfinite(x) && (double)x > lo && (double)x < hi) t = (double)x;
+    }
     for (int it = 0; it < 200; ++it) {
         double f, fp;
         secular_f(delta, zeta, kp, dorg, r, t, &f, &fp);
@@ -522,23 +767,25 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcNode* __restric
 
 // Loewner's formula: zh_i^2 = (lambda_last - delta_i) / r  prod_{j < i} (lambda_j - delta_i) / (delta_j - delta_i)
 //                              prod_{i <= j < last} (lambda_j - delta_i) / (delta_{j+1} - delta_i)
-__global__ void __launch_bounds__(128) dc_loewner_kernel(const DcNode* __restrict__ nodes, DcWork W) {
+// One warp per pole (eight per block): the lanes take the factors j, j + 32, ...
+__global__ void __launch_bounds__(256) dc_loewner_kernel(const DcNode* __restrict__ nodes, DcWork W) {
     const DcNode nd = nodes[blockIdx.y];
     const int l = nd.l, kp = W.node_kp[blockIdx.y];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= kp) return;
     const double r = W.node_r[blockIdx.y];
     const double* delta = W.delta + l;
     const int* org = W.org + l;
     const double* tau = W.tau + l;
     const double di = delta[i];
-    double acc = ((delta[org[kp - 1]] - di) + tau[kp - 1]) / r;
-    for (int j = 0; j < kp - 1; ++j) {
+    double acc = lane == 0 ? ((delta[org[kp - 1]] - di) + tau[kp - 1]) / r : 1.0;
+    for (int j = lane; j < kp - 1; j += 32) {
         const double num = (delta[org[j]] - di) + tau[j];
         const double den = j < i ? delta[j] - di : delta[j + 1] - di;
         acc *= num / den;
     }
-    W.zh[l + i] = copysign(sqrt(fmax(acc, 0.0)), W.zeta[l + i]);
+    for (int o = 16; o; o >>= 1) acc *= __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) W.zh[l + i] = copysign(sqrt(fmax(acc, 0.0)), W.zeta[l + i]);
 }
 
 // Eigenvectors of D + r z z^T: column j = zh / (delta - lambda_j), normalised; written as rows of
@@ -552,29 +799,38 @@ __global__ void __launch_bounds__(256) dc_vec_kernel(const DcNode* __restrict__ 
     const double* delta = W.delta + l;
     const double* zh = W.zh + l;
     const double dorg = delta[W.org[l + j]], t = W.tau[l + j];
+    double* row = WT + (size_t)(l + j) * n + l;
     double ss = 0.0;
     for (int i = lane; i < kp; i += 32) {
         const double v = zh[i] / ((delta[i] - dorg) - t);
+        row[i] = v;
         ss = fma(v, v, ss);
     }
     ss = warp_sum(ss);
     const double inv = 1.0 / sqrt(ss);
-    double* row = WT + (size_t)(l + j) * n + l;
-    for (int i = lane; i < kp; i += 32) row[i] = inv * (zh[i] / ((delta[i] - dorg) - t));
+    for (int i = lane; i < kp; i += 32) row[i] *= inv;
 }
 
-// Gathered eigenvector matrix of the halves: G[row][fcol[q]] = QA[row][l + perm[q]], then the
-// deflation rotations on its columns, in order.  One thread per row of the node.
-__global__ void __launch_bounds__(128) dc_gather_kernel(const DcNode* __restrict__ nodes, DcWork W, int n,
+// Gathered eigenvector matrix of the halves: G[row][fcol[q]] = QA[row][l + perm[q]], one warp per row.
+__global__ void __launch_bounds__(256) dc_gather_kernel(const DcNode* __restrict__ nodes, DcWork W, int n,
                                                         const double* __restrict__ QA, double* __restrict__ G) {
     const DcNode nd = nodes[blockIdx.y];
     const int l = nd.l, K = nd.r - nd.l;
-    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (row >= K) return;
     const double* src = QA + (size_t)(l + row) * n + l;
     double* dst = G + (size_t)(l + row) * n + l;
-    for (int q = 0; q < K; ++q) dst[W.fcol[l + q]] = src[W.perm[l + q]];
-    const int nrot = W.node_nrot[blockIdx.y];
+    for (int q = threadIdx.x & 31; q < K; q += 32) dst[W.fcol[l + q]] = src[W.perm[l + q]];
+}
+
+// The deflation rotations on the gathered columns, in order (few matrices have any).  One thread per row.
+__global__ void __launch_bounds__(128) dc_rotate_kernel(const DcNode* __restrict__ nodes, DcWork W, int n,
+                                                        double* __restrict__ G) {
+    const DcNode nd = nodes[blockIdx.y];
+    const int l = nd.l, K = nd.r - nd.l, nrot = W.node_nrot[blockIdx.y];
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (nrot == 0 || row >= K) return;
+    double* dst = G + (size_t)(l + row) * n + l;
     for (int k = 0; k < nrot; ++k) {
         const int cp = W.fcol[l + W.rot_p[l + k]], ci = W.fcol[l + W.rot_i[l + k]];
         const double c = W.rot_c[l + k], s = W.rot_s[l + k];
@@ -584,38 +840,77 @@ __global__ void __launch_bounds__(128) dc_gather_kernel(const DcNode* __restrict
     }
 }
 
-// Final order of a node's eigenvalues: roots (ascending) merged with the deflated values
-// (insertion-sorted first: they arrive nearly in order).  Thread 0 per node.
-__global__ void dc_order_kernel(const DcNode* __restrict__ nodes, DcWork W) {
-    if (threadIdx.x) return;
+// New eigenvectors of the small nodes of a level in one launch: columns j < kp of X = G WT^T, the
+// deflated ones copied.  32 x 32 tiles, grid (tiles, tiles, nodes), 2 x 2 outputs per thread.
+constexpr int kMergeBatch = 256;        // largest node of the batched form
+__global__ void __launch_bounds__(256) dc_merge_kernel(const DcNode* __restrict__ nodes, DcWork W, int n,
+                                                       const double* __restrict__ G, const double* __restrict__ WT,
+                                                       double* __restrict__ X) {
+    const DcNode nd = nodes[blockIdx.z];
+    const int l = nd.l, K = nd.r - nd.l, kp = W.node_kp[blockIdx.z];
+    const int bm = blockIdx.y * 32, bn = blockIdx.x * 32;
+    if (bm >= K || bn >= K) return;
+    __shared__ double As[16][33], Bs[16][33];
+    const size_t off = (size_t)l * n + l;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double acc[2][2] = {};
+    if (bn < kp)
+        for (int k0 = 0; k0 < kp; k0 += 16) {
+            for (int q = threadIdx.x; q < 512; q += 256) {
+                const int m = q >> 4, k = q & 15;
+                As[k][m] = (bm + m < K && k0 + k < kp) ? G[off + (size_t)(bm + m) * n + k0 + k] : 0.0;
+                Bs[k][m] = (bn + m < kp && k0 + k < kp) ? WT[off + (size_t)(bn + m) * n + k0 + k] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) acc[i][j] = fma(As[k][ty + 16 * i], Bs[k][tx + 16 * j], acc[i][j]);
+            __syncthreads();
+        }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int row = bm + ty + 16 * i, col = bn + tx + 16 * j;
+            if (row >= K || col >= K) continue;
+            const size_t at = off + (size_t)row * n + col;
+            X[at] = col < kp ? acc[i][j] : G[at];
+        }
+}
+
+// Final order of a node's eigenvalues: roots (ascending) merged with the deflated values, every entry
+// by its rank.  One block per node.
+__global__ void __launch_bounds__(kPrepThreads) dc_order_kernel(const DcNode* __restrict__ nodes, DcWork W) {
     const DcNode nd = nodes[blockIdx.x];
     const int l = nd.l, K = nd.r - nd.l, kp = W.node_kp[blockIdx.x];
     const int nd_ = K - kp;
-    double* dv = W.defl_val + l;
-    int* idx = W.perm + l;                 // reused: deflated order (column offsets)
-    for (int q = 0; q < nd_; ++q) idx[q] = q;
-    for (int q = 1; q < nd_; ++q) {
-        const int x = idx[q];
-        const double v = dv[x];
-        int p = q - 1;
-        while (p >= 0 && dv[idx[p]] > v) {
-            idx[p + 1] = idx[p];
-            --p;
-        }
-        idx[p + 1] = x;
-    }
+    const double* dv = W.defl_val + l;
     const double* root = W.root + l;
-    int a = 0, b = 0, o = 0;
-    while (a < kp || b < nd_) {
-        const bool tr = b >= nd_ || (a < kp && root[a] <= dv[idx[b]]);
-        if (tr) {
-            W.lam_out[l + o] = root[a];
-            W.oper[l + o] = a++;
-        } else {
-            W.lam_out[l + o] = dv[idx[b]];
-            W.oper[l + o] = kp + idx[b++];
+    double* sorted = W.delta + l;          // the poles are not needed any more
+    int* idx = W.perm + l;
+    for (int q = threadIdx.x; q < nd_; q += kPrepThreads) {
+        const double x = dv[q];
+        int rank = 0;
+        for (int p = 0; p < nd_; ++p) rank += dv[p] < x || (dv[p] == x && p < q);
+        sorted[rank] = x;
+        idx[rank] = q;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < K; q += kPrepThreads) {
+        const bool is_root = q < kp;
+        const double x = is_root ? root[q] : sorted[q - kp];
+        const double* other = is_root ? sorted : root;
+        int lo = 0, hi = is_root ? nd_ : kp;
+        while (lo < hi) {                  // ties: roots first
+            const int mid = (lo + hi) / 2;
+            if (is_root ? other[mid] < x : other[mid] <= x) lo = mid + 1; else hi = mid;
         }
-        ++o;
+        const int o = (is_root ? q : q - kp) + lo;
+        W.lam_out[l + o] = x;
+        W.oper[l + o] = is_root ? q : kp + idx[q - kp];
     }
 }
 
@@ -632,29 +927,42 @@ __global__ void __launch_bounds__(256) dc_permute_kernel(const DcNode* __restric
 }
 
 // ------------------------------------------------------- back-transformation
-// Rows j of Wt (nb x n): u_{k0 + j} (zeros up to column k0 + j, then v_k from row k0 + j of A).
-__global__ void wy_rows_kernel(const double* __restrict__ A, int n, int k0, int nb, double* __restrict__ Wt) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (c >= n || j >= nb) return;
-    const int k = k0 + j;
-    Wt[(size_t)j * n + c] = c <= k ? 0.0 : A[(size_t)k * n + c];
+// Rows k of Wt (nref x n): u_k (zeros up to column k, then v_k from row k of A).
+__global__ void wy_rows_kernel(const double* __restrict__ A, int n, int nref, double* __restrict__ Wt) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (c >= n || k >= nref) return;
+    Wt[(size_t)k * n + c] = c <= k ? 0.0 : A[(size_t)k * n + c];
 }
 
-// T (nb x nb, upper) of H_{k0} ... H_{k0+nb-1} = I - W T W^T from S = Wt Wt^T:
-// T[j][j] = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] S[0:j, j].  One thread.
-__global__ void wy_t_kernel(const double* __restrict__ S, const double* __restrict__ tau, int k0, int nb,
-                            double* __restrict__ T) {
-    if (threadIdx.x || blockIdx.x) return;
-    for (int i = 0; i < nb * nb; ++i) T[i] = 0.0;
+// T (upper triangular, pitch kWyBlock) of H_{k0} ... H_{k0+nb-1} = I - W T W^T from S = Wt Wt^T:
+// T[j][j] = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] S[0:j, j].  One block per group of reflectors (all
+// groups in one launch), thread i holds row i of T in shared memory; four partial sums per entry.
+__global__ void __launch_bounds__(kWyBlock) wy_t_kernel(const double* __restrict__ S_all, const double* __restrict__ tau,
+                                                        int nref, double* __restrict__ T_all) {
+    extern __shared__ double t[];                         // [kWyBlock][kWyBlock + 1]
+    __shared__ double sj[kWyBlock];
+    constexpr int P = kWyBlock + 1;
+    const int k0 = blockIdx.x * kWyBlock, nb = min(kWyBlock, nref - k0), i = threadIdx.x;
+    const double* S = S_all + (size_t)blockIdx.x * kWyBlock * kWyBlock;
+    double* T = T_all + (size_t)blockIdx.x * kWyBlock * kWyBlock;
     for (int j = 0; j < nb; ++j) {
         const double tj = tau[k0 + j];
-        for (int i = 0; i < j; ++i) {
-            double acc = 0.0;
-            for (int q = i; q < j; ++q) acc = fma(T[i * nb + q], S[q * nb + j], acc);
-            T[i * nb + j] = -tj * acc;
+        __syncthreads();
+        if (i < j) sj[i] = S[(size_t)i * kWyBlock + j];
+        __syncthreads();
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        if (i < j) {
+            int q = i;
+            for (; q + 3 < j; q += 4)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) a[u] = fma(t[i * P + q + u], sj[q + u], a[u]);
+            for (; q < j; ++q) a[0] = fma(t[i * P + q], sj[q], a[0]);
         }
-        T[j * nb + j] = tj;
+        if (i < nb) t[i * P + j] = i < j ? -tj * ((a[0] + a[1]) + (a[2] + a[3])) : (i == j ? tj : 0.0);
     }
+    __syncthreads();
+    for (int j = 0; j < nb; ++j)
+        if (i < nb) T[(size_t)j * kWyBlock + i] = t[j * P + i];
 }
 
 }  // namespace
@@ -663,6 +971,7 @@ __global__ void wy_t_kernel(const double* __restrict__ S, const double* __restri
 void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err) {
     if (n <= 0) return;
     DBuf<double> d, e, tau, vk, p;
+    DBuf<unsigned> bar;
     d.alloc(n);
     e.alloc(n);
     tau.alloc(n);
@@ -674,29 +983,48 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         allow_dyn_smem(trd_small_kernel, sh);
         trd_small_kernel<<<1, 1024, sh, s>>>(A, n, d.p, e.p, tau.p);
     } else {
-        for (int k = 0; k + 2 < n; ++k) {
-            const int m = n - k - 1;
-            trd_house_kernel<<<1, 1024, 0, s>>>(A, n, k, vk.p, d.p, e.p, tau.p);
-            trd_symv_kernel<<<(m + 7) / 8, 256, 0, s>>>(A, n, k, vk.p, tau.p, p.p);
-            trd_w_kernel<<<1, 1024, 0, s>>>(n, k, vk.p, tau.p, p.p);
-            trd_syr2_kernel<<<dim3((m + 255) / 256, (m + 3) / 4), 256, 0, s>>>(A, n, k, vk.p, p.p);
+        int dev = 0, n_sm = 0, optin = 0;
+        WT_CUDA(cudaGetDevice(&dev));
+        WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+        WT_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        const size_t sh = 3 * (size_t)n * sizeof(double);
+        if (sh + 1024 <= (size_t)optin) {
+            allow_dyn_smem(trd_kernel, sh);
+            bar.alloc(2);
+            bar.zero(s);
+            p.alloc(2 * (size_t)n);
+            // about one row per warp: more blocks than that only lengthen the barrier
+            int blocks = std::max(1, std::min(n_sm, (n + 7) / 8)), nn = n;
+            void* args[] = {&A, &nn, &d.p, &e.p, &tau.p, &p.p, &bar.p, &d_err};
+            WT_CUDA(cudaLaunchCooperativeKernel((const void*)trd_kernel, dim3(blocks), dim3(kTrdThreads), args, sh, s));
+        } else {
+            for (int k = 0; k + 2 < n; ++k) {
+                const int m = n - k - 1;
+                trd_house_kernel<<<1, 1024, 0, s>>>(A, n, k, vk.p, d.p, e.p, tau.p);
+                trd_symv_kernel<<<(m + 7) / 8, 256, 0, s>>>(A, n, k, vk.p, tau.p, p.p);
+                trd_w_kernel<<<1, 1024, 0, s>>>(n, k, vk.p, tau.p, p.p);
+                trd_syr2_kernel<<<dim3((m + 255) / 256, (m + 3) / 4), 256, 0, s>>>(A, n, k, vk.p, p.p);
+            }
+            trd_tail_kernel<<<1, 32, 0, s>>>(A, n, d.p, e.p, tau.p);
         }
-        trd_tail_kernel<<<1, 32, 0, s>>>(A, n, d.p, e.p, tau.p);
     }
     WT_LAUNCH("tridiagonalisation");
     vk.release();
-    p.release();
 
-    // 2. divide and conquer: tree by halving, leaves <= kLeaf rows
+    // 2. divide and conquer: tree by halving
     std::vector<int> leaves;            // starts, plus n
     std::vector<std::vector<DcNode>> levels;
     std::vector<int> splits;
     struct Item { int l, r, depth; };
     std::vector<Item> stack{{0, n, 0}};
+    // every node is split down to the same depth (sizes of a level differ by one at most), so every
+    // level merges all rows
+    int depth = 0;
+    while (((n - 1) >> depth) + 1 > kLeaf) ++depth;
     while (!stack.empty()) {
         const Item it = stack.back();
         stack.pop_back();
-        if (it.r - it.l <= kLeaf) {
+        if (it.depth == depth) {
             leaves.push_back(it.l);
             continue;
         }
@@ -762,53 +1090,53 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         Wk.lam_out = fbuf.p + 9 * nn;
         Wk.node_r = fbuf.p + 10 * nn;
         DBuf<DcNode> dnodes;
+        std::vector<DcNode> all;
+        std::vector<size_t> level_at;
+        for (const auto& nodes : levels) {
+            level_at.push_back(all.size());
+            all.insert(all.end(), nodes.begin(), nodes.end());
+        }
+        dnodes.upload(all.data(), all.size(), s);
         double *qa = QA.p, *qb = QB.p, *la = lamA.p, *lb = lamB.p;
         for (int lev = (int)levels.size() - 1; lev >= 0; --lev) {
             const std::vector<DcNode>& nodes = levels[lev];
             const int nn_ = (int)nodes.size();
-            dnodes.upload(nodes.data(), nodes.size(), s);
+            const DcNode* dn = dnodes.p + level_at[lev];
             int kmax = 0;
             for (const DcNode& nd : nodes) kmax = std::max(kmax, nd.r - nd.l);
-            dc_prep_kernel<<<nn_, 256, 0, s>>>(dnodes.p, e.p, la, qa, n, Wk, zbuf.p);
+            dc_prep_kernel<<<nn_, kPrepThreads, 0, s>>>(dn, e.p, la, qa, n, Wk, zbuf.p);
             WT_LAUNCH("dc_prep");
-            dc_secular_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dnodes.p, Wk);
+            dc_secular_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dn, Wk);
             WT_LAUNCH("dc_secular");
-            dc_loewner_kernel<<<dim3((kmax + 127) / 128, nn_), 128, 0, s>>>(dnodes.p, Wk);
+            dc_loewner_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dn, Wk);
             WT_LAUNCH("dc_loewner");
-            dc_vec_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dnodes.p, Wk, n, WT.p);
+            dc_vec_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dn, Wk, n, WT.p);
             WT_LAUNCH("dc_vec");
-            dc_gather_kernel<<<dim3((kmax + 127) / 128, nn_), 128, 0, s>>>(dnodes.p, Wk, n, qa, G.p);
+            dc_gather_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dn, Wk, n, qa, G.p);
+            dc_rotate_kernel<<<dim3((kmax + 127) / 128, nn_), 128, 0, s>>>(dn, Wk, n, G.p);
             WT_LAUNCH("dc_gather");
-            std::vector<int> kp(nn_);
-            WT_CUDA(cudaMemcpyAsync(kp.data(), Wk.node_kp, nn_ * sizeof(int), cudaMemcpyDeviceToHost, s));
-            WT_CUDA(cudaStreamSynchronize(s));
-            for (int q = 0; q < nn_; ++q) {
-                const DcNode& nd = nodes[q];
-                const int K = nd.r - nd.l, k1 = kp[q];
-                const size_t off = (size_t)nd.l * n + nd.l;
-                if (k1 > 0) dgemm(s, false, true, K, k1, k1, 1.0, G.p + off, n, WT.p + off, n, 0.0, qa + off, n);
-                if (K > k1) copy_block(s, G.p + off + k1, n, qa + off + k1, n, K, K - k1);
+            if (kmax <= kMergeBatch) {
+                const int tiles = (kmax + 31) / 32;
+                dc_merge_kernel<<<dim3(tiles, tiles, nn_), 256, 0, s>>>(dn, Wk, n, G.p, WT.p, qa);
+                WT_LAUNCH("dc_merge");
+            } else {
+                std::vector<int> kp(nn_);
+                WT_CUDA(cudaMemcpyAsync(kp.data(), Wk.node_kp, nn_ * sizeof(int), cudaMemcpyDeviceToHost, s));
+                WT_CUDA(cudaStreamSynchronize(s));
+                for (int q = 0; q < nn_; ++q) {
+                    const DcNode& nd = nodes[q];
+                    const int K = nd.r - nd.l, k1 = kp[q];
+                    const size_t off = (size_t)nd.l * n + nd.l;
+                    if (k1 > 0) dgemm(s, false, true, K, k1, k1, 1.0, G.p + off, n, WT.p + off, n, 0.0, qa + off, n);
+                    if (K > k1) copy_block(s, G.p + off + k1, n, qa + off + k1, n, K, K - k1);
+                }
             }
-            dc_order_kernel<<<nn_, 32, 0, s>>>(dnodes.p, Wk);
+            dc_order_kernel<<<nn_, kPrepThreads, 0, s>>>(dn, Wk);
             WT_LAUNCH("dc_order");
-            dc_permute_kernel<<<dim3((kmax + 255) / 256, kmax, nn_), 256, 0, s>>>(dnodes.p, Wk, n, qa, qb, lb);
+            dc_permute_kernel<<<dim3((kmax + 255) / 256, kmax, nn_), 256, 0, s>>>(dn, Wk, n, qa, qb, lb);
             WT_LAUNCH("dc_permute");
-            // rows and eigenvalues of the leaves/nodes not merged at this level carry over
-            WT_CUDA(cudaStreamSynchronize(s));
             std::swap(qa, qb);
             std::swap(la, lb);
-            // untouched blocks: copy the ones that did not take part (nodes of shallower leaves)
-            std::vector<char> cov(n, 0);
-            for (const DcNode& nd : nodes)
-                for (int i = nd.l; i < nd.r; ++i) cov[i] = 1;
-            for (int i = 0; i < n;) {
-                if (cov[i]) { ++i; continue; }
-                int j = i;
-                while (j < n && !cov[j]) ++j;
-                copy_block(s, qb + (size_t)i * n + i, n, qa + (size_t)i * n + i, n, j - i, j - i);
-                WT_CUDA(cudaMemcpyAsync(la + i, lb + i, (j - i) * sizeof(double), cudaMemcpyDeviceToDevice, s));
-                i = j;
-            }
         }
         if (qa != QA.p) {
             copy_block(s, qa, n, QA.p, n, n, n);
@@ -824,23 +1152,31 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
     const int nref = std::max(0, n - 2);
     if (nref > 0) {
         DBuf<double> Wt, S, T, Y, Y2;
-        Wt.alloc((size_t)kWyBlock * n);
-        S.alloc((size_t)kWyBlock * kWyBlock);
-        T.alloc((size_t)kWyBlock * kWyBlock);
+        const int nblk = (nref + kWyBlock - 1) / kWyBlock;
+        constexpr size_t tt = (size_t)kWyBlock * kWyBlock;
+        Wt.alloc((size_t)nref * n);
+        S.alloc(nblk * tt);
+        T.alloc(nblk * tt);
         Y.alloc((size_t)kWyBlock * n);
         Y2.alloc((size_t)kWyBlock * n);
-        const int nblk = (nref + kWyBlock - 1) / kWyBlock;
+        wy_rows_kernel<<<dim3((n + 255) / 256, nref), 256, 0, s>>>(A, n, nref, Wt.p);
+        WT_LAUNCH("wy_rows");
+        for (int bi = 0; bi < nblk; ++bi) {
+            const int k0 = bi * kWyBlock, nb = std::min(kWyBlock, nref - k0), m = n - k0 - 1;
+            const double* W0 = Wt.p + (size_t)k0 * n + k0 + 1;
+            dgemm(s, false, true, nb, nb, m, 1.0, W0, n, W0, n, 0.0, S.p + bi * tt, kWyBlock);
+        }
+        const size_t sh = (size_t)kWyBlock * (kWyBlock + 1) * sizeof(double);
+        allow_dyn_smem(wy_t_kernel, sh);
+        wy_t_kernel<<<nblk, kWyBlock, sh, s>>>(S.p, tau.p, nref, T.p);
+        WT_LAUNCH("wy_t");
         for (int bi = nblk - 1; bi >= 0; --bi) {
             const int k0 = bi * kWyBlock, nb = std::min(kWyBlock, nref - k0);
             const int m = n - k0 - 1;           // rows k0 + 1 .. n - 1
-            wy_rows_kernel<<<dim3((n + 255) / 256, nb), 256, 0, s>>>(A, n, k0, nb, Wt.p);
-            WT_LAUNCH("wy_rows");
-            dgemm(s, false, true, nb, nb, m, 1.0, Wt.p + k0 + 1, n, Wt.p + k0 + 1, n, 0.0, S.p, nb);
-            wy_t_kernel<<<1, 32, 0, s>>>(S.p, tau.p, k0, nb, T.p);
-            WT_LAUNCH("wy_t");
-            dgemm(s, false, false, nb, n, m, 1.0, Wt.p + k0 + 1, n, Z + (size_t)(k0 + 1) * n, n, 0.0, Y.p, n);
-            dgemm(s, false, false, nb, n, nb, 1.0, T.p, nb, Y.p, n, 0.0, Y2.p, n);
-            dgemm(s, true, false, m, n, nb, -1.0, Wt.p + k0 + 1, n, Y2.p, n, 1.0, Z + (size_t)(k0 + 1) * n, n);
+            const double* W0 = Wt.p + (size_t)k0 * n + k0 + 1;
+            dgemm(s, false, false, nb, n, m, 1.0, W0, n, Z + (size_t)(k0 + 1) * n, n, 0.0, Y.p, n);
+            dgemm(s, false, false, nb, n, nb, 1.0, T.p + bi * tt, kWyBlock, Y.p, n, 0.0, Y2.p, n);
+            dgemm(s, true, false, m, n, nb, -1.0, W0, n, Y2.p, n, 1.0, Z + (size_t)(k0 + 1) * n, n);
         }
     }
     copy_block(s, Z, n, V, n, n, n);
