@@ -70,53 +70,69 @@ __global__ void __launch_bounds__(256) features_kernel(const float* __restrict__
     for (int q = 0; q < 3; ++q) jl[q] = warp_max_int(jl[q]);
     const double sd = (double)s;
     auto Y = [&](int m) { return sd * (double)row[m]; };
-    const double fq[3] = {(double)fr.x, (double)fr.y, (double)fr.z};
-    if (lane == 0) {
+    // the FP64 expressions spread over the lanes: a warp instruction costs the FP64 units the same for
+    // one lane as for 32 (20 000 waveforms x 200 samples with four tangents: 721 -> 239 us)
+    const double den = (k > 0 && k < n - 1) ? Y(k - 1) - 2.0 * Y(k) + Y(k + 1) : 0.0;
+    if (lane < 4) {                                      // lane 0 the peak, 1..3 the crossings
         double* o = f + (size_t)tr * kNF;
-        double delta = 0.0;
-        if (k > 0 && k < n - 1) {
-            const double den = Y(k - 1) - 2.0 * Y(k) + Y(k + 1);
-            if (den != 0.0) delta = (Y(k - 1) - Y(k + 1)) / (2.0 * den);
+        const int q = lane - 1, j = lane == 0 ? -1 : (q == 0 ? jl[0] : q == 1 ? jl[1] : jl[2]);
+        const float l = q <= 0 ? lv[0] : q == 1 ? lv[1] : lv[2];
+        double num, d;
+        if (lane == 0) {
+            num = den != 0.0 ? Y(k - 1) - Y(k + 1) : 0.0;
+            d = den != 0.0 ? 2.0 * den : 1.0;
+        } else {
+            num = j < 0 ? 0.0 : (double)l - Y(j);
+            d = j < 0 ? 1.0 : Y(j + 1) - Y(j);
         }
-        o[0] = (double)A;
-        o[1] = t0 + dt * ((double)k + delta);
-        o[2] = dt * sum;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int j = jl[q];
-            o[3 + q] = j < 0 ? t0 : t0 + dt * ((double)j + ((double)lv[q] - Y(j)) / (Y(j + 1) - Y(j)));
+        const double quot = num / d;
+        if (lane == 0) {
+            o[0] = (double)A;
+            o[1] = t0 + dt * ((double)k + quot);
+            o[2] = dt * sum;
+        } else {
+            o[2 + lane] = j < 0 ? t0 : t0 + dt * ((double)j + quot);
         }
     }
-    for (int d = 0; d < n_dir; ++d) {
-        const float* drow = dx + ((size_t)d * n_tracks + tr) * n;
-        double dsum = 0.0;
-        for (int m = lane; m < n; m += 32) dsum += (double)drow[m];
-        dsum = warp_sum(dsum);
-        if (lane == 0) {
+    if (n_dir == 0) return;
+    for (int d0 = 0; d0 < n_dir; d0 += 8) {              // lane = 4 d + part: the peak or a crossing of tangent d
+        const int nd = min(8, n_dir - d0);
+        double mysum = 0.0;
+        for (int d = 0; d < nd; ++d) {
+            const float* drow = dx + ((size_t)(d0 + d) * n_tracks + tr) * n;
+            double dsum = 0.0;
+            for (int m = lane; m < n; m += 32) dsum += (double)drow[m];
+            dsum = warp_sum(dsum);
+            if (lane >> 2 == d) mysum = dsum;
+        }
+        const int d = lane >> 2, part = lane & 3;
+        if (d < nd) {
+            const float* drow = dx + ((size_t)(d0 + d) * n_tracks + tr) * n;
+            double* o = df + ((size_t)(d0 + d) * n_tracks + tr) * kNF;
             auto dY = [&](int m) { return sd * (double)drow[m]; };
-            double* o = df + ((size_t)d * n_tracks + tr) * kNF;
-            double dpk = 0.0;
-            if (k > 0 && k < n - 1) {
-                const double den = Y(k - 1) - 2.0 * Y(k) + Y(k + 1);
+            const int q = part - 1, j = part == 0 ? -1 : (q == 0 ? jl[0] : q == 1 ? jl[1] : jl[2]);
+            const float l = q <= 0 ? lv[0] : q == 1 ? lv[1] : lv[2];
+            double num = 0.0, dd = 1.0;
+            if (part == 0) {
                 if (den != 0.0) {
-                    const double num = Y(k - 1) - Y(k + 1);
+                    const double pn = Y(k - 1) - Y(k + 1);
                     const double dnum = dY(k - 1) - dY(k + 1);
                     const double dden = dY(k - 1) - 2.0 * dY(k) + dY(k + 1);
-                    dpk = dt * (dnum * den - num * dden) / (2.0 * den * den);
+                    num = dt * (dnum * den - pn * dden);
+                    dd = 2.0 * den * den;
                 }
+            } else if (j >= 0) {
+                const double e = Y(j + 1) - Y(j), fq = q == 0 ? (double)fr.x : q == 1 ? (double)fr.y : (double)fr.z;
+                num = dt * ((fq * dY(k) - dY(j)) * e - ((double)l - Y(j)) * (dY(j + 1) - dY(j)));
+                dd = e * e;
             }
-            o[0] = (double)drow[k];
-            o[1] = dpk;
-            o[2] = dt * dsum;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int j = jl[q];
-                double v = 0.0;
-                if (j >= 0) {
-                    const double dd = Y(j + 1) - Y(j);
-                    v = dt * ((fq[q] * dY(k) - dY(j)) * dd - ((double)lv[q] - Y(j)) * (dY(j + 1) - dY(j))) / (dd * dd);
-                }
-                o[3 + q] = v;
+            const double quot = num / dd;
+            if (part == 0) {
+                o[0] = (double)drow[k];
+                o[1] = quot;
+                o[2] = dt * mysum;
+            } else {
+                o[2 + part] = quot;
             }
         }
     }
