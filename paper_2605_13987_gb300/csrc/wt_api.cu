@@ -39,10 +39,9 @@ void add_column_vector(cudaStream_t, double*, int, int, const double*);
 void to_float(cudaStream_t, const double*, size_t, double, float*);
 void check_finite(cudaStream_t, const double*, size_t, int*);
 void expand_simt(cudaStream_t, const float*, int, const float*, int, int, size_t, float*);
-void sample_lateral(cudaStream_t, const double*, int, const double*, int, int, int, int, double, double,
-                    const double*, double*);
-void sample_contract(cudaStream_t, const double*, const double*, const double*, int, int, int, int, double, double,
-                     double*);
+void sample_points(cudaStream_t, const double*, int, const double*, const double*, const int*, int, int, int, int, int,
+                   double, double, double, double, const double*, const double*, int, double*, double*, double*,
+                   double*);
 void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, double, const float*, const float*,
                 const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
                 double, const void*, int, float*);
@@ -1189,15 +1188,32 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
     column_ztransform<double>(s, Qt.p, nt, ns, ns, c->zcos.p, c->d_col_off.p, ncol, g.Nz, Zc.p);
     T.alloc((size_t)(g.Nx / 2) * (g.Ny / 2) * g.Nz);
     green_invk2(s, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, T.p);
-    const int chunk = 512;
-    Lat.alloc((size_t)std::min(n, chunk) * ncol * g.Nz * 3);
-    o.alloc((size_t)nt * std::min(n, chunk) * 3);
+    // distinct column x coordinates
+    std::vector<double> hux;
+    std::vector<int> hcu(ncol);
+    for (int k = 0; k < ncol; ++k) {
+        const double x = c->cols[k].x;
+        hcu[k] = (int)(std::find(hux.begin(), hux.end(), x) - hux.begin());
+        if (hcu[k] == (int)hux.size()) hux.push_back(x);
+    }
+    const int nux = (int)hux.size();
+    DBuf<double> ux, F, G;
+    DBuf<int> cu;
+    ux.upload(hux.data(), nux, s);
+    cu.upload(hcu.data(), ncol, s);
+    // points per chunk: 512, fewer where their k_x sums would take more than 1 GB
+    const size_t per_point = (size_t)2 * nux * (g.Ny / 2) * g.Nz * sizeof(double);
+    const int chunk = std::min(n, (int)std::max<size_t>(1, std::min<size_t>(512, ((size_t)1 << 30) / per_point)));
+    F.alloc((size_t)2 * chunk * nux * (g.Nx / 2));
+    G.alloc((size_t)chunk * per_point / sizeof(double));
+    Lat.alloc((size_t)chunk * ncol * g.Nz * 3);
+    o.alloc((size_t)nt * chunk * 3);
     std::vector<double> hbuf;
     for (int p0 = 0; p0 < n; p0 += chunk) {
         const int np = std::min(chunk, n - p0);
         pts.upload(xyz + 3 * (size_t)p0, 3 * (size_t)np, s);
-        sample_lateral(s, pts.p, np, c->sp64.col_xy.p, ncol, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, T.p, Lat.p);
-        sample_contract(s, pts.p, Lat.p, Zc.p, np, nt, ncol, g.Nz, g.Lz, c->pref, o.p);
+        sample_points(s, pts.p, np, c->sp64.col_xy.p, ux.p, cu.p, ncol, nux, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz,
+                      c->pref, T.p, Zc.p, nt, F.p, G.p, Lat.p, o.p);
         hbuf.resize((size_t)nt * np * 3);
         o.download(hbuf.data(), hbuf.size(), s);
         WT_CUDA(cudaStreamSynchronize(s));
