@@ -1,0 +1,81 @@
+// FP64 helpers with short dependent chains, and the barrier of cooperative launches (k_dense.cu,
+// k_eigen.cu).
+#pragma once
+
+#include "wt_internal.cuh"
+
+namespace wt {
+
+// 1 / sqrt(x) of a positive x by Newton's iteration y <- y + y (1 - x y^2) / 2 from the FP32 value (24
+// bits, 46, then the FP64 rounding level), x normalised by its exponent.  A chain of about ten FP64
+// operations, each of which costs a warp 16 cycles of GB300's FP64 units.
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
+    const int e = (ex - 1023) & ~1;                            // x = m 2^e, 1 <= m < 4
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
+    double y = (double)rsqrtf((float)m);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
+}
+// 1 / x likewise, y <- y + y (1 - x y).
+__device__ __forceinline__ double rcp_newton(double x) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+    if (ex <= 2 || ex >= 0x7fd) return 1.0 / x;
+    const int e = ex - 1023;
+    const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
+    double y = (double)__frcp_rn((float)m);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) y = fma(y, fma(-m, y, 1.0), y);
+    return __hiloint2double(__double2hiint(y) - (e << 20), __double2loint(y));
+}
+
+// Barrier of the co-resident blocks of a cooperative launch: `round` counts them from 1.  bar:
+// kBarrierWords words, zeroed before the launch (a counter that every block adds to, and a word that says
+// that a block has given up, after two seconds: error word set, and everybody leaves).  A flag per block,
+// every block polling all of them, measured slower (152 blocks: 3 us more).
+constexpr unsigned long long kGridWaitNs = 2000000000ull;
+constexpr int kBarrierWords = 2;
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int* err) {
+    __syncthreads();
+    __shared__ int ok_sh;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const unsigned want = round * gridDim.x;
+        volatile unsigned* vb = bar;
+        volatile unsigned* gone = bar + 1;
+        int ok = 1;
+        if (*vb < want) {
+            unsigned long long t0, t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+            while (*vb < want) {
+                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+                if (t - t0 > 20000 && *gone) { ok = 0; break; }
+                if (t - t0 > kGridWaitNs) {
+                    *gone = 1;
+                    atomicMax(err, (int)DERR_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        ok_sh = ok;
+    }
+    __syncthreads();
+    return ok_sh != 0;
+}
+
+// Blocks of `kernel` that can be resident at once on the current device.
+template <class K>
+int coresident_blocks(K* kernel, int threads, size_t smem) {
+    int dev = 0, n_sm = 0, per = 0;
+    WT_CUDA(cudaGetDevice(&dev));
+    WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    WT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem));
+    return n_sm * per;
+}
+
+}  // namespace wt

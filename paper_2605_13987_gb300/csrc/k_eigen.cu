@@ -22,7 +22,7 @@
 //      working precision, and one GEMM per merge for the new eigenvectors.
 //   3. Back-transformation V = H_0 H_1 ... H_{n-3} Z in blocks of 128
 //      reflectors (compact WY form I - W T W^T, three GEMMs per block).
-#include "wt_internal.cuh"
+#include "coop.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -61,54 +61,6 @@ __device__ double block_sum(double v, double* sh) {
 }
 
 // ------------------------------------------------------ tridiagonalisation
-// 1 / x and 1 / sqrt(x) by Newton's iteration from the FP32 value (24 -> 48 -> FP64's rounding level):
-// short chains where every FP64 operation costs a warp 16 cycles.  x is normalised by its exponent.
-__device__ __forceinline__ double rsqrt_newton(double x) {
-    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
-    if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
-    const int e = (ex - 1023) & ~1;
-    const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
-    double y = (double)rsqrtf((float)m);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
-    return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
-}
-
-// Barrier of the co-resident blocks of a cooperative launch: `round` counts them.  Gives up after two
-// seconds (or when another block has): error word set, every later barrier passes at once, and the
-// caller leaves.
-constexpr unsigned long long kGridWaitNs = 2000000000ull;
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int* err) {
-    __syncthreads();
-    __shared__ int ok_sh;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        const unsigned want = round * gridDim.x;
-        volatile unsigned* vb = bar;
-        volatile unsigned* gone = bar + 1;
-        int ok = 1;
-        if (*vb < want) {
-            unsigned long long t0, t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-            while (*vb < want) {
-                if (*gone) { ok = 0; break; }
-                asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-                if (t - t0 > kGridWaitNs) {
-                    *gone = 1;
-                    atomicMax(err, (int)DERR_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        ok_sh = ok;
-    }
-    __syncthreads();
-    return ok_sh != 0;
-}
-
 // All columns in one cooperative launch (one block per SM, rows dealt out cyclically, one warp per
 // row).  Step k, with v, w of step k - 1 in shared memory:
 //   every block forms row k of the updated matrix, A[k] - v[k] w - w[k] v, and its reflector (the
@@ -120,7 +72,20 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int*
 // n = 2304 94 ms before.  p alternates between two buffers, so that a block still reading one is not
 // overtaken.  The reflector of step k is written into row k one step later, when no block reads that
 // row any more.
-constexpr int kTrdThreads = 512;
+//
+// The vectors are worked on by the first four warps only, one per SM quarter: a quarter does an FP64
+// warp instruction in 64 cycles, so more warps add nothing to the sums and four times the shuffle steps
+// to the reductions.
+constexpr int kTrdThreads = 512, kTrdVec = 128;
+// sum over the first kTrdVec threads, for all threads of the block (red: 4 values)
+__device__ __forceinline__ double trd_sum(double v, double* red) {
+    if (threadIdx.x < kTrdVec) {
+        v = warp_sum(v);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    }
+    __syncthreads();
+    return (red[0] + red[1]) + (red[2] + red[3]);
+}
 __global__ void __launch_bounds__(kTrdThreads, 1)
     trd_kernel(double* A, int n, double* __restrict__ d, double* __restrict__ e, double* __restrict__ tau_out,
                double* p, unsigned* bar, int* err) {
@@ -128,8 +93,8 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
     double* v = sm;
     double* w = sm + n;
     double* vn = sm + 2 * (size_t)n;
-    __shared__ double red[33];
-    __shared__ double par[4];
+    __shared__ double red[2][4];
+    __shared__ double par[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int T = kTrdThreads, NW = T / 32;
     const int nblk = gridDim.x, blk = blockIdx.x;
@@ -139,12 +104,13 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
         // row k of the current matrix, and the squares below its subdiagonal entry
         const double vk = v[k], wk = w[k];
         double ss = 0.0;
-        for (int j = k + tid; j < n; j += T) {
+        const int vt = tid < kTrdVec ? tid : n;          // the vector threads' start
+        for (int j = k + vt; j < n; j += kTrdVec) {
             const double x = fma(-wk, v[j], fma(-vk, w[j], __ldcg(A + (size_t)k * n + j)));
             vn[j] = x;
             if (j >= k + 2) ss = fma(x, x, ss);
         }
-        ss = block_sum(ss, red);
+        ss = trd_sum(ss, red[0]);
         if (tid == 0) {
             const double x0 = vn[k + 1];
             double t = 0.0, beta = x0, scale = 0.0;
@@ -152,7 +118,7 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
                 const double q = fma(x0, x0, ss), rq = rsqrt_newton(q), nrm = q * rq;
                 beta = -copysign(nrm, x0);
                 t = fma(fabs(x0), rq, 1.0);                    // (beta - x0) / beta
-                scale = 1.0 / (x0 - beta);
+                scale = rcp_newton(x0 - beta);
             }
             par[0] = t;
             par[1] = scale;
@@ -164,7 +130,7 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
         }
         __syncthreads();
         const double t = par[0], scale = par[1];
-        for (int j = k + 1 + tid; j < n; j += T) vn[j] = j == k + 1 ? 1.0 : vn[j] * scale;
+        for (int j = k + 1 + vt; j < n; j += kTrdVec) vn[j] = j == k + 1 ? 1.0 : vn[j] * scale;
         if (k > 0 && (k - 1) % nblk == blk)
             for (int j = k + tid; j < n; j += T) A[(size_t)(k - 1) * n + j] = v[j];
         __syncthreads();
@@ -190,14 +156,14 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
             __syncthreads();
         }
         double sp = 0.0;
-        for (int j = k + 1 + tid; j < n; j += T) {
+        for (int j = k + 1 + vt; j < n; j += kTrdVec) {
             const double x = __ldcg(pk + j);
             w[j] = x;
             sp = fma(x, vn[j], sp);
         }
-        sp = block_sum(sp, red);
+        sp = trd_sum(sp, red[1]);
         const double al = 0.5 * t * sp;
-        for (int j = k + 1 + tid; j < n; j += T) w[j] = fma(-al, vn[j], w[j]);
+        for (int j = k + 1 + vt; j < n; j += kTrdVec) w[j] = fma(-al, vn[j], w[j]);
         double* x = v;
         v = vn;
         vn = x;
@@ -662,22 +628,25 @@ __global__ void __launch_bounds__(kPrepThreads) dc_prep_kernel(const DcNode* __r
     }
 }
 
-// f(tau) = 1 + r sum_i zeta_i^2 / ((delta_i - delta_org) - tau) and its derivative, summed by the
-// 32 lanes of a warp (lane k takes the poles k, k + 32, ...).  The xor butterfly gives every lane
-// the same bits, so the iteration that uses them stays uniform across the warp.
+// f(tau) = 1 + r sum_i zeta_i^2 / ((delta_i - delta_org) - tau), its derivative and the sum of its
+// terms' sizes, summed by the 32 lanes of a warp (lane k takes the poles k, k + 32, ...).  The xor
+// butterfly gives every lane the same bits, so the iteration that uses them stays uniform across the warp.
 __device__ __forceinline__ void secular_f(const double* __restrict__ delta, const double* __restrict__ zeta, int kp,
-                                          double dorg, double r, double tau, double* f, double* fp) {
-    double s = 0.0, sp = 0.0;
+                                          double dorg, double r, double tau, double* f, double* fp, double* size) {
+    double s = 0.0, sp = 0.0, sa = 0.0;
     for (int i = threadIdx.x & 31; i < kp; i += 32) {
-        const double q = 1.0 / ((delta[i] - dorg) - tau);
-        const double z2 = zeta[i] * zeta[i];
-        s = fma(z2, q, s);
-        sp = fma(z2 * q, q, sp);
+        const double q = rcp_newton((delta[i] - dorg) - tau);
+        const double t = zeta[i] * zeta[i] * q;
+        s += t;
+        sa += fabs(t);
+        sp = fma(t, q, sp);
     }
     s = warp_sum(s);
     sp = warp_sum(sp);
+    sa = warp_sum(sa);
     *f = fma(r, s, 1.0);
     *fp = r * sp;
+    *size = fma(r, sa, 1.0);
 }
 
 // The same in FP32 on differences taken in FP64 (their rounding is relative, so near poles keep their
@@ -716,8 +685,8 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcNode* __restric
     double lo, hi;
     if (j < kp - 1) {
         const double gap = delta[j + 1] - delta[j];
-        double f, fp;
-        secular_f(delta, zeta, kp, delta[j], r, 0.5 * gap, &f, &fp);
+        double f, fp, size;
+        secular_f(delta, zeta, kp, delta[j], r, 0.5 * gap, &f, &fp, &size);
         if (f > 0.0) { org = j; lo = 0.0; hi = 0.5 * gap; }
         else { org = j + 1; lo = -0.5 * gap; hi = 0.0; }
     } else {
@@ -745,9 +714,11 @@ __global__ void __launch_bounds__(256) dc_secular_kernel(const DcNode* __restric
         if (isfinite(x) && (double)x > lo && (double)x < hi) t = (double)x;
     }
     for (int it = 0; it < 200; ++it) {
-        double f, fp;
-        secular_f(delta, zeta, kp, dorg, r, t, &f, &fp);
-        if (f == 0.0) { lo = hi = t; break; }
+        double f, fp, size;
+        secular_f(delta, zeta, kp, dorg, r, t, &f, &fp, &size);
+        // f at its own rounding level (the sum of 32 lanes' partial sums): no step beyond this one is
+        // more than noise, and Newton's would wander there until the bracket closed
+        if (fabs(f) <= 2.0 * kEps * size) { lo = hi = t; break; }
         if (f > 0.0) hi = t; else lo = t;
         const double w = hi - lo;
         if (w <= 4.0 * kEps * fmax(fabs(lo), fabs(hi))) break;
@@ -990,7 +961,7 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         const size_t sh = 3 * (size_t)n * sizeof(double);
         if (sh + 1024 <= (size_t)optin) {
             allow_dyn_smem(trd_kernel, sh);
-            bar.alloc(2);
+            bar.alloc(kBarrierWords);
             bar.zero(s);
             p.alloc(2 * (size_t)n);
             // about one row per warp: more blocks than that only lengthen the barrier

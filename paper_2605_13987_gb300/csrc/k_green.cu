@@ -9,6 +9,8 @@
 // w = 1 for index 0 and 2 otherwise (the +- mode pairs).
 #include "wt_internal.cuh"
 
+#include <algorithm>
+
 namespace wt {
 
 // T[mx][my][mz] = 1 / |k|^2 for mx < Nx/2, my < Ny/2, mz < Nz; 0 at the origin.
@@ -157,8 +159,43 @@ void green_cos_table(cudaStream_t s, const double* z, int n, int Nz, double Lz, 
     cos_table_kernel<<<(tot + 255) / 256, 256, 0, s>>>(z, n, Nz, Lz, C);
     WT_LAUNCH("cos_table");
 }
-void green_pblocks(cudaStream_t s, const void* blocks, int n_blocks, int max_rows, int max_cols, const double* Ct,
-                   const double* Cs, const double* L, int Nz, double pref, double* P, int ldp) {
+// Left factor of one source column's part of P, for all collocation rows:
+// X[row0 + p][m] = 2 pref w(m) L[combo][m] Ct[ct0 + p][m], block (target group, piece of its rows).
+__global__ void __launch_bounds__(256) pfactor_kernel(const PBlock* __restrict__ blocks, int stride, int col,
+                                                      const double* __restrict__ Ct, const double* __restrict__ Lt,
+                                                      int nz, double pref2, double* __restrict__ X) {
+    const PBlock B = blocks[(size_t)blockIdx.x * stride + col];
+    const double* L = Lt + (size_t)B.combo * nz;
+    const size_t tot = (size_t)B.nrow * nz;
+    for (size_t e = (size_t)blockIdx.y * blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.y * blockDim.x) {
+        const int m = (int)(e % nz);
+        X[(size_t)B.row0 * nz + e] = pref2 * (m ? 2.0 : 1.0) * L[m] * Ct[(size_t)B.ct0 * nz + e];
+    }
+}
+
+// blocks: [target group][source column], on the device and (hblocks) on the host; nc rows in all.
+// Every block is a product over m_z.  The small ones run in one launch; where a source column's part
+// (all rows x its sources) is worth a tensor-core product, column by column: 18 columns x 18 432 rows x
+// 128 sources, N_z = 128: 9.2 -> 1.9 ms.
+void green_pblocks(cudaStream_t s, const void* blocks, const void* hblocks, int n_blocks, int n_cols, int nc,
+                   int max_rows, int max_cols, const double* Ct, const double* Cs, const double* L, int Nz, double pref,
+                   double* P, int ldp) {
+    const PBlock* hb = static_cast<const PBlock*>(hblocks);
+    if ((double)nc * max_cols * Nz > 6e7) {        // above 100 us a column on the CUDA cores
+        const int n_tg = n_blocks / n_cols;
+        DBuf<double> X;
+        X.alloc((size_t)nc * Nz);
+        const int pieces = (int)std::max<size_t>(1, std::min<size_t>(64, ((size_t)max_rows * Nz + 1023) / 1024));
+        for (int k = 0; k < n_cols; ++k) {
+            pfactor_kernel<<<dim3(n_tg, pieces), 256, 0, s>>>(static_cast<const PBlock*>(blocks), n_cols, k, Ct, L, Nz,
+                                                              2.0 * pref, X.p);
+            WT_LAUNCH("pfactor");
+            dgemm(s, false, true, nc, hb[k].ncol, Nz, 1.0, X.p, Nz, Cs + (size_t)hb[k].cs0 * Nz, Nz, 0.0,
+                  P + hb[k].col0, ldp);
+        }
+        WT_CUDA(cudaStreamSynchronize(s));         // X goes out of scope
+        return;
+    }
     dim3 grid((max_cols + 63) / 64, (max_rows + 63) / 64, n_blocks);
     pblock_kernel<<<grid, 256, 0, s>>>(static_cast<const PBlock*>(blocks), Ct, Cs, L, Nz, 2.0 * pref, P, ldp);
     WT_LAUNCH("pblock");

@@ -26,7 +26,8 @@ namespace wt {
 void green_invk2(cudaStream_t, int, int, int, double, double, double, double*);
 void green_lateral(cudaStream_t, const double*, int, int, int, int, double, double, const double*, double*);
 void green_cos_table(cudaStream_t, const double*, int, int, double, double*);
-void green_pblocks(cudaStream_t, const void*, int, int, int, const double*, const double*, const double*, int, double,
+void green_pblocks(cudaStream_t, const void*, const void*, int, int, int, int, int, const double*, const double*,
+                   const double*, int, double,
                    double*, int);
 size_t pblock_size();
 void pack_pblock(void*, int, int, int, int, int, int, int);
@@ -412,7 +413,7 @@ void do_fit(wt_ctx* c) {
     DBuf<unsigned char> dblocks;
     dblocks.upload(blocks.data(), blocks.size(), s);
     P.alloc((size_t)nc * ns);
-    green_pblocks(s, dblocks.p, n_combo, max_rows, max_cols, Ct.p, Cs.p, L.p, g.Nz, c->pref, P.p, ns);
+    green_pblocks(s, dblocks.p, blocks.data(), n_combo, ncol, nc, max_rows, max_cols, Ct.p, Cs.p, L.p, g.Nz, c->pref, P.p, ns);
     Ct.release(); Cs.release(); L.release();
 
     // --- S3: neutral basis (Householder), offset column, column scaling
@@ -629,7 +630,8 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
                       double& trunc_out) {
     cudaStream_t s = c->s;
     const int ns = c->ns;
-    const bool pre = ns >= nt;                    // column-pivoted QR first
+    const bool pre = ns >= nt && qrcp_fits(ns, nt);      // column-pivoted QR first
+    clear_err(c);
     DBuf<double> A, V, sig, Rm;
     DBuf<int> dpiv;
     int nr = nt;                                  // rows of R that are not negligible
@@ -640,14 +642,15 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     if (pre) {
         Rm.alloc((size_t)nt * nt);
         dpiv.alloc(nt);
-        nr = qrcp_r(s, A.p, ns, nt, ns, Rm.p, dpiv.p);
+        nr = std::max(1, qrcp_r(s, A.p, ns, nt, ns, Rm.p, dpiv.p, c->d_err.p));
         A.release();
     } else {
         V.alloc((size_t)nt * nt);
     }
-    clear_err(c);
     double coupling = 0.0;
-    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nr, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling)
+    // rows of R below 1e-13 of the history carry nothing the basis could use (its target is 1e-7 of a
+    // sample, the smallest sample counted 1e-6 of the largest): they need not be orthogonal to each other
+    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nr, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling, 1e-13)
                            : onesided_jacobi_rows(s, A.p, nt, ns, ns, V.p, sig.p, c->d_err.p, 40, &coupling);
     if (read_err(c)) {
         char msg[160];
@@ -656,16 +659,18 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
                       sweeps, coupling);
         fail(WT_ERR_TIMEOUT, msg);
     }
-    std::vector<double> hs(nt), hv((size_t)nt * nt);
+    const int rows = pre ? nr : nt;               // the other singular values are zero
+    std::vector<double> hs(nt), hv((size_t)rows * nt);
     sig.download(hs.data(), nt, s);
     if (pre) {
         // hv[k][P_i] = S[k][i] / sigma_k: the coefficient of u_k in sample P_i over sigma_k
-        std::vector<double> hS((size_t)nt * nt);
+        std::vector<double> hS((size_t)rows * nt);
         std::vector<int> hp(nt);
         Rm.download(hS.data(), hS.size(), s);
         dpiv.download(hp.data(), nt, s);
         WT_CUDA(cudaStreamSynchronize(s));
-        for (int k = 0; k < nt; ++k) {
+        for (int k = rows; k < nt; ++k) hs[k] = 0.0;
+        for (int k = 0; k < rows; ++k) {
             const double inv = hs[k] > 0.0 ? 1.0 / hs[k] : 0.0;
             for (int i = 0; i < nt; ++i) hv[(size_t)k * nt + hp[i]] = hS[(size_t)k * nt + i] * inv;
         }
@@ -676,14 +681,15 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     std::vector<int> ord(nt);
     std::iota(ord.begin(), ord.end(), 0);
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return hs[a] > hs[b]; });
-    // per-sample squared norms and suffix (tail) sums, smallest terms first
-    auto term = [&](int j, int n) {
-        const double x = hs[ord[j]] * hv[(size_t)ord[j] * nt + n];
-        return x * x;
+    // per-sample squared norms and suffix (tail) sums, smallest terms first, a row at a time
+    auto add_terms = [&](int j, std::vector<double>& sum) {
+        if (ord[j] >= rows) return;
+        const double sg = hs[ord[j]];
+        const double* v = hv.data() + (size_t)ord[j] * nt;
+        for (int n = 0; n < nt; ++n) sum[n] += (sg * v[n]) * (sg * v[n]);
     };
     std::vector<double> norm2(nt, 0.0);
-    for (int n = 0; n < nt; ++n)
-        for (int j = nt - 1; j >= 0; --j) norm2[n] += term(j, n);
+    for (int j = nt - 1; j >= 0; --j) add_terms(j, norm2);
     double nmax = 0.0;
     for (double v : norm2) nmax = std::max(nmax, std::sqrt(v));
     const int r_cap = std::min(fault_enabled("rank_cap") ? 4 : 32, nt);    // WT_FAULT=rank_cap: the guard's test
@@ -691,7 +697,7 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     std::vector<double> worst(r_cap + 1, 0.0);
     std::vector<double> tail(nt, 0.0);
     for (int j = nt - 1; j >= 0; --j) {
-        for (int n = 0; n < nt; ++n) tail[n] += term(j, n);
+        add_terms(j, tail);
         if (j <= r_cap) {
             double w = 0.0;
             for (int n = 0; n < nt; ++n)
@@ -1585,7 +1591,8 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
             duxy.upload(uxy.data(), uxy.size(), s);
             green_lateral_deriv(s, ddxy.p, duxy.p, c->f_ncombo, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, 1.0, p - 2, Ld.p);
             dP.alloc((size_t)nc * ns);
-            green_pblocks(s, dblocks.p, c->f_ncombo, c->f_maxrows, c->f_maxcols, Ct.p, Cs.p, Ld.p, g.Nz, c->pref,
+            green_pblocks(s, dblocks.p, c->f_blocks.data(), c->f_ncombo, ncol, nc, c->f_maxrows, c->f_maxcols, Ct.p, Cs.p,
+                          Ld.p, g.Nz, c->pref,
                           dP.p, ns);
             house_right(c, dP.p, nc);
             set_column(s, dP.p, nc, ns, 0, 0.0);

@@ -163,14 +163,16 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
 // orthogonal (row i = sigma_i u_i^T), V [m][m] holds the accumulated rotations
 // (A_in = V^T A_out; V = NULL: not accumulated) and sigma[m] the row norms (unsorted).  Returns the number
 // of sweeps; sets d_err (DERR_TIMEOUT) when max_sweeps do not converge (unless the largest
-// relative coupling still rotated in the last sweep is below 1e-10; coupling_out returns it).
+// relative coupling still rotated in the last sweep is below 1e-10; coupling_out returns it).  Pairs whose
+// coupling is below (floor_rel ||A||_F)^2 are not rotated.
 int onesided_jacobi_rows(cudaStream_t s, double* A, int m, int n, int lda, double* V, double* sigma, int* d_err,
-                         int max_sweeps = 40, double* coupling_out = nullptr);
+                         int max_sweeps = 40, double* coupling_out = nullptr, double floor_rel = 1e-15);
 // Householder QR with column pivoting, M P = Q1 R, of the ns x nt matrix whose column j is row j of
 // the row-major array M [nt][ld] (ns >= nt; M is destroyed): R [nt][nt] row-major upper triangular,
 // piv[i] (device) = the column of M that became column i.  Only R and P are formed.  Returns the
 // number of steps taken: the rows of R past it are zero (negligible columns, see k_dense.cu).
-int qrcp_r(cudaStream_t s, double* M, int ns, int nt, int ld, double* R, int* piv);
+bool qrcp_fits(int ns, int nt);      // whether its reflector fits a block's shared memory
+int qrcp_r(cudaStream_t s, double* M, int ns, int nt, int ld, double* R, int* piv, int* d_err);
 // out[r][n] = scale[r] * A[idx[r]][:]  (idx, scale: device arrays of `rows`)
 void gather_rows_scaled(cudaStream_t s, const double* A, int n, int lda, const int* idx, const double* scale,
                         int rows, double* out);
