@@ -40,9 +40,9 @@ constexpr int EQ1_MC = 16;   // track steps per chunk
 __device__ __forceinline__ float eq1_interp(const float* __restrict__ fj, int nt, Eq1Lag lg) {
     return fmaf(lg.w0, fj[lg.n], lg.w1 * fj[min(lg.n + 1, nt - 1)]);
 }
-// f: [mc][nt] (nt: the row stride, also the clamp of sample n + 1); outputs m < c0 take nothing
+// f: [mc] rows of stride ld, nt the clamp of sample n + 1; outputs m < c0 take nothing
 // from this chunk, so the threads start at c0.
-__device__ __forceinline__ void eq1_increments(const float* __restrict__ f, int nt, int mc, int c0, int n_out,
+__device__ __forceinline__ void eq1_increments(const float* __restrict__ f, int ld, int nt, int mc, int c0, int n_out,
                                                const Eq1Lag* __restrict__ lags, double* __restrict__ D) {
     for (int m = c0 + threadIdx.x; m < n_out; m += blockDim.x) {
         const int jmax = min(mc - 1, m - c0);
@@ -52,7 +52,7 @@ __device__ __forceinline__ void eq1_increments(const float* __restrict__ f, int 
         Eq1Lag hi = lags[L];
         float d = 0.f;
         for (int j = 0; j <= jmax; ++j, --L) {
-            const float* fj = f + j * nt;
+            const float* fj = f + j * ld;
             const float g_hi = eq1_interp(fj, nt, hi);
             if (L == 0) {
                 d += g_hi;
@@ -66,72 +66,130 @@ __device__ __forceinline__ void eq1_increments(const float* __restrict__ f, int 
     }
 }
 
-// T: field type; L: lag table entry; TO: current type
+// Cell and weights of one track step, and W(x, t_n) . v from a stored field.
+template <class T>
+struct Eq1Cell {
+    T vx = 0, vy = 0, vz = 0, wx = 0, wy = 0, wz = 0;
+    size_t a00 = 0, a01 = 0, a10 = 0, a11 = 0;
+    __device__ __forceinline__ void set(T x, T y, T z, int Nx, int Ny, int Nz, T inv_hx, T inv_hy, T inv_hz) {
+        const T fx = x * inv_hx, fy = y * inv_hy;
+        T fz = z * inv_hz - (T)0.5;
+        fz = fz < (T)0 ? (T)0 : (fz > (T)(Nz - 1) ? (T)(Nz - 1) : fz);
+        const T flx = floor(fx), fly = floor(fy);
+        const int k0 = min((int)floor(fz), Nz - 2);
+        wx = fx - flx;
+        wy = fy - fly;
+        wz = fz - (T)k0;
+        const int i0 = ((int)flx % Nx + Nx) % Nx, j0 = ((int)fly % Ny + Ny) % Ny;
+        const int i1 = (i0 + 1) % Nx, j1 = (j0 + 1) % Ny;
+        a00 = ((size_t)i0 * Ny + j0) * Nz + k0;
+        a01 = ((size_t)i0 * Ny + j1) * Nz + k0;
+        a10 = ((size_t)i1 * Ny + j0) * Nz + k0;
+        a11 = ((size_t)i1 * Ny + j1) * Nz + k0;
+    }
+    __device__ __forceinline__ bool moving() const { return vx != 0 || vy != 0 || vz != 0; }
+    // hb: the three component planes of one time sample
+    __device__ __forceinline__ T dot(const T* __restrict__ hb, size_t npts) const {
+        const T one = 1;
+        T w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const T* h = hb + (size_t)c * npts;
+            const T v00 = (one - wz) * h[a00] + wz * h[a00 + 1];
+            const T v01 = (one - wz) * h[a01] + wz * h[a01 + 1];
+            const T v10 = (one - wz) * h[a10] + wz * h[a10 + 1];
+            const T v11 = (one - wz) * h[a11] + wz * h[a11 + 1];
+            w[c] = (one - wx) * ((one - wy) * v00 + wy * v01) + wx * ((one - wy) * v10 + wy * v11);
+        }
+        return w[0] * vx + w[1] * vy + w[2] * vz;
+    }
+};
+
+// G[n][step] = W(x_step, t_n) . v_step for all steps of all tracks, the time sample in the slow grid
+// index: the blocks that run together read one or two time planes, which stay in L2 (96 x 96 x 192: 21
+// MB), where a block per track drew sectors of every plane from memory (a step of an inclined track
+// lies in a cell of its own: 12 sectors a sample, 49 GB for 1e6 steps x 128 samples).
+__global__ void __launch_bounds__(256) eq1_stage_kernel(const float* __restrict__ H, int Nx, int Ny, int Nz,
+                                                        float inv_hx, float inv_hy, float inv_hz,
+                                                        const float* __restrict__ X, const float* __restrict__ Y,
+                                                        const float* __restrict__ Z, const float* __restrict__ VX,
+                                                        const float* __restrict__ VY, const float* __restrict__ VZ,
+                                                        size_t steps, float* __restrict__ G) {
+    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= steps) return;
+    const size_t npts = (size_t)Nx * Ny * Nz;
+    Eq1Cell<float> c;
+    c.vx = VX[s];
+    c.vy = VY[s];
+    c.vz = VZ[s];
+    c.set(X[s], Y[s], Z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
+    const size_t n = blockIdx.y;
+    G[n * steps + s] = c.moving() ? c.dot(H + n * 3 * npts, npts) : 0.f;
+}
+
+// T: field type; L: lag table entry; TO: current type.  nu: time samples the lag table reads
+// (samples n >= nu are never staged).  G: the dot products of eq1_stage_kernel, or NULL to take them
+// here (a call that may not allocate, the FP64 field, few steps): lanes over track steps, warps over
+// time samples, a lane keeping its step's cell for all samples, so that neighbouring steps share
+// sectors (lanes over time samples: every read a sector of its own).
+// 1e4 tracks x 100 steps, 96 x 96 x 192, 128 samples: 38.1 ms with lanes over samples, 16.0 with lanes
+// over steps, 5.5 through G.  A stage holds `steps` steps (32, or 16 where 32 rows of samples
+// do not fit), accumulated 16 at a time.
 template <class T, class L, class TO>
-// nu: time samples the lag table reads (samples n >= nu are never staged)
 __global__ void __launch_bounds__(256) eq1_kernel(const T* __restrict__ H, int Nx, int Ny, int Nz, int nt, int nu,
                                                   T inv_hx, T inv_hy, T inv_hz,
                                                   const float* __restrict__ X, const float* __restrict__ Y,
                                                   const float* __restrict__ Z, const float* __restrict__ VX,
                                                   const float* __restrict__ VY, const float* __restrict__ VZ,
                                                   const float* __restrict__ qtrack, float qconst, int n_steps,
-                                                  int n_out, double dt, double inv_vw,
+                                                  int n_out, double dt, double inv_vw, int steps, int ld,
+                                                  const float* __restrict__ G, size_t g_steps,
                                                   const L* __restrict__ lags, TO* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* f = reinterpret_cast<T*>(smem_raw);                               // [EQ1_MC][nt]
-    double* Q = reinterpret_cast<double*>(smem_raw + (((size_t)EQ1_MC * nt * sizeof(T) + 15) & ~(size_t)15));   // [n_out]
+    T* f = reinterpret_cast<T*>(smem_raw);                               // [steps][ld]
+    double* Q = reinterpret_cast<double*>(smem_raw + (((size_t)steps * ld * sizeof(T) + 15) & ~(size_t)15));   // [n_out]
     const int tr = blockIdx.x;
     const size_t npts = (size_t)Nx * Ny * Nz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int per = 32 / steps;                                          // time samples per warp and turn
     for (int m = threadIdx.x; m < n_out; m += blockDim.x) Q[m] = 0.0;
-    for (int c0 = 0; c0 < n_steps; c0 += EQ1_MC) {
-        const int mc = min(EQ1_MC, n_steps - c0);
-        __syncthreads();
-        for (int e = threadIdx.x; e < mc * nu; e += blockDim.x) {
-            const int j = e / nu, n = e % nu;
-            const size_t s = (size_t)tr * n_steps + c0 + j;
-            const T vx = VX[s], vy = VY[s], vz = VZ[s];
-            T acc = 0;
-            if (vx != 0 || vy != 0 || vz != 0) {
-                const T one = 1;
-                const T fx = (T)X[s] * inv_hx, fy = (T)Y[s] * inv_hy;
-                T fz = (T)Z[s] * inv_hz - (T)0.5;
-                fz = fz < (T)0 ? (T)0 : (fz > (T)(Nz - 1) ? (T)(Nz - 1) : fz);
-                const T flx = floor(fx), fly = floor(fy);
-                int k0 = min((int)floor(fz), Nz - 2);
-                const T wx = fx - flx, wy = fy - fly, wz = fz - (T)k0;
-                int i0 = ((int)flx % Nx + Nx) % Nx, j0 = ((int)fly % Ny + Ny) % Ny;
-                const int i1 = (i0 + 1) % Nx, j1 = (j0 + 1) % Ny;
-                const T* hb = H + (size_t)n * 3 * npts;
-                T w[3] = {0, 0, 0};
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const T* h = hb + (size_t)c * npts;
-                    const size_t a00 = ((size_t)i0 * Ny + j0) * Nz + k0, a01 = ((size_t)i0 * Ny + j1) * Nz + k0;
-                    const size_t a10 = ((size_t)i1 * Ny + j0) * Nz + k0, a11 = ((size_t)i1 * Ny + j1) * Nz + k0;
-                    const T v00 = (one - wz) * h[a00] + wz * h[a00 + 1];
-                    const T v01 = (one - wz) * h[a01] + wz * h[a01 + 1];
-                    const T v10 = (one - wz) * h[a10] + wz * h[a10 + 1];
-                    const T v11 = (one - wz) * h[a11] + wz * h[a11 + 1];
-                    w[c] = (one - wx) * ((one - wy) * v00 + wy * v01) + wx * ((one - wy) * v10 + wy * v11);
-                }
-                acc = w[0] * vx + w[1] * vy + w[2] * vz;
-            }
-            f[j * nt + n] = acc;
+    for (int s0 = 0; s0 < n_steps; s0 += steps) {
+        const int j = lane % steps;
+        const bool in = s0 + j < n_steps;
+        Eq1Cell<T> cell;
+        const size_t s = (size_t)tr * n_steps + s0 + j;
+        if (in && !G) {
+            cell.vx = VX[s];
+            cell.vy = VY[s];
+            cell.vz = VZ[s];
+            cell.set((T)X[s], (T)Y[s], (T)Z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
         }
         __syncthreads();
-        if constexpr (std::is_same<T, float>::value) {
-            // FP32 field: increments D(m) = Q(tau_m) - Q(tau_{m-1}) over dt, accumulated in Q
-            eq1_increments(f, nt, mc, c0, n_out, lags, Q);
-        } else {
-            for (int m = threadIdx.x; m < n_out; m += blockDim.x) {
-                double q = 0.0;
-                const int jmax = min(mc - 1, m - c0);
-                for (int j = 0; j <= jmax; ++j) {
-                    const L lg = lags[m - (c0 + j)];
-                    q += (double)lg.w0 * (double)f[j * nt + lg.n] +
-                         (double)lg.w1 * (double)f[j * nt + min(lg.n + 1, nt - 1)];
+        for (int n = warp * per + lane / steps; n < nu; n += nwarps * per) {
+            if (!in) continue;
+            if (G) f[j * ld + n] = (T)G[(size_t)n * g_steps + s];
+            else f[j * ld + n] = cell.moving() ? cell.dot(H + (size_t)n * 3 * npts, npts) : (T)0;
+        }
+        __syncthreads();
+        for (int c0 = s0; c0 < min(n_steps, s0 + steps); c0 += EQ1_MC) {
+            const int mc = min(EQ1_MC, n_steps - c0);
+            const T* fc = f + (size_t)(c0 - s0) * ld;
+            if constexpr (std::is_same<T, float>::value) {
+                // FP32 field: increments D(m) = Q(tau_m) - Q(tau_{m-1}) over dt, accumulated in Q; a
+                // thread keeps its outputs across the chunks, shifted by EQ1_MC, so order them
+                eq1_increments(fc, ld, nt, mc, c0, n_out, lags, Q);
+                __syncthreads();
+            } else {
+                for (int m = threadIdx.x; m < n_out; m += blockDim.x) {
+                    double q = 0.0;
+                    const int jmax = min(mc - 1, m - c0);
+                    for (int j = 0; j <= jmax; ++j) {
+                        const L lg = lags[m - (c0 + j)];
+                        q += (double)lg.w0 * (double)fc[j * ld + lg.n] +
+                             (double)lg.w1 * (double)fc[j * ld + min(lg.n + 1, nt - 1)];
+                    }
+                    Q[m] += q * dt;
                 }
-                Q[m] += q * dt;
             }
         }
     }
@@ -148,22 +206,48 @@ template <class T, class L, class TO>
 static void eq1_launch_t(cudaStream_t s, const T* H, int Nx, int Ny, int Nz, int nt, double Lx, double Ly, double Lz,
                          const float* x, const float* y, const float* z, const float* vx, const float* vy,
                          const float* vz, const float* q, float qconst, int n_tracks, int n_steps, int n_out,
-                         double dt, double v_w, const void* lags, int nu, TO* out) {
+                         double dt, double v_w, const void* lags, int nu, TO* out, const float* G = nullptr) {
     if (nu < 1 || nu > nt) fail(WT_ERR_ARG, "eq1: bad count of time samples in use");
-    size_t sh = (((size_t)EQ1_MC * nt * sizeof(T) + 15) & ~(size_t)15) + (size_t)n_out * sizeof(double);
-    if (sh > 200 * 1024) fail(WT_ERR_UNSUPPORTED, "eq1: n_t or n_out too large for shared memory");
+    // the limit of accepted sizes: 16 rows of nt samples and the outputs in 200 KB
+    if ((((size_t)EQ1_MC * nt * sizeof(T) + 15) & ~(size_t)15) + (size_t)n_out * sizeof(double) > 200 * 1024)
+        fail(WT_ERR_UNSUPPORTED, "eq1: n_t or n_out too large for shared memory");
+    // rows of the staged samples: an odd stride (lanes store down a column); nu + 1 entries may be read
+    const int ld = (std::min(nt, nu + 1)) | 1;
+    auto bytes = [&](int steps) {
+        return (((size_t)steps * ld * sizeof(T) + 15) & ~(size_t)15) + (size_t)n_out * sizeof(double);
+    };
+    // 32 steps per stage while four blocks fit an SM (or 16 would not give more)
+    const int steps = bytes(32) <= 56 * 1024 ? 32 : 16;
+    const size_t sh = bytes(steps);
     allow_dyn_smem(eq1_kernel<T, L, TO>, sh);
     eq1_kernel<T, L, TO><<<n_tracks, 256, sh, s>>>(H, Nx, Ny, Nz, nt, nu, (T)(Nx / Lx), (T)(Ny / Ly), (T)(Nz / Lz), x, y,
-                                                   z, vx, vy, vz, q, qconst, n_steps, n_out, dt, 1.0 / v_w,
-                                                   static_cast<const L*>(lags), out);
+                                                   z, vx, vy, vz, q, qconst, n_steps, n_out, dt, 1.0 / v_w, steps, ld,
+                                                   G, (size_t)n_tracks * n_steps, static_cast<const L*>(lags),
+                                                   out);
     WT_LAUNCH("eq1");
 }
 void eq1_launch(cudaStream_t s, const float* H, int Nx, int Ny, int Nz, int nt, double Lx, double Ly, double Lz,
                 const float* x, const float* y, const float* z, const float* vx, const float* vy, const float* vz,
                 const float* q, float qconst, int n_tracks, int n_steps, int n_out, double dt, double v_w,
-                const void* lags, int nu, float* out) {
-    eq1_launch_t<float, Eq1Lag, float>(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x, y, z, vx, vy, vz, q, qconst, n_tracks,
-                                       n_steps, n_out, dt, v_w, lags, nu, out);
+                const void* lags, int nu, float* out, float* G, size_t g_len) {
+    // G: workspace of g_len values (NULL: none) for the dot products of as many whole tracks at a time
+    const int per = (int)std::min<size_t>(n_tracks, g_len / ((size_t)nu * n_steps));
+    if (!G || per < 1) {
+        eq1_launch_t<float, Eq1Lag, float>(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x, y, z, vx, vy, vz, q, qconst, n_tracks,
+                                           n_steps, n_out, dt, v_w, lags, nu, out);
+        return;
+    }
+    for (int t0 = 0; t0 < n_tracks; t0 += per) {
+        const int n = std::min(per, n_tracks - t0);
+        const size_t o = (size_t)t0 * n_steps, steps = (size_t)n * n_steps;
+        eq1_stage_kernel<<<dim3((unsigned)((steps + 255) / 256), nu), 256, 0, s>>>(
+            H, Nx, Ny, Nz, (float)(Nx / Lx), (float)(Ny / Ly), (float)(Nz / Lz), x + o, y + o, z + o, vx + o, vy + o,
+            vz + o, steps, G);
+        WT_LAUNCH("eq1_stage");
+        eq1_launch_t<float, Eq1Lag, float>(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x + o, y + o, z + o, vx + o, vy + o, vz + o,
+                                           q ? q + t0 : nullptr, qconst, n, n_steps, n_out, dt, v_w, lags, nu,
+                                           out + (size_t)t0 * n_out, G);
+    }
 }
 // FP64 field (plain path): interpolation, time weights and currents in FP64 (lags: FP64 table).
 void eq1_launch64(cudaStream_t s, const double* H, int Nx, int Ny, int Nz, int nt, double Lx, double Ly, double Lz,
@@ -286,12 +370,233 @@ __global__ void __launch_bounds__(256) eq1_basis_kernel(const float* __restrict_
             default: eq1_stage_product<4>(sv, Wt, r, nq, nu, mc, f); break;
         }
         __syncthreads();
-        eq1_increments(f, nu, mc, c0, n_out, lg, Q);
+        eq1_increments(f, nu, nu, mc, c0, n_out, lg, Q);
     }
     __syncthreads();
     const float qc = qtrack ? qtrack[tr] : qconst;
     for (int m = threadIdx.x; m < n_out; m += blockDim.x)
         out[(size_t)tr * n_out + m] = (float)(-(double)qc * inv_vw * Q[m]);
+}
+
+// The same currents as a convolution.  With the lag table folded into the time coefficients,
+//   dV[L][m] = V[L][m] - V[L-1][m],  V[L][m] = w0(L) W[n(L)][m] + w1(L) W[n(L)+1][m],  V[-1] = 0,
+// the increment of output k is D(k) = sum_j sum_m s_m(j) dV[k - j][m], s_m(j) = E_m(x_j) . v_j: one FP32
+// multiply-add per (step, output, basis vector) in place of the staged product, its two lag reads and
+// their difference, and the small differences are formed once, in FP64, instead of from rounded values
+// per track (the error against 64 bits falls; 1e5 drifting carriers: 1.5e-6 -> 0.9e-6).  Bound by the FP32 units; one track per
+// block, blocks persistent with the table (32 x (n_out + pad) floats) in shared memory:
+//   * a thread holds 16 consecutive outputs and takes 8 steps and two basis vectors at a time: 23 table
+//     reads and 8 broadcast coefficients, all pairs, for 128 paired multiply-adds (fma.rn.f32x2: half
+//     the instructions, which bound the single form).  Table entry e lies at e + e / 16, so that lanes,
+//     16 outputs apart, read 17 pairs apart: no bank conflicts, and offsets within a thread are constants
+//     from three bases;
+//   * the steps of a chunk (8 per group of threads) are gathered first, a warp taking consecutive steps
+//     and keeping its cell's 24 corner values while the track stays in the cell (a drifting carrier: 11
+//     steps a cell);
+//   * groups are added in FP32, chunks in FP64.
+// 1e5 tracks x 200 steps, 400 outputs, rank 32: 20.3 -> 14.3 ms.
+constexpr int kConvThreads = 128, kConvOut = 16, kConvSteps = 8, kConvPad = 24;
+constexpr size_t kConvTableMax = 110 * 1024;
+struct ConvShape {
+    int tm;        // threads along the outputs
+    int ng;        // groups of steps
+    int row;       // entries of the table per basis vector
+    int jc;        // steps per chunk
+    int js;        // row stride of the gathered coefficients
+    size_t smem;
+};
+static bool conv_shape(int n_out, ConvShape* sh) {
+    sh->tm = (n_out + kConvOut - 1) / kConvOut;
+    if (sh->tm > kConvThreads) return false;
+    sh->ng = kConvThreads / sh->tm;
+    sh->row = 17 * (sh->tm + 2);
+    sh->jc = kConvSteps * std::min(sh->ng, 16);
+    sh->ng = sh->jc / kConvSteps;
+    sh->js = sh->jc + 4;
+    const size_t table = (size_t)32 * sh->row * sizeof(float);
+    sh->smem = table + (size_t)32 * sh->js * sizeof(float) + (size_t)sh->ng * sh->tm * kConvOut * sizeof(float) +
+               (size_t)sh->tm * kConvOut * sizeof(double) + 16;
+    return table <= kConvTableMax;
+}
+
+// dvt[m / 2][e + e / 16][m % 2] = dV[e - kConvPad][m] for 0 <= e - kConvPad < n_out, else 0.
+__global__ void eq1_dv_kernel(const double* __restrict__ W, int r, int nt, const Eq1Lag64* __restrict__ lags, int n_out,
+                              int row, float* __restrict__ dvt) {
+    const int pos = blockIdx.x * blockDim.x + threadIdx.x, m = blockIdx.y;
+    if (pos >= row) return;
+    const int L = pos - pos / 17 - kConvPad;              // the 17th of each group is not read
+    double d = 0.0;
+    if (pos % 17 < 16 && L >= 0 && L < n_out && m < r) {
+        auto V = [&](int l) {
+            const Eq1Lag64 g = lags[l];
+            return g.w0 * W[(size_t)g.n * 32 + m] + g.w1 * W[(size_t)min(g.n + 1, nt - 1) * 32 + m];
+        };
+        d = V(L) - (L > 0 ? V(L - 1) : 0.0);
+    }
+    dvt[((size_t)(m >> 1) * row + pos) * 2 + (m & 1)] = (float)d;
+}
+
+__device__ __forceinline__ unsigned long long fma_pair(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
+    const float* __restrict__ Ep, int r, const float* __restrict__ dvt, ConvShape C, int Nx, int Ny, int Nz, float inv_hx,
+    float inv_hy, float inv_hz, const float* __restrict__ X, const float* __restrict__ Y, const float* __restrict__ Z,
+    const float* __restrict__ VX, const float* __restrict__ VY, const float* __restrict__ VZ,
+    const float* __restrict__ qtrack, float qconst, int n_tracks, int n_steps, int n_out, double inv_vw,
+    float* __restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int row = C.row, nm = C.tm * kConvOut;
+    double* D = reinterpret_cast<double*>(smem_raw);              // [nm]
+    float* S = reinterpret_cast<float*>(D + nm);                  // [16][js][2]
+    float* tab = S + (size_t)32 * C.js;                           // [16][row][2]
+    float* P = tab + (size_t)32 * row;                            // [ng][nm]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < 32 * row; e += kConvThreads) tab[e] = dvt[e];
+    const int t = tid % C.tm, g = tid / C.tm;                     // outputs 16 t .., group of steps
+    const bool work = g < C.ng;
+    const int per_warp = (C.jc + kConvThreads / 32 - 1) / (kConvThreads / 32);
+    for (int tr = blockIdx.x; tr < n_tracks; tr += gridDim.x) {
+        for (int m = tid; m < nm; m += kConvThreads) D[m] = 0.0;
+        for (int c0 = 0; c0 < n_steps; c0 += C.jc) {
+            const int mc = min(C.jc, n_steps - c0);
+            __syncthreads();                                       // S and P of the last chunk are read, D is set
+            // a warp's steps are prepared a lane each (one coalesced read of the track arrays), then taken
+            // one after the other with a lane per basis field
+            for (int l0 = 0; l0 < per_warp; l0 += 32) {
+                const int js = warp * per_warp + l0 + lane;
+                Eq1Cell<float> cell;
+                if (l0 + lane < per_warp && js < mc) {
+                    const size_t st = (size_t)tr * n_steps + c0 + js;
+                    cell.vx = VX[st];
+                    cell.vy = VY[st];
+                    cell.vz = VZ[st];
+                    cell.set(X[st], Y[st], Z[st], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
+                }
+                const unsigned moving = __ballot_sync(0xffffffffu, cell.moving());
+                const int a00 = (int)cell.a00, a01 = (int)cell.a01, a10 = (int)cell.a10, a11 = (int)cell.a11;
+                int key = -1;
+                float v[24];
+                const int nl = min(32, per_warp - l0);
+                for (int l = 0; l < nl; ++l) {
+                    const int j = warp * per_warp + l0 + l;
+                    if (j >= C.jc) break;
+                    float acc = 0.f;
+                    if (moving >> l & 1) {
+                        const int k00 = __shfl_sync(0xffffffffu, a00, l);
+                        if (k00 != key) {
+                            key = k00;
+                            const int k01 = __shfl_sync(0xffffffffu, a01, l), k10 = __shfl_sync(0xffffffffu, a10, l),
+                                      k11 = __shfl_sync(0xffffffffu, a11, l);
+                            const float* p[4] = {Ep + (size_t)k00 * 96 + lane, Ep + (size_t)k01 * 96 + lane,
+                                                 Ep + (size_t)k10 * 96 + lane, Ep + (size_t)k11 * 96 + lane};
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                                for (int c = 0; c < 3; ++c) {
+                                    v[6 * q + 2 * c] = __ldg(p[q] + 32 * c);
+                                    v[6 * q + 2 * c + 1] = __ldg(p[q] + 96 + 32 * c);
+                                }
+                        }
+                        const float wx = __shfl_sync(0xffffffffu, cell.wx, l), wy = __shfl_sync(0xffffffffu, cell.wy, l),
+                                    wz = __shfl_sync(0xffffffffu, cell.wz, l);
+                        float w[3];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            float u[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                u[q] = (1.f - wz) * v[6 * q + 2 * c] + wz * v[6 * q + 2 * c + 1];
+                            w[c] = (1.f - wx) * ((1.f - wy) * u[0] + wy * u[1]) + wx * ((1.f - wy) * u[2] + wy * u[3]);
+                        }
+                        acc = w[0] * __shfl_sync(0xffffffffu, cell.vx, l) + w[1] * __shfl_sync(0xffffffffu, cell.vy, l) +
+                              w[2] * __shfl_sync(0xffffffffu, cell.vz, l);
+                    }
+                    S[((lane >> 1) * C.js + j) * 2 + (lane & 1)] = lane < r ? acc : 0.f;
+                }
+            }
+            __syncthreads();
+            const int j0 = kConvSteps * g, m0 = kConvOut * t;      // this thread's steps (in the chunk), outputs
+            const bool live = work && j0 < mc && m0 + kConvOut - 1 >= c0 + j0;
+            using pair = unsigned long long;
+            pair acc[kConvOut];
+#pragma unroll
+            for (int i = 0; i < kConvOut; ++i) acc[i] = 0;
+            if (live) {
+                // entries e0 .. e0 + 22 of a table row: dV[m0 + i - (c0 + j0 + jj)] at i - jj + 7; e0 mod 16 is 1
+                // or 9 (m0 is a multiple of 16, c0 + j0 of 8), so the skip of every 17th place falls at
+                // entry 15, or at 7
+                const int e0 = m0 - (c0 + j0) - (kConvSteps - 1) + kConvPad;
+                const pair* T = reinterpret_cast<const pair*>(tab) + e0 + (e0 >> 4);
+                const int skip = (e0 & 15) == 9 ? 1 : 0;
+                const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(S) + j0 / 2;
+                for (int m = 0; m < r; m += 2, T += row, sp += C.js / 2) {
+                    pair sj[kConvSteps], w[kConvOut + kConvSteps - 1];
+#pragma unroll
+                    for (int k = 0; k < kConvSteps / 2; ++k) {
+                        const ulonglong2 x = sp[k];
+                        sj[2 * k] = x.x;
+                        sj[2 * k + 1] = x.y;
+                    }
+#pragma unroll
+                    for (int k = 0; k < kConvOut + kConvSteps - 1; ++k) w[k] = k < 7 ? T[k] : k < 15 ? T[k + skip] : T[k + 1];
+#pragma unroll
+                    for (int jj = 0; jj < kConvSteps; ++jj)
+#pragma unroll
+                        for (int i = 0; i < kConvOut; ++i) acc[i] = fma_pair(sj[jj], w[i - jj + kConvSteps - 1], acc[i]);
+                }
+            }
+            if (work)
+#pragma unroll
+                for (int i = 0; i < kConvOut; ++i)
+                    P[(size_t)g * nm + i * C.tm + t] = __uint_as_float((unsigned)acc[i]) +
+                                                       __uint_as_float((unsigned)(acc[i] >> 32));
+            __syncthreads();
+            for (int e = tid; e < nm; e += kConvThreads) {         // e = i tm + t: output 16 t + i
+                const int m = (e % C.tm) * kConvOut + e / C.tm;
+                if (m < c0) continue;
+                float d = 0.f;
+                for (int q = 0; q < C.ng; ++q) d += P[(size_t)q * nm + e];
+                D[e] += (double)d;
+            }
+        }
+        __syncthreads();
+        const float qc = qtrack ? qtrack[tr] : qconst;
+        for (int m = tid; m < n_out; m += kConvThreads)
+            out[(size_t)tr * n_out + m] = (float)(-(double)qc * inv_vw * D[(m % kConvOut) * C.tm + m / kConvOut]);
+        __syncthreads();
+    }
+}
+
+// Floats of the table of eq1_conv_launch, 0 where it does not take n_out outputs.
+size_t eq1_conv_table(int n_out) {
+    ConvShape C;
+    return conv_shape(n_out, &C) ? (size_t)32 * C.row : 0;
+}
+// Ep: point-major basis fields; W: [nt][32] FP64 time coefficients; lags: the FP64 lag table; dvt: workspace.
+void eq1_conv_launch(cudaStream_t s, const float* Ep, int r, const double* W, int Nx, int Ny, int Nz, int nt, double Lx,
+                     double Ly, double Lz, const float* x, const float* y, const float* z, const float* vx,
+                     const float* vy, const float* vz, const float* q, float qconst, int n_tracks, int n_steps,
+                     int n_out, double v_w, const void* lags, float* dvt, float* out) {
+    if (r < 1 || r > 32) fail(WT_ERR_ARG, "eq1: basis rank out of range");
+    ConvShape C;
+    if (!conv_shape(n_out, &C)) fail(WT_ERR_UNSUPPORTED, "eq1: n_out too large for the convolution's table");
+    if (n_tracks < 1) return;
+    eq1_dv_kernel<<<dim3((C.row + 127) / 128, 32), 128, 0, s>>>(W, r, nt, static_cast<const Eq1Lag64*>(lags), n_out,
+                                                               C.row, dvt);
+    WT_LAUNCH("eq1_dv");
+    allow_dyn_smem(eq1_conv_kernel, C.smem);
+    int dev = 0, n_sm = 0, per = 0;
+    WT_CUDA(cudaGetDevice(&dev));
+    WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    WT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, eq1_conv_kernel, kConvThreads, C.smem));
+    eq1_conv_kernel<<<std::min(n_tracks, n_sm * std::max(1, per)), kConvThreads, C.smem, s>>>(
+        Ep, r, dvt, C, Nx, Ny, Nz, (float)(Nx / Lx), (float)(Ny / Ly), (float)(Nz / Lz), x, y, z, vx, vy, vz, q, qconst,
+        n_tracks, n_steps, n_out, 1.0 / v_w, out);
+    WT_LAUNCH("eq1_conv");
 }
 
 // Point-major copy of the basis fields for eq1_basis_kernel: Ep[p][c][m] = E[c][m][p] for m < r, 0 for
@@ -328,21 +633,30 @@ void eq1_point_major(cudaStream_t s, const float* E, int r, size_t npts, float* 
     WT_LAUNCH("eq1_point_major");
 }
 
-void eq1_basis_launch(cudaStream_t s, const float* Ep, int r, const float* W32, int Nx, int Ny, int Nz, int nt,
-                      double Lx, double Ly, double Lz, const float* x, const float* y, const float* z,
-                      const float* vx, const float* vy, const float* vz, const float* q, float qconst, int n_tracks,
-                      int n_steps, int n_out, double dt, double v_w, const void* lags, int nu, float* out) {
-    if (r < 1 || r > 32) fail(WT_ERR_ARG, "eq1: basis rank out of range");
-    if (nu < 1 || nu > nt) fail(WT_ERR_ARG, "eq1: bad count of time samples in use");
+// Shared memory of eq1_basis_kernel; the lag table goes beside the rest when it is small (12 B per output).
+static size_t eq1_basis_smem(int r, int nu, int n_out, int* nb_out, bool* stage_lags_out) {
     // time samples per thread in the staged product: the fewest that keep the (samples / nb) x
     // (steps / 4) items within one pass of the 256 threads
     const int nb = std::min(4, std::max(1, (nu + 63) / 64));
     const size_t ldw = (size_t)nb * ((nu + nb - 1) / nb);
     const size_t base = ((((size_t)r * ldw + EQ1_MC * 32 + (size_t)EQ1_MC * nu) * sizeof(float) + 15) & ~(size_t)15) +
                         (size_t)n_out * sizeof(double);
-    // the lag table goes into shared memory beside the rest when it is small (12 B per output)
     const bool stage_lags = (size_t)n_out * sizeof(Eq1Lag) <= 16384;
-    const size_t sh = base + (stage_lags ? (size_t)n_out * sizeof(Eq1Lag) : 0);
+    if (nb_out) *nb_out = nb;
+    if (stage_lags_out) *stage_lags_out = stage_lags;
+    return base + (stage_lags ? (size_t)n_out * sizeof(Eq1Lag) : 0);
+}
+// Whether eq1_basis_launch takes up to nt time samples and n_out outputs, at any rank.
+bool eq1_basis_fits(int nt, int n_out) { return eq1_basis_smem(32, nt, n_out, nullptr, nullptr) <= 200 * 1024; }
+void eq1_basis_launch(cudaStream_t s, const float* Ep, int r, const float* W32, int Nx, int Ny, int Nz, int nt,
+                      double Lx, double Ly, double Lz, const float* x, const float* y, const float* z,
+                      const float* vx, const float* vy, const float* vz, const float* q, float qconst, int n_tracks,
+                      int n_steps, int n_out, double dt, double v_w, const void* lags, int nu, float* out) {
+    if (r < 1 || r > 32) fail(WT_ERR_ARG, "eq1: basis rank out of range");
+    if (nu < 1 || nu > nt) fail(WT_ERR_ARG, "eq1: bad count of time samples in use");
+    int nb = 0;
+    bool stage_lags = false;
+    const size_t sh = eq1_basis_smem(r, nu, n_out, &nb, &stage_lags);
     if (sh > 200 * 1024) fail(WT_ERR_UNSUPPORTED, "eq1: n_t or n_out too large for shared memory");
     allow_dyn_smem(eq1_basis_kernel, sh);
     if (n_tracks > 0)
@@ -459,7 +773,7 @@ void eq1_noalloc_launch(cudaStream_t s, int device, const float* H, int Nx, int 
     eq1_lag_table_kernel<<<(n_out + 127) / 128, 128, 0, s>>>(d_times, nt, dt, n_out, lags);
     WT_LAUNCH("eq1_lag_table");
     eq1_launch(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x, y, z, vx, vy, vz, q, qconst, n_tracks, n_steps, n_out, dt, v_w,
-               lags, nu, out);
+               lags, nu, out, nullptr, 0);
 }
 
 }  // namespace wt

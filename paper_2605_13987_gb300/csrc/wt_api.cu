@@ -45,7 +45,7 @@ void sample_points(cudaStream_t, const double*, int, const double*, const double
                    double*);
 void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, double, const float*, const float*,
                 const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
-                double, const void*, int, float*);
+                double, const void*, int, float*, float*, size_t);
 size_t eq1_lag_size();
 void eq1_launch64(cudaStream_t, const double*, int, int, int, int, double, double, double, const float*, const float*,
                   const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
@@ -70,6 +70,11 @@ void eq1_point_major(cudaStream_t, const float*, int, size_t, float*);
 void eq1_basis_launch(cudaStream_t, const float*, int, const float*, int, int, int, int, double, double, double,
                       const float*, const float*, const float*, const float*, const float*, const float*,
                       const float*, float, int, int, int, double, double, const void*, int, float*);
+bool eq1_basis_fits(int, int);
+size_t eq1_conv_table(int);
+void eq1_conv_launch(cudaStream_t, const float*, int, const double*, int, int, int, int, double, double, double,
+                     const float*, const float*, const float*, const float*, const float*, const float*,
+                     const float*, float, int, int, int, double, const void*, float*, float*);
 void features_launch(cudaStream_t, const float*, int, int, double, double, float, float, float, const float*, int,
                      double*, double*);
 void add_f32(cudaStream_t, size_t, const float*, float*);
@@ -125,6 +130,7 @@ struct wt_ctx {
     int rank = 0, r_pad = 0;
     DBuf<double> Ub;                      // [r][ns] basis charge vectors
     DBuf<float> W32;                      // [nt][r_pad] time coefficients
+    DBuf<double> W64;                     // the same before rounding
     // spectral
     DBuf<double> d_zsrc;
     DBuf<double> zcos;                   // [ns][Nz] 2 cos(pi m z_j / Lz)
@@ -621,13 +627,13 @@ void charges_at(wt_ctx* c, const double* d_t, int nt, double* Q) {
 // the smallest term up.  Samples whose charge is below kTruncFloor of the
 // largest one are measured against that floor (tangent histories can vanish
 // at some times).  Outputs: basis charge vectors Ub [r][ns] (unit norm),
-// FP32 coefficients W32 [nt][32] = sigma_m v_m[n], r, and the largest
+// coefficients W32, W64 [nt][32] = sigma_m v_m[n], r, and the largest
 // per-sample truncation at r (trunc_out).
 constexpr double kTruncTarget = 1e-7;
 constexpr double kTruncLimit = 1e-6;     // the FP32 field paths refuse a basis truncated beyond this
 constexpr double kTruncFloor = 1e-6;
-void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf<float>& W32, int& rank_out,
-                      double& trunc_out) {
+void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf<float>& W32, DBuf<double>& W64,
+                      int& rank_out, double& trunc_out) {
     cudaStream_t s = c->s;
     const int ns = c->ns;
     const bool pre = ns >= nt && qrcp_fits(ns, nt);      // column-pivoted QR first
@@ -720,7 +726,7 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
         for (int n = 0; n < nt; ++n) coef[(size_t)n * rp + m] = sg * hv[(size_t)ord[m] * nt + n];
     }
     DBuf<int> didx;
-    DBuf<double> dscale, dcoef;
+    DBuf<double> dscale;
     Ub.alloc((size_t)r * ns);
     if (pre) {
         // u_m = Q v_m / sigma_m: Ub [r][ns] = (V_r / sigma) Q^T
@@ -736,9 +742,9 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
         dscale.upload(scale.data(), r, s);
         gather_rows_scaled(s, A.p, ns, ns, didx.p, dscale.p, r, Ub.p);
     }
-    dcoef.upload(coef.data(), coef.size(), s);
+    W64.upload(coef.data(), coef.size(), s);
     W32.alloc(coef.size());
-    to_float(s, dcoef.p, coef.size(), 1.0, W32.p);
+    to_float(s, W64.p, coef.size(), 1.0, W32.p);
     WT_CUDA(cudaStreamSynchronize(s));
 }
 
@@ -885,7 +891,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     if (read_err(c)) fail(WT_ERR_NAN, "non-finite charges");
     // S5b: time basis of the charge history (Gram matrix + Jacobi)
     c->r_pad = 32;
-    compress_history(c, Q.p, nt, c->Ub, c->W32, c->rank, c->info.trunc_rel);
+    compress_history(c, Q.p, nt, c->Ub, c->W32, c->W64, c->rank, c->info.trunc_rel);
     c->info.n_t = nt;
     c->info.rank = c->rank;
     c->info.relax_seconds = secs(t0);
@@ -1306,10 +1312,26 @@ void eq1_run(wt_ctx* c, const void* H, bool h64, const TrackDev& t, void* out, c
         eq1_launch64(s, static_cast<const double*>(H), g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx,
                      t.vy, vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, t.dt, c->opts.v_w, dlag.p, nu,
                      static_cast<double*>(out));
-    else
+    else {
+        // workspace of the staged dot products: all of them, or 1 GB of tracks at a time (a large field
+        // is then read once per GB); few steps go without (their sectors stay in L2 anyway)
+        constexpr size_t kMost = (size_t)1 << 28, kFew = (size_t)1 << 20;
+        const size_t all = (size_t)t.n_tracks * t.n_steps * nu;
+        DBuf<float> G;
+        const bool staged = all >= kFew && (size_t)t.n_steps * nu <= kMost && nu <= 65535;
+        if (staged) {
+            try {
+                G.alloc(std::min(all, kMost));
+            } catch (const Error&) {       // no memory for it: the one-kernel form
+                if (fault_enabled("alloc")) throw;
+            }
+        }
         eq1_launch(s, static_cast<const float*>(H), g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx, t.vy,
                    vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, t.dt, c->opts.v_w, dlag.p, nu,
-                   static_cast<float*>(out));
+                   static_cast<float*>(out), G.p, G.n);
+        WT_CUDA(cudaStreamSynchronize(s));
+        return;
+    }
     WT_CUDA(cudaStreamSynchronize(s));   // the lag table is freed on return
 }
 
@@ -1336,11 +1358,24 @@ void do_eq1(wt_ctx* c, const void* H, const wt_tracks* tr, float* iout, cudaStre
 // Eq. 1 from the rank-r form of the FP32 field (the context's basis fields E32 and time
 // coefficients W32), without writing H; the basis fields are computed when E32 does not hold
 // them already.
-void eq1_basis_run(wt_ctx* c, const float* E, int r, const float* W32, const TrackDev& t, float* out, cudaStream_t s,
-                   const float* vz_override = nullptr) {
+void eq1_basis_run(wt_ctx* c, const float* E, int r, const float* W32, const double* W64, const TrackDev& t, float* out,
+                   cudaStream_t s, const float* vz_override = nullptr) {
     const wt_grid& g = c->grid;
     const int nt = (int)c->times.size();
     DBuf<unsigned char> dlag;
+    if (const size_t table = eq1_conv_table(t.n_out)) {
+        build_lags(c, t.dt, t.n_out, dlag, s, true);
+        DBuf<float> dvt;
+        dvt.alloc(table);
+        const size_t np = (size_t)g.Nx * g.Ny * g.Nz;
+        c->Ep32.alloc(np * 96);
+        eq1_point_major(s, E, r, np, c->Ep32.p);
+        eq1_conv_launch(s, c->Ep32.p, r, W64, g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx, t.vy,
+                        vz_override ? vz_override : t.vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, c->opts.v_w,
+                        dlag.p, dvt.p, out);
+        WT_CUDA(cudaStreamSynchronize(s));   // the tables are freed on return
+        return;
+    }
     const int nu = build_lags(c, t.dt, t.n_out, dlag, s, false);
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     c->Ep32.alloc(npts * 96);
@@ -1378,7 +1413,7 @@ void do_eq1_direct(wt_ctx* c, const wt_tracks* tr, float* iout, cudaStream_t us)
     DBuf<float> dout;
     float* o = iout;
     if (!dev_out) { dout.alloc((size_t)tr->n_tracks * tr->n_out); o = dout.p; }
-    eq1_basis_run(c, c->E32.p, c->rank, c->W32.p, td, o, s);
+    eq1_basis_run(c, c->E32.p, c->rank, c->W32.p, c->W64.p, td, o, s);
     if (!dev_out) {
         dout.download(iout, (size_t)tr->n_tracks * tr->n_out, s);
         WT_CUDA(cudaStreamSynchronize(s));
@@ -1426,7 +1461,7 @@ double do_loss(wt_ctx* c, wt_precision prec, const wt_tracks* tr) {
         ensure_base_fields(c, s);
         DBuf<float> I;
         I.alloc(nI);
-        eq1_basis_run(c, c->E32.p, c->rank, c->W32.p, td, I.p, s);
+        eq1_basis_run(c, c->E32.p, c->rank, c->W32.p, c->W64.p, td, I.p, s);
         sum = dot_f32(s, I.p, I.p, nI, c->d_scr.p);
     }
     if (read_err(c)) fail(WT_ERR_TIMEOUT, "device wait timed out");
@@ -1520,13 +1555,37 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     clock.on = c->timing;
     for (double& v : c->grad_ms) v = 0.0;
     clock.mark(-1);
-    // base field and currents
-    c->stage32.alloc((size_t)nt * 3 * npts);
-    extend32_basis(c, c->Ub.p, c->rank, c->W32.p, nt, c->stage32.p, s, 0, &launches, false);
-    DBuf<float> I, dI;
+    // Currents of a charge history's field, in its rank-r form: no field is expanded over time (1 000
+    // tracks x 100 steps, 256 times: 0.98 ms and the expansion per field before).  Outputs that do
+    // not fit that form's shared memory go through the expanded field, whose limit on the time samples
+    // holds for both.
+    if (c->use_tc && expand_tc_available() && nt > 512)
+        fail(WT_ERR_UNSUPPORTED, "tensor-core expansion handles 1 to 512 time samples");
+    const bool rank_r = eq1_conv_table(td.n_out) > 0 || eq1_basis_fits(nt, td.n_out);
+    DBuf<float> Hx;
+    auto field_currents = [&](const double* Ub, int r, const float* W, const double* Wd, int mode, float* out,
+                              const float* vz_override) {
+        if (rank_r) {
+            if (Ub == c->Ub.p && mode == 0) ensure_base_fields(c, s);
+            else basis_fields32(c, Ub, r, s, mode, &launches, false);
+            eq1_basis_run(c, c->E32.p, r, W, Wd, td, out, s, vz_override);
+        } else {
+            Hx.alloc((size_t)nt * 3 * npts);
+            extend32_basis(c, Ub, r, W, nt, Hx.p, s, mode, &launches, false);
+            eq1_run(c, Hx.p, false, td, out, s, vz_override);
+        }
+    };
+    DBuf<float> I, dI, I0;
     I.alloc(nI);
     dI.alloc(nI);
-    eq1_run(c, c->stage32.p, false, td, I.p, s);
+    field_currents(c->Ub.p, c->rank, c->W32.p, c->W64.p, 0, I.p, nullptr);
+    if (!delta) {      // the base field with the lateral velocities only, for the lateral scale
+        DBuf<float> zeros;
+        I0.alloc(nI);
+        zeros.alloc((size_t)td.n_tracks * td.n_steps);
+        zeros.zero(s);
+        field_currents(c->Ub.p, c->rank, c->W32.p, c->W64.p, 0, I0.p, zeros.p);
+    }
     if (I_out) WT_CUDA(cudaMemcpyAsync(I_out, I.p, nI * sizeof(float), cudaMemcpyDeviceToDevice, s));
     *loss = dot_f32(s, I.p, I.p, nI, c->d_scr.p) / (double)nI;
     const double gscale = 2.0 / (double)nI;
@@ -1567,10 +1626,6 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     ddxy.upload(c->f_dxy.data(), c->f_dxy.size(), s);
     dblocks.upload(c->f_blocks.data(), c->f_blocks.size(), s);
     Ld.alloc((size_t)c->f_ncombo * g.Nz);
-    DBuf<float> dH, zeros;
-    dH.alloc((size_t)nt * 3 * npts);
-    zeros.alloc((size_t)td.n_tracks * td.n_steps);
-    zeros.zero(s);
     clock.mark(1);
     DBuf<double> dCn, dKt, T, tmp, dP, Sh, Ah, Om, Mm, cm, dz, dQ, dQq, dgv, dqi;
     // parameters 0..3 (s_R, s_B, r, lambda), or 4: the node-resistivity direction delta
@@ -1693,25 +1748,23 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
         // field and current tangents
         DBuf<double> dUb;
         DBuf<float> dW;
+        DBuf<double> dWd;
         int dr = 0;
         double dtr = 0.0;
-        compress_history(c, dQq.p, nt, dUb, dW, dr, dtr);
+        compress_history(c, dQq.p, nt, dUb, dW, dWd, dr, dtr);
         clock.mark(4);
         c->info.grad_trunc_rel = std::max(c->info.grad_trunc_rel, dtr);
-        extend32_basis(c, dUb.p, dr, dW.p, nt, dH.p, s, 0, &launches, false);
-        eq1_run(c, dH.p, false, td, dI.p, s);
+        field_currents(dUb.p, dr, dW.p, dWd.p, 0, dI.p, nullptr);
         float* dIo = (dI_out && p < 4) ? dI_out + (size_t)p * nI : nullptr;
         if (dIo) WT_CUDA(cudaMemcpyAsync(dIo, dI.p, nI * sizeof(float), cudaMemcpyDeviceToDevice, s));
         double acc = dot_f32(s, I.p, dI.p, nI, c->d_scr.p);
         if (p == 3) {
             // derivative of the field operator itself, and of the lateral velocities
-            extend32_basis(c, c->Ub.p, c->rank, c->W32.p, nt, dH.p, s, 1, &launches, false);
-            eq1_run(c, dH.p, false, td, dI.p, s);
+            field_currents(c->Ub.p, c->rank, c->W32.p, c->W64.p, 1, dI.p, nullptr);
             acc += dot_f32(s, I.p, dI.p, nI, c->d_scr.p);
             if (dIo) add_f32(s, nI, dI.p, dIo);
-            eq1_run(c, c->stage32.p, false, td, dI.p, s, zeros.p);
-            acc += dot_f32(s, I.p, dI.p, nI, c->d_scr.p);
-            if (dIo) add_f32(s, nI, dI.p, dIo);
+            acc += dot_f32(s, I.p, I0.p, nI, c->d_scr.p);
+            if (dIo) add_f32(s, nI, I0.p, dIo);
         }
         grad[p - p_first] = gscale * acc;
         clock.mark(5);

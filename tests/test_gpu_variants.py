@@ -65,3 +65,46 @@ def test_gradient_with_many_time_samples(env, n_t):
     r = w.columns[0].radius * np.array([0, 0, 1, 0]) + np.array([1, 1, 0, 1])
     scale = np.max(np.abs(fd * r))
     assert np.max(np.abs(g - fd) * r) < 1e-4 * scale        # the bound of the derivative's other tests
+
+
+@pytest.mark.parametrize("order", [0, 1, 2, 3, 4, 5, 20])
+@pytest.mark.parametrize("n_tracks,n", [(3, 1), (3, 33), (2, 300), (6000, 33), (2100, 200), (9000, 64)])
+def test_shaping_forms(env, order, n_tracks, n):
+    """Tap by tap (few tracks) and by recursion (many), in place, and rows with an infinity or a NaN,
+    which must reach as far as the taps do and no further."""
+    from oracle import electronics as E
+    torch, P, w, s = env
+    dt, tau = 1e-11, 0.7e-11 if order < 3 else 2.3e-11
+    rng = np.random.default_rng(order)
+    i = rng.standard_normal((n_tracks, n)).astype(np.float32)
+    x = torch.tensor(i, device="cuda")
+    v = s.shape(x, dt, tau, order, gain=2.0)
+    rows = np.unique(np.concatenate([[0, n_tracks - 1], rng.integers(0, n_tracks, 8)]))
+    ref = E.shape(i[rows], dt, tau, order, gain=2.0)
+    # FP32 rounding of the result: 2^-24 of each value
+    got = v[torch.tensor(rows, device="cuda")].cpu().numpy()
+    assert np.linalg.norm(got - ref) <= 1e-7 * np.linalg.norm(ref)      # one sample of order > 0: zero
+    bad = x.clone()
+    bad[0, n // 2] = float("inf")
+    bad[-1, 0] = float("nan")
+    alone = s.shape(bad[[0, n_tracks - 1]].contiguous(), dt, tau, order, gain=2.0)
+    many = s.shape(bad, dt, tau, order, gain=2.0)
+    assert torch.equal(many[1:-1], v[1:-1])
+    assert torch.allclose(many[[0, n_tracks - 1]], alone, rtol=1e-6, atol=0.0, equal_nan=True)
+    y = bad.clone()
+    s.shape(y, dt, tau, order, gain=2.0, out=y)
+    assert torch.equal(torch.nan_to_num(y), torch.nan_to_num(many))
+
+
+@pytest.mark.parametrize("n_tracks,n_steps", [(2000, 60), (700, 100), (1, 33)])
+def test_eq1_on_the_field_staged_and_not(env, n_tracks, n_steps):
+    """The staged form (large calls) and the one-kernel form (the allocation-free call) interpolate and
+    sum in the same order: equal bits."""
+    torch, P, w, s = env
+    H = s.extend("fp32")
+    tr = device_tracks(W.configs.mip_tracks(w.grid, n_tracks, n_steps, np.random.default_rng(1)), torch)
+    a = s.eq1(H, tr)
+    b = torch.empty_like(a)
+    P.wt_eq1_noalloc(s.ctx, H, tr, b)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
