@@ -599,32 +599,88 @@ static void residues(cudaStream_t s, const double* X, int ld, bool trans, int ro
 
 }  // namespace tcg
 
-static thread_local DenseScratch* t_scratch = nullptr;
-DenseScratch::DenseScratch(int* err) : d_err(err), outer(t_scratch) { t_scratch = this; }
-DenseScratch::~DenseScratch() {
-    t_scratch = outer;
-    if (p) cudaFree(p);
+static thread_local CallMemory* t_memory = nullptr;
+CallMemory::CallMemory(int* err) : d_err(err), outer(t_memory) { t_memory = this; }
+CallMemory::~CallMemory() {
+    t_memory = outer;
+    if (ws) cudaFree(ws);
+    for (void* c : chunks) cudaFree(c);
 }
-unsigned char* DenseScratch::get(size_t bytes) {
-    if (bytes <= cap) return p;
+CallMemory* CallMemory::current() { return t_memory; }
+unsigned char* CallMemory::products(size_t bytes) {
+    if (bytes <= ws_cap) return ws;
     if (fault_enabled("alloc")) return nullptr;
-    if (p) cudaFree(p);                          // waits for the products that still use it
-    p = nullptr;
-    cap = 0;
-    if (cudaMalloc(reinterpret_cast<void**>(&p), bytes) != cudaSuccess) {
+    if (ws) cudaFree(ws);                        // waits for the products that still use it
+    ws = nullptr;
+    ws_cap = 0;
+    if (cudaMalloc(reinterpret_cast<void**>(&ws), bytes) != cudaSuccess) {
         cudaGetLastError();
-        p = nullptr;
+        ws = nullptr;
         return nullptr;
     }
-    cap = bytes;
+    ws_cap = bytes;
+    return ws;
+}
+// Best fit among the free pieces, else a chunk of its own size (at least 16 MB, shared by small ones).
+void* CallMemory::take(size_t bytes) {
+    const size_t need = (bytes + 511) & ~(size_t)511;
+    int best = -1;
+    for (size_t k = 0; k < pieces.size(); ++k)
+        if (!pieces[k].used && pieces[k].size >= need && (best < 0 || pieces[k].size < pieces[best].size)) best = (int)k;
+    if (best < 0) {
+        size_t size = std::max(need, (size_t)16 << 20);
+        void* c = nullptr;
+        if (cudaMalloc(&c, size) != cudaSuccess) {
+            // give back the chunks that nothing uses and ask for no more than is needed
+            cudaGetLastError();
+            for (size_t k = 0; k < chunks.size(); ++k) {
+                bool used = !chunks[k];
+                for (const Piece& q : pieces) used = used || (q.chunk == (int)k && q.used);
+                if (used) continue;
+                cudaFree(chunks[k]);
+                chunks[k] = nullptr;
+                pieces.erase(std::remove_if(pieces.begin(), pieces.end(), [&](const Piece& q) { return q.chunk == (int)k; }),
+                             pieces.end());
+            }
+            size = need;
+            if (cudaMalloc(&c, size) != cudaSuccess) {
+                cudaGetLastError();
+                return nullptr;
+            }
+        }
+        chunks.push_back(c);
+        pieces.push_back({static_cast<unsigned char*>(c), size, (int)chunks.size() - 1, false});
+        best = (int)pieces.size() - 1;
+    }
+    Piece& q = pieces[best];
+    const Piece rest{q.p + need, q.size - need, q.chunk, false};
+    q.used = true;
+    q.size = need;
+    void* p = q.p;
+    if (rest.size) pieces.insert(pieces.begin() + best + 1, rest);
     return p;
+}
+void CallMemory::give(void* p) {
+    for (size_t k = 0; k < pieces.size(); ++k) {
+        if (pieces[k].p != p) continue;
+        pieces[k].used = false;
+        if (k + 1 < pieces.size() && !pieces[k + 1].used && pieces[k + 1].chunk == pieces[k].chunk) {
+            pieces[k].size += pieces[k + 1].size;
+            pieces.erase(pieces.begin() + k + 1);
+        }
+        if (k > 0 && !pieces[k - 1].used && pieces[k - 1].chunk == pieces[k].chunk) {
+            pieces[k - 1].size += pieces[k].size;
+            pieces.erase(pieces.begin() + k);
+        }
+        return;
+    }
 }
 
 // True when the product was launched; false: the caller's FP64 kernel takes it.
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only) {
     using namespace tcg;
-    DenseScratch* ws = t_scratch;
+    CallMemory* ws = t_memory;
     if (!ws || !ws->d_err || std::fabs(alpha) != 1.0) return false;
     // op(A) rows and op(B) columns that are the same vectors are converted once
     const bool same = A == B && lda == ldb && ta != tb && M == N;
@@ -637,7 +693,7 @@ bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alph
     const size_t b_e = up((size_t)(M + N) * 4), b_s = up((size_t)(M + N) * 8);
     const size_t b_a = up((size_t)NMOD * M * Kp * 2), b_b = same ? 0 : up((size_t)NMOD * N * Kp * 2);
     const size_t b_t = up((size_t)NMOD * M * Tp);
-    unsigned char* p = ws->get(b_e + b_s + b_a + b_b + b_t);
+    unsigned char* p = ws->products(b_e + b_s + b_a + b_b + b_t);
     if (!p) return false;
     unsigned* ea = reinterpret_cast<unsigned*>(p);
     unsigned* eb = same ? ea : ea + M;

@@ -941,8 +941,8 @@ __global__ void __launch_bounds__(kWyBlock) wy_t_kernel(const double* __restrict
 // Eigendecomposition of the symmetric A (n x n row-major, destroyed): w ascending, V columns.
 void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err) {
     if (n <= 0) return;
-    DBuf<double> d, e, tau, vk, p;
-    DBuf<unsigned> bar;
+    TBuf<double> d, e, tau, vk, p;
+    TBuf<unsigned> bar;
     d.alloc(n);
     e.alloc(n);
     tau.alloc(n);
@@ -1009,34 +1009,32 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
     std::sort(leaves.begin(), leaves.end());
     const int n_leaves = (int)leaves.size();
     leaves.push_back(n);
-    DBuf<double> lamA, lamB, QA, QB, G;
+    TBuf<double> lamA, lamB, QA, QB, G;
     lamA.alloc(n);
     lamB.alloc(n);
     QA.alloc((size_t)n * n);
     QA.zero(s);
     if (!splits.empty()) {
-        DBuf<int> dsp;
+        TBuf<int> dsp;
         dsp.upload(splits.data(), splits.size(), s);
         dc_split_kernel<<<1, 32, 0, s>>>(d.p, e.p, dsp.p, (int)splits.size());
         WT_LAUNCH("dc_split");
-        WT_CUDA(cudaStreamSynchronize(s));
     }
     {
-        DBuf<int> dst;
+        TBuf<int> dst;
         dst.upload(leaves.data(), leaves.size(), s);
         dc_leaf_kernel<<<(n_leaves + 3) / 4, 128, 0, s>>>(d.p, e.p, dst.p, n_leaves, n, lamA.p, QA.p, d_err);
         WT_LAUNCH("dc_leaf");
-        WT_CUDA(cudaStreamSynchronize(s));
     }
     if (!levels.empty()) {
         QB.alloc((size_t)n * n);
         G.alloc((size_t)n * n);
         QB.zero(s);
-        DBuf<int> ibuf;
-        DBuf<double> fbuf;
+        TBuf<int> ibuf;
+        TBuf<double> fbuf;
         ibuf.alloc((size_t)n * 8);
         fbuf.alloc((size_t)n * 12);
-        DBuf<double> WT, zbuf;
+        TBuf<double> WT, zbuf;
         WT.alloc((size_t)n * n);
         zbuf.alloc(n);
         const size_t nn = n;
@@ -1060,7 +1058,7 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         Wk.defl_val = fbuf.p + 8 * nn;
         Wk.lam_out = fbuf.p + 9 * nn;
         Wk.node_r = fbuf.p + 10 * nn;
-        DBuf<DcNode> dnodes;
+        TBuf<DcNode> dnodes;
         std::vector<DcNode> all;
         std::vector<size_t> level_at;
         for (const auto& nodes : levels) {
@@ -1122,7 +1120,7 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
     double* Z = QA.p;
     const int nref = std::max(0, n - 2);
     if (nref > 0) {
-        DBuf<double> Wt, S, T, Y, Y2;
+        TBuf<double> Wt, S, T, Y, Y2;
         const int nblk = (nref + kWyBlock - 1) / kWyBlock;
         constexpr size_t tt = (size_t)kWyBlock * kWyBlock;
         Wt.alloc((size_t)nref * n);

@@ -183,7 +183,7 @@ void green_pblocks(cudaStream_t s, const void* blocks, const void* hblocks, int 
     const PBlock* hb = static_cast<const PBlock*>(hblocks);
     if ((double)nc * max_cols * Nz > 6e7) {        // above 100 us a column on the CUDA cores
         const int n_tg = n_blocks / n_cols;
-        DBuf<double> X;
+        TBuf<double> X;
         X.alloc((size_t)nc * Nz);
         const int pieces = (int)std::max<size_t>(1, std::min<size_t>(64, ((size_t)max_rows * Nz + 1023) / 1024));
         for (int k = 0; k < n_cols; ++k) {
@@ -193,7 +193,6 @@ void green_pblocks(cudaStream_t s, const void* blocks, const void* hblocks, int 
             dgemm(s, false, true, nc, hb[k].ncol, Nz, 1.0, X.p, Nz, Cs + (size_t)hb[k].cs0 * Nz, Nz, 0.0,
                   P + hb[k].col0, ldp);
         }
-        WT_CUDA(cudaStreamSynchronize(s));         // X goes out of scope
         return;
     }
     dim3 grid((max_cols + 63) / 64, (max_rows + 63) / 64, n_blocks);

@@ -193,7 +193,7 @@ wt_status run(wt_ctx* ctx, const char* fn, F&& body) {
             cudaError_t e = cudaSetDevice(ctx->dev);
             if (e != cudaSuccess) fail(WT_ERR_CUDA, std::string("cudaSetDevice: ") + cudaGetErrorString(e));
         }
-        DenseScratch scratch(ctx ? ctx->d_err.p : nullptr);
+        CallMemory memory(ctx ? ctx->d_err.p : nullptr);
         body();
         if (ctx) ctx->err.clear();
         return WT_OK;
@@ -324,26 +324,6 @@ void build_layout(wt_ctx* c) {
             for (int j = c->col_off[k]; j < c->col_off[k + 1]; ++j) c->phi_dc[j] = c->opts.v_w;
 }
 
-// H M H for symmetric M (n x n, in place), H = I - beta v v^T.
-void householder_two_sided(wt_ctx* c, double* M, int n) {
-    DBuf<double> u;
-    u.alloc(n);
-    dgemv(c->s, false, n, n, 1.0, M, n, c->hv.p, 0.0, u.p);
-    std::vector<double> hu(n), hv(n);
-    u.download(hu.data(), n, c->s);
-    c->hv.download(hv.data(), n, c->s);
-    WT_CUDA(cudaStreamSynchronize(c->s));
-    double gamma = 0;
-    for (int i = 0; i < n; ++i) gamma += hv[i] * hu[i];
-    std::vector<double> w(n);
-    for (int i = 0; i < n; ++i) w[i] = c->beta * hu[i] - 0.5 * c->beta * c->beta * gamma * hv[i];
-    DBuf<double> dw;
-    dw.upload(w.data(), n, c->s);
-    rank1(c->s, n, n, -1.0, c->hv.p, dw.p, M, n);
-    rank1(c->s, n, n, -1.0, dw.p, c->hv.p, M, n);
-    WT_CUDA(cudaStreamSynchronize(c->s));
-}
-
 void do_fit(wt_ctx* c) {
     auto t0 = clk::now();
     validate_geometry(c);
@@ -358,7 +338,8 @@ void do_fit(wt_ctx* c) {
     clear_err(c);
 
     // --- S2: fundamental-solution tables and the fit matrix P
-    DBuf<double> T, L, dxy, Ct, Cs, zc_all, zs_all, P;
+    TBuf<double> T, L, dxy, Ct, Cs, zc_all, zs_all;
+    DBuf<double> P, dcol, G;                       // kept by the context
     T.alloc((size_t)(g.Nx / 2) * (g.Ny / 2) * g.Nz);
     green_invk2(s, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, T.p);
     const int n_tg = ncol * n_az;                  // target lateral groups
@@ -416,7 +397,7 @@ void do_fit(wt_ctx* c) {
     c->f_ncombo = n_combo;
     c->f_maxrows = max_rows;
     c->f_maxcols = max_cols;
-    DBuf<unsigned char> dblocks;
+    TBuf<unsigned char> dblocks;
     dblocks.upload(blocks.data(), blocks.size(), s);
     P.alloc((size_t)nc * ns);
     green_pblocks(s, dblocks.p, blocks.data(), n_combo, ncol, nc, max_rows, max_cols, Ct.p, Cs.p, L.p, g.Nz, c->pref, P.p, ns);
@@ -429,7 +410,7 @@ void do_fit(wt_ctx* c) {
     for (double x : hv) vtv += x * x;
     c->beta = 2.0 / vtv;
     c->hv.upload(hv.data(), ns, s);
-    DBuf<double> w, dcol;
+    TBuf<double> w;
     w.alloc(nc);
     dgemv(s, false, nc, ns, 1.0, P.p, ns, c->hv.p, 0.0, w.p);
     rank1(s, nc, ns, -c->beta, w.p, c->hv.p, P.p, ns);     // P H
@@ -450,25 +431,25 @@ void do_fit(wt_ctx* c) {
     scale_columns(s, P.p, nc, ns, ns, dcol.p);               // A_s = A D
 
     // normal matrix G = A_s^T A_s (+ ridge on the charge part)
-    DBuf<double> G, R, Y;
+    TBuf<double> R, Y;
     G.alloc((size_t)ns * ns);
     dgemm(s, true, false, ns, ns, nc, 1.0, P.p, ns, P.p, ns, 0.0, G.p, ns, true);
     symmetrize_from_lower(s, G.p, ns, ns);
     if (c->opts.tikhonov > 0.0) {
         std::vector<double> ridge(ns, 0.0);
         for (int k = 1; k < ns; ++k) ridge[k] = c->opts.tikhonov * max_sq * hd[k] * hd[k];
-        DBuf<double> dr;
+        TBuf<double> dr;
         dr.upload(ridge.data(), ns, s);
         // G[k][k] += ridge[k]: a rank-1 of diagonal form via a strided axpy
-        DBuf<double> diag;
+        TBuf<double> diag;
         diag.alloc(ns);
         get_diag(s, G.p, ns, ns, diag.p);
         axpy(s, ns, 1.0, dr.p, diag.p);
         copy_block(s, diag.p, 1, G.p, ns + 1, ns, 1);
     }
     // right-hand sides R = A_s^T S
-    DBuf<int> sp, si;
-    DBuf<double> sw;
+    TBuf<int> sp, si;
+    TBuf<double> sw;
     sp.upload(c->s_ptr.data(), c->s_ptr.size(), s);
     si.upload(c->s_idx.data(), c->s_idx.size(), s);
     sw.upload(c->s_w.data(), c->s_w.size(), s);
@@ -507,7 +488,7 @@ void do_fit(wt_ctx* c) {
         for (int j = 0; j < ns; ++j)
             for (int e = c->s_ptr[j]; e < c->s_ptr[j + 1]; ++e)
                 for (int k = 0; k < kp; ++k) hsz[(size_t)c->s_idx[e] * kp + k] += c->s_w[e] * hz[(size_t)j * kp + k];
-        DBuf<double> Z, Yz, Rz, Cz;
+        TBuf<double> Z, Yz, Rz, Cz;
         Z.upload(hz.data(), hz.size(), s);
         Rz.upload(hsz.data(), hsz.size(), s);                    // S Z
         Yz.alloc((size_t)ns * kp);
@@ -523,7 +504,7 @@ void do_fit(wt_ctx* c) {
         refine = !(correction <= kRefineSkip);
     }
     if (refine) {
-        DBuf<double> Res;
+        TBuf<double> Res;
         Res.alloc((size_t)nc * ns);
         dgemm(s, false, false, nc, ns, ns, -1.0, P.p, ns, Y.p, ns, 0.0, Res.p, ns);
         fit_add_s(s, Res.p, ns, ns, sp.p, si.p, sw.p, 1.0);
@@ -538,7 +519,7 @@ void do_fit(wt_ctx* c) {
     c->info.fit_refined = refine ? 1 : 0;
     // DC boundary residual || A_s (Y phi) - S phi || / || S phi ||
     {
-        DBuf<double> dphi, yphi, r;
+        TBuf<double> dphi, yphi, r;
         dphi.upload(c->phi_dc.data(), ns, s);
         yphi.alloc(ns);
         r.alloc(nc);
@@ -555,7 +536,7 @@ void do_fit(wt_ctx* c) {
     }
     // condition estimate from the Cholesky diagonal of the scaled normal matrix
     {
-        DBuf<double> dg;
+        TBuf<double> dg;
         dg.alloc(ns);
         get_diag(s, G.p, ns, ns, dg.p);
         std::vector<double> h(ns);
@@ -575,7 +556,7 @@ void do_fit(wt_ctx* c) {
     c->offset.alloc(ns);
     copy_block(s, Y.p, ns, c->offset.p, ns, 1, ns);
     fill(s, Y.p, ns, 0.0);
-    DBuf<double> u;
+    TBuf<double> u;
     u.alloc(ns);
     dgemv(s, true, ns, ns, 1.0, Y.p, ns, c->hv.p, 0.0, u.p);
     rank1(s, ns, ns, -c->beta, c->hv.p, u.p, Y.p, ns);      // F in Y
@@ -599,7 +580,7 @@ void do_fit(wt_ctx* c) {
 void charges_at(wt_ctx* c, const double* d_t, int nt, double* Q) {
     cudaStream_t s = c->s;
     const int ns = c->ns, n1 = ns - 1;
-    DBuf<double> E, Zf, vz;
+    TBuf<double> E, Zf, vz;
     E.alloc((size_t)n1 * nt);
     modal_factors(s, c->amp.p, c->mu.p, n1, d_t, nt, E.p);
     Zf.alloc((size_t)ns * nt);
@@ -638,8 +619,8 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     const int ns = c->ns;
     const bool pre = ns >= nt && qrcp_fits(ns, nt);      // column-pivoted QR first
     clear_err(c);
-    DBuf<double> A, V, sig, Rm;
-    DBuf<int> dpiv;
+    TBuf<double> A, V, sig, Rm;
+    TBuf<int> dpiv;
     int nr = nt;                                  // rows of R that are not negligible
     A.alloc((size_t)nt * ns);
     transpose(s, Q, ns, nt, A.p);                 // rows = time samples (the columns of Q)
@@ -725,15 +706,15 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
         scale[m] = sg > 0 ? 1.0 / sg : 0.0;
         for (int n = 0; n < nt; ++n) coef[(size_t)n * rp + m] = sg * hv[(size_t)ord[m] * nt + n];
     }
-    DBuf<int> didx;
-    DBuf<double> dscale;
+    TBuf<int> didx;
+    TBuf<double> dscale;
     Ub.alloc((size_t)r * ns);
     if (pre) {
         // u_m = Q v_m / sigma_m: Ub [r][ns] = (V_r / sigma) Q^T
         std::vector<double> vr((size_t)r * nt);
         for (int m = 0; m < r; ++m)
             for (int n = 0; n < nt; ++n) vr[(size_t)m * nt + n] = hv[(size_t)idx[m] * nt + n] * scale[m];
-        DBuf<double> dvr;
+        TBuf<double> dvr;
         dvr.upload(vr.data(), vr.size(), s);
         dgemm(s, false, true, r, ns, nt, 1.0, dvr.p, nt, Q, nt, 0.0, Ub.p, ns);
         WT_CUDA(cudaStreamSynchronize(s));
@@ -791,7 +772,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     c->k_k1 = k1;
     double s1 = 0;
     for (double x : k1) s1 += x;
-    DBuf<double> dd, doff, dk1, K, Am, Sm;
+    TBuf<double> dd, doff, dk1, K, Am, Sm;
     dd.upload(diag.data(), ns, s);
     doff.upload(off.data(), ns, s);
     dk1.upload(k1.data(), ns, s);
@@ -799,11 +780,11 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     build_k(s, dd.p, doff.p, ns, K.p);
     rank1(s, ns, ns, -1.0 / s1, dk1.p, dk1.p, K.p, ns);     // K~ = K - K1 1^T K / (1^T K 1)
     // reduced pencil on the neutral subspace: Am = (H Cn H)[1:,1:], Sm = -(H K~ H)[1:,1:]
-    DBuf<double> HC;
+    TBuf<double> HC;
     HC.alloc((size_t)ns * ns);
     copy_block(s, c->Cn.p, ns, HC.p, ns, ns, ns);
-    householder_two_sided(c, HC.p, ns);
-    householder_two_sided(c, K.p, ns);
+    householder_both(s, HC.p, ns, c->hv.p, c->beta);
+    householder_both(s, K.p, ns, c->hv.p, c->beta);
     Am.alloc((size_t)n1 * n1);
     Sm.alloc((size_t)n1 * n1);
     copy_block(s, HC.p + ns + 1, ns, Am.p, n1, n1, n1);
@@ -812,7 +793,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     K.release();
     dscal(s, (size_t)n1 * n1, -1.0, Sm.p);                  // Sm = -B^T K~ B
     {
-        DBuf<double> tmp;
+        TBuf<double> tmp;
         tmp.alloc((size_t)n1 * n1);
         symmetrize_avg(s, Am.p, tmp.p, n1);
         copy_block(s, tmp.p, n1, Am.p, n1, n1, n1);
@@ -823,7 +804,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     cholesky(s, Am.p, n1, n1, c->d_err.p);
     if (read_err(c)) fail(WT_ERR_NOT_SPD, "fitted capacitance is not positive definite on the neutral subspace");
     // Shat = L^-1 Sm L^-T (symmetric positive definite)
-    DBuf<double> Y, Yt;
+    TBuf<double> Y, Yt;
     Y.alloc((size_t)n1 * n1);
     Yt.alloc((size_t)n1 * n1);
     copy_block(s, Sm.p, n1, Y.p, n1, n1, n1);
@@ -832,7 +813,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     trsm_lower(s, Am.p, n1, n1, Yt.p, n1, n1);
     symmetrize_avg(s, Yt.p, Y.p, n1);
     c->mu.alloc(n1);
-    DBuf<double> U;
+    TBuf<double> U;
     U.alloc((size_t)n1 * n1);
     // modes: tridiagonalisation + divide and conquer; WT_EIGEN=jacobi selects the two-sided
     // Jacobi solver instead (a cross-check)
@@ -855,7 +836,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     c->info.mu_min = mn;
     c->info.mu_max = mx;
     // q_inf = Cn phi_DC; amplitudes amp = V^T B^T (-q_inf)
-    DBuf<double> dphi, g;
+    TBuf<double> dphi, g;
     dphi.upload(c->phi_dc.data(), ns, s);
     c->qinf.alloc(ns);
     dgemv(s, false, ns, ns, 1.0, c->Cn.p, ns, dphi.p, 0.0, c->qinf.p);
@@ -881,7 +862,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     }
     if (!c->ev_noalloc) WT_CUDA(cudaEventCreateWithFlags(&c->ev_noalloc, cudaEventDisableTiming));
     c->d_times.upload(t, nt, s);
-    DBuf<double> Q;
+    TBuf<double> Q;
     Q.alloc((size_t)ns * nt);
     charges_at(c, c->d_times.p, nt, Q.p);
     c->Qt.alloc((size_t)nt * ns);
@@ -1190,7 +1171,7 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
         if (!(t[i] >= 0.0) || !std::isfinite(t[i])) fail(WT_ERR_ARG, "sample times must be finite and >= 0");
     for (int i = 0; i < 3 * n; ++i)
         if (!std::isfinite(xyz[i])) fail(WT_ERR_NAN, "non-finite sample point");
-    DBuf<double> dt_, Q, Qt, Zc, T, Lat, pts, o;
+    TBuf<double> dt_, Q, Qt, Zc, T, Lat, pts, o;
     dt_.upload(t, nt, s);
     Q.alloc((size_t)ns * nt);
     charges_at(c, dt_.p, nt, Q.p);
@@ -1209,8 +1190,8 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
         if (hcu[k] == (int)hux.size()) hux.push_back(x);
     }
     const int nux = (int)hux.size();
-    DBuf<double> ux, F, G;
-    DBuf<int> cu;
+    TBuf<double> ux, F, G;
+    TBuf<int> cu;
     ux.upload(hux.data(), nux, s);
     cu.upload(hcu.data(), ncol, s);
     // points per chunk: 512, fewer where their k_x sums would take more than 1 GB
@@ -1423,14 +1404,14 @@ void do_eq1_direct(wt_ctx* c, const wt_tracks* tr, float* iout, cudaStream_t us)
 
 // H M (right Householder product) for M rows x ns, in place.
 void house_right(wt_ctx* c, double* M, int rows) {
-    DBuf<double> w;
+    TBuf<double> w;
     w.alloc(rows);
     dgemv(c->s, false, rows, c->ns, 1.0, M, c->ns, c->hv.p, 0.0, w.p);
     rank1(c->s, rows, c->ns, -c->beta, w.p, c->hv.p, M, c->ns);
 }
 // H M (left Householder product) for M ns x cols, in place.
 void house_left(wt_ctx* c, double* M, int cols) {
-    DBuf<double> u;
+    TBuf<double> u;
     u.alloc(cols);
     dgemv(c->s, true, c->ns, cols, 1.0, M, cols, c->hv.p, 0.0, u.p);
     rank1(c->s, c->ns, cols, -c->beta, c->hv.p, u.p, M, cols);
@@ -1592,8 +1573,8 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     clock.mark(0);
 
     // shared pieces: fit residual, modal factors, inverse gaps, potentials Phi(t)
-    DBuf<int> sp, si;
-    DBuf<double> sw, Rs, E, AE, ones, invg, Phi, dphi;
+    TBuf<int> sp, si;
+    TBuf<double> sw, Rs, E, AE, ones, invg, Phi, dphi;
     sp.upload(c->s_ptr.data(), c->s_ptr.size(), s);
     si.upload(c->s_idx.data(), c->s_idx.size(), s);
     sw.upload(c->s_w.data(), c->s_w.size(), s);
@@ -1615,8 +1596,8 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     dphi.upload(c->phi_dc.data(), ns, s);
     add_row_const(s, Phi.p, ns, nt, dphi.p);
     // tables for the derivative of the fit matrix
-    DBuf<double> zc_all, zs_all, Ct, Cs, ddxy, duxy, Ld;
-    DBuf<unsigned char> dblocks;
+    TBuf<double> zc_all, zs_all, Ct, Cs, ddxy, duxy, Ld;
+    TBuf<unsigned char> dblocks;
     zc_all.upload(c->f_hzc.data(), c->f_hzc.size(), s);
     zs_all.upload(c->src_z.data(), ns, s);
     Ct.alloc(c->f_hzc.size() * g.Nz);
@@ -1627,7 +1608,7 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     dblocks.upload(c->f_blocks.data(), c->f_blocks.size(), s);
     Ld.alloc((size_t)c->f_ncombo * g.Nz);
     clock.mark(1);
-    DBuf<double> dCn, dKt, T, tmp, dP, Sh, Ah, Om, Mm, cm, dz, dQ, dQq, dgv, dqi;
+    TBuf<double> dCn, dKt, T, tmp, dP, Sh, Ah, Om, Mm, cm, dz, dQ, dQq, dgv, dqi;
     // parameters 0..3 (s_R, s_B, r, lambda), or 4: the node-resistivity direction delta
     const int p_first = delta ? 4 : 0, p_last = delta ? 4 : 3;
     for (int p = p_first; p <= p_last; ++p) {
@@ -1690,7 +1671,7 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
             }
             double s1 = 0, ds1 = 0;
             for (int j = 0; j < ns; ++j) { s1 += c->k_k1[j]; ds1 += dk1[j]; }
-            DBuf<double> d_dd, d_doff, d_dk1, d_k1;
+            TBuf<double> d_dd, d_doff, d_dk1, d_k1;
             d_dd.upload(dd.data(), ns, s);
             d_doff.upload(doff.data(), ns, s);
             d_dk1.upload(dk1.data(), ns, s);
@@ -1708,17 +1689,17 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
         Sh.alloc((size_t)n1 * n1);
         Sh.zero(s);
         if (has_dk) {
-            householder_two_sided(c, dKt.p, ns);
+            householder_both(s, dKt.p, ns, c->hv.p, c->beta);
             dgemm(s, false, false, n1, n1, n1, -1.0, dKt.p + ns + 1, ns, c->Vm.p, n1, 0.0, tmp.p, n1);   // dS_m V
             dgemm(s, true, false, n1, n1, n1, 1.0, c->Vm.p, n1, tmp.p, n1, 0.0, Sh.p, n1);
         }
         Ah.alloc((size_t)n1 * n1);
         Ah.zero(s);
         if (has_dc) {
-            DBuf<double> HC;
+            TBuf<double> HC;
             HC.alloc((size_t)ns * ns);
             copy_block(s, dCn.p, ns, HC.p, ns, ns, ns);
-            householder_two_sided(c, HC.p, ns);
+            householder_both(s, HC.p, ns, c->hv.p, c->beta);
             dgemm(s, false, false, n1, n1, n1, 1.0, HC.p + ns + 1, ns, c->Vm.p, n1, 0.0, tmp.p, n1);
             dgemm(s, true, false, n1, n1, n1, 1.0, c->Vm.p, n1, tmp.p, n1, 0.0, Ah.p, n1);
         }

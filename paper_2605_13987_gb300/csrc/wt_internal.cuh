@@ -112,28 +112,85 @@ struct DBuf {
     }
 };
 
+// Device memory of one library call: made by the C entry points, found through the calling thread,
+// given back when the call returns.  It serves the workspace of the tensor-core products (one, shared
+// by the products of a call in turn) and the call's temporaries (TBuf).  All of it is used on the
+// context's stream only, so that memory given back within the call can be handed out again at once;
+// cudaMalloc and cudaFree for each temporary cost the host 20 us apiece and a wait for the GPU (a
+// hundred of them in a fit and a relaxation).
+struct CallMemory {
+    int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
+    int n_sm = 0;                    // SMs of the device (0: not asked yet)
+    explicit CallMemory(int* err);
+    ~CallMemory();
+    CallMemory(const CallMemory&) = delete;
+    CallMemory& operator=(const CallMemory&) = delete;
+    static CallMemory* current();
+    unsigned char* products(size_t bytes);   // the products' workspace; NULL when the memory is not to be had
+    void* take(size_t bytes);                // a temporary; NULL when the memory is not to be had
+    void give(void* p);
+private:
+    struct Piece {
+        unsigned char* p;
+        size_t size;
+        int chunk;
+        bool used;
+    };
+    std::vector<Piece> pieces;               // by chunk, then by address
+    std::vector<void*> chunks;
+    unsigned char* ws = nullptr;
+    size_t ws_cap = 0;
+    CallMemory* outer;
+};
+
+// Temporary device buffer of one call, used on the context's stream only (DBuf's interface).
+template <class T>
+struct TBuf {
+    T* p = nullptr;
+    size_t n = 0;
+    TBuf() = default;
+    TBuf(const TBuf&) = delete;
+    TBuf& operator=(const TBuf&) = delete;
+    ~TBuf() { release(); }
+    void release() {
+        if (p) {
+            if (owner) owner->give(p);
+            else cudaFree(p);
+        }
+        p = nullptr;
+        n = 0;
+    }
+    void alloc(size_t count) {
+        if (count == n && p) return;
+        release();
+        if (count == 0) return;
+        if (fault_enabled("alloc")) fail(WT_ERR_OOM, "injected allocation failure (WT_FAULT=alloc)");
+        owner = CallMemory::current();
+        void* q = nullptr;
+        if (owner) q = owner->take(count * sizeof(T));
+        else if (cudaMalloc(&q, count * sizeof(T)) != cudaSuccess) { cudaGetLastError(); q = nullptr; }
+        if (!q) fail(WT_ERR_OOM, "device allocation of " + std::to_string(count * sizeof(T)) + " bytes failed");
+        p = static_cast<T*>(q);
+        n = count;
+    }
+    void zero(cudaStream_t s) { if (n) WT_CUDA(cudaMemsetAsync(p, 0, n * sizeof(T), s)); }
+    void upload(const T* host, size_t count, cudaStream_t s) {
+        alloc(count);
+        if (count) WT_CUDA(cudaMemcpyAsync(p, host, count * sizeof(T), cudaMemcpyHostToDevice, s));
+    }
+    void download(T* host, size_t count, cudaStream_t s) const {
+        if (count) WT_CUDA(cudaMemcpyAsync(host, p, count * sizeof(T), cudaMemcpyDeviceToHost, s));
+    }
+private:
+    CallMemory* owner = nullptr;
+};
+
 // ---------------------------------------------------------------- dense FP64
 // Row-major matrices.  op(A) is M x K, op(B) is K x N, C is M x N.  lower_only: entries above the
 // diagonal of C are left as they are.  Large products run on the tensor cores (fp64_cores: never).
 void dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
            const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
            bool lower_only = false, bool fp64_cores = false);
-// Device workspace of the tensor-core products of one library call: made by the C entry points,
-// found by dgemm through the calling thread, freed when the call returns.  Products of one call
-// run on one stream, so they share it in turn.
-struct DenseScratch {
-    int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
-    explicit DenseScratch(int* err);
-    ~DenseScratch();
-    DenseScratch(const DenseScratch&) = delete;
-    DenseScratch& operator=(const DenseScratch&) = delete;
-    unsigned char* get(size_t bytes);     // NULL when the memory is not to be had
-    int n_sm = 0;                    // SMs of the device (0: not asked yet)
-private:
-    unsigned char* p = nullptr;
-    size_t cap = 0;
-    DenseScratch* outer;
-};
 // dgemm on the tensor cores (k_dgemm_tc.cu); false when it does not take the product.
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only);
@@ -183,6 +240,8 @@ double dnrm2(cudaStream_t s, const double* x, size_t n, double* d_scratch);
 void fill(cudaStream_t s, double* x, size_t n, double v);
 void axpy(cudaStream_t s, size_t n, double a, const double* x, double* y);
 void dscal(cudaStream_t s, size_t n, double a, double* x);
+// M (n x n, symmetric) <- H M H, H = I - beta v v^T (v: device)
+void householder_both(cudaStream_t s, double* M, int n, const double* v, double beta);
 // A[i][j] += alpha * u[i] * v[j]
 void rank1(cudaStream_t s, int M, int N, double alpha, const double* u, const double* v, double* A, int lda);
 void copy_block(cudaStream_t s, const double* src, int lds, double* dst, int ldd, int rows, int cols);

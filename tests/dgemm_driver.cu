@@ -45,7 +45,7 @@ int main() {
         std::vector<double> R(C.size());
         bool taken;
         {
-            DenseScratch ws(err.p);
+            CallMemory ws(err.p);
             taken = dgemm_tc(0, ta, tb, M, N, K, -1.0, dA.p, ac, same ? dA.p : dB.p, bc, 1.0, dC.p, ldc, lower);
         }
         dC.download(R.data(), R.size(), 0);
