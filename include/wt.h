@@ -98,7 +98,7 @@ typedef struct {
  * the normal equations, corrected by one step of the semi-normal equations
  * (the residual taken in the collocation space) either always (1) or (0,
  * the default) only when the correction, probed on eight random
- * combinations of the right-hand sides, exceeds 1e-11 of the solution (1e-12
+ * combinations of the right-hand sides, exceeds 1e-11 of the solution (1e-13
  * from 512 sources on)
  * (wt_info.fit_correction, wt_info.fit_refined). */
 typedef struct {

@@ -520,7 +520,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
                                                       const unsigned long long* __restrict__ sa,
                                                       const unsigned* __restrict__ eb,
                                                       const unsigned long long* __restrict__ sb, double scale,
-                                                      double beta, double* __restrict__ C, int ldc, int lower) {
+                                                      double beta, double* __restrict__ C, int ldc, int lower,
+                                                      int mblk, size_t mstride) {
     const int n = 4 * (blockIdx.x * 64 + (threadIdx.x & 63)), m = blockIdx.y * 4 + (threadIdx.x >> 6);
     if (m >= M || n >= N || (lower && n > m)) return;
     constexpr Tables kT = make_tables();
@@ -560,7 +561,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
             else
                 v = scalbn((double)top * scale, h);
         }
-        double* c = C + (size_t)m * ldc + n + e;
+        double* c = C + (mblk ? (size_t)(m / mblk) * mstride + (size_t)(m % mblk) * ldc : (size_t)m * ldc) + n + e;
         *c = beta == 0.0 ? v : fma(beta, *c, v);
     }
 }
@@ -676,32 +677,58 @@ void CallMemory::give(void* p) {
     }
 }
 
-// True when the product was launched; false: the caller's FP64 kernel takes it.
-bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
-              const double* B, int ldb, double beta, double* C, int ldc, bool lower_only) {
+static size_t product_smem() {
+    return 1024 + (size_t)tcg::STAGES * (tcg::A_BYTES + tcg::B_BYTES) + sizeof(tcg::Smem);
+}
+// Shared-memory limit of the product kernel on the current device; returns its SMs.
+static int product_setup() {
+    int dev = 0, n_sm = 0;
+    WT_CUDA(cudaGetDevice(&dev));
+    WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    allow_dyn_smem(tcg::product_kernel, product_smem());
+    return n_sm;
+}
+
+// Workspace layout of one product: scales, residue planes of op(A) and op(B), residues of C.
+struct Layout {
+    bool same;
+    int kc, Kp, Tp;
+    size_t b_e, b_s, b_a, b_b, total;
+};
+static Layout layout(int M, int N, int K, bool same) {
     using namespace tcg;
-    CallMemory* ws = t_memory;
-    if (!ws || !ws->d_err || std::fabs(alpha) != 1.0) return false;
-    // op(A) rows and op(B) columns that are the same vectors are converted once
-    const bool same = A == B && lda == ldb && ta != tb && M == N;
+    Layout L{};
+    L.same = same;
     // terms per pass: residue planes of at most about 6 GB
     const size_t per_k = (size_t)(same ? M : M + N) * NMOD * 2;
-    int kc = K;
-    if (per_k * (size_t)K > ((size_t)6 << 30)) kc = (int)std::max<size_t>(CHUNK, (((size_t)6 << 30) / per_k) / CHUNK * CHUNK);
-    const int Kp = (std::min(K, kc) + 7) & ~7, Tp = (N + 15) & ~15;
+    L.kc = K;
+    if (per_k * (size_t)K > ((size_t)6 << 30))
+        L.kc = (int)std::max<size_t>(CHUNK, (((size_t)6 << 30) / per_k) / CHUNK * CHUNK);
+    L.Kp = (std::min(K, L.kc) + 7) & ~7;
+    L.Tp = (N + 15) & ~15;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t b_e = up((size_t)(M + N) * 4), b_s = up((size_t)(M + N) * 8);
-    const size_t b_a = up((size_t)NMOD * M * Kp * 2), b_b = same ? 0 : up((size_t)NMOD * N * Kp * 2);
-    const size_t b_t = up((size_t)NMOD * M * Tp);
-    unsigned char* p = ws->products(b_e + b_s + b_a + b_b + b_t);
-    if (!p) return false;
+    L.b_e = up((size_t)(M + N) * 4);
+    L.b_s = up((size_t)(M + N) * 8);
+    L.b_a = up((size_t)NMOD * M * L.Kp * 2);
+    L.b_b = same ? 0 : up((size_t)NMOD * N * L.Kp * 2);
+    L.total = L.b_e + L.b_s + L.b_a + L.b_b + up((size_t)NMOD * M * L.Tp);
+    return L;
+}
+
+// The product in workspace p.  mblk > 0: row m of C lies at (m / mblk) mstride + (m % mblk) ldc.
+static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
+                    const double* B, int ldb, double beta, double* C, int ldc, bool lower_only, int mblk, size_t mstride,
+                    const Layout& L, unsigned char* p, int n_sm, int* d_err) {
+    using namespace tcg;
+    const bool same = L.same;
+    const int kc = L.kc, Kp = L.Kp, Tp = L.Tp;
     unsigned* ea = reinterpret_cast<unsigned*>(p);
     unsigned* eb = same ? ea : ea + M;
-    unsigned long long* sa = reinterpret_cast<unsigned long long*>(p + b_e);
+    unsigned long long* sa = reinterpret_cast<unsigned long long*>(p + L.b_e);
     unsigned long long* sb = same ? sa : sa + M;
-    __nv_bfloat16* ra = reinterpret_cast<__nv_bfloat16*>(p + b_e + b_s);
-    __nv_bfloat16* rb = same ? ra : reinterpret_cast<__nv_bfloat16*>(p + b_e + b_s + b_a);
-    signed char* T = reinterpret_cast<signed char*>(p + b_e + b_s + b_a + b_b);
+    __nv_bfloat16* ra = reinterpret_cast<__nv_bfloat16*>(p + L.b_e + L.b_s);
+    __nv_bfloat16* rb = same ? ra : reinterpret_cast<__nv_bfloat16*>(p + L.b_e + L.b_s + L.b_a);
+    signed char* T = reinterpret_cast<signed char*>(p + L.b_e + L.b_s + L.b_a + L.b_b);
     // op(A) rows: k contiguous unless transposed; op(B) columns: k contiguous when transposed.  One
     // conversion launch up to K = kFusedK (2304 x 2304 x 256: 3 launches, 21 us against 9 and 47 us of
     // host time); beyond, 32 rows per block leave SMs idle.
@@ -711,7 +738,7 @@ bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alph
         convert_kernel<<<oa.blocks + (same ? 0 : ob.blocks), 256, 0, s>>>(oa, ob, K, Kp);
         WT_LAUNCH("residues");
     } else {
-        WT_CUDA(cudaMemsetAsync(p, 0, b_e + b_s, s));
+        WT_CUDA(cudaMemsetAsync(p, 0, L.b_e + L.b_s, s));
         scales(s, A, lda, ta, M, K, ea, sa);
         if (!same) scales(s, B, ldb, !tb, N, K, eb, sb);
     }
@@ -721,14 +748,7 @@ bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alph
     U.per_mod = U.tm * U.tn;
     U.n = U.per_mod * NMOD;
     U.lower = lower_only ? 1 : 0;
-    const size_t sh = 1024 + (size_t)STAGES * (A_BYTES + B_BYTES) + sizeof(Smem);
-    if (!ws->n_sm) {                                           // once per call of the library
-        int dev = 0;
-        WT_CUDA(cudaGetDevice(&dev));
-        WT_CUDA(cudaDeviceGetAttribute(&ws->n_sm, cudaDevAttrMultiProcessorCount, dev));
-        allow_dyn_smem(product_kernel, sh);
-    }
-    const int n_sm = ws->n_sm;
+    const size_t sh = product_smem();
     for (int k0 = 0; k0 < K; k0 += kc) {
         const int k1 = std::min(K, k0 + kc);
         if (!fused) {
@@ -739,16 +759,38 @@ bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alph
         encode_planes(&ma, ra, M, k1 - k0, Kp, BM);
         encode_planes(&mb, rb, N, k1 - k0, Kp, BN);
         product_kernel<<<std::min(n_sm, U.n), 64 + 32 * EPI_WARPS, sh, s>>>(ma, mb, U, M, N, k1 - k0, T, Tp, k0 > 0,
-                                                                          ws->d_err);
+                                                                          d_err);
         WT_LAUNCH("residue product");
     }
     unsigned __int128 P = 1;
     for (int m = 0; m < NMOD; ++m) P *= (unsigned)kMod[m];     // 117.4 bits, exact
     combine_kernel<<<dim3((N + 255) / 256, (M + 3) / 4), 256, 0, s>>>(T, Tp, M, N, ea, sa, eb, sb,
                                                                       std::ldexp((double)P, -64) * alpha, beta, C, ldc,
-                                                                      lower_only ? 1 : 0);
+                                                                      lower_only ? 1 : 0, mblk, mstride);
     WT_LAUNCH("residue combine");
+}
+
+// True when the product was launched; false: the caller's FP64 kernel takes it.
+bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
+              const double* B, int ldb, double beta, double* C, int ldc, bool lower_only) {
+    CallMemory* mem = t_memory;
+    if (!mem || !mem->d_err || std::fabs(alpha) != 1.0) return false;
+    // op(A) rows and op(B) columns that are the same vectors are converted once
+    const Layout L = layout(M, N, K, A == B && lda == ldb && ta != tb && M == N);
+    unsigned char* p = mem->products(L.total);
+    if (!p) return false;
+    if (!mem->n_sm) mem->n_sm = product_setup();              // once per call of the library
+    product(s, ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower_only, 0, 0, L, p, mem->n_sm, mem->d_err);
     return true;
+}
+
+// C[m / mblk][m % mblk][n] = sum_k A[k][m] B[n][k] for M = blocks x mblk rows, row block b of C at
+// b mstride: the z series of many lines.  Workspace from the caller (dgemm_tc_rows_bytes).
+size_t dgemm_tc_rows_bytes(int M, int N, int K) { return layout(M, N, K, false).total; }
+void dgemm_tc_rows(cudaStream_t s, int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
+                   int ldc, int mblk, size_t mstride, unsigned char* ws, int* d_err) {
+    product(s, true, true, M, N, K, 1.0, A, lda, B, ldb, 0.0, C, ldc, false, mblk, mstride, layout(M, N, K, false), ws,
+            product_setup(), d_err);
 }
 
 }  // namespace wt

@@ -43,6 +43,11 @@ void expand_simt(cudaStream_t, const float*, int, const float*, int, int, size_t
 void sample_points(cudaStream_t, const double*, int, const double*, const double*, const int*, int, int, int, int, int,
                    double, double, double, double, const double*, const double*, int, double*, double*, double*,
                    double*);
+void t64_build(cudaStream_t, const double*, const int*, const double*, int, int, int, int, int, double, double, double,
+               double, const double*, double*, double*, double*, double*, double*);
+size_t t64_work(int, int, int, int);
+void t64_fields(cudaStream_t, const double*, const double*, const double*, int, int, int, int, int, double*,
+                unsigned char*, int*, double*);
 void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, double, const float*, const float*,
                 const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
                 double, const void*, int, float*, float*, size_t);
@@ -146,6 +151,10 @@ struct wt_ctx {
     DBuf<float> T32, Rsl;
     bool t32_ready = false;
     DBuf<double> Zc64, G64;
+    // FP64 lateral tables ([n_cols][3][Nz][Nx Ny], geometry only; built once), the series matrices and the
+    // products' workspace
+    DBuf<double> T64, CS64;
+    DBuf<unsigned char> ws64;
     DBuf<float> stage32;
     DBuf<double> stage64;
     wt_info info{};
@@ -473,8 +482,8 @@ void do_fit(wt_ctx* c) {
     // ||dY|| / ||Y||, and the full step runs only when that exceeds kRefineSkip, a tenth of the
     // FP64 path's accuracy bound (1e-10): the normal equations alone err by about cond(A_s)^2 eps.
     // From 512 sources on, where the step's products run on the tensor cores (2 304 sources: 14 ms
-    // instead of 350) and round less, so that the estimate itself is smaller, a tenth of that.
-    const double kRefineSkip = ns >= 512 ? 1e-12 : 1e-11;
+    // instead of 350) and round less, so that the estimate itself is smaller, from 1e-13 on.
+    const double kRefineSkip = ns >= 512 ? 1e-13 : 1e-11;
     bool refine = c->opts.refine == 1;
     double correction = 0.0;
     if (!refine) {
@@ -1071,11 +1080,69 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
     if (timing) WT_CUDA(cudaEventRecord(c->ev[3], s));
 }
 
-// FP64 plain path: one spectral transform per time sample into out [nt][3][npts].
+// The tables of the FP64 field: held when they take at most 8 GiB and a quarter of the device's free
+// memory, and worth building from about n_cols N_y / 128 time samples on (their multiply-adds against
+// what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.35 ns per point and sample).
+bool tables64(wt_ctx* c, int nt) {
+    if (c->T64.p) return true;
+    const wt_grid& g = c->grid;
+    const int ncol = (int)c->cols.size();
+    if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;
+    const size_t nxy = (size_t)g.Nx * g.Ny, bytes = (size_t)ncol * 3 * g.Nz * nxy * sizeof(double);
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (bytes > ((size_t)8 << 30) || bytes > fr / 4 || nxy * 3 * g.Nz > (size_t)INT32_MAX / 4) return false;
+    if (t64_work(1, g.Nx, g.Ny, g.Nz) > fr / 8) return false;
+    cudaStream_t s = c->s;
+    std::vector<double> hux, hy(ncol);
+    std::vector<int> hcu(ncol);
+    for (int k = 0; k < ncol; ++k) {
+        hcu[k] = (int)(std::find(hux.begin(), hux.end(), c->cols[k].x) - hux.begin());
+        if (hcu[k] == (int)hux.size()) hux.push_back(c->cols[k].x);
+        hy[k] = c->cols[k].y;
+    }
+    const int nux = (int)hux.size();
+    TBuf<double> ux, cy, F, G, Y, ik2;
+    TBuf<int> cu;
+    ux.upload(hux.data(), nux, s);
+    cy.upload(hy.data(), ncol, s);
+    cu.upload(hcu.data(), ncol, s);
+    F.alloc((size_t)g.Nx * nux * g.Nx);
+    G.alloc((size_t)g.Nx * nux * g.Ny * g.Nz);
+    Y.alloc((size_t)ncol * g.Ny * g.Ny);
+    ik2.alloc((size_t)(g.Nx / 2) * (g.Ny / 2) * g.Nz);
+    green_invk2(s, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, ik2.p);
+    c->CS64.alloc((size_t)2 * g.Nz * g.Nz);
+    c->T64.alloc(bytes / sizeof(double));
+    t64_build(s, ux.p, cu.p, cy.p, ncol, nux, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, c->pref, ik2.p, F.p, G.p, Y.p,
+              c->T64.p, c->CS64.p);
+    WT_CUDA(cudaStreamSynchronize(s));
+    return true;
+}
+
+// FP64 plain path into out [nt][3][npts]: from the lateral tables, several time samples at a time
+// (intermediates of about 1 GB), or by one spectral transform per time sample.
 void extend64(wt_ctx* c, double* out, cudaStream_t s, int* launches) {
     const wt_grid& g = c->grid;
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const int nt = (int)c->times.size(), ncol = (int)c->cols.size();
+    if (tables64(c, nt)) {
+        const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
+        int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
+        nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
+        c->Zc64.alloc((size_t)std::max(nb, 4) * ncol * g.Nz);
+        c->G64.alloc(std::max(c->sp64.scratch_elems(4), (size_t)3 * nb * npts));
+        c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
+        for (int t0 = 0; t0 < nt; t0 += nb) {
+            const int b = std::min(nb, nt - t0);
+            column_ztransform<double>(s, c->Qt.p + (size_t)t0 * c->ns, b, c->ns, c->ns, c->zcos.p, c->d_col_off.p, ncol,
+                                      g.Nz, c->Zc64.p);
+            t64_fields(s, c->T64.p, c->CS64.p, c->Zc64.p, b, ncol, g.Nx, g.Ny, g.Nz, c->G64.p, c->ws64.p, c->d_err.p,
+                       out + (size_t)t0 * 3 * npts);
+            *launches += 2 + 3 * 3;
+        }
+        return;
+    }
     const int nb = 4;
     c->Zc64.alloc((size_t)nb * ncol * g.Nz);
     c->G64.alloc(c->sp64.scratch_elems(nb));

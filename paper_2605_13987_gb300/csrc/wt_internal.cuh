@@ -194,6 +194,9 @@ void dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
 // dgemm on the tensor cores (k_dgemm_tc.cu); false when it does not take the product.
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only);
+size_t dgemm_tc_rows_bytes(int M, int N, int K);
+void dgemm_tc_rows(cudaStream_t s, int M, int N, int K, const double* A, int lda, const double* B, int ldb, double* C,
+                   int ldc, int mblk, size_t mstride, unsigned char* ws, int* d_err);
 void symmetrize_from_lower(cudaStream_t s, double* A, int n, int lda);
 void symmetrize_avg(cudaStream_t s, const double* F, double* C, int n);   // C = (F + F^T)/2
 void transpose(cudaStream_t s, const double* A, int rows, int cols, double* At);

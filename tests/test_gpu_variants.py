@@ -108,3 +108,23 @@ def test_eq1_on_the_field_staged_and_not(env, n_tracks, n_steps):
     P.wt_eq1_noalloc(s.ctx, H, tr, b)
     torch.cuda.synchronize()
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nx,nz", [(16, 32), (20, 36), (36, 60)])
+def test_fp64_field_from_tables_and_per_sample(env, nx, nz):
+    """Few time samples take one spectral transform each, more the lateral tables and products."""
+    torch, P, _, _ = env
+    w = W.tiny_cell(nx=nx, nz=nz, n_t=12, radius=0.5 * 55e-6 / nx * (5 if nx > 20 else 1))
+    s = P.Sensor(w.grid, w.columns)
+    s.fit()
+    try:
+        s.relax(w.times[:3])
+        few = s.extend("fp64")
+        s.relax(w.times)
+        many = s.extend("fp64")
+        torch.cuda.synchronize()
+        for t in range(3):
+            # the charges of both relaxations agree to the FP64 path's bound
+            assert rel_l2(many[t].cpu().numpy(), few[t].cpu().numpy()) < 1e-10
+    finally:
+        s.close()
