@@ -30,9 +30,9 @@
 // until the MMAs of the previous job have completed and rewrites the
 // coefficient tiles in shared memory.
 //
-// Warp roles: two producer warps (warp 0 and the last warp; each loads its
-// half of the 128-point slice by TMA and splits it into hi/lo, with its own
-// TMA barriers, so neither waits on the other), warp 1 TMEM owner + MMA
+// Warp roles: two or four producer warps (warp 0 and the last ones; each loads
+// its part of the 128-point slice by TMA and splits it into hi/lo, with its own
+// TMA barriers, so none waits on another), warp 1 TMEM owner + MMA
 // issuer, warps 2 .. 1 + NEPI epilogue.  Every mbarrier wait gives up
 // after ~2 s (globaltimer), sets the device error word and lets the CTA
 // unwind: the producer waits (bounded) for the TMA loads it still has in
@@ -68,8 +68,18 @@ __device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long a, 
         " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
-constexpr int RAW_BYTES = KR * BM * 4;   // one raw FP32 slice [32 basis][128 points], two halves
-constexpr int HALF = BM / 2;             // points per producer warp
+constexpr int RAW_BYTES = KR * BM * 4;   // one raw FP32 slice [32 basis][128 points], in NPROD parts
+// Rows of E that a load brings (the basis vectors in use) and K steps of 8 of the products over them
+__host__ __device__ constexpr int raw_rows(int r) { return r > 1 ? r : 1; }
+__host__ __device__ constexpr int k_steps(int r) { return r > 8 ? (r + 7) / 8 : 1; }
+// Producer warps: the conversion of a unit (rank x 128 values read, split and written twice to shared
+// memory) bounds the kernel below about 100 time samples, not the memory: 96 x 96 x 144
+// points, rank 29, 60 samples took 419 us with two such warps and two slices in flight, 294 us with four
+// warps, 275 us with four slices in flight and loads and products that stop at the rank (floor 203 us).
+// Four beside eight epilogue warps; two beside twelve or sixteen, which the autotuner takes for long
+// time axes only and whose registers would spill (80 or 96 instead of 96 to 122 a thread).
+__host__ __device__ constexpr int producers(int nepi) { return nepi == 8 ? 4 : 2; }
+__host__ __device__ constexpr int threads(int nepi) { return 32 * (1 + producers(nepi) + nepi); }
 
 // 4 x 4 transposes within lane quads: on entry lane 4g + i holds v[4b + j] =
 // D[point 4g + i][time 4b + j]; on return v[4b + j] = D[point 4g + j][time 4b + i],
@@ -91,8 +101,8 @@ __device__ __forceinline__ void quad_transpose(float (&v)[32], int lane) {
 
 struct Smem {
     // tiles first (1024-byte aligned base):
-    // B_hi[nt_pad x 128 B], B_lo[...], A[2 stages][hi, lo], raw[2][32][128] FP32
-    unsigned long long a_full[2], a_empty[2], acc_full[2], acc_empty[2], raw_full[2][2], drain, b_free;
+    // B_hi[nt_pad x 128 B], B_lo[...], A[2 stages][hi, lo], raw[2 or 4][32][128] FP32
+    unsigned long long a_full[2], a_empty[2], acc_full[2], acc_empty[2], raw_full[4][4], drain, b_free;
     unsigned tmem_base;
     int abort_flag;
 };
@@ -145,27 +155,29 @@ __device__ __forceinline__ void pair_transpose(float (&v)[32], int lane) {
 }
 
 template <int NEPI, int VEC>
-__global__ void __launch_bounds__(96 + 32 * NEPI, 1)
-    expand_tc_kernel(const __grid_constant__ Jobs J, int nt_pad_max, int n_units, int nch, int stall,
+__global__ void __launch_bounds__(threads(NEPI), 1)
+    expand_tc_kernel(const __grid_constant__ Jobs J, int nt_pad_max, int n_units, int nch, int lraw, int stall,
                      int* __restrict__ d_err) {
+    constexpr int NPROD = producers(NEPI), PART = BM / NPROD;   // producer warps, points of each
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // align the tile region to 1024 bytes
     unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     unsigned char* b_hi = base;
     unsigned char* b_lo = b_hi + (size_t)nt_pad_max * 128;
     unsigned char* a_tiles = b_lo + (size_t)nt_pad_max * 128;      // [stage][hi|lo] x TILE_BYTES
-    float* raw = reinterpret_cast<float*>(a_tiles + 4 * TILE_BYTES);  // [2 stages][2 halves][KR][HALF]
-    Smem* S = reinterpret_cast<Smem*>(reinterpret_cast<unsigned char*>(raw) + 2 * RAW_BYTES);
+    float* raw = reinterpret_cast<float*>(a_tiles + 4 * TILE_BYTES);  // [nraw stages][NPROD][KR][PART]
+    Smem* S = reinterpret_cast<Smem*>(reinterpret_cast<unsigned char*>(raw) + ((size_t)RAW_BYTES << lraw));
+    const int nraw = 1 << lraw;              // raw slices in flight (2 or 4)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int job0 = job_of(J, blockIdx.x, 0);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&S->a_full[i], 64);            // both producer warps
+            mbar_init(&S->a_full[i], 32 * NPROD);    // every producer warp
             mbar_init(&S->a_empty[i], 1);
-            mbar_init(&S->raw_full[i][0], 1);
-            mbar_init(&S->raw_full[i][1], 1);
         }
+        for (int i = 0; i < nraw; ++i)
+            for (int k = 0; k < NPROD; ++k) mbar_init(&S->raw_full[i][k], 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&S->acc_full[i], 1);
             mbar_init(&S->acc_empty[i], 32 * NEPI);
@@ -190,49 +202,50 @@ __global__ void __launch_bounds__(96 + 32 * NEPI, 1)
     constexpr int nbuf = 2, bstride = TMEM_COLS / 2;
     volatile int* abort_flag = &S->abort_flag;
 
-    if (warp == 0 || warp == 2 + NEPI) {
-        // ---------------- producers: TMA loads of raw E half slices, hi/lo conversion into swizzled A tiles
-        const int h = warp == 0 ? 0 : 1;             // points h HALF .. h HALF + HALF - 1 of each unit
-        float* rawh = raw + h * KR * HALF;           // stage st at rawh + st * KR * BM
-        int issued = 0;          // raw loads issued (unit k of this CTA goes to buffer k & 1)
+    if (warp == 0 || warp >= 2 + NEPI) {
+        // ---------------- producers: TMA loads of raw E slice parts, hi/lo conversion into swizzled A tiles
+        const int h = warp == 0 ? 0 : warp - 1 - NEPI;   // points h PART .. h PART + PART - 1 of each unit
+        float* rawh = raw + h * KR * PART;           // stage st at rawh + st * KR * BM
+        int issued = 0;          // raw loads issued (unit k of this CTA goes to buffer k % nraw)
         if (lane == 0)
-            for (int jl = job0; issued < 2; ++issued) {
+            for (int jl = job0; issued < nraw; ++issued) {
                 const int u = blockIdx.x + issued * gridDim.x;
                 if (u >= n_units) break;
                 jl = job_of(J, u, jl);
                 const int v = u - unit0_of(J, jl);
-                mbar_expect_tx(&S->raw_full[issued][h], RAW_BYTES / 2);
-                tma_load_2d(rawh + issued * KR * BM, &J.emap[jl], (v / 3) * BM + h * HALF, (v % 3) * KR,
+                mbar_expect_tx(&S->raw_full[issued][h], raw_rows(J.r[jl]) * PART * 4);
+                tma_load_2d(rawh + issued * KR * BM, &J.emap[jl], (v / 3) * BM + h * PART, (v % 3) * KR,
                             &S->raw_full[issued][h]);
             }
         issued = __shfl_sync(0xffffffffu, issued, 0);
         int i = 0, cur = job0, jnext = job0, n_changes = 0;
         for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++i) {
-            const int st = i & 1;
+            const int st = i & 1, sr = i & (nraw - 1);
             const int j = job_of(J, u, cur);
             if (j != cur) {
                 // new job: wait until the MMAs of the previous one are done, then its coefficients
                 if (!mbar_wait(&S->b_free, n_changes & 1, abort_flag, d_err)) break;
                 ++n_changes;
-                load_coeffs(J.W[j], J.nt[j], pad32(J.nt[j]), b_hi, b_lo, h * 32 + lane, 64);
+                load_coeffs(J.W[j], J.nt[j], pad32(J.nt[j]), b_hi, b_lo, h * 32 + lane, 32 * NPROD);
                 cur = j;
             }
             if (!mbar_wait(&S->a_empty[st], ((i >> 1) & 1) ^ 1, abort_flag, d_err)) break;
-            if (!mbar_wait(&S->raw_full[st][h], (i >> 1) & 1, abort_flag, d_err)) break;
+            if (!mbar_wait(&S->raw_full[sr][h], (i >> lraw) & 1, abort_flag, d_err)) break;
             unsigned char* ah = a_tiles + (size_t)(2 * st) * TILE_BYTES;
             unsigned char* al = ah + TILE_BYTES;
-            const float* rb = rawh + st * KR * BM;               // [KR][HALF]
-            const int rk = J.r[cur];
+            const float* rb = rawh + sr * KR * BM;               // [KR][PART]
+            const int rk = J.r[cur], kc = 2 * k_steps(rk);
 #pragma unroll
-            for (int rr = 0; rr < HALF / 32; ++rr) {
-                const int hr = lane + 32 * rr;                    // lane = grid point of this half
-                const int row = h * HALF + hr;
+            for (int rr = 0; rr < PART / 32; ++rr) {
+                const int hr = lane + 32 * rr;                    // lane = grid point of this part
+                const int row = h * PART + hr;
 #pragma unroll
                 for (int c = 0; c < KR / 4; ++c) {
+                    if (c >= kc) break;                           // the products stop at k_steps(rk)
                     unsigned hi[4], lo[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float x = (4 * c + j) < rk ? rb[(4 * c + j) * HALF + hr] : 0.f;
+                        const float x = (4 * c + j) < rk ? rb[(4 * c + j) * PART + hr] : 0.f;
                         hi[j] = to_tf32(x);
                         lo[j] = to_tf32(x - __uint_as_float(hi[j]));
                     }
@@ -247,19 +260,19 @@ __global__ void __launch_bounds__(96 + 32 * NEPI, 1)
             }
             fence_proxy_async();     // A tiles for the tensor core; raw buffer reads before the TMA refill
             __syncwarp();
-            const int u2 = u + 2 * gridDim.x;
+            const int u2 = u + nraw * gridDim.x;
             if (u2 < n_units) jnext = job_of(J, u2, max(jnext, cur));
             if (lane == 0 && u2 < n_units) {
                 const int v2 = u2 - unit0_of(J, jnext);
-                mbar_expect_tx(&S->raw_full[st][h], RAW_BYTES / 2);
-                tma_load_2d(rawh + st * KR * BM, &J.emap[jnext], (v2 / 3) * BM + h * HALF, (v2 % 3) * KR,
-                            &S->raw_full[st][h]);
+                mbar_expect_tx(&S->raw_full[sr][h], raw_rows(J.r[jnext]) * PART * 4);
+                tma_load_2d(rawh + sr * KR * BM, &J.emap[jnext], (v2 / 3) * BM + h * PART, (v2 % 3) * KR,
+                            &S->raw_full[sr][h]);
             }
-            if (u + 2 * gridDim.x < n_units) ++issued;
+            if (u2 < n_units) ++issued;
             mbar_arrive(&S->a_full[st]);
         }
         // loads still in flight after an abort: wait for them (bounded) before the CTA exits
-        for (int k = i; k < issued; ++k) mbar_wait_drain(&S->raw_full[k & 1][h], (k >> 1) & 1, d_err);
+        for (int k = i; k < issued; ++k) mbar_wait_drain(&S->raw_full[k & (nraw - 1)][h], (k >> lraw) & 1, d_err);
     } else if (warp == 1) {
         // ---------------- MMA issuer (lane 0)
         int i = 0, g = 0, cur = job0;
@@ -268,7 +281,7 @@ __global__ void __launch_bounds__(96 + 32 * NEPI, 1)
             const int st = i & 1;
             cur = job_of(J, u, cur);
             const int nt_pad = pad32(J.nt[cur]);
-            const int n_chunks = (nt_pad + nch - 1) / nch;
+            const int n_chunks = (nt_pad + nch - 1) / nch, nk = k_steps(J.r[cur]);
             if (!mbar_wait(&S->a_full[st], (i >> 1) & 1, abort_flag, d_err)) { ok = false; break; }
             tc_fence_after();
             const unsigned a_hi = smem_u32(a_tiles + (size_t)(2 * st) * TILE_BYTES);
@@ -286,6 +299,7 @@ __global__ void __launch_bounds__(96 + 32 * NEPI, 1)
                     const unsigned d = tmem + (unsigned)(b * bstride);
 #pragma unroll
                     for (int ks = 0; ks < KR / 8; ++ks) {
+                        if (ks >= nk) break;
                         const unsigned off = ks * 32;   // 8 TF32 = 32 bytes along K
                         mma_tf32(d, sdesc(a_lo + off), sdesc(bh + off), idesc, ks > 0);
                         mma_tf32(d, sdesc(a_hi + off), sdesc(bl + off), idesc, 1);
@@ -387,9 +401,11 @@ __global__ void __launch_bounds__(96 + 32 * NEPI, 1)
 
 bool expand_tc_available() { return true; }
 
-size_t expand_tc_smem(int nt_pad) {
-    return 1024 + (size_t)2 * nt_pad * 128 + 4 * (size_t)tc::TILE_BYTES + 2 * (size_t)tc::RAW_BYTES + sizeof(tc::Smem);
+static size_t expand_smem(int nt_pad, int lraw) {
+    return 1024 + (size_t)2 * nt_pad * 128 + 4 * (size_t)tc::TILE_BYTES + ((size_t)tc::RAW_BYTES << lraw) +
+           sizeof(tc::Smem);
 }
+size_t expand_tc_smem(int nt_pad) { return expand_smem(nt_pad, 1); }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
@@ -404,12 +420,12 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-static void encode_basis_map(CUtensorMap* m, const float* E, size_t npts) {
-    // E viewed as 96 rows (component x basis index) of npts points; one box = 32 rows x 64 points
-    // (half a unit: each producer warp loads its own half)
+static void encode_basis_map(CUtensorMap* m, const float* E, size_t npts, int rank, int nepi) {
+    // E viewed as 96 rows (component x basis index) of npts points; one box = the r rows in use x the
+    // points of one producer warp (each loads its own part of a unit)
     cuuint64_t dims[2] = {(cuuint64_t)npts, (cuuint64_t)3 * tc::KR};
     cuuint64_t strides[1] = {(cuuint64_t)npts * sizeof(float)};
-    cuuint32_t box[2] = {tc::HALF, tc::KR};
+    cuuint32_t box[2] = {(cuuint32_t)(tc::BM / tc::producers(nepi)), (cuuint32_t)tc::raw_rows(rank)};
     cuuint32_t es[2] = {1, 1};
     CUresult r = tensor_map_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(E), dims, strides, box,
                                       es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -423,16 +439,16 @@ int expand_tc_max_jobs() { return tc::MAX_JOBS; }
 // expansions in one persistent launch of at most `max_ctas` CTAs (0: one per SM).
 template <int VEC>
 static void launch_expand(int nepi, int grid, size_t sh, cudaStream_t s, const tc::Jobs& J, int nt_pad_max, int units,
-                          int nch, int stall, int* d_err) {
+                          int nch, int lraw, int stall, int* d_err) {
     if (nepi == 8) {
         allow_dyn_smem(tc::expand_tc_kernel<8, VEC>, sh);
-        tc::expand_tc_kernel<8, VEC><<<grid, 96 + 32 * 8, sh, s>>>(J, nt_pad_max, units, nch, stall, d_err);
+        tc::expand_tc_kernel<8, VEC><<<grid, tc::threads(8), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
     } else if (nepi == 12) {
         allow_dyn_smem(tc::expand_tc_kernel<12, VEC>, sh);
-        tc::expand_tc_kernel<12, VEC><<<grid, 96 + 32 * 12, sh, s>>>(J, nt_pad_max, units, nch, stall, d_err);
+        tc::expand_tc_kernel<12, VEC><<<grid, tc::threads(12), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
     } else {
         allow_dyn_smem(tc::expand_tc_kernel<16, VEC>, sh);
-        tc::expand_tc_kernel<16, VEC><<<grid, 96 + 32 * 16, sh, s>>>(J, nt_pad_max, units, nch, stall, d_err);
+        tc::expand_tc_kernel<16, VEC><<<grid, tc::threads(16), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
     }
 }
 
@@ -441,6 +457,7 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
     if (n_jobs < 1) return;
     if (nch != 64 && nch != 128 && nch != 256) fail(WT_ERR_ARG, "expansion time chunk must be 64, 128 or 256");
     if (n_jobs > tc::MAX_JOBS) fail(WT_ERR_UNSUPPORTED, "too many expansion jobs for one launch");
+    if (nepi != 8 && nepi != 12 && nepi != 16) fail(WT_ERR_ARG, "expansion epilogue warps must be 8, 12 or 16");
     tc::Jobs J;             // kernel parameter block (about 10 KB)
     int nt_pad_max = 32, units = 0;
     for (int j = 0; j < n_jobs; ++j) {
@@ -454,7 +471,7 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
         if (reinterpret_cast<uintptr_t>(jb.H) % 16) fail(WT_ERR_ARG, "H must be 16-byte aligned");
         const size_t n_tiles = (jb.npts + tc::BM - 1) / tc::BM;
         if ((size_t)units + 3 * n_tiles > (size_t)INT32_MAX) fail(WT_ERR_UNSUPPORTED, "expansion batch too large");
-        encode_basis_map(&J.emap[j], jb.E, jb.npts);
+        encode_basis_map(&J.emap[j], jb.E, jb.npts, jb.r, nepi);
         J.W[j] = jb.W;
         J.H[j] = jb.H;
         J.npts[j] = jb.npts;
@@ -465,22 +482,23 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
         nt_pad_max = std::max(nt_pad_max, nt_pad);
     }
     J.n_jobs = n_jobs;
-    const size_t sh = expand_tc_smem(nt_pad_max);
     int dev = 0, n_sm = 0, max_sh = 0;
     WT_CUDA(cudaGetDevice(&dev));
     WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
     WT_CUDA(cudaDeviceGetAttribute(&max_sh, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // four raw slices in flight where shared memory has the room (up to 384 time samples)
+    const int lraw = expand_smem(nt_pad_max, 2) <= (size_t)max_sh ? 2 : 1;
+    const size_t sh = expand_smem(nt_pad_max, lraw);
     if (sh > (size_t)max_sh) fail(WT_ERR_UNSUPPORTED, "expansion tile does not fit shared memory");
-    if (nepi != 8 && nepi != 12 && nepi != 16) fail(WT_ERR_ARG, "expansion epilogue warps must be 8, 12 or 16");
     if (vec != 1 && vec != 2 && vec != 4) fail(WT_ERR_ARG, "expansion store width must be 1, 2 or 4 floats");
     int grid = std::min(n_sm, units);
     if (max_ctas > 0) grid = std::min(grid, max_ctas);
     // WT_FAULT=queue_stall: the MMA warp withholds its accumulator-ready signals, so the epilogue's
     // bounded waits run out and the kernel unwinds with DERR_TIMEOUT (tests of the failure path)
     const int stall = fault_enabled("queue_stall") ? 1 : 0;
-    if (vec == 4) launch_expand<4>(nepi, grid, sh, s, J, nt_pad_max, units, nch, stall, d_err);
-    else if (vec == 2) launch_expand<2>(nepi, grid, sh, s, J, nt_pad_max, units, nch, stall, d_err);
-    else launch_expand<1>(nepi, grid, sh, s, J, nt_pad_max, units, nch, stall, d_err);
+    if (vec == 4) launch_expand<4>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else if (vec == 2) launch_expand<2>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else launch_expand<1>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
     WT_LAUNCH("expand_tc");
 }
 

@@ -1,6 +1,6 @@
 // FP32 z pass of the bulk extension, two-pass shared-memory form for
 // Nz = A B with A in {8, 16} lanes per line pair and B built from the factors
-// 2, 3, 5, 7 (Nz = 64, 96, 128, 160, 192, 224, 256, 384): the same cosine
+// 2, 3, 5, 7 (17 lengths from 40 to 384, listed below): the same cosine
 // and sine series as the register-FFT z pass (k_fft32_z.cu, Makhoul's
 // reordering of the DCT-III with two real lines per complex FFT), with the
 // N-point FFT split as
@@ -166,23 +166,25 @@ __global__ void __launch_bounds__(256, zpass2_min_blocks(A, B)) f32_zpass2_kerne
     }
 }
 
-// Two-pass forms compiled in: (A, B) for Nz = 64, 96, 128, 160, 192, 224, 256, 384.
-#define WT_FOR_EACH_Z2(X) X(8, 8) X(8, 12) X(8, 16) X(8, 20) X(8, 24) X(16, 14) X(16, 16) X(16, 24)
+// Two-pass forms compiled in, one per length: eight lanes per line pair up to 128 (their pass 2 leaves
+// fewer lanes idle: 112 as 8 x 14 43 us, as 16 x 7 50 us per 8 basis fields of 56^2 lines; 80 as 8 x 10
+// 10.2 us, as 16 x 5 10.9), sixteen above (a DFT of 16 points or fewer keeps four blocks per SM: 160 as
+// 16 x 10 68 us, as 8 x 20 95 us; 192 as 16 x 12 317 us, as 8 x 24 518 us per 32 fields of 96^2 lines;
+// 144 as 16 x 9 77 us, as 8 x 18 90 us).  The register form they replace: 144 138 us, 240 670 -> 284 us,
+// 120 78 -> 63 us, 72 23.6 -> 15.0 us.
+#define WT_FOR_EACH_Z2(X) \
+    X(8, 5) X(8, 6) X(8, 7) X(8, 8) X(8, 9) X(8, 10) X(8, 12) X(8, 14) X(8, 15) X(8, 16) X(16, 9) X(16, 10) \
+    X(16, 12) X(16, 14) X(16, 15) X(16, 16) X(16, 24)
+#define WT_Z2_LENGTHS "40, 48, 56, 64, 72, 80, 96, 112, 120, 128, 144, 160, 192, 224, 240, 256, 384"
 
 static bool z2_shape(int nz, int* A, int* B) {
     switch (nz) {
-        case 64: *A = 8; break;
-        case 96: *A = 8; break;
-        case 128: *A = 8; break;
-        case 160: *A = 8; break;
-        case 192: *A = 8; break;
-        case 224: *A = 16; break;
-        case 256: *A = 16; break;
-        case 384: *A = 16; break;
+#define WT_CASE(AA, BB) \
+    case AA * BB: *A = AA; *B = BB; return true;
+        WT_FOR_EACH_Z2(WT_CASE)
+#undef WT_CASE
         default: return false;
     }
-    *B = nz / *A;
-    return true;
 }
 bool zpass2_supported(int nz) {
     int A, B;
@@ -192,7 +194,7 @@ bool zpass2_supported(int nz) {
 void zpass2_allow(int nz) {
     int A, B;
     if (!z2_shape(nz, &A, &B))
-        fail(WT_ERR_UNSUPPORTED, "two-pass z FFT needs Nz in {64, 96, 128, 160, 192, 224, 256, 384}");
+        fail(WT_ERR_UNSUPPORTED, "two-pass z FFT needs Nz in {" WT_Z2_LENGTHS "}");
     const size_t sz = zpass2_smem(A, B, 64);
 #define WT_CASE(AA, BB) \
     if (A == AA && B == BB) { \
@@ -208,7 +210,7 @@ void zpass2_launch(int lb, dim3 gz, cudaStream_t s, const GridDev& g, const floa
                    const C2<float>* zz, float* out, size_t out_sb, size_t out_sc, ZLines zl) {
     int A, B;
     if (!z2_shape(g.Nz, &A, &B))
-        fail(WT_ERR_UNSUPPORTED, "two-pass z FFT needs Nz in {64, 96, 128, 160, 192, 224, 256, 384}");
+        fail(WT_ERR_UNSUPPORTED, "two-pass z FFT needs Nz in {" WT_Z2_LENGTHS "}");
     const size_t sz = zpass2_smem(A, B, lb);
 #define WT_CASE(AA, BB) \
     if (A == AA && B == BB) { \
