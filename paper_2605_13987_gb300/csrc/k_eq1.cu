@@ -105,26 +105,148 @@ struct Eq1Cell {
     }
 };
 
-// G[n][step] = W(x_step, t_n) . v_step for all steps of all tracks, the time sample in the slow grid
-// index: the blocks that run together read one or two time planes, which stay in L2 (96 x 96 x 192: 21
-// MB), where a block per track drew sectors of every plane from memory (a step of an inclined track
-// lies in a cell of its own: 12 sectors a sample, 49 GB for 1e6 steps x 128 samples).
+// G[step][n] = W(x_step, t_n) . v_step for all steps of all tracks, eight time samples a thread (one
+// 32-byte sector of G).  What bounds it are the sectors drawn from L2: a step of an inclined track lies
+// in a cell of its own, 12 sectors a sample (49 GB for 1e6 steps x 128 samples of a 96 x 96 x 192
+// field), so the steps of a large call are taken in the order of their cells: a warp's 32 steps then
+// share the sectors of a few neighbouring cells.  That field and those steps: 16.0 ms with a block per
+// track, 4.55 ms a time plane at a time in the tracks' order, 1.24 ms in the cells' order (the sort
+// 0.055 ms).
+constexpr int kStageTimes = 8;
+struct Eq1Steps {
+    const float *x, *y, *z, *vx, *vy, *vz;
+    const unsigned* order;               // the step whose row of G a position fills (NULL: its own)
+    size_t n;
+};
 __global__ void __launch_bounds__(256) eq1_stage_kernel(const float* __restrict__ H, int Nx, int Ny, int Nz,
-                                                        float inv_hx, float inv_hy, float inv_hz,
-                                                        const float* __restrict__ X, const float* __restrict__ Y,
-                                                        const float* __restrict__ Z, const float* __restrict__ VX,
-                                                        const float* __restrict__ VY, const float* __restrict__ VZ,
-                                                        size_t steps, float* __restrict__ G) {
+                                                        float inv_hx, float inv_hy, float inv_hz, Eq1Steps st, int nu,
+                                                        int ldg, float* __restrict__ G) {
     const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= steps) return;
+    if (s >= st.n) return;
     const size_t npts = (size_t)Nx * Ny * Nz;
     Eq1Cell<float> c;
-    c.vx = VX[s];
-    c.vy = VY[s];
-    c.vz = VZ[s];
-    c.set(X[s], Y[s], Z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
-    const size_t n = blockIdx.y;
-    G[n * steps + s] = c.moving() ? c.dot(H + n * 3 * npts, npts) : 0.f;
+    c.vx = st.vx[s];
+    c.vy = st.vy[s];
+    c.vz = st.vz[s];
+    c.set(st.x[s], st.y[s], st.z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
+    const int n0 = blockIdx.y * kStageTimes;
+    float r[kStageTimes];
+#pragma unroll
+    for (int i = 0; i < kStageTimes; ++i)
+        r[i] = n0 + i < nu && c.moving() ? c.dot(H + (size_t)(n0 + i) * 3 * npts, npts) : 0.f;
+    float4* g = reinterpret_cast<float4*>(G + (st.order ? (size_t)st.order[s] : s) * ldg + n0);
+    g[0] = make_float4(r[0], r[1], r[2], r[3]);
+    g[1] = make_float4(r[4], r[5], r[6], r[7]);
+}
+
+// Order of the steps by their cells (counting sort): a bin is eight cells along z, one 32-byte sector of
+// each component plane; resting steps, which read nothing, have the last bin to themselves.  The order
+// within a bin is that of the atomics: it moves no value.
+__device__ __forceinline__ unsigned eq1_bin(const Eq1Steps& st, size_t s, int Nx, int Ny, int Nz, float inv_hx,
+                                            float inv_hy, float inv_hz, unsigned n_bins) {
+    Eq1Cell<float> c;
+    c.vx = st.vx[s];
+    c.vy = st.vy[s];
+    c.vz = st.vz[s];
+    if (!c.moving()) return n_bins - 1;
+    c.set(st.x[s], st.y[s], st.z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
+    const size_t col = c.a00 / Nz;
+    return (unsigned)(col * ((Nz + 7) / 8) + (c.a00 - col * Nz) / 8);
+}
+__global__ void __launch_bounds__(256) eq1_count_kernel(Eq1Steps st, int Nx, int Ny, int Nz, float inv_hx, float inv_hy,
+                                                        float inv_hz, unsigned n_bins, unsigned* __restrict__ count,
+                                                        unsigned* __restrict__ rank) {
+    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < st.n) rank[s] = atomicAdd(count + eq1_bin(st, s, Nx, Ny, Nz, inv_hx, inv_hy, inv_hz, n_bins), 1u);
+}
+// Exclusive sums within stretches of kScan bins (in place), and each stretch's total.
+constexpr int kScan = 4096;
+__device__ __forceinline__ unsigned block_exclusive(unsigned v, unsigned* warp_tot, unsigned* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_tot[w] = x;
+    __syncthreads();
+    if (w == 0) {
+        unsigned t = warp_tot[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        warp_tot[lane] = t;
+    }
+    __syncthreads();
+    *total = warp_tot[31];
+    const unsigned base = w ? warp_tot[w - 1] : 0u;
+    __syncthreads();
+    return base + x - v;
+}
+__global__ void __launch_bounds__(1024) eq1_scan_kernel(unsigned* __restrict__ count, unsigned n_bins,
+                                                        unsigned* __restrict__ total) {
+    __shared__ unsigned wt[32];
+    const unsigned b0 = blockIdx.x * kScan + 4 * threadIdx.x;
+    unsigned v[4], sum = 0, all;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[i] = b0 + i < n_bins ? count[b0 + i] : 0u;
+        sum += v[i];
+    }
+    unsigned at = block_exclusive(sum, wt, &all);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (b0 + i < n_bins) count[b0 + i] = at;
+        at += v[i];
+    }
+    if (threadIdx.x == 0) total[blockIdx.x] = all;
+}
+__global__ void __launch_bounds__(1024) eq1_scan_totals_kernel(unsigned* __restrict__ total, int n) {
+    __shared__ unsigned wt[32];
+    unsigned carry = 0;
+    for (int k0 = 0; k0 < n; k0 += 1024) {
+        const int k = k0 + threadIdx.x;
+        unsigned all;
+        const unsigned at = block_exclusive(k < n ? total[k] : 0u, wt, &all);
+        if (k < n) total[k] = carry + at;
+        carry += all;
+    }
+}
+__global__ void __launch_bounds__(256) eq1_order_kernel(Eq1Steps st, int Nx, int Ny, int Nz, float inv_hx, float inv_hy,
+                                                        float inv_hz, unsigned n_bins,
+                                                        const unsigned* __restrict__ count,
+                                                        const unsigned* __restrict__ total,
+                                                        const unsigned* __restrict__ rank, float* __restrict__ sorted,
+                                                        unsigned* __restrict__ order) {
+    const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= st.n) return;
+    const unsigned b = eq1_bin(st, s, Nx, Ny, Nz, inv_hx, inv_hy, inv_hz, n_bins);
+    const size_t at = (size_t)count[b] + total[b / kScan] + rank[s];
+    order[at] = (unsigned)s;
+    sorted[at] = st.x[s];
+    sorted[st.n + at] = st.y[s];
+    sorted[2 * st.n + at] = st.z[s];
+    sorted[3 * st.n + at] = st.vx[s];
+    sorted[4 * st.n + at] = st.vy[s];
+    sorted[5 * st.n + at] = st.vz[s];
+}
+
+// Workspace of the staged form: per step a row of G, its sorted copy, its place and its rank; the bins.
+static int eq1_ldg(int nu) { return (nu + kStageTimes - 1) / kStageTimes * kStageTimes; }
+static size_t eq1_bins(int Nx, int Ny, int Nz) { return (size_t)Nx * Ny * ((Nz + 7) / 8) + 1; }
+static size_t eq1_bin_bytes(size_t bins) { return (bins + (bins + kScan - 1) / kScan) * sizeof(unsigned); }
+static size_t eq1_step_bytes(int nu) { return (size_t)(eq1_ldg(nu) + 8) * sizeof(float); }
+size_t eq1_stage_bytes(size_t steps, int nu, int Nx, int Ny, int Nz) {
+    return steps * eq1_step_bytes(nu) + eq1_bin_bytes(eq1_bins(Nx, Ny, Nz));
+}
+// The sort pays for itself when there is a step for every eighth sector (a sector serves four cells), from
+// 2^21 values on (below, its launches take longer than the sectors it saves).  96 x 96 x 192, 128 samples:
+// 1e5 steps 982 -> 442 us, 4e4 steps 452 -> 375 us, 2e4 steps 226 -> 267 us (not sorted).
+static bool eq1_sort(size_t steps, int nu, size_t bins) {
+    return 8 * steps >= bins && steps * nu >= ((size_t)1 << 21) && bins < ((size_t)1 << 31);
 }
 
 // T: field type; L: lag table entry; TO: current type.  nu: time samples the lag table reads
@@ -133,7 +255,7 @@ __global__ void __launch_bounds__(256) eq1_stage_kernel(const float* __restrict_
 // time samples, a lane keeping its step's cell for all samples, so that neighbouring steps share
 // sectors (lanes over time samples: every read a sector of its own).
 // 1e4 tracks x 100 steps, 96 x 96 x 192, 128 samples: 38.1 ms with lanes over samples, 16.0 with lanes
-// over steps, 5.5 through G.  A stage holds `steps` steps (32, or 16 where 32 rows of samples
+// over steps, 1.6 through G.  A stage holds `steps` steps (32, or 16 where 32 rows of samples
 // do not fit), accumulated 16 at a time.
 template <class T, class L, class TO>
 __global__ void __launch_bounds__(256) eq1_kernel(const T* __restrict__ H, int Nx, int Ny, int Nz, int nt, int nu,
@@ -143,7 +265,7 @@ __global__ void __launch_bounds__(256) eq1_kernel(const T* __restrict__ H, int N
                                                   const float* __restrict__ VY, const float* __restrict__ VZ,
                                                   const float* __restrict__ qtrack, float qconst, int n_steps,
                                                   int n_out, double dt, double inv_vw, int steps, int ld,
-                                                  const float* __restrict__ G, size_t g_steps,
+                                                  const float* __restrict__ G, int ldg,
                                                   const L* __restrict__ lags, TO* __restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* f = reinterpret_cast<T*>(smem_raw);                               // [steps][ld]
@@ -165,10 +287,13 @@ __global__ void __launch_bounds__(256) eq1_kernel(const T* __restrict__ H, int N
             cell.set((T)X[s], (T)Y[s], (T)Z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
         }
         __syncthreads();
-        for (int n = warp * per + lane / steps; n < nu; n += nwarps * per) {
-            if (!in) continue;
-            if (G) f[j * ld + n] = (T)G[(size_t)n * g_steps + s];
-            else f[j * ld + n] = cell.moving() ? cell.dot(H + (size_t)n * 3 * npts, npts) : (T)0;
+        if (G) {
+            const float* g = G + ((size_t)tr * n_steps + s0) * ldg;
+            for (int q = warp; q < min(steps, n_steps - s0); q += nwarps)
+                for (int n = lane; n < nu; n += 32) f[q * ld + n] = (T)g[(size_t)q * ldg + n];
+        } else {
+            for (int n = warp * per + lane / steps; n < nu; n += nwarps * per)
+                if (in) f[j * ld + n] = cell.moving() ? cell.dot(H + (size_t)n * 3 * npts, npts) : (T)0;
         }
         __syncthreads();
         for (int c0 = s0; c0 < min(n_steps, s0 + steps); c0 += EQ1_MC) {
@@ -222,27 +347,47 @@ static void eq1_launch_t(cudaStream_t s, const T* H, int Nx, int Ny, int Nz, int
     allow_dyn_smem(eq1_kernel<T, L, TO>, sh);
     eq1_kernel<T, L, TO><<<n_tracks, 256, sh, s>>>(H, Nx, Ny, Nz, nt, nu, (T)(Nx / Lx), (T)(Ny / Ly), (T)(Nz / Lz), x, y,
                                                    z, vx, vy, vz, q, qconst, n_steps, n_out, dt, 1.0 / v_w, steps, ld,
-                                                   G, (size_t)n_tracks * n_steps, static_cast<const L*>(lags),
+                                                   G, eq1_ldg(nu), static_cast<const L*>(lags),
                                                    out);
     WT_LAUNCH("eq1");
 }
 void eq1_launch(cudaStream_t s, const float* H, int Nx, int Ny, int Nz, int nt, double Lx, double Ly, double Lz,
                 const float* x, const float* y, const float* z, const float* vx, const float* vy, const float* vz,
                 const float* q, float qconst, int n_tracks, int n_steps, int n_out, double dt, double v_w,
-                const void* lags, int nu, float* out, float* G, size_t g_len) {
-    // G: workspace of g_len values (NULL: none) for the dot products of as many whole tracks at a time
-    const int per = (int)std::min<size_t>(n_tracks, g_len / ((size_t)nu * n_steps));
-    if (!G || per < 1) {
+                const void* lags, int nu, float* out, unsigned char* ws, size_t ws_bytes) {
+    // ws: workspace (NULL: none) for the dot products of as many whole tracks at a time
+    const size_t bins = eq1_bins(Nx, Ny, Nz), fixed = eq1_bin_bytes(bins);
+    const int per = !ws || ws_bytes <= fixed ? 0 :
+        (int)std::min<size_t>(n_tracks, (ws_bytes - fixed) / (eq1_step_bytes(nu) * n_steps));
+    if (per < 1) {
         eq1_launch_t<float, Eq1Lag, float>(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x, y, z, vx, vy, vz, q, qconst, n_tracks,
                                            n_steps, n_out, dt, v_w, lags, nu, out);
         return;
     }
+    const float ix = (float)(Nx / Lx), iy = (float)(Ny / Ly), iz = (float)(Nz / Lz);
+    const int ldg = eq1_ldg(nu);
     for (int t0 = 0; t0 < n_tracks; t0 += per) {
         const int n = std::min(per, n_tracks - t0);
         const size_t o = (size_t)t0 * n_steps, steps = (size_t)n * n_steps;
-        eq1_stage_kernel<<<dim3((unsigned)((steps + 255) / 256), nu), 256, 0, s>>>(
-            H, Nx, Ny, Nz, (float)(Nx / Lx), (float)(Ny / Ly), (float)(Nz / Lz), x + o, y + o, z + o, vx + o, vy + o,
-            vz + o, steps, G);
+        const unsigned blocks = (unsigned)((steps + 255) / 256);
+        float* G = reinterpret_cast<float*>(ws);
+        Eq1Steps st{x + o, y + o, z + o, vx + o, vy + o, vz + o, nullptr, steps};
+        if (eq1_sort(steps, nu, bins)) {
+            float* sorted = G + steps * ldg;
+            unsigned* order = reinterpret_cast<unsigned*>(sorted + 6 * steps);
+            unsigned *rank = order + steps, *count = rank + steps, *total = count + bins;
+            const int stretches = (int)((bins + kScan - 1) / kScan);
+            WT_CUDA(cudaMemsetAsync(count, 0, bins * sizeof(unsigned), s));
+            eq1_count_kernel<<<blocks, 256, 0, s>>>(st, Nx, Ny, Nz, ix, iy, iz, (unsigned)bins, count, rank);
+            eq1_scan_kernel<<<stretches, 1024, 0, s>>>(count, (unsigned)bins, total);
+            eq1_scan_totals_kernel<<<1, 1024, 0, s>>>(total, stretches);
+            eq1_order_kernel<<<blocks, 256, 0, s>>>(st, Nx, Ny, Nz, ix, iy, iz, (unsigned)bins, count, total, rank,
+                                                    sorted, order);
+            WT_LAUNCH("eq1_order");
+            st = Eq1Steps{sorted, sorted + steps, sorted + 2 * steps, sorted + 3 * steps, sorted + 4 * steps,
+                          sorted + 5 * steps, order, steps};
+        }
+        eq1_stage_kernel<<<dim3(blocks, ldg / kStageTimes), 256, 0, s>>>(H, Nx, Ny, Nz, ix, iy, iz, st, nu, ldg, G);
         WT_LAUNCH("eq1_stage");
         eq1_launch_t<float, Eq1Lag, float>(s, H, Nx, Ny, Nz, nt, Lx, Ly, Lz, x + o, y + o, z + o, vx + o, vy + o, vz + o,
                                            q ? q + t0 : nullptr, qconst, n, n_steps, n_out, dt, v_w, lags, nu,

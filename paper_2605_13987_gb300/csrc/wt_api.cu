@@ -50,7 +50,8 @@ void t64_fields(cudaStream_t, const double*, const double*, const double*, int, 
                 unsigned char*, int*, double*);
 void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, double, const float*, const float*,
                 const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
-                double, const void*, int, float*, float*, size_t);
+                double, const void*, int, float*, unsigned char*, size_t);
+size_t eq1_stage_bytes(size_t, int, int, int, int);
 size_t eq1_lag_size();
 void eq1_launch64(cudaStream_t, const double*, int, int, int, int, double, double, double, const float*, const float*,
                   const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
@@ -1363,20 +1364,20 @@ void eq1_run(wt_ctx* c, const void* H, bool h64, const TrackDev& t, void* out, c
     else {
         // workspace of the staged dot products: all of them, or 1 GB of tracks at a time (a large field
         // is then read once per GB); few steps go without (their sectors stay in L2 anyway)
-        constexpr size_t kMost = (size_t)1 << 28, kFew = (size_t)1 << 20;
-        const size_t all = (size_t)t.n_tracks * t.n_steps * nu;
-        DBuf<float> G;
-        const bool staged = all >= kFew && (size_t)t.n_steps * nu <= kMost && nu <= 65535;
-        if (staged) {
+        constexpr size_t kMost = (size_t)1 << 30, kFew = (size_t)1 << 20;
+        const size_t steps = (size_t)t.n_tracks * t.n_steps;
+        DBuf<unsigned char> ws;
+        if (steps * nu >= kFew && eq1_stage_bytes(t.n_steps, nu, g.Nx, g.Ny, g.Nz) <= kMost && nu <= 65535) {
+            const size_t all = eq1_stage_bytes(steps, nu, g.Nx, g.Ny, g.Nz);
             try {
-                G.alloc(std::min(all, kMost));
+                ws.alloc(std::min(all, kMost));
             } catch (const Error&) {       // no memory for it: the one-kernel form
                 if (fault_enabled("alloc")) throw;
             }
         }
         eq1_launch(s, static_cast<const float*>(H), g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx, t.vy,
                    vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, t.dt, c->opts.v_w, dlag.p, nu,
-                   static_cast<float*>(out), G.p, G.n);
+                   static_cast<float*>(out), ws.p, ws.n);
         WT_CUDA(cudaStreamSynchronize(s));
         return;
     }

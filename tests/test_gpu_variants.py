@@ -128,3 +128,26 @@ def test_fp64_field_from_tables_and_per_sample(env, nx, nz):
             assert rel_l2(many[t].cpu().numpy(), few[t].cpu().numpy()) < 1e-10
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("n_tracks,n_steps", [(5000, 70), (20000, 16)])
+def test_eq1_steps_in_cell_order(env, n_tracks, n_steps):
+    """Enough steps to be taken in the order of their cells: random cells, resting steps, positions outside
+    of the box and on its faces; equal bits to the one-kernel form, which keeps the tracks' order."""
+    torch, P, w, s = env
+    H = s.extend("fp32")
+    t = W.configs.mip_tracks(w.grid, n_tracks, n_steps, np.random.default_rng(2))
+    rng = np.random.default_rng(3)
+    shape = t.x.shape
+    t.x[:] = rng.uniform(-1.0, 2.0, shape) * w.grid.Lx
+    t.y[:] = rng.uniform(-1.0, 2.0, shape) * w.grid.Ly
+    t.z[:] = np.clip(rng.uniform(-0.2, 1.2, shape), 0.0, 1.0) * w.grid.Lz
+    rest = rng.uniform(size=shape) < 0.2
+    for v in (t.vx, t.vy, t.vz):
+        v[rest] = 0.0
+    tr = device_tracks(t, torch)
+    a = s.eq1(H, tr)
+    b = torch.empty_like(a)
+    P.wt_eq1_noalloc(s.ctx, H, tr, b)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
