@@ -538,8 +538,11 @@ __global__ void __launch_bounds__(256) eq1_basis_kernel(const float* __restrict_
 //   * the steps of a chunk (8 per group of threads) are gathered first, a warp taking consecutive steps
 //     and keeping its cell's 24 corner values while the track stays in the cell (a drifting carrier: 11
 //     steps a cell);
-//   * groups are added in FP32, chunks in FP64.
-// 1e5 tracks x 200 steps, 400 outputs, rank 32: 20.3 -> 14.3 ms.
+//   * groups are added in FP32, chunks in FP64;
+//   * groups of 8 steps in which the track rests (a carrier that has arrived, a track that has left the
+//     sensor) are left out: the chunks take the moving groups only.
+// 1e5 tracks x 200 steps, 400 outputs, rank 32: 20.3 -> 14.3 ms, without the resting
+// groups 10.5 ms (carriers that drift 20 um on average of the 30 that 200 steps allow).
 constexpr int kConvThreads = 128, kConvOut = 16, kConvSteps = 8, kConvPad = 24;
 constexpr size_t kConvTableMax = 110 * 1024;
 struct ConvShape {
@@ -599,6 +602,9 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
     float* S = reinterpret_cast<float*>(D + nm);                  // [16][js][2]
     float* tab = S + (size_t)32 * C.js;                           // [16][row][2]
     float* P = tab + (size_t)32 * row;                            // [ng][nm]
+    __shared__ unsigned bits[kConvThreads / 4];
+    __shared__ unsigned char list[kConvThreads];
+    __shared__ int n_list;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int e = tid; e < 32 * row; e += kConvThreads) tab[e] = dvt[e];
     const int t = tid % C.tm, g = tid / C.tm;                     // outputs 16 t .., group of steps
@@ -606,106 +612,141 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
     const int per_warp = (C.jc + kConvThreads / 32 - 1) / (kConvThreads / 32);
     for (int tr = blockIdx.x; tr < n_tracks; tr += gridDim.x) {
         for (int m = tid; m < nm; m += kConvThreads) D[m] = 0.0;
-        for (int c0 = 0; c0 < n_steps; c0 += C.jc) {
-            const int mc = min(C.jc, n_steps - c0);
-            __syncthreads();                                       // S and P of the last chunk are read, D is set
-            // a warp's steps are prepared a lane each (one coalesced read of the track arrays), then taken
-            // one after the other with a lane per basis field
-            for (int l0 = 0; l0 < per_warp; l0 += 32) {
-                const int js = warp * per_warp + l0 + lane;
-                Eq1Cell<float> cell;
-                if (l0 + lane < per_warp && js < mc) {
-                    const size_t st = (size_t)tr * n_steps + c0 + js;
-                    cell.vx = VX[st];
-                    cell.vy = VY[st];
-                    cell.vz = VZ[st];
-                    cell.set(X[st], Y[st], Z[st], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
-                }
-                const unsigned moving = __ballot_sync(0xffffffffu, cell.moving());
-                const int a00 = (int)cell.a00, a01 = (int)cell.a01, a10 = (int)cell.a10, a11 = (int)cell.a11;
-                int key = -1;
-                float v[24];
-                const int nl = min(32, per_warp - l0);
-                for (int l = 0; l < nl; ++l) {
-                    const int j = warp * per_warp + l0 + l;
-                    if (j >= C.jc) break;
-                    float acc = 0.f;
-                    if (moving >> l & 1) {
-                        const int k00 = __shfl_sync(0xffffffffu, a00, l);
-                        if (k00 != key) {
-                            key = k00;
-                            const int k01 = __shfl_sync(0xffffffffu, a01, l), k10 = __shfl_sync(0xffffffffu, a10, l),
-                                      k11 = __shfl_sync(0xffffffffu, a11, l);
-                            const float* p[4] = {Ep + (size_t)k00 * 96 + lane, Ep + (size_t)k01 * 96 + lane,
-                                                 Ep + (size_t)k10 * 96 + lane, Ep + (size_t)k11 * 96 + lane};
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    v[6 * q + 2 * c] = __ldg(p[q] + 32 * c);
-                                    v[6 * q + 2 * c + 1] = __ldg(p[q] + 96 + 32 * c);
-                                }
-                        }
-                        const float wx = __shfl_sync(0xffffffffu, cell.wx, l), wy = __shfl_sync(0xffffffffu, cell.wy, l),
-                                    wz = __shfl_sync(0xffffffffu, cell.wz, l);
-                        float w[3];
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            float u[4];
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                u[q] = (1.f - wz) * v[6 * q + 2 * c] + wz * v[6 * q + 2 * c + 1];
-                            w[c] = (1.f - wx) * ((1.f - wy) * u[0] + wy * u[1]) + wx * ((1.f - wy) * u[2] + wy * u[3]);
-                        }
-                        acc = w[0] * __shfl_sync(0xffffffffu, cell.vx, l) + w[1] * __shfl_sync(0xffffffffu, cell.vy, l) +
-                              w[2] * __shfl_sync(0xffffffffu, cell.vz, l);
-                    }
-                    S[((lane >> 1) * C.js + j) * 2 + (lane & 1)] = lane < r ? acc : 0.f;
-                }
+        for (int b0 = 0; b0 < n_steps; b0 += kConvSteps * kConvThreads) {
+            // the groups of 8 steps in which the track moves at all, in order: a bit per group, then its place
+            __syncthreads();                                           // the last list is used
+            if (tid < kConvThreads / 4) bits[tid] = 0;
+            __syncthreads();
+            const int lim = min(n_steps - b0, kConvSteps * kConvThreads);
+            for (int j = b0 + tid; j - lane < b0 + lim; j += kConvThreads) {
+                const size_t st = (size_t)tr * n_steps + j;
+                const bool mv = j < n_steps && (VX[st] != 0.f || VY[st] != 0.f || VZ[st] != 0.f);
+                const unsigned any = __ballot_sync(0xffffffffu, mv);
+                if (lane == 0)                                         // 32 steps: four groups
+                    bits[(j - b0) >> 5] = (any & 0xffu ? 1u : 0u) | (any & 0xff00u ? 2u : 0u) | (any & 0xff0000u ? 4u : 0u) |
+                                          (any & 0xff000000u ? 8u : 0u);
             }
             __syncthreads();
-            const int j0 = kConvSteps * g, m0 = kConvOut * t;      // this thread's steps (in the chunk), outputs
-            const bool live = work && j0 < mc && m0 + kConvOut - 1 >= c0 + j0;
-            using pair = unsigned long long;
-            pair acc[kConvOut];
-#pragma unroll
-            for (int i = 0; i < kConvOut; ++i) acc[i] = 0;
-            if (live) {
-                // entries e0 .. e0 + 22 of a table row: dV[m0 + i - (c0 + j0 + jj)] at i - jj + 7; e0 mod 16 is 1
-                // or 9 (m0 is a multiple of 16, c0 + j0 of 8), so the skip of every 17th place falls at
-                // entry 15, or at 7
-                const int e0 = m0 - (c0 + j0) - (kConvSteps - 1) + kConvPad;
-                const pair* T = reinterpret_cast<const pair*>(tab) + e0 + (e0 >> 4);
-                const int skip = (e0 & 15) == 9 ? 1 : 0;
-                const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(S) + j0 / 2;
-                for (int m = 0; m < r; m += 2, T += row, sp += C.js / 2) {
-                    pair sj[kConvSteps], w[kConvOut + kConvSteps - 1];
-#pragma unroll
-                    for (int k = 0; k < kConvSteps / 2; ++k) {
-                        const ulonglong2 x = sp[k];
-                        sj[2 * k] = x.x;
-                        sj[2 * k + 1] = x.y;
-                    }
-#pragma unroll
-                    for (int k = 0; k < kConvOut + kConvSteps - 1; ++k) w[k] = k < 7 ? T[k] : k < 15 ? T[k + skip] : T[k + 1];
-#pragma unroll
-                    for (int jj = 0; jj < kConvSteps; ++jj)
-#pragma unroll
-                        for (int i = 0; i < kConvOut; ++i) acc[i] = fma_pair(sj[jj], w[i - jj + kConvSteps - 1], acc[i]);
+            if (warp == 0) {
+                const unsigned mine = bits[lane];
+                int at = __popc(mine);
+    #pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += y;
                 }
+                if (lane == 31) n_list = at;
+                at -= __popc(mine);
+    #pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (mine >> q & 1) list[at++] = (unsigned char)(4 * lane + q);
             }
-            if (work)
-#pragma unroll
-                for (int i = 0; i < kConvOut; ++i)
-                    P[(size_t)g * nm + i * C.tm + t] = __uint_as_float((unsigned)acc[i]) +
-                                                       __uint_as_float((unsigned)(acc[i] >> 32));
             __syncthreads();
-            for (int e = tid; e < nm; e += kConvThreads) {         // e = i tm + t: output 16 t + i
-                const int m = (e % C.tm) * kConvOut + e / C.tm;
-                if (m < c0) continue;
-                float d = 0.f;
-                for (int q = 0; q < C.ng; ++q) d += P[(size_t)q * nm + e];
-                D[e] += (double)d;
+            const int n_act = n_list;
+            for (int k0 = 0; k0 < n_act; k0 += C.ng) {
+                const int nk = min(C.ng, n_act - k0), c0 = b0 + kConvSteps * list[k0];
+                if (k0) __syncthreads();                               // S and P of the last chunk are read
+                // a warp's steps are prepared a lane each (one coalesced read of the track arrays), then taken
+                // one after the other with a lane per basis field
+                for (int l0 = 0; l0 < per_warp; l0 += 32) {
+                    const int js = warp * per_warp + l0 + lane;
+                    Eq1Cell<float> cell;
+                    const int step =
+                        js < kConvSteps * nk ? b0 + kConvSteps * list[k0 + js / kConvSteps] + js % kConvSteps : n_steps;
+                    if (l0 + lane < per_warp && step < n_steps) {
+                        const size_t st = (size_t)tr * n_steps + step;
+                        cell.vx = VX[st];
+                        cell.vy = VY[st];
+                        cell.vz = VZ[st];
+                        cell.set(X[st], Y[st], Z[st], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
+                    }
+                    const unsigned moving = __ballot_sync(0xffffffffu, cell.moving());
+                    const int a00 = (int)cell.a00, a01 = (int)cell.a01, a10 = (int)cell.a10, a11 = (int)cell.a11;
+                    int key = -1;
+                    float v[24];
+                    const int nl = min(32, per_warp - l0);
+                    for (int l = 0; l < nl; ++l) {
+                        const int j = warp * per_warp + l0 + l;
+                        if (j >= C.jc) break;
+                        float acc = 0.f;
+                        if (moving >> l & 1) {
+                            const int k00 = __shfl_sync(0xffffffffu, a00, l);
+                            if (k00 != key) {
+                                key = k00;
+                                const int k01 = __shfl_sync(0xffffffffu, a01, l), k10 = __shfl_sync(0xffffffffu, a10, l),
+                                          k11 = __shfl_sync(0xffffffffu, a11, l);
+                                const float* p[4] = {Ep + (size_t)k00 * 96 + lane, Ep + (size_t)k01 * 96 + lane,
+                                                     Ep + (size_t)k10 * 96 + lane, Ep + (size_t)k11 * 96 + lane};
+    #pragma unroll
+                                for (int q = 0; q < 4; ++q)
+    #pragma unroll
+                                    for (int c = 0; c < 3; ++c) {
+                                        v[6 * q + 2 * c] = __ldg(p[q] + 32 * c);
+                                        v[6 * q + 2 * c + 1] = __ldg(p[q] + 96 + 32 * c);
+                                    }
+                            }
+                            const float wx = __shfl_sync(0xffffffffu, cell.wx, l), wy = __shfl_sync(0xffffffffu, cell.wy, l),
+                                        wz = __shfl_sync(0xffffffffu, cell.wz, l);
+                            float w[3];
+    #pragma unroll
+                            for (int c = 0; c < 3; ++c) {
+                                float u[4];
+    #pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    u[q] = (1.f - wz) * v[6 * q + 2 * c] + wz * v[6 * q + 2 * c + 1];
+                                w[c] = (1.f - wx) * ((1.f - wy) * u[0] + wy * u[1]) + wx * ((1.f - wy) * u[2] + wy * u[3]);
+                            }
+                            acc = w[0] * __shfl_sync(0xffffffffu, cell.vx, l) + w[1] * __shfl_sync(0xffffffffu, cell.vy, l) +
+                                  w[2] * __shfl_sync(0xffffffffu, cell.vz, l);
+                        }
+                        S[((lane >> 1) * C.js + j) * 2 + (lane & 1)] = lane < r ? acc : 0.f;
+                    }
+                }
+                __syncthreads();
+                // this thread's steps (in the chunk and in the track) and outputs
+                const int j0 = kConvSteps * g, js0 = work && g < nk ? b0 + kConvSteps * list[k0 + g] : 0, m0 = kConvOut * t;
+                const bool live = work && g < nk && m0 + kConvOut - 1 >= js0;
+                using pair = unsigned long long;
+                pair acc[kConvOut];
+    #pragma unroll
+                for (int i = 0; i < kConvOut; ++i) acc[i] = 0;
+                if (live) {
+                    // entries e0 .. e0 + 22 of a table row: dV[m0 + i - (js0 + jj)] at i - jj + 7; e0 mod 16 is 1
+                    // or 9 (m0 is a multiple of 16, js0 of 8), so the skip of every 17th place falls at
+                    // entry 15, or at 7
+                    const int e0 = m0 - js0 - (kConvSteps - 1) + kConvPad;
+                    const pair* T = reinterpret_cast<const pair*>(tab) + e0 + (e0 >> 4);
+                    const int skip = (e0 & 15) == 9 ? 1 : 0;
+                    const ulonglong2* sp = reinterpret_cast<const ulonglong2*>(S) + j0 / 2;
+                    for (int m = 0; m < r; m += 2, T += row, sp += C.js / 2) {
+                        pair sj[kConvSteps], w[kConvOut + kConvSteps - 1];
+    #pragma unroll
+                        for (int k = 0; k < kConvSteps / 2; ++k) {
+                            const ulonglong2 x = sp[k];
+                            sj[2 * k] = x.x;
+                            sj[2 * k + 1] = x.y;
+                        }
+    #pragma unroll
+                        for (int k = 0; k < kConvOut + kConvSteps - 1; ++k) w[k] = k < 7 ? T[k] : k < 15 ? T[k + skip] : T[k + 1];
+    #pragma unroll
+                        for (int jj = 0; jj < kConvSteps; ++jj)
+    #pragma unroll
+                            for (int i = 0; i < kConvOut; ++i) acc[i] = fma_pair(sj[jj], w[i - jj + kConvSteps - 1], acc[i]);
+                    }
+                }
+                if (work)
+    #pragma unroll
+                    for (int i = 0; i < kConvOut; ++i)
+                        P[(size_t)g * nm + i * C.tm + t] = __uint_as_float((unsigned)acc[i]) +
+                                                           __uint_as_float((unsigned)(acc[i] >> 32));
+                __syncthreads();
+                for (int e = tid; e < nm; e += kConvThreads) {         // e = i tm + t: output 16 t + i
+                    const int m = (e % C.tm) * kConvOut + e / C.tm;
+                    if (m < c0) continue;
+                    float d = 0.f;
+                    for (int q = 0; q < nk; ++q) d += P[(size_t)q * nm + e];
+                    D[e] += (double)d;
+                }
             }
         }
         __syncthreads();

@@ -151,3 +151,30 @@ def test_eq1_steps_in_cell_order(env, n_tracks, n_steps):
     P.wt_eq1_noalloc(s.ctx, H, tr, b)
     torch.cuda.synchronize()
     assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_steps,n_out", [(8, 16), (33, 40), (200, 400), (1030, 700), (2100, 750)])
+def test_eq1_direct_leaves_out_resting_steps(env, n_steps, n_out):
+    """Tracks that rest now and then, at any step, or always, or never, over one list of groups and over
+    several: against the stored field's form, which takes every step.  Both sum FP32 products of the same
+    FP32 basis fields: 1e-5 of the norm, as between the two forms elsewhere."""
+    torch, P, w, s = env
+    H = s.extend("fp32")
+    t = W.configs.mip_tracks(w.grid, 40, n_steps, np.random.default_rng(4))
+    rng = np.random.default_rng(5)
+    t.n_out = n_out
+    v = 1e5 * (1 + rng.uniform(size=t.x.shape))
+    rest = np.repeat(rng.uniform(size=(40, (n_steps + 10) // 11)) < 0.6, 11, axis=1)[:, :n_steps]
+    rest[0] = True
+    rest[1] = False
+    rest[2, 1:] = True
+    t.x[:] = rng.uniform(0, 1, t.x.shape) * w.grid.Lx
+    t.z[:] = rng.uniform(0, 1, t.x.shape) * w.grid.Lz
+    t.vx[:] = np.where(rest, 0.0, v)
+    t.vy[:] = np.where(rest, 0.0, -0.5 * v)
+    t.vz[:] = 0.0
+    tr = device_tracks(t, torch)
+    a = s.eq1_direct(tr).cpu().numpy()
+    b = s.eq1(H, tr).cpu().numpy()
+    assert np.all(a[0] == 0.0)
+    assert rel_l2(a, b) < 1e-5
