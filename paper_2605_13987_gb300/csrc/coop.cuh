@@ -8,7 +8,7 @@ namespace wt {
 
 // 1 / sqrt(x) of a positive x by Newton's iteration y <- y + y (1 - x y^2) / 2 from the FP32 value (24
 // bits, 46, then the FP64 rounding level), x normalised by its exponent.  A chain of about ten FP64
-// operations, each of which costs a warp 16 cycles of GB300's FP64 units.
+// operations, each of which costs a warp 64 cycles of GB300's FP64 units.
 __device__ __forceinline__ double rsqrt_newton(double x) {
     const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
     if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
@@ -41,16 +41,19 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int*
     __syncthreads();
     __shared__ int ok_sh;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         const unsigned want = round * gridDim.x;
-        volatile unsigned* vb = bar;
+        auto count = [&] {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            return v;
+        };
         volatile unsigned* gone = bar + 1;
         int ok = 1;
-        if (*vb < want) {
+        if (count() < want) {
             unsigned long long t0, t;
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
-            while (*vb < want) {
+            while (count() < want) {
                 asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
                 if (t - t0 > 20000 && *gone) { ok = 0; break; }
                 if (t - t0 > kGridWaitNs) {
@@ -61,7 +64,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned round, int*
                 }
             }
         }
-        __threadfence();
         ok_sh = ok;
     }
     __syncthreads();

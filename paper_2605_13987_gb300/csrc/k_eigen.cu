@@ -61,22 +61,27 @@ __device__ double block_sum(double v, double* sh) {
 }
 
 // ------------------------------------------------------ tridiagonalisation
-// All columns in one cooperative launch (one block per SM, rows dealt out cyclically, one warp per
-// row).  Step k, with v, w of step k - 1 in shared memory:
-//   every block forms row k of the updated matrix, A[k] - v[k] w - w[k] v, and its reflector (the
-//   same work in every block: 3 m operations, cheaper than a barrier);
-//   a warp takes a row i > k: A[i] -= v[i] w + w[i] v and, on the same pass, p[i] = tau A[i] . vn;
-//   barrier; every block reads p and forms w = p - (tau (p . vn) / 2) vn.
-// One barrier per column and one pass over the trailing block (three FP64 operations per entry: the
-// FP64 units bound it, 2 per clock and SM), where four launches a column took three passes:
-// n = 2304 94 ms before.  p alternates between two buffers, so that a block still reading one is not
-// overtaken.  The reflector of step k is written into row k one step later, when no block reads that
-// row any more.
+// All columns in one cooperative launch (one block per SM, rows dealt out cyclically).  Step k, with the
+// vector u of step k - 1 (unscaled: H = 1 - t u u^T) and p = t A u in shared memory, A' = A - u p^T - c u^T,
+// c = p - (t p.u) u:
+//   every block forms row k of A' and the squares below its subdiagonal entry (the same work in every
+//   block: 4 m operations, cheaper than a barrier);
+//   four warps take a row i > k, a quarter of its entries each: A[i] = A'[i], and on the same pass
+//   acc = A'[i] . A'[k].  A warp of its own meanwhile works out the reflector (beta, t); it enters
+//   the product through its first entry only, u = A'[k] - beta e_{k+1}, so p_i = t (acc - beta A'[i][k+1]);
+//   barrier; every block reads p.
+// One barrier per column and one pass over the trailing block.  What bounds it: three FP64 operations per
+// entry of the trailing block (2 per clock and SM: n^3 in all, 21 of the 43.5 ms at n = 2304; the four
+// warps of a row sit on the four quarters of the SM, so that a few rows load them alike), and about six
+// us a column of latency (barrier, loads, two sums).  Four launches a column: 94 ms at n = 2304; the same
+// launch with normalised vectors, a warp per row: 46.7.
+// p alternates between two buffers, so that a block still reading one is not overtaken.  The reflector of
+// step k is written into row k one step later, when no block reads that row any more.
 //
-// The vectors are worked on by the first four warps only, one per SM quarter: a quarter does an FP64
+// The sums over vectors are taken by the first four warps only, one per SM quarter: a quarter does an FP64
 // warp instruction in 64 cycles, so more warps add nothing to the sums and four times the shuffle steps
 // to the reductions.
-constexpr int kTrdThreads = 512, kTrdVec = 128;
+constexpr int kTrdThreads = 544, kTrdRowThreads = 512, kTrdVec = 128, kTrdRows = 64;
 // sum over the first kTrdVec threads, for all threads of the block (red: 4 values)
 __device__ __forceinline__ double trd_sum(double v, double* red) {
     if (threadIdx.x < kTrdVec) {
@@ -90,92 +95,124 @@ __global__ void __launch_bounds__(kTrdThreads, 1)
     trd_kernel(double* A, int n, double* __restrict__ d, double* __restrict__ e, double* __restrict__ tau_out,
                double* p, unsigned* bar, int* err) {
     extern __shared__ double sm[];
-    double* v = sm;
-    double* w = sm + n;
-    double* vn = sm + 2 * (size_t)n;
+    double* u = sm;
+    double* w = sm + n;                                  // p of the last step
+    double* x = sm + 2 * (size_t)n;                      // row k, then the next u
     __shared__ double red[2][4];
-    __shared__ double par[2];
+    __shared__ double par[2];                            // t, scale of the last reflector
+    __shared__ double part[kTrdRows][5];                 // per own row: sums of its quarters, entry k + 1
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int T = kTrdThreads, NW = T / 32;
     const int nblk = gridDim.x, blk = blockIdx.x;
-    for (int j = tid; j < n; j += T) { v[j] = 0.0; w[j] = 0.0; }
+    const int vt = tid < kTrdVec ? tid : n;              // the vector threads' start
+    for (int j = tid; j < n; j += kTrdThreads) { u[j] = 0.0; w[j] = 0.0; }
+    if (tid == 0) { par[0] = 0.0; par[1] = 0.0; }
+    double ref = 0.0;                                    // largest entry so far (scalar warp)
     __syncthreads();
+    double al2 = 0.0;                                    // t (p . u) of the last step
+    // p and row k of the last step's matrix into shared memory, then al2 (all threads; k: first index in use)
+    auto take_p = [&](int k) {
+        const double* pk = p + (size_t)((k - 1) & 1) * n;
+        for (int j = k + tid; j < n; j += kTrdThreads) w[j] = __ldcg(pk + j);
+    };
+    auto sum_pu = [&](int k) {
+        double sp = 0.0;
+        for (int j = k + vt; j < n; j += kTrdVec) sp = fma(w[j], u[j], sp);
+        al2 = par[0] * trd_sum(sp, red[0]);
+    };
     for (int k = 0; k + 2 < n; ++k) {
-        // row k of the current matrix, and the squares below its subdiagonal entry
-        const double vk = v[k], wk = w[k];
-        double ss = 0.0;
-        const int vt = tid < kTrdVec ? tid : n;          // the vector threads' start
-        for (int j = k + vt; j < n; j += kTrdVec) {
-            const double x = fma(-wk, v[j], fma(-vk, w[j], __ldcg(A + (size_t)k * n + j)));
-            vn[j] = x;
-            if (j >= k + 2) ss = fma(x, x, ss);
-        }
-        ss = trd_sum(ss, red[0]);
-        if (tid == 0) {
-            const double x0 = vn[k + 1];
-            double t = 0.0, beta = x0, scale = 0.0;
-            if (ss > 0.0) {
-                const double q = fma(x0, x0, ss), rq = rsqrt_newton(q), nrm = q * rq;
-                beta = -copysign(nrm, x0);
-                t = fma(fabs(x0), rq, 1.0);                    // (beta - x0) / beta
-                scale = rcp_newton(x0 - beta);
+        for (int j = k + tid; j < n; j += kTrdThreads) x[j] = __ldcg(A + (size_t)k * n + j);
+        if (k > 0) take_p(k);
+        __syncthreads();
+        if (k > 0) sum_pu(k);
+        const double scale = par[1];                     // of step k - 1
+        {
+            const double uk = u[k], ck = fma(-al2, uk, w[k]);
+            double ss = 0.0;
+            for (int j = k + vt; j < n; j += kTrdVec) {
+                const double y = fma(-ck, u[j], fma(-uk, w[j], x[j]));
+                x[j] = y;
+                if (j >= k + 2) ss = fma(y, y, ss);
             }
-            par[0] = t;
-            par[1] = scale;
+            if (tid < kTrdVec) {
+                ss = warp_sum(ss);
+                if (lane == 0) red[1][warp] = ss;
+            }
+        }
+        __syncthreads();
+        const int first = k + 1 + ((blk - (k + 1)) % nblk + nblk) % nblk;
+        double beta = 0.0;
+        if (warp < kTrdRowThreads / 32) {
+            // rows below k: quarter q of row first + r nblk
+            const int q = warp & 3;
+            for (int i = first + (warp >> 2) * nblk, r = warp >> 2; i < n; i += 4 * nblk, r += 4) {
+                const double ui = u[i], ci = fma(-al2, ui, w[i]);
+                double* row = A + (size_t)i * n;
+                double acc = 0.0;
+#pragma unroll 4
+                for (int j = k + 1 + 32 * q + lane; j < n; j += 128) {
+                    const double y = fma(-ci, u[j], fma(-ui, w[j], row[j]));
+                    row[j] = y;
+                    acc = fma(y, x[j], acc);
+                    if (j == k + 1) part[r][4] = y;
+                }
+                acc = warp_sum(acc);
+                if (lane == 0) part[r][q] = acc;
+            }
+            if (k > 0 && (k - 1) % nblk == blk)
+                for (int j = k + tid; j < n; j += kTrdRowThreads)
+                    A[(size_t)(k - 1) * n + j] = j == k ? 1.0 : u[j] * scale;
+        } else if (lane == 0) {
+            const double ss = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]), x0 = x[k + 1], dk = x[k];
+            const double sq = fma(x0, x0, ss);
+            double t = 0.0, sc = 0.0;
+            beta = x0;
+            // a row below 1e-100 of the entries so far couples nothing, and its square would leave the range
+            if (ss > 0.0 && !(sq < 1e-200 * ref * ref)) {
+                const double rq = rsqrt_newton(sq);
+                beta = -copysign(sq * rq, x0);
+                sc = rcp_newton(x0 - beta);
+                t = fma(fabs(x0), rq, 1.0);                        // (beta - x0) / beta
+            }
+            ref = fmax(ref, fmax(fabs(dk), fabs(beta)));
+            par[0] = t * sc * sc;
+            par[1] = sc;
+            red[0][0] = beta;
             if (blk == 0) {
-                d[k] = vn[k];
+                d[k] = dk;
                 e[k] = beta;
                 tau_out[k] = t;
             }
         }
         __syncthreads();
-        const double t = par[0], scale = par[1];
-        for (int j = k + 1 + vt; j < n; j += kTrdVec) vn[j] = j == k + 1 ? 1.0 : vn[j] * scale;
-        if (k > 0 && (k - 1) % nblk == blk)
-            for (int j = k + tid; j < n; j += T) A[(size_t)(k - 1) * n + j] = v[j];
-        __syncthreads();
-        // own rows below k
-        double* pk = p + (size_t)(k & 1) * n;
-        const int first = k + 1 + ((blk - (k + 1)) % nblk + nblk) % nblk;
-        for (int i = first + warp * nblk; i < n; i += NW * nblk) {
-            const double vi = v[i], wi = w[i];
-            double* row = A + (size_t)i * n;
-            double acc = 0.0;
-#pragma unroll 4
-            for (int j = k + 1 + lane; j < n; j += 32) {
-                const double x = fma(-wi, v[j], fma(-vi, w[j], row[j]));
-                row[j] = x;
-                acc = fma(x, vn[j], acc);
-            }
-            acc = warp_sum(acc);
-            if (lane == 0) __stcg(pk + i, t * acc);
-        }
+        beta = red[0][0];
+        if (tid == kTrdRowThreads) x[k + 1] -= beta;               // the rows have been taken with row k itself
+        const int i = first + tid * nblk;
+        if (tid < kTrdRows && i < n)
+            __stcg(p + (size_t)(k & 1) * n + i,
+                   par[0] * fma(-beta, part[tid][4], (part[tid][0] + part[tid][1]) + (part[tid][2] + part[tid][3])));
         if (nblk > 1) {
             if (!grid_barrier(bar, k + 1, err)) return;
         } else {
             __syncthreads();
         }
-        double sp = 0.0;
-        for (int j = k + 1 + vt; j < n; j += kTrdVec) {
-            const double x = __ldcg(pk + j);
-            w[j] = x;
-            sp = fma(x, vn[j], sp);
-        }
-        sp = trd_sum(sp, red[1]);
-        const double al = 0.5 * t * sp;
-        for (int j = k + 1 + vt; j < n; j += kTrdVec) w[j] = fma(-al, vn[j], w[j]);
-        double* x = v;
-        v = vn;
-        vn = x;
-        __syncthreads();
+        double* y = u;
+        u = x;
+        x = y;
     }
     // the last 2 x 2 block and the last reflector (its row was read before the last barrier)
     if (blk == 0) {
-        if (n > 2)
-            for (int j = n - 2 + tid; j < n; j += T) A[(size_t)(n - 3) * n + j] = v[j];
+        if (n > 2) {
+            take_p(n - 2);
+            __syncthreads();
+            sum_pu(n - 2);
+            for (int j = n - 2 + tid; j < n; j += kTrdThreads)
+                A[(size_t)(n - 3) * n + j] = j == n - 2 ? 1.0 : u[j] * par[1];
+        }
         if (tid == 0) {
             const int a = n - 2, b = n - 1;
-            auto at = [&](int i, int j) { return fma(-w[i], v[j], fma(-v[i], w[j], __ldcg(A + (size_t)i * n + j))); };
+            auto at = [&](int i, int j) {
+                return fma(-fma(-al2, u[i], w[i]), u[j], fma(-u[i], w[j], __ldcg(A + (size_t)i * n + j)));
+            };
             if (n >= 2) {
                 d[a] = at(a, a);
                 e[a] = at(a, b);
@@ -959,13 +996,13 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         WT_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
         WT_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         const size_t sh = 3 * (size_t)n * sizeof(double);
-        if (sh + 1024 <= (size_t)optin) {
+        // about one row per warp: more blocks than that only lengthen the barrier
+        int blocks = std::max(1, std::min(n_sm, (n + 7) / 8)), nn = n;
+        if (sh + 4096 <= (size_t)optin && (n + blocks - 1) / blocks <= kTrdRows) {
             allow_dyn_smem(trd_kernel, sh);
             bar.alloc(kBarrierWords);
             bar.zero(s);
             p.alloc(2 * (size_t)n);
-            // about one row per warp: more blocks than that only lengthen the barrier
-            int blocks = std::max(1, std::min(n_sm, (n + 7) / 8)), nn = n;
             void* args[] = {&A, &nn, &d.p, &e.p, &tau.p, &p.p, &bar.p, &d_err};
             WT_CUDA(cudaLaunchCooperativeKernel((const void*)trd_kernel, dim3(blocks), dim3(kTrdThreads), args, sh, s));
         } else {
