@@ -326,8 +326,9 @@ typedef struct {
     int nepi;       /* expansion epilogue warps: 8, 12, 16 */
     int r_xy, r_z;  /* elements per lane of the lateral and z register FFTs */
     int x_direct;   /* 1: the x transforms store from registers (else staged) */
-    int two_pass;   /* two-pass shared-memory FFTs in use, a bit mask: 1 the z pass (Nz of 64, 96,
-                       128, 160, 192, 224, 256 or 384; r_z then unused), 2 the y transforms (Ny of 64 or 128; r_xy then
+    int two_pass;   /* two-pass shared-memory FFTs in use, a bit mask: 1 the z pass (Nz of 40, 48,
+                       56, 64, 72, 80, 96, 112, 120, 128, 144, 160, 192, 224, 240, 256 or 384; r_z then
+                       unused), 2 the y transforms (Ny of 64 or 128; r_xy then
                        sets the x transforms only), 4 the x transforms too (with 2, Nx = Ny;
                        r_xy and x_direct then unused) */
     int store_vec;  /* floats per expansion store: 4 (4 x 4 lane-quad transposes), 2 (2 x 2

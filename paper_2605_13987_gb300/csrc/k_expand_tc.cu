@@ -75,11 +75,11 @@ __host__ __device__ constexpr int k_steps(int r) { return r > 8 ? (r + 7) / 8 : 
 // Producer warps: the conversion of a unit (rank x 128 values read, split and written twice to shared
 // memory) bounds the kernel below about 100 time samples, not the memory: 96 x 96 x 144
 // points, rank 29, 60 samples took 419 us with two such warps and two slices in flight, 294 us with four
-// warps, 275 us with four slices in flight and loads and products that stop at the rank (floor 203 us).
-// Four beside eight epilogue warps; two beside twelve or sixteen, which the autotuner takes for long
-// time axes only and whose registers would spill (80 or 96 instead of 96 to 122 a thread).
-__host__ __device__ constexpr int producers(int nepi) { return nepi == 8 ? 4 : 2; }
-__host__ __device__ constexpr int threads(int nepi) { return 32 * (1 + producers(nepi) + nepi); }
+// warps, 275 us with four slices in flight and loads and products that stop at the rank (floor 208 us).
+// Four beside eight epilogue warps up to 384 samples; two on longer axes, where the stores bound the kernel
+// (128 x 128 x 256 points, 512 samples: 4.43 ms with two, 4.52 with four), and beside twelve or sixteen,
+// whose registers would spill (80 or 96 instead of 96 to 122 a thread).
+__host__ __device__ constexpr int threads(int nepi, int nprod) { return 32 * (1 + nprod + nepi); }
 
 // 4 x 4 transposes within lane quads: on entry lane 4g + i holds v[4b + j] =
 // D[point 4g + i][time 4b + j]; on return v[4b + j] = D[point 4g + j][time 4b + i],
@@ -154,11 +154,11 @@ __device__ __forceinline__ void pair_transpose(float (&v)[32], int lane) {
     }
 }
 
-template <int NEPI, int VEC>
-__global__ void __launch_bounds__(threads(NEPI), 1)
+template <int NEPI, int VEC, int NPROD>
+__global__ void __launch_bounds__(threads(NEPI, NPROD), 1)
     expand_tc_kernel(const __grid_constant__ Jobs J, int nt_pad_max, int n_units, int nch, int lraw, int stall,
                      int* __restrict__ d_err) {
-    constexpr int NPROD = producers(NEPI), PART = BM / NPROD;   // producer warps, points of each
+    constexpr int PART = BM / NPROD;         // points of each producer warp
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // align the tile region to 1024 bytes
     unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -420,12 +420,12 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-static void encode_basis_map(CUtensorMap* m, const float* E, size_t npts, int rank, int nepi) {
+static void encode_basis_map(CUtensorMap* m, const float* E, size_t npts, int rank, int nprod) {
     // E viewed as 96 rows (component x basis index) of npts points; one box = the r rows in use x the
     // points of one producer warp (each loads its own part of a unit)
     cuuint64_t dims[2] = {(cuuint64_t)npts, (cuuint64_t)3 * tc::KR};
     cuuint64_t strides[1] = {(cuuint64_t)npts * sizeof(float)};
-    cuuint32_t box[2] = {(cuuint32_t)(tc::BM / tc::producers(nepi)), (cuuint32_t)tc::raw_rows(rank)};
+    cuuint32_t box[2] = {(cuuint32_t)(tc::BM / nprod), (cuuint32_t)tc::raw_rows(rank)};
     cuuint32_t es[2] = {1, 1};
     CUresult r = tensor_map_encoder()(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(E), dims, strides, box,
                                       es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -437,19 +437,20 @@ int expand_tc_max_jobs() { return tc::MAX_JOBS; }
 
 // jobs[j]: E [3][32][npts] FP32, W [nt][32] FP32, H [nt][3][npts] FP32; all
 // expansions in one persistent launch of at most `max_ctas` CTAs (0: one per SM).
+template <int NEPI, int VEC, int NPROD>
+static void launch_expand_n(int grid, size_t sh, cudaStream_t s, const tc::Jobs& J, int nt_pad_max, int units, int nch,
+                            int lraw, int stall, int* d_err) {
+    allow_dyn_smem(tc::expand_tc_kernel<NEPI, VEC, NPROD>, sh);
+    tc::expand_tc_kernel<NEPI, VEC, NPROD><<<grid, tc::threads(NEPI, NPROD), sh, s>>>(J, nt_pad_max, units, nch, lraw,
+                                                                                    stall, d_err);
+}
 template <int VEC>
-static void launch_expand(int nepi, int grid, size_t sh, cudaStream_t s, const tc::Jobs& J, int nt_pad_max, int units,
-                          int nch, int lraw, int stall, int* d_err) {
-    if (nepi == 8) {
-        allow_dyn_smem(tc::expand_tc_kernel<8, VEC>, sh);
-        tc::expand_tc_kernel<8, VEC><<<grid, tc::threads(8), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
-    } else if (nepi == 12) {
-        allow_dyn_smem(tc::expand_tc_kernel<12, VEC>, sh);
-        tc::expand_tc_kernel<12, VEC><<<grid, tc::threads(12), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
-    } else {
-        allow_dyn_smem(tc::expand_tc_kernel<16, VEC>, sh);
-        tc::expand_tc_kernel<16, VEC><<<grid, tc::threads(16), sh, s>>>(J, nt_pad_max, units, nch, lraw, stall, d_err);
-    }
+static void launch_expand(int nepi, int nprod, int grid, size_t sh, cudaStream_t s, const tc::Jobs& J, int nt_pad_max,
+                          int units, int nch, int lraw, int stall, int* d_err) {
+    if (nepi == 8 && nprod == 4) launch_expand_n<8, VEC, 4>(grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else if (nepi == 8) launch_expand_n<8, VEC, 2>(grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else if (nepi == 12) launch_expand_n<12, VEC, 2>(grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else launch_expand_n<16, VEC, 2>(grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
 }
 
 void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_ctas, int nch, int* d_err, int nepi,
@@ -458,6 +459,9 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
     if (nch != 64 && nch != 128 && nch != 256) fail(WT_ERR_ARG, "expansion time chunk must be 64, 128 or 256");
     if (n_jobs > tc::MAX_JOBS) fail(WT_ERR_UNSUPPORTED, "too many expansion jobs for one launch");
     if (nepi != 8 && nepi != 12 && nepi != 16) fail(WT_ERR_ARG, "expansion epilogue warps must be 8, 12 or 16");
+    int nt_max = 0;
+    for (int j = 0; j < n_jobs; ++j) nt_max = std::max(nt_max, jobs[j].nt);
+    const int nprod = nepi == 8 && nt_max <= 384 ? 4 : 2;
     tc::Jobs J;             // kernel parameter block (about 10 KB)
     int nt_pad_max = 32, units = 0;
     for (int j = 0; j < n_jobs; ++j) {
@@ -471,7 +475,7 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
         if (reinterpret_cast<uintptr_t>(jb.H) % 16) fail(WT_ERR_ARG, "H must be 16-byte aligned");
         const size_t n_tiles = (jb.npts + tc::BM - 1) / tc::BM;
         if ((size_t)units + 3 * n_tiles > (size_t)INT32_MAX) fail(WT_ERR_UNSUPPORTED, "expansion batch too large");
-        encode_basis_map(&J.emap[j], jb.E, jb.npts, jb.r, nepi);
+        encode_basis_map(&J.emap[j], jb.E, jb.npts, jb.r, nprod);
         J.W[j] = jb.W;
         J.H[j] = jb.H;
         J.npts[j] = jb.npts;
@@ -496,9 +500,9 @@ void expand_tc_jobs(cudaStream_t s, const ExpandJob* jobs, int n_jobs, int max_c
     // WT_FAULT=queue_stall: the MMA warp withholds its accumulator-ready signals, so the epilogue's
     // bounded waits run out and the kernel unwinds with DERR_TIMEOUT (tests of the failure path)
     const int stall = fault_enabled("queue_stall") ? 1 : 0;
-    if (vec == 4) launch_expand<4>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
-    else if (vec == 2) launch_expand<2>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
-    else launch_expand<1>(nepi, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    if (vec == 4) launch_expand<4>(nepi, nprod, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else if (vec == 2) launch_expand<2>(nepi, nprod, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
+    else launch_expand<1>(nepi, nprod, grid, sh, s, J, nt_pad_max, units, nch, lraw, stall, d_err);
     WT_LAUNCH("expand_tc");
 }
 
