@@ -94,38 +94,55 @@ __global__ void t64_series_kernel(int nz, double* __restrict__ CS) {
     CS[(size_t)nz * nz + e] = sn;
 }
 
-// R[a][kz][t][xy] for nb time samples, sixteen per thread and pass; grid (xy, kz, a).
-constexpr int kT64B = 16;
+// R[a][kz][t][xy] for nb time samples, kB of them per thread and pass; grid (xy, kz, a).  The FP64 units
+// bound it, so kB is the one of 2, 4, 8, 12, 16 that leaves the fewest samples of a pass empty (18 columns,
+// 128 x 128 x 256, three samples at a time: 5.8 ms with kB = 16, 1.45 with 4).
+template <int kB>
 __global__ void __launch_bounds__(128) t64_combine_kernel(const double* __restrict__ T, const double* __restrict__ Zc,
                                                           int n_cols, int nz, size_t nxy, int nb,
                                                           double* __restrict__ R) {
-    extern __shared__ __align__(16) double zs[];   // [n_cols][kT64B]
+    extern __shared__ __align__(16) double zs[];   // [n_cols][kB]
     const int kz = blockIdx.y, a = blockIdx.z;
     const size_t xy = (size_t)blockIdx.x * 128 + threadIdx.x;
     const bool in = xy < nxy;
     const double* t = T + ((size_t)a * nz + kz) * nxy + (in ? xy : 0);
     double* r = R + ((size_t)a * nz + kz) * nb * nxy + (in ? xy : 0);
-    for (int b0 = 0; b0 < nb; b0 += kT64B) {
+    for (int b0 = 0; b0 < nb; b0 += kB) {
         __syncthreads();
-        for (int e = threadIdx.x; e < n_cols * kT64B; e += 128) {
-            const int b = b0 + e % kT64B;
-            zs[e] = b < nb ? Zc[((size_t)b * n_cols + e / kT64B) * nz + kz] : 0.0;
+        for (int e = threadIdx.x; e < n_cols * kB; e += 128) {
+            const int b = b0 + e % kB;
+            zs[e] = b < nb ? Zc[((size_t)b * n_cols + e / kB) * nz + kz] : 0.0;
         }
         __syncthreads();
         if (!in) continue;
-        double acc[kT64B];
+        double acc[kB];
 #pragma unroll
-        for (int b = 0; b < kT64B; ++b) acc[b] = 0.0;
+        for (int b = 0; b < kB; ++b) acc[b] = 0.0;
 #pragma unroll 2
         for (int c = 0; c < n_cols; ++c) {
             const double v = t[(size_t)c * 3 * nz * nxy];
 #pragma unroll
-            for (int b = 0; b < kT64B; ++b) acc[b] = fma(zs[c * kT64B + b], v, acc[b]);
+            for (int b = 0; b < kB; ++b) acc[b] = fma(zs[c * kB + b], v, acc[b]);
         }
 #pragma unroll
-        for (int b = 0; b < kT64B; ++b)
+        for (int b = 0; b < kB; ++b)
             if (b0 + b < nb) r[(size_t)(b0 + b) * nxy] = acc[b];
     }
+}
+
+static int t64_pass(int nb) {
+    int best = 16;
+    for (int q : {12, 8, 4, 2})
+        if ((nb + q - 1) / q * q < (nb + best - 1) / best * best) best = q;
+    return best;
+}
+template <int kB>
+static void t64_combine(cudaStream_t s, const double* T, const double* Zc, int n_cols, int nz, size_t nxy, int nb,
+                        double* R) {
+    const size_t sh = (size_t)n_cols * kB * sizeof(double);
+    allow_dyn_smem(t64_combine_kernel<kB>, sh);
+    t64_combine_kernel<kB><<<dim3((unsigned)((nxy + 127) / 128), nz, 3), 128, sh, s>>>(T, Zc, n_cols, nz, nxy, nb, R);
+    WT_LAUNCH("t64_combine");
 }
 
 // Tables T [n_cols][3][Nz][Nx Ny] and the series matrices CS [2][Nz][Nz].  hux: distinct column x, hcu[c]
@@ -157,10 +174,13 @@ size_t t64_work(int nb, int Nx, int Ny, int Nz) { return dgemm_tc_rows_bytes(nb 
 void t64_fields(cudaStream_t s, const double* T, const double* CS, const double* Zc, int nb, int n_cols, int Nx, int Ny,
                 int Nz, double* R, unsigned char* ws, int* d_err, double* out) {
     const size_t nxy = (size_t)Nx * Ny, npts = nxy * Nz;
-    const size_t sh = (size_t)n_cols * kT64B * sizeof(double);
-    allow_dyn_smem(t64_combine_kernel, sh);
-    t64_combine_kernel<<<dim3((unsigned)((nxy + 127) / 128), Nz, 3), 128, sh, s>>>(T, Zc, n_cols, Nz, nxy, nb, R);
-    WT_LAUNCH("t64_combine");
+    switch (t64_pass(nb)) {
+        case 2: t64_combine<2>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
+        case 4: t64_combine<4>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
+        case 8: t64_combine<8>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
+        case 12: t64_combine<12>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
+        default: t64_combine<16>(s, T, Zc, n_cols, Nz, nxy, nb, R);
+    }
     const int M = (int)(nb * nxy);
     for (int a = 0; a < 3; ++a)
         dgemm_tc_rows(s, M, Nz, Nz, R + (size_t)a * Nz * M, M, CS + (a == 2 ? (size_t)Nz * Nz : 0), Nz,

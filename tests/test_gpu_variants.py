@@ -178,3 +178,23 @@ def test_eq1_direct_leaves_out_resting_steps(env, n_steps, n_out):
     b = s.eq1(H, tr).cpu().numpy()
     assert np.all(a[0] == 0.0)
     assert rel_l2(a, b) < 1e-5
+
+
+@pytest.mark.parametrize("n_t", [13, 18, 23, 30])
+def test_fp64_field_from_tables_by_any_count(env, n_t):
+    """Counts of time samples that the combination takes by 4, 8, 12 or 16 with some of a pass left empty."""
+    torch, P, _, _ = env
+    w = W.tiny_cell(nx=16, nz=32, n_t=n_t, radius=0.5 * 55e-6 / 16)
+    s = P.Sensor(w.grid, w.columns)
+    s.fit()
+    try:
+        s.relax(w.times)
+        many = s.extend("fp64")
+        for t in (0, n_t // 2, n_t - 1):
+            s.relax(w.times[t:t + 1])
+            one = s.extend("fp64")
+            torch.cuda.synchronize()
+            # the charges of both relaxations agree to the FP64 path's bound
+            assert rel_l2(many[t].cpu().numpy(), one[0].cpu().numpy()) < 1e-10
+    finally:
+        s.close()
