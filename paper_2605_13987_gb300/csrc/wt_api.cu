@@ -151,6 +151,7 @@ struct wt_ctx {
     // and the slab buffer of the combined planes ([32][3][Nz][ys][Nx])
     DBuf<float> T32, Rsl;
     bool t32_ready = false;
+    DBuf<unsigned char> eq1_ws;      // kept workspace of Eq. 1 on a stored field (eq1_run)
     DBuf<double> Zc64, G64;
     // FP64 lateral tables ([n_cols][3][Nz][Nx Ny], geometry only; built once), the series matrices and the
     // products' workspace
@@ -1084,8 +1085,12 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 // The tables of the FP64 field: held when they take at most 8 GiB and a quarter of the device's free
 // memory, and worth building from about n_cols N_y / 128 time samples on (their multiply-adds against
 // what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.35 ns per point and sample).
-bool tables64(wt_ctx* c, int nt) {
+// A capture on us takes what its warm-up call took: nothing is built then.
+bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     if (c->T64.p) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(us, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) return false;
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
     if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;
@@ -1127,7 +1132,7 @@ void extend64(wt_ctx* c, double* out, cudaStream_t s, int* launches) {
     const wt_grid& g = c->grid;
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const int nt = (int)c->times.size(), ncol = (int)c->cols.size();
-    if (tables64(c, nt)) {
+    if (tables64(c, nt, s)) {
         const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
         int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
         nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
@@ -1363,21 +1368,29 @@ void eq1_run(wt_ctx* c, const void* H, bool h64, const TrackDev& t, void* out, c
                      static_cast<double*>(out));
     else {
         // workspace of the staged dot products: all of them, or 1 GB of tracks at a time (a large field
-        // is then read once per GB); few steps go without (their sectors stay in L2 anyway)
+        // is then read once per GB); few steps go without (their sectors stay in L2 anyway).  Up to 64 MB
+        // stay with the context (the call has finished with them when it returns): an allocation and its
+        // release take 0.2 ms, as long as a small call.
         constexpr size_t kMost = (size_t)1 << 30, kFew = (size_t)1 << 20;
         const size_t steps = (size_t)t.n_tracks * t.n_steps;
-        DBuf<unsigned char> ws;
+        constexpr size_t kKeep = (size_t)64 << 20;
+        DBuf<unsigned char> own;
+        DBuf<unsigned char>* ws = nullptr;
         if (steps * nu >= kFew && eq1_stage_bytes(t.n_steps, nu, g.Nx, g.Ny, g.Nz) <= kMost && nu <= 65535) {
             const size_t all = eq1_stage_bytes(steps, nu, g.Nx, g.Ny, g.Nz);
             try {
-                ws.alloc(std::min(all, kMost));
+                ws = all <= kKeep ? &c->eq1_ws : &own;
+                if (ws->n < std::min(all, kMost)) {
+                    const size_t piece = (size_t)4 << 20;
+                    ws->alloc(ws == &own ? std::min(all, kMost) : (all + piece - 1) / piece * piece);
+                }
             } catch (const Error&) {       // no memory for it: the one-kernel form
                 if (fault_enabled("alloc")) throw;
             }
         }
         eq1_launch(s, static_cast<const float*>(H), g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx, t.vy,
                    vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, t.dt, c->opts.v_w, dlag.p, nu,
-                   static_cast<float*>(out), ws.p, ws.n);
+                   static_cast<float*>(out), ws ? ws->p : nullptr, ws ? ws->n : 0);
         WT_CUDA(cudaStreamSynchronize(s));
         return;
     }
