@@ -6,29 +6,47 @@
 
 namespace wt {
 
-// 1 / sqrt(x) of a positive x by Newton's iteration y <- y + y (1 - x y^2) / 2 from the FP32 value (24
-// bits, 46, then the FP64 rounding level), x normalised by its exponent.  A chain of about ten FP64
-// operations, each of which costs a warp 64 cycles of GB300's FP64 units.
+// 1 / sqrt(x) of a positive x from the FP32 value by one third-order step, y <- y + y e (1/2 + 3/8 e) with
+// e = 1 - x y^2 (the binomial series: e of 2^-21 leaves 2^-64), x normalised by its exponent.  A chain of
+// five FP64 operations, each of which costs a warp 64 cycles of GB300's FP64 units; Newton's two steps
+// take eight.
 __device__ __forceinline__ double rsqrt_newton(double x) {
     const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
     if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
     const int e = (ex - 1023) & ~1;                            // x = m 2^e, 1 <= m < 4
     const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
     double y = (double)rsqrtf((float)m);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) y = fma(0.5 * y, fma(-m * y, y, 1.0), y);
+    const double c = fma(-m * y, y, 1.0);
+    y = fma(y * c, fma(0.375, c, 0.5), y);
     return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
 }
-// 1 / x likewise, y <- y + y (1 - x y).
+// 1 / x likewise, y <- y + y (e + e^2) with e = 1 - x y.
 __device__ __forceinline__ double rcp_newton(double x) {
     const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
     if (ex <= 2 || ex >= 0x7fd) return 1.0 / x;
     const int e = ex - 1023;
     const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
     double y = (double)__frcp_rn((float)m);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) y = fma(y, fma(-m, y, 1.0), y);
+    const double c = fma(-m, y, 1.0);
+    y = fma(y, fma(c, c, c), y);
     return __hiloint2double(__double2hiint(y) - (e << 20), __double2loint(y));
+}
+
+// Sums of a, b and c over the warp: lanes 0, 8 and 16 return those of a, b and c (the two first steps halve
+// the values a lane carries: six FP64 additions a lane instead of fifteen).
+__device__ __forceinline__ double warp_sum3(double a, double b, double c) {
+    const int lane = threadIdx.x & 31;
+    // lanes below 16 go on with a and b, the others with c
+    const bool up = lane & 16;
+    const double s0 = up ? a : c, s1 = up ? b : 0.0;
+    double x = (up ? c : a) + __shfl_xor_sync(0xffffffffu, s0, 16);
+    double y = (up ? 0.0 : b) + __shfl_xor_sync(0xffffffffu, s1, 16);
+    // lanes with bit 3 go on with b
+    const bool hi = lane & 8;
+    double v = (hi ? y : x) + __shfl_xor_sync(0xffffffffu, hi ? x : y, 8);
+#pragma unroll
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // Barrier of the co-resident blocks of a cooperative launch: `round` counts them from 1.  bar:
