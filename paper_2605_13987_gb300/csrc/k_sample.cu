@@ -14,7 +14,7 @@ namespace wt {
 // so the k_x sums are taken once per (point, distinct x), as one FP64 product (on the tensor cores)
 //   G[p][u][my][mz] = sum_mx F[p][u][mx] T[mx][my][mz],   F = wx cos(kx dx) and 2 kx sin(kx dx),
 // the k_y sums and the z factors per (point, column, mz), and the sum over columns and mz for all times
-// as another product.  500 points, 16 times, 18 columns, 64 x 64 x 128: 38.4 -> 0.9 ms of kernels.
+// as another product.  500 points, 16 times, 18 columns, 64 x 64 x 128: 38.4 -> 1.1 ms of kernels.
 
 // F[(p, u, f)][mx], f = 0: wx cos, 1: 2 kx sin.
 __global__ void sample_xfactor_kernel(const double* __restrict__ pts, const double* __restrict__ ux, int n_pts,

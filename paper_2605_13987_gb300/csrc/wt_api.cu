@@ -1084,7 +1084,7 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 
 // The tables of the FP64 field: held when they take at most 8 GiB and a quarter of the device's free
 // memory, and worth building from about n_cols N_y / 128 time samples on (their multiply-adds against
-// what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.35 ns per point and sample).
+// what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.21 ns per point and sample against 0.50).
 // A capture on us takes what its warm-up call took: nothing is built then.
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     if (c->T64.p) return true;
