@@ -110,7 +110,7 @@ struct Eq1Cell {
 // in a cell of its own, 12 sectors a sample (49 GB for 1e6 steps x 128 samples of a 96 x 96 x 192
 // field), so the steps of a large call are taken in the order of their cells: a warp's 32 steps then
 // share the sectors of a few neighbouring cells.  That field and those steps: 16.0 ms with a block per
-// track, 4.55 ms a time plane at a time in the tracks' order, 1.24 ms in the cells' order (the sort
+// track, 4.55 ms a time plane at a time in the tracks' order, 1.16 ms in the cells' order (the sort
 // 0.055 ms).
 constexpr int kStageTimes = 8;
 struct Eq1Steps {
@@ -118,7 +118,7 @@ struct Eq1Steps {
     const unsigned* order;               // the step whose row of G a position fills (NULL: its own)
     size_t n;
 };
-__global__ void __launch_bounds__(256) eq1_stage_kernel(const float* __restrict__ H, int Nx, int Ny, int Nz,
+__global__ void __launch_bounds__(256, 4) eq1_stage_kernel(const float* __restrict__ H, int Nx, int Ny, int Nz,
                                                         float inv_hx, float inv_hy, float inv_hz, Eq1Steps st, int nu,
                                                         int ldg, float* __restrict__ G) {
     const size_t s = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -130,10 +130,15 @@ __global__ void __launch_bounds__(256) eq1_stage_kernel(const float* __restrict_
     c.vz = st.vz[s];
     c.set(st.x[s], st.y[s], st.z[s], Nx, Ny, Nz, inv_hx, inv_hy, inv_hz);
     const int n0 = blockIdx.y * kStageTimes;
-    float r[kStageTimes];
+    float r[kStageTimes] = {};
+    if (c.moving()) {
+        // no branch between the samples, so that their loads overlap; the ones past nu read the last plane
 #pragma unroll
-    for (int i = 0; i < kStageTimes; ++i)
-        r[i] = n0 + i < nu && c.moving() ? c.dot(H + (size_t)(n0 + i) * 3 * npts, npts) : 0.f;
+        for (int i = 0; i < kStageTimes; ++i) r[i] = c.dot(H + (size_t)min(n0 + i, nu - 1) * 3 * npts, npts);
+#pragma unroll
+        for (int i = 0; i < kStageTimes; ++i)
+            if (n0 + i >= nu) r[i] = 0.f;
+    }
     float4* g = reinterpret_cast<float4*>(G + (st.order ? (size_t)st.order[s] : s) * ldg + n0);
     g[0] = make_float4(r[0], r[1], r[2], r[3]);
     g[1] = make_float4(r[4], r[5], r[6], r[7]);
