@@ -42,6 +42,7 @@ constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
 constexpr int CHUNK = 1024;               // terms per accumulator: 1024 x 127^2 < 2^24
 constexpr int EPI_WARPS = 8;
 constexpr int kFusedK = 1024;             // longest K whose operands one launch converts
+constexpr int kMostTerms = 65535 * 64 / CHUNK * CHUNK;    // per pass: 64 of them per block of the residues' grid
 constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
 
 // pairwise coprime: 3 5 17, 11 23, 251, 13 19, 241, 239, 233, 229, 227, 223, 7 31, 211, 199, 197, 193
@@ -514,7 +515,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI_WARPS, 1)
 // ---------------------------------------------------------------- combine
 // sum a' b' = P x frac(sum_m r_m y_m / p_m), the fraction to 84 bits in three 28-bit limbs, taken
 // as signed; its top 64 bits to FP64 (2^-63 P is 2^-61 of ||a'|| ||b'||).  scale = alpha P 2^-64.
-// Four outputs per thread.
+// Four outputs per thread.  Blocks of 4 rows x 256 columns in one grid dimension: the rows of a field of
+// many time samples (samples x lateral points) pass the 65 535 blocks of the others.
 __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restrict__ T, int Tp, int M, int N,
                                                       const unsigned* __restrict__ ea,
                                                       const unsigned long long* __restrict__ sa,
@@ -522,7 +524,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
                                                       const unsigned long long* __restrict__ sb, double scale,
                                                       double beta, double* __restrict__ C, int ldc, int lower,
                                                       int mblk, size_t mstride) {
-    const int n = 4 * (blockIdx.x * 64 + (threadIdx.x & 63)), m = blockIdx.y * 4 + (threadIdx.x >> 6);
+    const int nblk = (N + 255) / 256;
+    const int n = 4 * (blockIdx.x % nblk * 64 + (threadIdx.x & 63)), m = blockIdx.x / nblk * 4 + (threadIdx.x >> 6);
     if (m >= M || n >= N || (lower && n > m)) return;
     constexpr Tables kT = make_tables();
     long long acc[4][3];
@@ -704,6 +707,7 @@ static Layout layout(int M, int N, int K, bool same) {
     L.kc = K;
     if (per_k * (size_t)K > ((size_t)6 << 30))
         L.kc = (int)std::max<size_t>(CHUNK, (((size_t)6 << 30) / per_k) / CHUNK * CHUNK);
+    L.kc = std::min(L.kc, kMostTerms);
     L.Kp = (std::min(K, L.kc) + 7) & ~7;
     L.Tp = (N + 15) & ~15;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
@@ -764,9 +768,8 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
     }
     unsigned __int128 P = 1;
     for (int m = 0; m < NMOD; ++m) P *= (unsigned)kMod[m];     // 117.4 bits, exact
-    combine_kernel<<<dim3((N + 255) / 256, (M + 3) / 4), 256, 0, s>>>(T, Tp, M, N, ea, sa, eb, sb,
-                                                                      std::ldexp((double)P, -64) * alpha, beta, C, ldc,
-                                                                      lower_only ? 1 : 0, mblk, mstride);
+    combine_kernel<<<(unsigned)((size_t)((N + 255) / 256) * ((M + 3) / 4)), 256, 0, s>>>(
+        T, Tp, M, N, ea, sa, eb, sb, std::ldexp((double)P, -64) * alpha, beta, C, ldc, lower_only ? 1 : 0, mblk, mstride);
     WT_LAUNCH("residue combine");
 }
 
@@ -774,7 +777,7 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only) {
     CallMemory* mem = t_memory;
-    if (!mem || !mem->d_err || std::fabs(alpha) != 1.0) return false;
+    if (!mem || !mem->d_err || std::fabs(alpha) != 1.0 || K > 65535 * tcg::SC_K) return false;
     // op(A) rows and op(B) columns that are the same vectors are converted once
     const Layout L = layout(M, N, K, A == B && lda == ldb && ta != tb && M == N);
     unsigned char* p = mem->products(L.total);
