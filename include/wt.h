@@ -182,6 +182,9 @@ wt_status wt_relax(wt_ctx* ctx, const double* t, int n_t);
  * point-sample).  H may be device memory (written on cuda_stream, a
  * cudaStream_t or NULL; asynchronous) or host memory (the library computes
  * into an internal device buffer and copies out; returns after the copy).
+ * An asynchronous extension goes on using the context's buffers after the
+ * call; later calls on the context, on whatever stream, wait for it on the
+ * GPU (a graph captured from the call is ordered by whoever launches it).
  * H_bytes must be >= n_t * 3 * Nx*Ny*Nz * sizeof(element), else WT_ERR_ARG.
  * The first FP32 extension of a context (unless wt_batch_run came first)
  * runs the autotuner of wt_batch_run on it, writing trial results into H,
@@ -250,7 +253,7 @@ wt_status wt_eq1_noalloc(wt_ctx* ctx, const float* H, const wt_tracks* tracks, f
  * call overwrote them).  Track arrays and i: host or device memory (as in
  * wt_eq1).  Ordered after the caller's work on cuda_stream; returns when i
  * is written.  Shares the FP32 work buffers of wt_extend and wt_batch_run:
- * do not run them concurrently on one context. */
+ * do not call them on one context from several threads at once. */
 wt_status wt_eq1_direct(wt_ctx* ctx, const wt_tracks* tracks, float* i, void* cuda_stream);
 
 /* Loss of Eq. 1 currents, L = mean over tracks and output times of i(tau)^2
@@ -312,9 +315,10 @@ wt_status wt_eq1_loss_grad_profile(wt_ctx* ctx, const wt_tracks* tracks, const d
  * keeps the fastest for the process (see wt_get_tuning); tuning writes into
  * that context's H buffer.  The results equal wt_extend's bit for bit.
  * FP64: the plain path of each context in turn.  Asynchronous on
- * cuda_stream, ordered after the contexts' own pending work; the contexts'
- * FP32 work buffers are shared with wt_extend, so do not run either on the
- * same context concurrently. */
+ * cuda_stream, ordered after the contexts' own pending work and their earlier
+ * extensions on other streams; the contexts' FP32 work buffers are shared with
+ * wt_extend, so do not call either on the same context from several threads at
+ * once. */
 wt_status wt_batch_run(wt_ctx* const* ctxs, int n, wt_precision prec, void* const* H, void* cuda_stream);
 
 /* Launch shapes the FP32 path of this context uses, set by the autotuner

@@ -171,6 +171,7 @@ struct wt_ctx {
     bool timing = false;
     bool use_tc = true;          // WT_EXPAND=simt selects the FP32 FMA expansion
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t ev_user = nullptr;       // last extension on a caller's stream (UserWork)
     cudaEvent_t ev_noalloc = nullptr;    // last wt_eq1_noalloc call, on the caller's stream
     bool noalloc_pending = false;
     bool ev_recorded = false;
@@ -225,6 +226,32 @@ int read_err(wt_ctx* c) {
     return h;
 }
 void clear_err(wt_ctx* c) { WT_CUDA(cudaMemsetAsync(c->d_err.p, 0, sizeof(int), c->s)); }
+
+// An extension on the caller's stream uses the context's buffers (charges, basis fields, tables) after the call
+// has returned: whatever uses them next, on the context's stream or another caller's, waits for it there.  A
+// captured extension is ordered by whoever launches the graph.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+    return cap != cudaStreamCaptureStatusNone;
+}
+void after_user_work(wt_ctx* c, cudaStream_t s) {
+    if (c->ev_user && !capturing(s)) WT_CUDA(cudaStreamWaitEvent(s, c->ev_user, 0));
+}
+struct UserWork {
+    wt_ctx* c;
+    cudaStream_t s;
+    UserWork(wt_ctx* c_, cudaStream_t s_) : c(c_), s(s_) {
+        if (capturing(s)) { c = nullptr; return; }
+        after_user_work(c, s);
+        if (!c->ev_user) WT_CUDA(cudaEventCreateWithFlags(&c->ev_user, cudaEventDisableTiming));
+    }
+    UserWork(const UserWork&) = delete;
+    UserWork& operator=(const UserWork&) = delete;
+    ~UserWork() {
+        if (c && cudaEventRecord(c->ev_user, s) != cudaSuccess) cudaGetLastError();
+    }
+};
 
 bool is_device_ptr(const void* p) {
     cudaPointerAttributes a{};
@@ -755,6 +782,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     cudaStream_t s = c->s;
     const int ns = c->ns, n1 = ns - 1;
     if (n1 < 1) fail(WT_ERR_GEOMETRY, "need at least two sources");
+    after_user_work(c, s);
     clear_err(c);
     c->times.assign(t, t + nt);
     // resistive lines (Sec. 5): G_seg = pi r^2 / (rho Delta), terminal 2 G_seg
@@ -1088,9 +1116,7 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 // A capture on us takes what its warm-up call took: nothing is built then.
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     if (c->T64.p) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(us, &cap) != cudaSuccess) cudaGetLastError();
-    if (cap != cudaStreamCaptureStatusNone) return false;
+    if (capturing(us)) return false;
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
     if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;
@@ -1179,7 +1205,7 @@ void do_extend(wt_ctx* c, wt_precision prec, void* H, size_t bytes, cudaStream_t
         if (prec == WT_FP64) c->stage64.alloc((size_t)nt * 3 * npts);
         else c->stage32.alloc((size_t)nt * 3 * npts);
     }
-    const int ncol = (int)c->cols.size();
+    UserWork use(c, s);
     if (c->timing) {
         for (int k = 0; k < 4; ++k)
             if (!c->ev[k]) WT_CUDA(cudaEventCreate(&c->ev[k]));
@@ -1238,6 +1264,7 @@ void do_extend(wt_ctx* c, wt_precision prec, void* H, size_t bytes, cudaStream_t
 void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, double* out) {
     ensure_spectral(c);
     cudaStream_t s = c->s;
+    after_user_work(c, s);
     const wt_grid& g = c->grid;
     const int ns = c->ns, ncol = (int)c->cols.size();
     for (int i = 0; i < nt; ++i)
@@ -1469,6 +1496,7 @@ void do_eq1_direct(wt_ctx* c, const wt_tracks* tr, float* iout, cudaStream_t us)
         WT_CUDA(cudaStreamWaitEvent(s, ev, 0));
         cudaEventDestroy(ev);
     }
+    after_user_work(c, s);
     DBuf<float> keep[7];
     const TrackDev td = stage_tracks(c, tr, keep, s);
     ensure_base_fields(c, s);
@@ -1506,6 +1534,7 @@ double do_loss(wt_ctx* c, wt_precision prec, const wt_tracks* tr) {
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const int nt = (int)c->times.size();
     if (tr->n_tracks == 0) return 0.0;
+    after_user_work(c, s);
     DBuf<float> keep[7];
     const TrackDev td = stage_tracks(c, tr, keep, s);
     int launches = 0;
@@ -1606,6 +1635,7 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
     for (int k = 0; k < n_out_params; ++k) grad[k] = 0.0;
     *loss = 0.0;
     if (tr->n_tracks == 0) return;
+    after_user_work(c, s);
     DBuf<float> keep[7];
     const TrackDev td = stage_tracks(c, tr, keep, s);
     const size_t nI = (size_t)tr->n_tracks * tr->n_out;
@@ -2152,6 +2182,7 @@ void do_batch(wt_ctx* const* ctxs, int n, wt_precision prec, void* const* H, cud
     for (int i = 0; i < n; ++i) {
         wt_ctx* c = ctxs[i];
         ensure_spectral(c);
+        after_user_work(c, c->s);            // its tuning uses the buffers, and the graph comes after that
         const TuneKey k = tune_key(c);
         if (!shapes.count(k)) shapes[k] = autotune(c, static_cast<float*>(H[i]));
         apply_tuning(c, shapes[k]);
@@ -2200,6 +2231,8 @@ void do_batch(wt_ctx* const* ctxs, int n, wt_precision prec, void* const* H, cud
         WT_CUDA(cudaStreamWaitEvent(us, ev, 0));
     }
     cudaEventDestroy(ev);
+    std::vector<std::unique_ptr<UserWork>> use;
+    for (int i = 0; i < n; ++i) use.push_back(std::make_unique<UserWork>(ctxs[i], us));
     WT_CUDA(cudaGraphLaunch(plan->exec, us));
 }
 
@@ -2447,6 +2480,7 @@ wt_status wt_static_field(wt_ctx* ctx, const double* phi_cols, wt_precision prec
             if (!std::isfinite(phi_cols[k])) fail(WT_ERR_ARG, "non-finite potential");
             for (int j = ctx->col_off[k]; j < ctx->col_off[k + 1]; ++j) phi[j] = phi_cols[k];
         }
+        after_user_work(ctx, s);
         DBuf<double> dphi, q;
         dphi.upload(phi.data(), ns, s);
         q.alloc(ns);
@@ -2659,6 +2693,10 @@ void wt_destroy(wt_ctx* ctx) {
         }
         cudaEventDestroy(ctx->ev_fork);
         cudaStreamDestroy(ctx->s_aux);
+    }
+    if (ctx->ev_user) {
+        cudaEventSynchronize(ctx->ev_user);
+        cudaEventDestroy(ctx->ev_user);
     }
     if (ctx->ev_noalloc) {
         cudaEventSynchronize(ctx->ev_noalloc);
