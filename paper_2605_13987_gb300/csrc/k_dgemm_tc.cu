@@ -515,8 +515,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI_WARPS, 1)
 // ---------------------------------------------------------------- combine
 // sum a' b' = P x frac(sum_m r_m y_m / p_m), the fraction to 84 bits in three 28-bit limbs, taken
 // as signed; its top 64 bits to FP64 (2^-63 P is 2^-61 of ||a'|| ||b'||).  scale = alpha P 2^-64.
-// Four outputs per thread.  Blocks of 4 rows x 256 columns in one grid dimension: the rows of a field of
-// many time samples (samples x lateral points) pass the 65 535 blocks of the others.
+// Four outputs per thread.  The row blocks are the grid's first dimension: the rows of a field of many time
+// samples (samples x lateral points) pass the 65 535 blocks of the others.
 __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restrict__ T, int Tp, int M, int N,
                                                       const unsigned* __restrict__ ea,
                                                       const unsigned long long* __restrict__ sa,
@@ -524,8 +524,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
                                                       const unsigned long long* __restrict__ sb, double scale,
                                                       double beta, double* __restrict__ C, int ldc, int lower,
                                                       int mblk, size_t mstride) {
-    const int nblk = (N + 255) / 256;
-    const int n = 4 * (blockIdx.x % nblk * 64 + (threadIdx.x & 63)), m = blockIdx.x / nblk * 4 + (threadIdx.x >> 6);
+    const int n = 4 * (blockIdx.y * 64 + (threadIdx.x & 63)), m = blockIdx.x * 4 + (threadIdx.x >> 6);
     if (m >= M || n >= N || (lower && n > m)) return;
     constexpr Tables kT = make_tables();
     long long acc[4][3];
@@ -768,7 +767,7 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
     }
     unsigned __int128 P = 1;
     for (int m = 0; m < NMOD; ++m) P *= (unsigned)kMod[m];     // 117.4 bits, exact
-    combine_kernel<<<(unsigned)((size_t)((N + 255) / 256) * ((M + 3) / 4)), 256, 0, s>>>(
+    combine_kernel<<<dim3((M + 3) / 4, (N + 255) / 256), 256, 0, s>>>(
         T, Tp, M, N, ea, sa, eb, sb, std::ldexp((double)P, -64) * alpha, beta, C, ldc, lower_only ? 1 : 0, mblk, mstride);
     WT_LAUNCH("residue combine");
 }
@@ -777,7 +776,7 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only) {
     CallMemory* mem = t_memory;
-    if (!mem || !mem->d_err || std::fabs(alpha) != 1.0 || K > 65535 * tcg::SC_K) return false;
+    if (!mem || !mem->d_err || std::fabs(alpha) != 1.0 || K > 65535 * tcg::SC_K || N > 65535 * 256) return false;
     // op(A) rows and op(B) columns that are the same vectors are converted once
     const Layout L = layout(M, N, K, A == B && lda == ldb && ta != tb && M == N);
     unsigned char* p = mem->products(L.total);
