@@ -153,9 +153,10 @@ struct wt_ctx {
     bool t32_ready = false;
     DBuf<unsigned char> eq1_ws;      // kept workspace of Eq. 1 on a stored field (eq1_run)
     DBuf<double> Zc64, G64;
-    // FP64 lateral tables ([n_cols][3][Nz][Nx Ny], geometry only; built once), the series matrices and the
-    // products' workspace
-    DBuf<double> T64, CS64;
+    // FP64 lateral tables ([n_cols][3][Nz][Nx Ny], geometry only; built once), the series matrices, and the
+    // buffers of a field from them: column transforms, combined planes, the products' workspace.  No other
+    // call uses them, so that a captured wt_extend stays valid (their sizes follow the time samples)
+    DBuf<double> T64, CS64, Zt64, R64;
     DBuf<unsigned char> ws64;
     DBuf<float> stage32;
     DBuf<double> stage64;
@@ -1162,14 +1163,14 @@ void extend64(wt_ctx* c, double* out, cudaStream_t s, int* launches) {
         const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
         int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
         nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
-        c->Zc64.alloc((size_t)std::max(nb, 4) * ncol * g.Nz);
-        c->G64.alloc(std::max(c->sp64.scratch_elems(4), (size_t)3 * nb * npts));
+        c->Zt64.alloc((size_t)nb * ncol * g.Nz);
+        c->R64.alloc((size_t)3 * nb * npts);
         c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
         for (int t0 = 0; t0 < nt; t0 += nb) {
             const int b = std::min(nb, nt - t0);
             column_ztransform<double>(s, c->Qt.p + (size_t)t0 * c->ns, b, c->ns, c->ns, c->zcos.p, c->d_col_off.p, ncol,
-                                      g.Nz, c->Zc64.p);
-            t64_fields(s, c->T64.p, c->CS64.p, c->Zc64.p, b, ncol, g.Nx, g.Ny, g.Nz, c->G64.p, c->ws64.p, c->d_err.p,
+                                      g.Nz, c->Zt64.p);
+            t64_fields(s, c->T64.p, c->CS64.p, c->Zt64.p, b, ncol, g.Nx, g.Ny, g.Nz, c->R64.p, c->ws64.p, c->d_err.p,
                        out + (size_t)t0 * 3 * npts);
             *launches += 2 + 3 * 3;
         }
