@@ -1116,11 +1116,11 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 // what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.21 ns per point and sample against 0.50).
 // A capture on us takes what its warm-up call took: nothing is built then.
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
-    if (c->T64.p) return true;
-    if (capturing(us)) return false;
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
-    if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;
+    if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;      // also when they exist: the same call, the same bits
+    if (c->T64.p) return true;
+    if (capturing(us)) return false;
     const size_t nxy = (size_t)g.Nx * g.Ny, bytes = (size_t)ncol * 3 * g.Nz * nxy * sizeof(double);
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); return false; }
