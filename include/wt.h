@@ -437,7 +437,10 @@ wt_status wt_features(wt_ctx* ctx, const float* x, int n_tracks, int n, double t
  * Failure injection for tests: the environment variable WT_FAULT, a comma
  * separated list of fit_singular (wt_fit reports WT_ERR_NOT_SPD),
  * alloc (every device allocation fails with WT_ERR_OOM), nan_q (wt_relax
- * meets a non-finite charge: WT_ERR_NAN) and queue_stall (the tensor-core
+ * meets a non-finite charge: WT_ERR_NAN), tables_oom and tables_timeout (the
+ * lateral tables of the FP64 field find no memory: one transform per sample;
+ * or a wait of their product runs out: WT_ERR_TIMEOUT, and they are built
+ * again) and queue_stall (the tensor-core
  * expansion withholds its accumulator signals, its bounded waits run out
  * after about 2 s and the call reports WT_ERR_TIMEOUT). */
 wt_status wt_sync(wt_ctx* ctx, void* cuda_stream);

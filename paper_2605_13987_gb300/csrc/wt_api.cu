@@ -158,6 +158,8 @@ struct wt_ctx {
     // call uses them, so that a captured wt_extend stays valid (their sizes follow the time samples)
     DBuf<double> T64, CS64, Zt64, R64;
     DBuf<unsigned char> ws64;
+    bool t64_ready = false;          // the tables are complete
+    int t64_nt = 0, t64_nb = 0;      // samples of the last field from them, samples per piece
     DBuf<float> stage32;
     DBuf<double> stage64;
     wt_info info{};
@@ -1114,19 +1116,14 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 // The tables of the FP64 field: held when they take at most 8 GiB and a quarter of the device's free
 // memory, and worth building from about n_cols N_y / 128 time samples on (their multiply-adds against
 // what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.21 ns per point and sample against 0.50).
-// A capture on us takes what its warm-up call took: nothing is built then.
+// A capture on us takes what its warm-up call took: nothing is built then.  False: one transform per
+// sample, also where the memory is not to be had (it needs far less).
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
     if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;      // also when they exist: the same call, the same bits
-    if (c->T64.p) return true;
+    if (c->t64_ready) return true;
     if (capturing(us)) return false;
-    const size_t nxy = (size_t)g.Nx * g.Ny, bytes = (size_t)ncol * 3 * g.Nz * nxy * sizeof(double);
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); return false; }
-    if (bytes > ((size_t)8 << 30) || bytes > fr / 4 || nxy * 3 * g.Nz > (size_t)INT32_MAX / 4) return false;
-    if (t64_work(1, g.Nx, g.Ny, g.Nz) > fr / 8) return false;
-    cudaStream_t s = c->s;
     std::vector<double> hux, hy(ncol);
     std::vector<int> hcu(ncol);
     for (int k = 0; k < ncol; ++k) {
@@ -1135,22 +1132,79 @@ bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
         hy[k] = c->cols[k].y;
     }
     const int nux = (int)hux.size();
-    TBuf<double> ux, cy, F, G, Y, ik2;
-    TBuf<int> cu;
-    ux.upload(hux.data(), nux, s);
-    cy.upload(hy.data(), ncol, s);
-    cu.upload(hcu.data(), ncol, s);
-    F.alloc((size_t)g.Nx * nux * g.Nx);
-    G.alloc((size_t)g.Nx * nux * g.Ny * g.Nz);
-    Y.alloc((size_t)ncol * g.Ny * g.Ny);
-    ik2.alloc((size_t)(g.Nx / 2) * (g.Ny / 2) * g.Nz);
-    green_invk2(s, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, ik2.p);
-    c->CS64.alloc((size_t)2 * g.Nz * g.Nz);
-    c->T64.alloc(bytes / sizeof(double));
-    t64_build(s, ux.p, cu.p, cy.p, ncol, nux, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, c->pref, ik2.p, F.p, G.p, Y.p,
-              c->T64.p, c->CS64.p);
-    WT_CUDA(cudaStreamSynchronize(s));
+    const size_t nxy = (size_t)g.Nx * g.Ny, nT = (size_t)ncol * 3 * g.Nz * nxy, nF = (size_t)g.Nx * nux * g.Nx,
+                 nG = (size_t)g.Nx * nux * g.Ny * g.Nz, nY = (size_t)ncol * g.Ny * g.Ny, nK = nxy / 4 * g.Nz;
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (nT * sizeof(double) > ((size_t)8 << 30) || nT * sizeof(double) > fr / 4 ||
+        (nF + nG + nY + nK) * sizeof(double) > fr / 4 || nxy * 3 * g.Nz > (size_t)INT32_MAX / 4 ||
+        t64_work(1, g.Nx, g.Ny, g.Nz) > fr / 8)
+        return false;
+    cudaStream_t s = c->s;
+    int* build_err = c->d_err.p + 1;         // the build's own error word
+    int err = 0;
+    try {
+        CallMemory memory(build_err);
+        WT_CUDA(cudaMemsetAsync(build_err, 0, sizeof(int), s));
+        TBuf<double> ux, cy, F, G, Y, ik2;
+        TBuf<int> cu;
+        ux.upload(hux.data(), nux, s);
+        cy.upload(hy.data(), ncol, s);
+        cu.upload(hcu.data(), ncol, s);
+        F.alloc(nF);
+        G.alloc(nG);
+        Y.alloc(nY);
+        ik2.alloc(nK);
+        green_invk2(s, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, ik2.p);
+        c->CS64.alloc((size_t)2 * g.Nz * g.Nz);
+        c->T64.alloc(nT);
+        if (fault_enabled("tables_oom")) fail(WT_ERR_OOM, "injected allocation failure (WT_FAULT=tables_oom)");
+        t64_build(s, ux.p, cu.p, cy.p, ncol, nux, g.Nx, g.Ny, g.Nz, g.Lx, g.Ly, g.Lz, c->pref, ik2.p, F.p, G.p, Y.p,
+                  c->T64.p, c->CS64.p);
+        if (fault_enabled("tables_timeout")) {   // injected: as if a bounded wait of the build's product had run out
+            const int v = DERR_TIMEOUT;
+            WT_CUDA(cudaMemcpyAsync(build_err, &v, sizeof(int), cudaMemcpyHostToDevice, s));
+        }
+        WT_CUDA(cudaMemcpyAsync(&err, build_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        WT_CUDA(cudaStreamSynchronize(s));
+        if (err) fail(WT_ERR_TIMEOUT, "device wait timed out while building the FP64 tables");
+    } catch (const Error& e) {
+        c->T64.release();
+        c->CS64.release();
+        if (e.code != WT_ERR_OOM) throw;
+        return false;
+    }
+    c->t64_ready = true;
     return true;
+}
+
+// Buffers of a field of nt samples from the tables: pieces of about 1 GB of intermediates, smaller ones where
+// the memory is not to be had.  Samples per piece; 0 when not even one sample's are to be had.
+int tables64_piece(wt_ctx* c, int nt) {
+    if (c->t64_nt == nt) return c->t64_nb;       // as before (a capture allocates nothing)
+    const wt_grid& g = c->grid;
+    const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
+    const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
+    int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
+    c->t64_nt = 0;
+    for (;; nb = nb / 2) {
+        nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
+        try {
+            c->Zt64.alloc((size_t)nb * c->cols.size() * g.Nz);
+            c->R64.alloc((size_t)3 * nb * npts);
+            c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
+            break;
+        } catch (const Error& e) {
+            c->Zt64.release();
+            c->R64.release();
+            c->ws64.release();
+            if (e.code != WT_ERR_OOM) throw;
+            if (nb == 1) return 0;
+        }
+    }
+    c->t64_nt = nt;
+    c->t64_nb = nb;
+    return nb;
 }
 
 // FP64 plain path into out [nt][3][npts]: from the lateral tables, several time samples at a time
@@ -1159,13 +1213,7 @@ void extend64(wt_ctx* c, double* out, cudaStream_t s, int* launches) {
     const wt_grid& g = c->grid;
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const int nt = (int)c->times.size(), ncol = (int)c->cols.size();
-    if (tables64(c, nt, s)) {
-        const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
-        int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
-        nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
-        c->Zt64.alloc((size_t)nb * ncol * g.Nz);
-        c->R64.alloc((size_t)3 * nb * npts);
-        c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
+    if (const int nb = tables64(c, nt, s) ? tables64_piece(c, nt) : 0) {
         for (int t0 = 0; t0 < nt; t0 += nb) {
             const int b = std::min(nb, nt - t0);
             column_ztransform<double>(s, c->Qt.p + (size_t)t0 * c->ns, b, c->ns, c->ns, c->zcos.p, c->d_col_off.p, ncol,
