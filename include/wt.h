@@ -440,7 +440,8 @@ wt_status wt_features(wt_ctx* ctx, const float* x, int n_tracks, int n, double t
  * meets a non-finite charge: WT_ERR_NAN), tables_oom and tables_timeout (the
  * lateral tables of the FP64 field find no memory: one transform per sample;
  * or a wait of their product runs out: WT_ERR_TIMEOUT, and they are built
- * again) and queue_stall (the tensor-core
+ * again), product_timeout (a wait of an FP64 product on the tensor cores runs
+ * out, with WT_FAULT_AT=n that of the call's n-th: WT_ERR_TIMEOUT) and queue_stall (the tensor-core
  * expansion withholds its accumulator signals, its bounded waits run out
  * after about 2 s and the call reports WT_ERR_TIMEOUT). */
 wt_status wt_sync(wt_ctx* ctx, void* cuda_stream);

@@ -770,6 +770,15 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
     combine_kernel<<<dim3((M + 3) / 4, (N + 255) / 256), 256, 0, s>>>(
         T, Tp, M, N, ea, sa, eb, sb, std::ldexp((double)P, -64) * alpha, beta, C, ldc, lower_only ? 1 : 0, mblk, mstride);
     WT_LAUNCH("residue combine");
+    // WT_FAULT=product_timeout: as if a wait of the product had run out (WT_FAULT_AT=n: of the call's n-th product)
+    if (fault_enabled("product_timeout")) {
+        const char* at = std::getenv("WT_FAULT_AT");
+        CallMemory* mem = CallMemory::current();
+        if (!at || (mem && ++mem->n_products == std::atoi(at))) {
+            const int v = DERR_TIMEOUT;
+            WT_CUDA(cudaMemcpyAsync(d_err, &v, sizeof(int), cudaMemcpyHostToDevice, s));
+        }
+    }
 }
 
 // True when the product was launched; false: the caller's FP64 kernel takes it.

@@ -222,13 +222,22 @@ wt_status run(wt_ctx* ctx, const char* fn, F&& body) {
     }
 }
 
+void clear_err(wt_ctx* c) { WT_CUDA(cudaMemsetAsync(c->d_err.p, 0, sizeof(int), c->s)); }
+// The device error word; an error is reported once.
 int read_err(wt_ctx* c) {
     int h = 0;
     WT_CUDA(cudaMemcpyAsync(&h, c->d_err.p, sizeof(int), cudaMemcpyDeviceToHost, c->s));
     WT_CUDA(cudaStreamSynchronize(c->s));
+    if (h) clear_err(c);
     return h;
 }
-void clear_err(wt_ctx* c) { WT_CUDA(cudaMemsetAsync(c->d_err.p, 0, sizeof(int), c->s)); }
+// Fails with `code` and `msg` on a device error, with WT_ERR_TIMEOUT when a bounded wait (of a product, a
+// cooperative launch or the expansion) gave up.
+void fail_on_err(wt_ctx* c, wt_status code, const char* msg) {
+    const int e = read_err(c);
+    if (e == DERR_TIMEOUT && code != WT_ERR_TIMEOUT) fail(WT_ERR_TIMEOUT, "device wait timed out");
+    if (e) fail(code, msg);
+}
 
 // An extension on the caller's stream uses the context's buffers (charges, basis fields, tables) after the call
 // has returned: whatever uses them next, on the context's stream or another caller's, waits for it there.  A
@@ -504,7 +513,7 @@ void do_fit(wt_ctx* c) {
         const int v = DERR_NOT_SPD;
         WT_CUDA(cudaMemcpyAsync(c->d_err.p, &v, sizeof(int), cudaMemcpyHostToDevice, s));
     }
-    if (read_err(c)) fail(WT_ERR_NOT_SPD, "normal matrix of the fit is not positive definite (rank-deficient fit)");
+    fail_on_err(c, WT_ERR_NOT_SPD, "normal matrix of the fit is not positive definite (rank-deficient fit)");
     copy_block(s, R.p, ns, Y.p, ns, ns, ns);
     trsm_lower(s, G.p, ns, ns, Y.p, ns, ns);
     trsm_lower_t(s, G.p, ns, ns, Y.p, ns, ns);
@@ -609,7 +618,7 @@ void do_fit(wt_ctx* c) {
     double nA = dnrm2(s, R.p, (size_t)ns * ns, c->d_scr.p);
     c->info.asymmetry = nF > 0 ? nA / nF : 0.0;
     check_finite(s, c->Cn.p, (size_t)ns * ns, c->d_err.p);
-    if (read_err(c)) fail(WT_ERR_NAN, "non-finite capacitance");
+    fail_on_err(c, WT_ERR_NAN, "non-finite capacitance");
     c->fitD.take(dcol);
     c->info.n_columns = ncol;
     c->info.n_sources = ns;
@@ -659,7 +668,7 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
     cudaStream_t s = c->s;
     const int ns = c->ns;
     const bool pre = ns >= nt && qrcp_fits(ns, nt);      // column-pivoted QR first
-    clear_err(c);
+    fail_on_err(c, WT_ERR_NAN, "non-finite charge history");
     TBuf<double> A, V, sig, Rm;
     TBuf<int> dpiv;
     int nr = nt;                                  // rows of R that are not negligible
@@ -758,7 +767,7 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
         TBuf<double> dvr;
         dvr.upload(vr.data(), vr.size(), s);
         dgemm(s, false, true, r, ns, nt, 1.0, dvr.p, nt, Q, nt, 0.0, Ub.p, ns);
-        WT_CUDA(cudaStreamSynchronize(s));
+        fail_on_err(c, WT_ERR_NAN, "time basis");
     } else {
         didx.upload(idx.data(), r, s);
         dscale.upload(scale.data(), r, s);
@@ -844,7 +853,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     }
     // Cholesky of the capacitance pencil side
     cholesky(s, Am.p, n1, n1, c->d_err.p);
-    if (read_err(c)) fail(WT_ERR_NOT_SPD, "fitted capacitance is not positive definite on the neutral subspace");
+    fail_on_err(c, WT_ERR_NOT_SPD, "fitted capacitance is not positive definite on the neutral subspace");
     // Shat = L^-1 Sm L^-T (symmetric positive definite)
     TBuf<double> Y, Yt;
     Y.alloc((size_t)n1 * n1);
@@ -911,7 +920,7 @@ void do_relax(wt_ctx* c, const double* t, int nt) {
     transpose(s, Q.p, ns, nt, c->Qt.p);
     if (fault_enabled("nan_q")) fill(s, c->Qt.p, 1, std::nan(""));     // injected non-finite charge
     check_finite(s, c->Qt.p, (size_t)nt * ns, c->d_err.p);
-    if (read_err(c)) fail(WT_ERR_NAN, "non-finite charges");
+    fail_on_err(c, WT_ERR_NAN, "non-finite charges");
     // S5b: time basis of the charge history (Gram matrix + Jacobi)
     c->r_pad = 32;
     compress_history(c, Q.p, nt, c->Ub, c->W32, c->W64, c->rank, c->info.trunc_rel);
@@ -1320,6 +1329,11 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
         if (!(t[i] >= 0.0) || !std::isfinite(t[i])) fail(WT_ERR_ARG, "sample times must be finite and >= 0");
     for (int i = 0; i < 3 * n; ++i)
         if (!std::isfinite(xyz[i])) fail(WT_ERR_NAN, "non-finite sample point");
+    // an error word of its own: the context's may still hold that of an extension under way
+    int* err = c->d_err.p + 2;
+    int h_err = 0;
+    CallMemory memory(err);
+    WT_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     TBuf<double> dt_, Q, Qt, Zc, T, Lat, pts, o;
     dt_.upload(t, nt, s);
     Q.alloc((size_t)ns * nt);
@@ -1358,7 +1372,9 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
                       c->pref, T.p, Zc.p, nt, F.p, G.p, Lat.p, o.p);
         hbuf.resize((size_t)nt * np * 3);
         o.download(hbuf.data(), hbuf.size(), s);
+        WT_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         WT_CUDA(cudaStreamSynchronize(s));
+        if (h_err) fail(WT_ERR_TIMEOUT, "device wait timed out in the point evaluation");
         for (int tt = 0; tt < nt; ++tt)
             std::memcpy(out + ((size_t)tt * n + p0) * 3, hbuf.data() + (size_t)tt * np * 3, sizeof(double) * np * 3);
     }
@@ -1909,7 +1925,7 @@ void do_loss_grad(wt_ctx* c, const wt_tracks* tr, double* loss, double* grad, co
         }
         grad[p - p_first] = gscale * acc;
         clock.mark(5);
-        if (read_err(c)) fail(WT_ERR_NAN, "non-finite or timed-out tangent");
+        fail_on_err(c, WT_ERR_NAN, "non-finite tangent");
     }
     clock.finish(c->grad_ms, 6);
 }

@@ -39,7 +39,8 @@ struct Error {
 [[noreturn]] void fail(wt_status code, const std::string& msg);
 
 // Host-side fault injection: WT_FAULT is a comma-separated list of names
-// (fit_singular, alloc, nan_q, queue_stall); each forces one error path.
+// (fit_singular, alloc, nan_q, tables_oom, tables_timeout, product_timeout, queue_stall); each forces one
+// error path.
 inline bool fault_enabled(const char* name) {
     const char* env = std::getenv("WT_FAULT");
     if (!env) return false;
@@ -121,6 +122,7 @@ struct DBuf {
 struct CallMemory {
     int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
     int n_sm = 0;                    // SMs of the device (0: not asked yet)
+    int n_products = 0;              // tensor-core products so far, counted for an injected failure
     explicit CallMemory(int* err);
     ~CallMemory();
     CallMemory(const CallMemory&) = delete;
