@@ -573,6 +573,13 @@ __global__ void __launch_bounds__(kPrepThreads) dc_prep_kernel(const DcNode* __r
     int* flag = W.oper + l;                // 1 = deflated (oper is written after the merge)
     const double* lam = lamA + l;
     if (tid == 0) { any_close = 0; n_rot = 0; }
+    // a NaN has no rank: the positions that nobody takes then keep an index of the node
+    for (int i = tid; i < K; i += kPrepThreads) {
+        perm[i] = i;
+        ds[i] = 0.0;
+        zs[i] = 0.0;
+    }
+    __syncthreads();
     double dmax = 0.0;
     for (int i = tid; i < K; i += kPrepThreads) {
         const double x = lam[i];
@@ -933,6 +940,15 @@ __global__ void __launch_bounds__(kPrepThreads) dc_order_kernel(const DcNode* __
     const double* root = W.root + l;
     double* sorted = W.delta + l;          // the poles are not needed any more
     int* idx = W.perm + l;
+    for (int q = threadIdx.x; q < nd_; q += kPrepThreads) {      // for the ranks that a NaN leaves open
+        idx[q] = q;
+        sorted[q] = 0.0;
+    }
+    for (int q = threadIdx.x; q < K; q += kPrepThreads) {
+        W.oper[l + q] = q;
+        W.lam_out[l + q] = 0.0;
+    }
+    __syncthreads();
     for (int q = threadIdx.x; q < nd_; q += kPrepThreads) {
         const double x = dv[q];
         int rank = 0;
