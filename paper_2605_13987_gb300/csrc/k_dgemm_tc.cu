@@ -610,18 +610,45 @@ CallMemory::~CallMemory() {
     for (void* c : chunks) cudaFree(c);
 }
 CallMemory* CallMemory::current() { return t_memory; }
+bool CallMemory::trim() {
+    bool any = false;
+    for (CallMemory* m = this; m; m = m->outer) {
+        if (m->ws) {
+            cudaFree(m->ws);                     // waits for the products that still use it
+            m->ws = nullptr;
+            m->ws_cap = 0;
+            any = true;
+        }
+        for (size_t k = 0; k < m->chunks.size(); ++k) {
+            bool used = !m->chunks[k];
+            for (const Piece& q : m->pieces) used = used || (q.chunk == (int)k && q.used);
+            if (used) continue;
+            cudaFree(m->chunks[k]);
+            m->chunks[k] = nullptr;
+            m->pieces.erase(std::remove_if(m->pieces.begin(), m->pieces.end(), [&](const Piece& q) { return q.chunk == (int)k; }),
+                            m->pieces.end());
+            any = true;
+        }
+    }
+    return any;
+}
+// cudaMalloc, once more after trim(); NULL when the memory is not to be had.
+static void* malloc_or_trim(CallMemory* m, size_t bytes) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    if (m->trim() && cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+}
 unsigned char* CallMemory::products(size_t bytes) {
     if (bytes <= ws_cap) return ws;
     if (fault_enabled("alloc")) return nullptr;
     if (ws) cudaFree(ws);                        // waits for the products that still use it
     ws = nullptr;
     ws_cap = 0;
-    if (cudaMalloc(reinterpret_cast<void**>(&ws), bytes) != cudaSuccess) {
-        cudaGetLastError();
-        ws = nullptr;
-        return nullptr;
-    }
-    ws_cap = bytes;
+    ws = static_cast<unsigned char*>(malloc_or_trim(this, bytes));
+    if (ws) ws_cap = bytes;
     return ws;
 }
 // Best fit among the free pieces, else a chunk of its own size (at least 16 MB, shared by small ones).
@@ -633,23 +660,11 @@ void* CallMemory::take(size_t bytes) {
     if (best < 0) {
         size_t size = std::max(need, (size_t)16 << 20);
         void* c = nullptr;
-        if (cudaMalloc(&c, size) != cudaSuccess) {
-            // give back the chunks that nothing uses and ask for no more than is needed
+        if (cudaMalloc(&c, size) != cudaSuccess) {           // then no more than is needed
             cudaGetLastError();
-            for (size_t k = 0; k < chunks.size(); ++k) {
-                bool used = !chunks[k];
-                for (const Piece& q : pieces) used = used || (q.chunk == (int)k && q.used);
-                if (used) continue;
-                cudaFree(chunks[k]);
-                chunks[k] = nullptr;
-                pieces.erase(std::remove_if(pieces.begin(), pieces.end(), [&](const Piece& q) { return q.chunk == (int)k; }),
-                             pieces.end());
-            }
             size = need;
-            if (cudaMalloc(&c, size) != cudaSuccess) {
-                cudaGetLastError();
-                return nullptr;
-            }
+            c = malloc_or_trim(this, size);
+            if (!c) return nullptr;
         }
         chunks.push_back(c);
         pieces.push_back({static_cast<unsigned char*>(c), size, (int)chunks.size() - 1, false});

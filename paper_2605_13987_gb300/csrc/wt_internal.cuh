@@ -69,6 +69,40 @@ void allow_dyn_smem(K* kernel, size_t bytes) {
                    "cudaFuncSetAttribute");
 }
 
+// Device memory of one library call: made by the C entry points, found through the calling thread,
+// given back when the call returns.  It serves the workspace of the tensor-core products (one, shared
+// by the products of a call in turn) and the call's temporaries (TBuf).  All of it is used on the
+// context's stream only, so that memory given back within the call can be handed out again at once;
+// cudaMalloc and cudaFree for each temporary cost the host 20 us apiece and a wait for the GPU (a
+// hundred of them in a fit and a relaxation).  An allocation of the call that finds no memory, here or in
+// DBuf, has it give back what nothing uses and tries again.
+struct CallMemory {
+    int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
+    int n_sm = 0;                    // SMs of the device (0: not asked yet)
+    int n_products = 0;              // tensor-core products so far, counted for an injected failure
+    explicit CallMemory(int* err);
+    ~CallMemory();
+    CallMemory(const CallMemory&) = delete;
+    CallMemory& operator=(const CallMemory&) = delete;
+    static CallMemory* current();
+    unsigned char* products(size_t bytes);   // the products' workspace; NULL when the memory is not to be had
+    void* take(size_t bytes);                // a temporary; NULL when the memory is not to be had
+    void give(void* p);
+    bool trim();                             // frees what nothing uses, of the outer calls too; whether there was any
+private:
+    struct Piece {
+        unsigned char* p;
+        size_t size;
+        int chunk;
+        bool used;
+    };
+    std::vector<Piece> pieces;               // by chunk, then by address
+    std::vector<void*> chunks;
+    unsigned char* ws = nullptr;
+    size_t ws_cap = 0;
+    CallMemory* outer;
+};
+
 // Owning device buffer.
 template <class T>
 struct DBuf {
@@ -91,6 +125,11 @@ struct DBuf {
         cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&p), count * sizeof(T));
         if (e != cudaSuccess) {
             cudaGetLastError();
+            CallMemory* m = CallMemory::current();
+            if (m && m->trim()) e = cudaMalloc(reinterpret_cast<void**>(&p), count * sizeof(T));
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
             p = nullptr;
             fail(WT_ERR_OOM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed");
         }
@@ -111,38 +150,6 @@ struct DBuf {
     void download(T* host, size_t count, cudaStream_t s) const {
         if (count) WT_CUDA(cudaMemcpyAsync(host, p, count * sizeof(T), cudaMemcpyDeviceToHost, s));
     }
-};
-
-// Device memory of one library call: made by the C entry points, found through the calling thread,
-// given back when the call returns.  It serves the workspace of the tensor-core products (one, shared
-// by the products of a call in turn) and the call's temporaries (TBuf).  All of it is used on the
-// context's stream only, so that memory given back within the call can be handed out again at once;
-// cudaMalloc and cudaFree for each temporary cost the host 20 us apiece and a wait for the GPU (a
-// hundred of them in a fit and a relaxation).
-struct CallMemory {
-    int* d_err;                      // error word for the kernels' bounded waits (NULL: no tensor-core products)
-    int n_sm = 0;                    // SMs of the device (0: not asked yet)
-    int n_products = 0;              // tensor-core products so far, counted for an injected failure
-    explicit CallMemory(int* err);
-    ~CallMemory();
-    CallMemory(const CallMemory&) = delete;
-    CallMemory& operator=(const CallMemory&) = delete;
-    static CallMemory* current();
-    unsigned char* products(size_t bytes);   // the products' workspace; NULL when the memory is not to be had
-    void* take(size_t bytes);                // a temporary; NULL when the memory is not to be had
-    void give(void* p);
-private:
-    struct Piece {
-        unsigned char* p;
-        size_t size;
-        int chunk;
-        bool used;
-    };
-    std::vector<Piece> pieces;               // by chunk, then by address
-    std::vector<void*> chunks;
-    unsigned char* ws = nullptr;
-    size_t ws_cap = 0;
-    CallMemory* outer;
 };
 
 // Temporary device buffer of one call, used on the context's stream only (DBuf's interface).
