@@ -1357,13 +1357,23 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
     TBuf<int> cu;
     ux.upload(hux.data(), nux, s);
     cu.upload(hcu.data(), ncol, s);
-    // points per chunk: 512, fewer where their k_x sums would take more than 1 GB
+    // points per chunk: 512, fewer where their k_x sums would take more than 1 GB, or the memory is not to be had
     const size_t per_point = (size_t)2 * nux * (g.Ny / 2) * g.Nz * sizeof(double);
-    const int chunk = std::min(n, (int)std::max<size_t>(1, std::min<size_t>(512, ((size_t)1 << 30) / per_point)));
-    F.alloc((size_t)2 * chunk * nux * (g.Nx / 2));
-    G.alloc((size_t)chunk * per_point / sizeof(double));
-    Lat.alloc((size_t)chunk * ncol * g.Nz * 3);
-    o.alloc((size_t)nt * chunk * 3);
+    int chunk = std::min(n, (int)std::max<size_t>(1, std::min<size_t>(512, ((size_t)1 << 30) / per_point)));
+    for (;; chunk = (chunk + 1) / 2) {
+        try {
+            F.alloc((size_t)2 * chunk * nux * (g.Nx / 2));
+            G.alloc((size_t)chunk * per_point / sizeof(double));
+            Lat.alloc((size_t)chunk * ncol * g.Nz * 3);
+            o.alloc((size_t)nt * chunk * 3);
+            break;
+        } catch (const Error& e) {
+            if (e.code != WT_ERR_OOM || chunk == 1) throw;
+            F.release();
+            G.release();
+            Lat.release();
+        }
+    }
     std::vector<double> hbuf;
     for (int p0 = 0; p0 < n; p0 += chunk) {
         const int np = std::min(chunk, n - p0);
