@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
     float* P = tab + (size_t)32 * row;                            // [ng][nm]
     __shared__ unsigned bits[kConvThreads / 4];
     __shared__ unsigned char list[kConvThreads];
-    __shared__ int n_list;
+    __shared__ int n_list, bad_step;                              // first step with a non-finite coefficient
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int e = tid; e < 32 * row; e += kConvThreads) tab[e] = dvt[e];
     const int t = tid % C.tm, g = tid / C.tm;                     // outputs 16 t .., group of steps
@@ -617,6 +617,7 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
     const int per_warp = (C.jc + kConvThreads / 32 - 1) / (kConvThreads / 32);
     for (int tr = blockIdx.x; tr < n_tracks; tr += gridDim.x) {
         for (int m = tid; m < nm; m += kConvThreads) D[m] = 0.0;
+        if (tid == 0) bad_step = n_out;
         for (int b0 = 0; b0 < n_steps; b0 += kConvSteps * kConvThreads) {
             // the groups of 8 steps in which the track moves at all, in order: a bit per group, then its place
             __syncthreads();                                           // the last list is used
@@ -667,7 +668,7 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
                     }
                     const unsigned moving = __ballot_sync(0xffffffffu, cell.moving());
                     const int a00 = (int)cell.a00, a01 = (int)cell.a01, a10 = (int)cell.a10, a11 = (int)cell.a11;
-                    int key = -1;
+                    int key = -1, bad_j = C.jc;
                     float v[24];
                     const int nl = min(32, per_warp - l0);
                     for (int l = 0; l < nl; ++l) {
@@ -704,8 +705,14 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
                             acc = w[0] * __shfl_sync(0xffffffffu, cell.vx, l) + w[1] * __shfl_sync(0xffffffffu, cell.vy, l) +
                                   w[2] * __shfl_sync(0xffffffffu, cell.vz, l);
                         }
-                        S[((lane >> 1) * C.js + j) * 2 + (lane & 1)] = lane < r ? acc : 0.f;
+                        // a step that is not finite counts nothing here (0 x infinity would reach the outputs before
+                        // it) and makes every output from its own on NaN at the end
+                        const bool use = lane < r && isfinite(acc);
+                        if (lane < r && !use) bad_j = min(bad_j, j);
+                        S[((lane >> 1) * C.js + j) * 2 + (lane & 1)] = use ? acc : 0.f;
                     }
+                    if (bad_j < C.jc)
+                        atomicMin(&bad_step, b0 + kConvSteps * list[k0 + bad_j / kConvSteps] + bad_j % kConvSteps);
                 }
                 __syncthreads();
                 // this thread's steps (in the chunk and in the track) and outputs
@@ -757,7 +764,8 @@ __global__ void __launch_bounds__(kConvThreads) eq1_conv_kernel(
         __syncthreads();
         const float qc = qtrack ? qtrack[tr] : qconst;
         for (int m = tid; m < n_out; m += kConvThreads)
-            out[(size_t)tr * n_out + m] = (float)(-(double)qc * inv_vw * D[(m % kConvOut) * C.tm + m / kConvOut]);
+            out[(size_t)tr * n_out + m] = m >= bad_step ? __int_as_float(0x7fffffff)
+                                                        : (float)(-(double)qc * inv_vw * D[(m % kConvOut) * C.tm + m / kConvOut]);
         __syncthreads();
     }
 }
