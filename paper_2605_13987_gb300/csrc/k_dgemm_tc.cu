@@ -104,9 +104,25 @@ __device__ __forceinline__ float mod_centred(float x, float p, float inv) {
 
 // ------------------------------------------------------------------ scale
 // Element (r, k) of an operand: TRANS false X[r ld + k], true X[k ld + r].  Largest biased
-// exponent per row, then the sum of squares relative to it (2^30 fixed point: the integer sums do
+// exponent per row, then the sum of squares relative to it (2^20 fixed point: the integer sums do
 // not depend on the order).  Blocks of 32 rows x 256 k.
 constexpr int SC_R = 32, SC_K = 256;
+
+// Biased exponent of x; 1 (its unit's) for a subnormal x, 0 for zero.
+__device__ __forceinline__ unsigned exponent_of(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+    const unsigned ex = hi >> 20;
+    return ex ? ex : (unsigned)((hi | lo) != 0);
+}
+// |x| 2^-(em - 1023) from the top 24 bits of x, for an x of at most the exponent em
+__device__ __forceinline__ float scaled_top(double x, unsigned em) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+    const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const int ex = (int)(hi >> 20), d = max(ex, 1) - (int)em;  // <= 0
+    if (d < -60) return 0.f;
+    if (ex == 0) return (float)m * __uint_as_float((unsigned)(104 + d) << 23);
+    return __uint_as_float(((unsigned)(127 + d) << 23) | m);
+}
 template <bool TRANS, bool SUM>
 __global__ void __launch_bounds__(256) scale_kernel(const double* __restrict__ X, int ld, int rows, int K,
                                                     unsigned* __restrict__ emax, unsigned long long* __restrict__ ss) {
@@ -116,14 +132,9 @@ __global__ void __launch_bounds__(256) scale_kernel(const double* __restrict__ X
     __shared__ unsigned sh_e[8][33];
     __shared__ float sh_s[8][33];
     auto add = [&](double x, unsigned em, unsigned& e, float& s) {
-        const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
-        const unsigned ex = hi >> 20;
-        if (!SUM) e = max(e, ex);
+        if (!SUM) e = max(e, exponent_of(x));
         else {
-            const int d = (int)ex - (int)em;                   // <= 0
-            const unsigned lo = (unsigned)__double2loint(x);
-            const float f = (ex == 0 || d < -60) ? 0.f
-                : __uint_as_float(((unsigned)(127 + d) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+            const float f = scaled_top(x, em);
             s = fmaf(f, f, s);
         }
     };
@@ -166,7 +177,8 @@ __global__ void __launch_bounds__(256) scale_kernel(const double* __restrict__ X
 }
 
 // Power of two by which a row is scaled: 2^sh with ||a 2^sh|| <= 2^58 (a margin of 2^-9 covers the
-// rounding of the sum and of a' itself).  kZeroRow: nothing in the row; kBadRow: an infinity or a NaN in it.
+// rounding of the sum and of a' itself).  kZeroRow: nothing in the row; kBadRow: an infinity or a NaN in it
+// (its products are summed in FP64, see combine_kernel).
 constexpr int kZeroRow = 1 << 20, kBadRow = 1 << 21;
 __device__ __forceinline__ int row_shift(unsigned emax, unsigned long long ss) {
     if (emax == 0) return kZeroRow;
@@ -188,10 +200,10 @@ __device__ __forceinline__ void residues_of(const double (&x)[2], int sh, __nv_b
     for (int j = 0; j < 2; ++j) {
         const unsigned hi = (unsigned)__double2hiint(x[j]);
         const int ex = (int)((hi >> 20) & 0x7ff);
-        unsigned long long mant = ((unsigned long long)(hi & 0xfffffu) << 32) | (unsigned)__double2loint(x[j]) |
-                                  (1ull << 52);
-        const int s = ex - 1075 + sh;                          // a' = round(mant 2^s), s <= 58 - 52
-        if (sh >= kZeroRow / 2 || ex == 0 || s < -54) mant = 0;
+        unsigned long long mant = ((unsigned long long)(hi & 0xfffffu) << 32) | (unsigned)__double2loint(x[j]);
+        if (ex) mant |= 1ull << 52;
+        const int s = max(ex, 1) - 1075 + sh;                  // a' = round(mant 2^s) <= 2^58
+        if (sh >= kZeroRow / 2 || s < -54) mant = 0;
         else if (s >= 0) mant <<= s;
         else mant = (mant + (1ull << (-s - 1))) >> -s;
         const float sg = (hi >> 31) ? -1.f : 1.f;
@@ -264,17 +276,14 @@ __global__ void __launch_bounds__(256) convert_kernel(Operand A, Operand B, int 
     if (threadIdx.x < 32) { e_sh[threadIdx.x] = 0; s_sh[threadIdx.x] = 0; }
     __syncthreads();
     auto at = [&](int r, int k) { return P.trans ? P.X[(size_t)k * P.ld + r0 + r] : P.X[(size_t)(r0 + r) * P.ld + k]; };
-    auto square = [](double x, unsigned em) {                  // (x 2^-(em - 1023))^2 from the top 24 bits
-        const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
-        const int ex = (int)(hi >> 20), d = ex - (int)em;
-        const float f = (ex == 0 || d < -60) ? 0.f
-            : __uint_as_float(((unsigned)(127 + d) << 23) | ((hi & 0xfffffu) << 3) | ((unsigned)__double2loint(x) >> 29));
+    auto square = [](double x, unsigned em) {
+        const float f = scaled_top(x, em);
         return f * f;
     };
     if (P.trans) {
         if (r0 + lane < P.rows) {
             unsigned e = 0;
-            for (int k = w; k < K; k += 8) e = max(e, ((unsigned)__double2hiint(at(lane, k)) >> 20) & 0x7ffu);
+            for (int k = w; k < K; k += 8) e = max(e, exponent_of(at(lane, k)));
             atomicMax(&e_sh[lane], e);
         }
         __syncthreads();
@@ -286,7 +295,7 @@ __global__ void __launch_bounds__(256) convert_kernel(Operand A, Operand B, int 
     } else {
         for (int i = w; i < 32 && r0 + i < P.rows; i += 8) {
             unsigned e = 0;
-            for (int k = lane; k < K; k += 32) e = max(e, ((unsigned)__double2hiint(at(i, k)) >> 20) & 0x7ffu);
+            for (int k = lane; k < K; k += 32) e = max(e, exponent_of(at(i, k)));
             e = __reduce_max_sync(0xffffffffu, e);
             float s = 0.f;
             for (int k = lane; k < K; k += 32) s += square(at(i, k), e);
@@ -517,13 +526,20 @@ __global__ void __launch_bounds__(64 + 32 * EPI_WARPS, 1)
 // as signed; its top 64 bits to FP64 (2^-63 P is 2^-61 of ||a'|| ||b'||).  scale = alpha P 2^-64.
 // Four outputs per thread.  The row blocks are the grid's first dimension: the rows of a field of many time
 // samples (samples x lateral points) pass the 65 535 blocks of the others.
+//
+// An output whose row of op(A) or column of op(B) holds an infinity or a NaN is the FP64 sum itself.
+struct Factors {
+    const double *A, *B;
+    int lda, ldb, K;
+    bool ta, tb;
+};
 __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restrict__ T, int Tp, int M, int N,
                                                       const unsigned* __restrict__ ea,
                                                       const unsigned long long* __restrict__ sa,
                                                       const unsigned* __restrict__ eb,
                                                       const unsigned long long* __restrict__ sb, double scale,
                                                       double beta, double* __restrict__ C, int ldc, int lower,
-                                                      int mblk, size_t mstride) {
+                                                      int mblk, size_t mstride, Factors F, double alpha) {
     const int n = 4 * (blockIdx.y * 64 + (threadIdx.x & 63)), m = blockIdx.x * 4 + (threadIdx.x >> 6);
     if (m >= M || n >= N || (lower && n > m)) return;
     constexpr Tables kT = make_tables();
@@ -545,6 +561,10 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
             for (int l = 0; l < 3; ++l) acc[e][l] += (long long)r * kT.limb[k][l];
         }
     const int sm = row_shift(ea[m], sa[m]);
+    auto out = [&](int e) {
+        return C + (mblk ? (size_t)(m / mblk) * mstride + (size_t)(m % mblk) * ldc : (size_t)m * ldc) + n + e;
+    };
+    int bad = 0;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         if (n + e >= N || (lower && n + e > m)) break;
@@ -554,8 +574,11 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
         const long long top = (long long)(((unsigned long long)a2 << 36) | ((unsigned long long)mid << 8) | (lo >> 20));
         const int sn = row_shift(eb[n + e], sb[n + e]);
         double v;
-        if (sm >= kBadRow || sn >= kBadRow) v = __longlong_as_double(0x7ff8000000000000ll);
-        else if (sm >= kZeroRow || sn >= kZeroRow) v = 0.0;
+        if (sm >= kBadRow || sn >= kBadRow) {
+            bad |= 1 << e;
+            continue;
+        }
+        if (sm >= kZeroRow || sn >= kZeroRow) v = 0.0;
         else {
             const int h = -(sm + sn);
             if (abs(h) < 900)                    // scale 2^h by its exponent bits (scale is +-2^53.4)
@@ -563,8 +586,17 @@ __global__ void __launch_bounds__(256) combine_kernel(const signed char* __restr
             else
                 v = scalbn((double)top * scale, h);
         }
-        double* c = C + (mblk ? (size_t)(m / mblk) * mstride + (size_t)(m % mblk) * ldc : (size_t)m * ldc) + n + e;
+        double* c = out(e);
         *c = beta == 0.0 ? v : fma(beta, *c, v);
+    }
+    for (int e = 0; bad >> e; ++e) {
+        if (!(bad >> e & 1)) continue;
+        const double *a = F.A + (F.ta ? (size_t)m : (size_t)m * F.lda), *b = F.B + (F.tb ? (size_t)(n + e) * F.ldb : (size_t)(n + e));
+        const size_t da = F.ta ? F.lda : 1, db = F.tb ? 1 : F.ldb;
+        double v = 0.0;
+        for (int k = 0; k < F.K; ++k, a += da, b += db) v = fma(*a, *b, v);
+        double* c = out(e);
+        *c = beta == 0.0 ? alpha * v : fma(beta, *c, alpha * v);
     }
 }
 
@@ -783,7 +815,8 @@ static void product(cudaStream_t s, bool ta, bool tb, int M, int N, int K, doubl
     unsigned __int128 P = 1;
     for (int m = 0; m < NMOD; ++m) P *= (unsigned)kMod[m];     // 117.4 bits, exact
     combine_kernel<<<dim3((M + 3) / 4, (N + 255) / 256), 256, 0, s>>>(
-        T, Tp, M, N, ea, sa, eb, sb, std::ldexp((double)P, -64) * alpha, beta, C, ldc, lower_only ? 1 : 0, mblk, mstride);
+        T, Tp, M, N, ea, sa, eb, sb, std::ldexp((double)P, -64) * alpha, beta, C, ldc, lower_only ? 1 : 0, mblk, mstride,
+        Factors{A, B, lda, ldb, K, ta, tb}, alpha);
     WT_LAUNCH("residue combine");
     // WT_FAULT=product_timeout: as if a wait of the product had run out (WT_FAULT_AT=n: of the call's n-th product)
     if (fault_enabled("product_timeout")) {
