@@ -240,7 +240,6 @@ int onesided_jacobi_rows(cudaStream_t s, double* A, int m, int n, int lda, doubl
 // the row-major array M [nt][ld] (ns >= nt; M is destroyed): R [nt][nt] row-major upper triangular,
 // piv[i] (device) = the column of M that became column i.  Only R and P are formed.  Returns the
 // number of steps taken: the rows of R past it are zero (negligible columns, see k_dense.cu).
-bool qrcp_fits(int ns, int nt);      // whether its reflector fits a block's shared memory
 int qrcp_r(cudaStream_t s, double* M, int ns, int nt, int ld, double* R, int* piv, int* d_err);
 // out[r][n] = scale[r] * A[idx[r]][:]  (idx, scale: device arrays of `rows`)
 void gather_rows_scaled(cudaStream_t s, const double* A, int n, int lda, const int* idx, const double* scale,
