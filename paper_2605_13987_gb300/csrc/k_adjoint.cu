@@ -79,7 +79,7 @@ void modal_inv_gap(cudaStream_t s, const double* mu, int n, double* inv) {
 // divided difference F_kl(t) = (E_k - E_l)/(mu_k - mu_l), F_kk = -t E_k, near-degenerate pairs
 // -t (E_k + E_l)/2.  (Daleckii-Krein derivative of the matrix exponential.)  Four rows k per block,
 // threads over t: the weights Om amp / gap of the four rows sit in shared memory (0 for the pairs
-// without a gap, which a list adds afterwards), so a pair costs one FP64 subtraction and one
+// without a gap, which are added afterwards in the order of l, from a bit each), so a pair costs one FP64 subtraction and one
 // multiply-add, and an E_l serves four rows (n = 1 151, 256 times: 3.99 -> 1.27 ms).
 constexpr int kModalRows = 4, kModalTile = 1024;
 __global__ void __launch_bounds__(256) modal_tangent_kernel(const double* __restrict__ Om,
@@ -90,8 +90,7 @@ __global__ void __launch_bounds__(256) modal_tangent_kernel(const double* __rest
                                                             const double* __restrict__ c, int n, int nt,
                                                             double* __restrict__ out) {
     __shared__ double wt[kModalTile][kModalRows];
-    __shared__ int near_l[kModalTile];
-    __shared__ int n_near;
+    __shared__ unsigned near_l[kModalTile / 32];
     const int k0 = blockIdx.x * kModalRows;
     // a pass of the tile loop per block of 256 times keeps the sums in registers
     for (int j0 = 0; j0 < nt; j0 += 256) {
@@ -106,22 +105,21 @@ __global__ void __launch_bounds__(256) modal_tangent_kernel(const double* __rest
         for (int l0 = 0; l0 < n; l0 += kModalTile) {
             const int nl = min(kModalTile, n - l0);
             __syncthreads();
-            if (threadIdx.x == 0) n_near = 0;
-            __syncthreads();
-            for (int e = threadIdx.x; e < nl; e += 256) {
+            for (int e = threadIdx.x; e < kModalTile; e += 256) {
                 const int l = l0 + e;
                 bool near = false;
 #pragma unroll
                 for (int q = 0; q < kModalRows; ++q) {
                     double x = 0.0;
-                    if (k0 + q < n) {
+                    if (k0 + q < n && e < nl) {
                         const double iv = inv[(size_t)(k0 + q) * n + l];
                         x = Om[(size_t)(k0 + q) * n + l] * amp[l] * iv;
                         near = near || iv == 0.0;
                     }
                     wt[e][q] = x;
                 }
-                if (near) near_l[atomicAdd(&n_near, 1)] = l;
+                const unsigned bits = __ballot_sync(0xffffffffu, near);
+                if ((threadIdx.x & 31) == 0) near_l[e >> 5] = bits;
             }
             __syncthreads();
             if (j < nt) {
@@ -131,17 +129,18 @@ __global__ void __launch_bounds__(256) modal_tangent_kernel(const double* __rest
 #pragma unroll
                     for (int q = 0; q < kModalRows; ++q) acc[q] = fma(wt[e][q], ek[q] - el, acc[q]);
                 }
-                for (int e = 0; e < n_near; ++e) {
-                    const int l = near_l[e];
-                    const double el = E[(size_t)l * nt + j];
+                for (int w = 0; 32 * w < nl; ++w)
+                    for (unsigned bits = near_l[w]; bits; bits &= bits - 1) {
+                        const int l = l0 + 32 * w + __ffs(bits) - 1;
+                        const double el = E[(size_t)l * nt + j];
 #pragma unroll
-                    for (int q = 0; q < kModalRows; ++q) {
-                        const int k = k0 + q;
-                        if (k >= n || inv[(size_t)k * n + l] != 0.0) continue;
-                        const double f = l == k ? -tj * ek[q] : -tj * 0.5 * (ek[q] + el);
-                        acc[q] = fma(Om[(size_t)k * n + l] * amp[l], f, acc[q]);
+                        for (int q = 0; q < kModalRows; ++q) {
+                            const int k = k0 + q;
+                            if (k >= n || inv[(size_t)k * n + l] != 0.0) continue;
+                            const double f = l == k ? -tj * ek[q] : -tj * 0.5 * (ek[q] + el);
+                            acc[q] = fma(Om[(size_t)k * n + l] * amp[l], f, acc[q]);
+                        }
                     }
-                }
             }
         }
         if (j < nt)
