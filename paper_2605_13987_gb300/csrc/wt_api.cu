@@ -685,9 +685,7 @@ void compress_history(wt_ctx* c, const double* Q, int nt, DBuf<double>& Ub, DBuf
         V.alloc((size_t)nt * nt);
     }
     double coupling = 0.0;
-    // rows of R below 1e-13 of the history carry nothing the basis could use (its target is 1e-7 of a
-    // sample, the smallest sample counted 1e-6 of the largest): they need not be orthogonal to each other
-    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nr, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling, 1e-13)
+    const int sweeps = pre ? onesided_jacobi_rows(s, Rm.p, nr, nt, nt, nullptr, sig.p, c->d_err.p, 40, &coupling)
                            : onesided_jacobi_rows(s, A.p, nt, ns, ns, V.p, sig.p, c->d_err.p, 40, &coupling);
     if (read_err(c)) {
         char msg[160];

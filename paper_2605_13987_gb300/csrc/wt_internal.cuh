@@ -232,10 +232,9 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
 // orthogonal (row i = sigma_i u_i^T), V [m][m] holds the accumulated rotations
 // (A_in = V^T A_out; V = NULL: not accumulated) and sigma[m] the row norms (unsorted).  Returns the number
 // of sweeps; sets d_err (DERR_TIMEOUT) when max_sweeps do not converge (unless the largest
-// relative coupling still rotated in the last sweep is below 1e-10; coupling_out returns it).  Pairs whose
-// coupling is below (floor_rel ||A||_F)^2 are not rotated.
+// relative coupling still rotated in the last sweep is below 1e-10; coupling_out returns it).
 int onesided_jacobi_rows(cudaStream_t s, double* A, int m, int n, int lda, double* V, double* sigma, int* d_err,
-                         int max_sweeps = 40, double* coupling_out = nullptr, double floor_rel = 1e-15);
+                         int max_sweeps = 40, double* coupling_out = nullptr);
 // Householder QR with column pivoting, M P = Q1 R, of the ns x nt matrix whose column j is row j of
 // the row-major array M [nt][ld] (ns >= nt; M is destroyed): R [nt][nt] row-major upper triangular,
 // piv[i] (device) = the column of M that became column i.  Only R and P are formed.  Returns the
