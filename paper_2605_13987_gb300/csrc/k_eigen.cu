@@ -556,8 +556,7 @@ constexpr int kPrepThreads = 1024;
 __global__ void __launch_bounds__(kPrepThreads) dc_prep_kernel(const DcNode* __restrict__ nodes,
                                                                const double* __restrict__ e,
                                                                const double* __restrict__ lamA,
-                                                               const double* __restrict__ QA, int n, DcWork W,
-                                                               double* zbuf) {
+                                                               const double* __restrict__ QA, int n, DcWork W) {
     __shared__ int sh_i[32];
     __shared__ double sh_d[32];
     __shared__ int any_close, n_rot;
@@ -1121,9 +1120,8 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
         TBuf<double> fbuf;
         ibuf.alloc((size_t)n * 8);
         fbuf.alloc((size_t)n * 12);
-        TBuf<double> WT, zbuf;
+        TBuf<double> WT;
         WT.alloc((size_t)n * n);
-        zbuf.alloc(n);
         const size_t nn = n;
         DcWork Wk{};
         Wk.perm = ibuf.p;
@@ -1160,7 +1158,7 @@ void sym_eig(cudaStream_t s, double* A, int n, double* w, double* V, int* d_err)
             const DcNode* dn = dnodes.p + level_at[lev];
             int kmax = 0;
             for (const DcNode& nd : nodes) kmax = std::max(kmax, nd.r - nd.l);
-            dc_prep_kernel<<<nn_, kPrepThreads, 0, s>>>(dn, e.p, la, qa, n, Wk, zbuf.p);
+            dc_prep_kernel<<<nn_, kPrepThreads, 0, s>>>(dn, e.p, la, qa, n, Wk);
             WT_LAUNCH("dc_prep");
             dc_secular_kernel<<<dim3((kmax + 7) / 8, nn_), 256, 0, s>>>(dn, Wk);
             WT_LAUNCH("dc_secular");

@@ -405,7 +405,6 @@ static size_t expand_smem(int nt_pad, int lraw) {
     return 1024 + (size_t)2 * nt_pad * 128 + 4 * (size_t)tc::TILE_BYTES + ((size_t)tc::RAW_BYTES << lraw) +
            sizeof(tc::Smem);
 }
-size_t expand_tc_smem(int nt_pad) { return expand_smem(nt_pad, 1); }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {

@@ -196,10 +196,10 @@ private:
 
 // ---------------------------------------------------------------- dense FP64
 // Row-major matrices.  op(A) is M x K, op(B) is K x N, C is M x N.  lower_only: entries above the
-// diagonal of C are left as they are.  Large products run on the tensor cores (fp64_cores: never).
+// diagonal of C are left as they are.  Large products run on the tensor cores.
 void dgemm(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha,
            const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
-           bool lower_only = false, bool fp64_cores = false);
+           bool lower_only = false);
 // dgemm on the tensor cores (k_dgemm_tc.cu); false when it does not take the product.
 bool dgemm_tc(cudaStream_t s, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
               const double* B, int ldb, double beta, double* C, int ldc, bool lower_only);
