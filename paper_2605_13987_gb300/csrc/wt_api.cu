@@ -1073,7 +1073,7 @@ void basis_fields32(wt_ctx* c, const double* Ub, int r, cudaStream_t s, int mode
         }
     }
     if (timing) WT_CUDA(cudaEventRecord(c->ev[2], s));
-    if (mode == 0 && Ub == c->Ub.p && r == c->rank) c->e32_stamp = c->version;
+    if (mode == 0 && Ub == c->Ub.p && r == c->rank && !capturing(s)) c->e32_stamp = c->version;   // captured: not run yet
 }
 
 void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt, float* out, cudaStream_t s, int mode,
