@@ -175,7 +175,9 @@ void shape_launch(cudaStream_t s, const float* cur, int n_tracks, int n_out, dou
     const double nn = n_out, mean_taps = n_taps >= n_out ? 0.5 * nn : n_taps * (1.0 - 0.5 * n_taps / nn);
     const double t_direct = std::max(std::ceil(nn / 256) * n_taps * 0.13, n_tracks * (0.024 + nn * mean_taps / 1.4e5));
     const double t_rec = nn * (order <= 4 ? 0.5 + 0.11 * order : 3.3) + 1.6e-5 * nn * n_tracks;
-    if (n_tracks > 0 && t_direct <= t_rec) {
+    // (dt / tau)^n, which the recursion's coefficients hold, must be a normal number (order 20: dt / tau of 1e-15 to
+    // 1e15); the taps hold it times a power of the lag and e^-t
+    if (n_tracks > 0 && (t_direct <= t_rec || !std::isnormal(step))) {
         const size_t sh = (size_t)n_taps * sizeof(double) + (size_t)n_out * sizeof(float);
         allow_dyn_smem(shape_direct_kernel, sh);
         shape_direct_kernel<<<n_tracks, 256, sh, s>>>(cur, n_out, n_taps, dt, tau, order, scale, noise_rms, noise, v);
