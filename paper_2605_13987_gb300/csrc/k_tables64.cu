@@ -96,7 +96,8 @@ __global__ void t64_series_kernel(int nz, double* __restrict__ CS) {
 
 // R[a][kz][t][xy] for nb time samples, kB of them per thread and pass; grid (xy, kz, a).  The FP64 units
 // bound it, so kB is the one of 2, 4, 8, 12, 16 that leaves the fewest samples of a pass empty (18 columns,
-// 128 x 128 x 256, three samples at a time: 5.8 ms with kB = 16, 1.45 with 4).
+// 128 x 128 x 256, three samples at a time: 5.8 ms with kB = 16, 1.45 with 4) among those whose coefficients
+// of all columns fit a block's shared memory (16 up to 1 600 columns).
 template <int kB>
 __global__ void __launch_bounds__(128) t64_combine_kernel(const double* __restrict__ T, const double* __restrict__ Zc,
                                                           int n_cols, int nz, size_t nxy, int nb,
@@ -130,12 +131,15 @@ __global__ void __launch_bounds__(128) t64_combine_kernel(const double* __restri
     }
 }
 
-static int t64_pass(int nb) {
-    int best = 16;
-    for (int q : {12, 8, 4, 2})
-        if ((nb + q - 1) / q * q < (nb + best - 1) / best * best) best = q;
+constexpr size_t kT64Coefs = 200 * 1024;
+static int t64_pass(int nb, int n_cols) {
+    int best = 2;
+    for (int q : {4, 8, 12, 16})
+        if ((size_t)n_cols * q * sizeof(double) <= kT64Coefs && (nb + q - 1) / q * q <= (nb + best - 1) / best * best) best = q;
     return best;
 }
+// Whether the combination takes so many columns.
+bool t64_takes(int n_cols) { return (size_t)n_cols * 2 * sizeof(double) <= kT64Coefs; }
 template <int kB>
 static void t64_combine(cudaStream_t s, const double* T, const double* Zc, int n_cols, int nz, size_t nxy, int nb,
                         double* R) {
@@ -174,7 +178,7 @@ size_t t64_work(int nb, int Nx, int Ny, int Nz) { return dgemm_tc_rows_bytes(nb 
 void t64_fields(cudaStream_t s, const double* T, const double* CS, const double* Zc, int nb, int n_cols, int Nx, int Ny,
                 int Nz, double* R, unsigned char* ws, int* d_err, double* out) {
     const size_t nxy = (size_t)Nx * Ny, npts = nxy * Nz;
-    switch (t64_pass(nb)) {
+    switch (t64_pass(nb, n_cols)) {
         case 2: t64_combine<2>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
         case 4: t64_combine<4>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;
         case 8: t64_combine<8>(s, T, Zc, n_cols, Nz, nxy, nb, R); break;

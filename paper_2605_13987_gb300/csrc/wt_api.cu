@@ -46,6 +46,7 @@ void sample_points(cudaStream_t, const double*, int, const double*, const double
 void t64_build(cudaStream_t, const double*, const int*, const double*, int, int, int, int, int, double, double, double,
                double, const double*, double*, double*, double*, double*, double*);
 size_t t64_work(int, int, int, int);
+bool t64_takes(int);
 void t64_fields(cudaStream_t, const double*, const double*, const double*, int, int, int, int, int, double*,
                 unsigned char*, int*, double*);
 void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, double, const float*, const float*,
@@ -1128,7 +1129,7 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
-    if (nt < std::max(4, ncol * (g.Ny / 2) / 64)) return false;      // also when they exist: the same call, the same bits
+    if (nt < std::max(4, ncol * (g.Ny / 2) / 64) || !t64_takes(ncol)) return false;      // also when they exist: the same call, the same bits
     if (c->t64_ready) return true;
     if (capturing(us)) return false;
     std::vector<double> hux, hy(ncol);
