@@ -175,9 +175,14 @@ wt_status wt_fit(wt_ctx* ctx, const wt_fit_opts* opts, double* cond_estimate_out
 wt_status wt_relax(wt_ctx* ctx, const double* t, int n_t);
 
 /* Bulk extension (Abstract; Sec. 1 DFT; Sec. 3 |k|^2 spectral division):
- * writes H[t][c][x][y][z] for all n_t times.  WT_FP64: plain path, one
- * FP64 spectral transform per time sample, H as double (24 B per
- * point-sample).  WT_FP32: fast path, FP32 basis fields of the rank-r
+ * writes H[t][c][x][y][z] for all n_t times.  WT_FP64: FP64 throughout, H
+ * as double (24 B per point-sample): of a few time samples by one spectral
+ * transform each; of more (from about columns x Ny / 128 on, at least 4) from
+ * lateral tables that the context builds once, several samples at a time.
+ * The context then holds until wt_destroy the tables (24 B x columns x grid
+ * points, at most 8 GiB and a quarter of the memory free when they are built)
+ * and about 1 GB of intermediates; where the memory is not to be had it takes
+ * one transform per sample.  WT_FP32: fast path, FP32 basis fields of the rank-r
  * time basis and a tensor-core expansion, H as float (12 B per
  * point-sample).  H may be device memory (written on cuda_stream, a
  * cudaStream_t or NULL; asynchronous) or host memory (the library computes
@@ -209,7 +214,9 @@ wt_status wt_sample_H(wt_ctx* ctx, const double* xyz, int n, const double* t, in
  * first/last grid plane) and linear interpolation in time (H = 0 at t = 0,
  * held after the last sample).  H must be device memory.  Track arrays and
  * i ([n_tracks][n_out] float32) may be device or host memory; the call
- * returns after the result is written. */
+ * returns after the result is written.  Its workspace is up to 1 GB of device
+ * memory, of which the context keeps up to 64 MB until wt_destroy; without it
+ * the call runs in the form of wt_eq1_noalloc. */
 wt_status wt_eq1(wt_ctx* ctx, const void* H, const wt_tracks* tracks, float* i, void* cuda_stream);
 
 /* Eq. 1 without any allocation.  Same result as wt_eq1, for callers that
@@ -259,7 +266,7 @@ wt_status wt_eq1_direct(wt_ctx* ctx, const wt_tracks* tracks, float* i, void* cu
 /* Loss of Eq. 1 currents, L = mean over tracks and output times of i(tau)^2
  * (Sec. 4's current of each track with its own charge, Eq. 1), computed in
  * one call: the field of the relaxed charges (WT_FP32: the fast path of
- * wt_extend; WT_FP64: the plain FP64 path) into an internal buffer, then
+ * wt_extend; WT_FP64: wt_extend's FP64 field) into an internal buffer, then
  * Eq. 1 on it.  Track arrays may be host or device memory (layout as in
  * wt_eq1).  Synchronous; *loss written on success.  Needs wt_relax. */
 wt_status wt_eq1_loss(wt_ctx* ctx, wt_precision prec, const wt_tracks* tracks, double* loss);
@@ -314,7 +321,7 @@ wt_status wt_eq1_loss_grad_profile(wt_ctx* ctx, const wt_tracks* tracks, const d
  * n_t) the autotuner times the candidate launch shapes on that context and
  * keeps the fastest for the process (see wt_get_tuning); tuning writes into
  * that context's H buffer.  The results equal wt_extend's bit for bit.
- * FP64: the plain path of each context in turn.  Asynchronous on
+ * FP64: wt_extend of each context in turn.  Asynchronous on
  * cuda_stream, ordered after the contexts' own pending work and their earlier
  * extensions on other streams; the contexts' FP32 work buffers are shared with
  * wt_extend, so do not call either on the same context from several threads at
