@@ -261,7 +261,7 @@ static bool eq1_sort(size_t steps, int nu, size_t bins) {
 // sectors (lanes over time samples: every read a sector of its own).
 // 1e4 tracks x 100 steps, 96 x 96 x 192, 128 samples: 38.1 ms with lanes over samples, 16.0 with lanes
 // over steps, 1.6 through G.  A stage holds `steps` steps (32, or 16 where 32 rows of samples
-// do not fit), accumulated 16 at a time.
+// do not fit, or the power of two that holds all of them), accumulated 16 at a time.
 template <class T, class L, class TO>
 __global__ void __launch_bounds__(256) eq1_kernel(const T* __restrict__ H, int Nx, int Ny, int Nz, int nt, int nu,
                                                   T inv_hx, T inv_hy, T inv_hz,
@@ -346,8 +346,11 @@ static void eq1_launch_t(cudaStream_t s, const T* H, int Nx, int Ny, int Nz, int
     auto bytes = [&](int steps) {
         return (((size_t)steps * ld * sizeof(T) + 15) & ~(size_t)15) + (size_t)n_out * sizeof(double);
     };
-    // 32 steps per stage while four blocks fit an SM (or 16 would not give more)
-    const int steps = bytes(32) <= 56 * 1024 ? 32 : 16;
+    // 32 steps per stage while four blocks fit an SM (or 16 would not give more); a power of two that holds
+    // the steps where they are fewer, so that all lanes have a time sample to take (one step, 200 samples: 55 us
+    // with 32, 41 with one; 100 tracks x 4 steps: 139 and 61)
+    int steps = bytes(32) <= 56 * 1024 ? 32 : 16;
+    while (steps / 2 >= n_steps) steps /= 2;
     const size_t sh = bytes(steps);
     allow_dyn_smem(eq1_kernel<T, L, TO>, sh);
     eq1_kernel<T, L, TO><<<n_tracks, 256, sh, s>>>(H, Nx, Ny, Nz, nt, nu, (T)(Nx / Lx), (T)(Ny / Ly), (T)(Nz / Lz), x, y,
