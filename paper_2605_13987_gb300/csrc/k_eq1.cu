@@ -247,11 +247,23 @@ static size_t eq1_step_bytes(int nu) { return (size_t)(eq1_ldg(nu) + 8) * sizeof
 size_t eq1_stage_bytes(size_t steps, int nu, int Nx, int Ny, int Nz) {
     return steps * eq1_step_bytes(nu) + eq1_bin_bytes(eq1_bins(Nx, Ny, Nz));
 }
+// Whether the staged form pays, kept: its workspace is there already.  From 2^20 values on (2^19 with more than
+// 64 samples); below, where a track has so many values that its one block takes long over them: one track
+// of 50 steps, 200 samples 132 -> 56 us, 100 of them 296 -> 119 us, 64 samples 73 -> 54 us; with 300 tracks
+// the blocks fill the chip and it takes four times the values (31 steps, 128 samples: 188 us without, 211
+// with).  Few samples are not worth an allocation of 0.25 ms below 2^24 values: 1 000 tracks x 1 000 steps, 12
+// samples 522 us without, 758 with.
+bool eq1_staged(int n_tracks, int n_steps, int nu, bool kept) {
+    const size_t per = (size_t)n_steps * nu, all = per * n_tracks;
+    if (nu > 65535 || (!kept && nu < 32 && all < ((size_t)1 << 24))) return false;
+    return all >= (nu > 64 ? (size_t)1 << 19 : (size_t)1 << 20) || per >= (n_tracks <= 200 ? 1000 : 4000);
+}
 // The sort pays for itself when there is a step for every eighth sector (a sector serves four cells), from
 // 2^21 values on (below, its launches take longer than the sectors it saves).  96 x 96 x 192, 128 samples:
-// 1e5 steps 982 -> 442 us, 4e4 steps 452 -> 375 us, 2e4 steps 226 -> 267 us (not sorted).
+// 1e5 steps 982 -> 442 us, 4e4 steps 452 -> 375 us, 2e4 steps 226 -> 267 us (not sorted).  A field of at most 4 096
+// bins stays in L1: 16 x 16 x 32, 3e5 steps x 12 samples 263 us, sorted 310.
 static bool eq1_sort(size_t steps, int nu, size_t bins) {
-    return 8 * steps >= bins && steps * nu >= ((size_t)1 << 21) && bins < ((size_t)1 << 31);
+    return 8 * steps >= bins && steps * nu >= ((size_t)1 << 21) && bins > 4096 && bins < ((size_t)1 << 31);
 }
 
 // T: field type; L: lag table entry; TO: current type.  nu: time samples the lag table reads

@@ -53,6 +53,7 @@ void eq1_launch(cudaStream_t, const float*, int, int, int, int, double, double, 
                 const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
                 double, const void*, int, float*, unsigned char*, size_t);
 size_t eq1_stage_bytes(size_t, int, int, int, int);
+bool eq1_staged(int, int, int, bool);
 size_t eq1_lag_size();
 void eq1_launch64(cudaStream_t, const double*, int, int, int, int, double, double, double, const float*, const float*,
                   const float*, const float*, const float*, const float*, const float*, float, int, int, int, double,
@@ -1469,16 +1470,15 @@ void eq1_run(wt_ctx* c, const void* H, bool h64, const TrackDev& t, void* out, c
                      static_cast<double*>(out));
     else {
         // workspace of the staged dot products: all of them, or 1 GB of tracks at a time (a large field
-        // is then read once per GB); few steps go without (their sectors stay in L2 anyway).  Up to 64 MB
-        // stay with the context (the call has finished with them when it returns): an allocation and its
-        // release take 0.2 ms, as long as a small call.
-        constexpr size_t kMost = (size_t)1 << 30, kFew = (size_t)1 << 20;
+        // is then read once per GB).  Up to 64 MB stay with the context (the call has finished with them when it
+        // returns): an allocation and its release take 0.25 ms, as long as a small call.
+        constexpr size_t kMost = (size_t)1 << 30, kKeep = (size_t)64 << 20;
         const size_t steps = (size_t)t.n_tracks * t.n_steps;
-        constexpr size_t kKeep = (size_t)64 << 20;
         DBuf<unsigned char> own;
         DBuf<unsigned char>* ws = nullptr;
-        if (steps * nu >= kFew && eq1_stage_bytes(t.n_steps, nu, g.Nx, g.Ny, g.Nz) <= kMost && nu <= 65535) {
-            const size_t all = eq1_stage_bytes(steps, nu, g.Nx, g.Ny, g.Nz);
+        const size_t all = eq1_stage_bytes(steps, nu, g.Nx, g.Ny, g.Nz);
+        if (eq1_staged(t.n_tracks, t.n_steps, nu, all <= kKeep) &&
+            eq1_stage_bytes(t.n_steps, nu, g.Nx, g.Ny, g.Nz) <= kMost) {
             try {
                 ws = all <= kKeep ? &c->eq1_ws : &own;
                 if (ws->n < std::min(all, kMost)) {
