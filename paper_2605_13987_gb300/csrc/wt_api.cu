@@ -154,6 +154,7 @@ struct wt_ctx {
     DBuf<float> T32, Rsl;
     bool t32_ready = false;
     DBuf<unsigned char> eq1_ws;      // kept workspace of Eq. 1 on a stored field (eq1_run)
+    DBuf<float> eq1_dvt;             // kept table of Eq. 1 from the rank-r form (eq1_basis_run)
     DBuf<double> Zc64, G64;
     // FP64 lateral tables ([n_cols][3][Nz][Nx Ny], geometry only; built once), the series matrices, and the
     // buffers of a field from them: column transforms, combined planes, the products' workspace.  No other
@@ -1526,17 +1527,20 @@ void eq1_basis_run(wt_ctx* c, const float* E, int r, const float* W32, const dou
     const wt_grid& g = c->grid;
     const int nt = (int)c->times.size();
     DBuf<unsigned char> dlag;
-    if (const size_t table = eq1_conv_table(t.n_out)) {
+    // tracks of up to 8 steps leave the convolution's groups of 8 steps and its table without use: 1 000 tracks of
+    // 4 steps 140 us against 122, 10 000 of one step 170 against 82 (the errors of both forms are equal there)
+    const bool few = t.n_steps <= 8 && eq1_basis_fits(nt, t.n_out);
+    if (const size_t table = few ? 0 : eq1_conv_table(t.n_out)) {
         build_lags(c, t.dt, t.n_out, dlag, s, true);
-        DBuf<float> dvt;
-        dvt.alloc(table);
+        DBuf<float>& dvt = c->eq1_dvt;           // kept: at most 110 KB, and an allocation is half of a small call
+        if (dvt.n < table) dvt.alloc(table);
         const size_t np = (size_t)g.Nx * g.Ny * g.Nz;
         c->Ep32.alloc(np * 96);
         eq1_point_major(s, E, r, np, c->Ep32.p);
         eq1_conv_launch(s, c->Ep32.p, r, W64, g.Nx, g.Ny, g.Nz, nt, g.Lx, g.Ly, g.Lz, t.x, t.y, t.z, t.vx, t.vy,
                         vz_override ? vz_override : t.vz, t.q, t.qconst, t.n_tracks, t.n_steps, t.n_out, c->opts.v_w,
                         dlag.p, dvt.p, out);
-        WT_CUDA(cudaStreamSynchronize(s));   // the tables are freed on return
+        WT_CUDA(cudaStreamSynchronize(s));   // the lag table is freed on return
         return;
     }
     const int nu = build_lags(c, t.dt, t.n_out, dlag, s, false);
