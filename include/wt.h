@@ -177,8 +177,9 @@ wt_status wt_relax(wt_ctx* ctx, const double* t, int n_t);
 /* Bulk extension (Abstract; Sec. 1 DFT; Sec. 3 |k|^2 spectral division):
  * writes H[t][c][x][y][z] for all n_t times.  WT_FP64: FP64 throughout, H
  * as double (24 B per point-sample): of a few time samples by one spectral
- * transform each; of more (from about columns x Ny / 128 on, at least 4) from
- * lateral tables that the context builds once, several samples at a time.
+ * transform each; of more (a single cell of 32 x 32 x 64 points: from 9 on,
+ * a 3 x 3 matrix of 128 x 128 x 256: from 18) from lateral tables that the
+ * context builds once, several samples at a time.
  * The context then holds until wt_destroy the tables (24 B x columns x grid
  * points, at most 8 GiB and a quarter of the memory free when they are built)
  * and about 1 GB of intermediates; where the memory is not to be had it takes

@@ -162,7 +162,7 @@ struct wt_ctx {
     DBuf<double> T64, CS64, Zt64, R64;
     DBuf<unsigned char> ws64;
     bool t64_ready = false;          // the tables are complete
-    int t64_nt = 0, t64_nb = 0;      // samples of the last field from them, samples per piece
+    int t64_nb = 0, t64_tried = 0;   // samples that a field's buffers hold, samples they were last wanted for
     DBuf<float> stage32;
     DBuf<double> stage64;
     wt_info info{};
@@ -1125,14 +1125,22 @@ void extend32_basis(wt_ctx* c, const double* Ub, int r, const float* W32, int nt
 
 // The tables of the FP64 field: held when they take at most 8 GiB and a quarter of the device's free
 // memory, and worth building from about n_cols N_y / 128 time samples on (their multiply-adds against
-// what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.21 ns per point and sample against 0.50).
+// what a sample saves; 3 x 3 cell, 128 x 128 x 256: 25 ms once, 0.21 ns per point and sample against 0.50),
+// where a first and a second field together do not take longer than without them.  In us, fitted to fields of
+// 16 x 16 x 32 to 128 x 128 x 256 points and 2 to 18 columns: a sample 12 + 0.5 ns a point by its own
+// transform, a third of that and 60 a field from the tables, the build 400 and its multiply-adds at 580 per ns
+// (single cell, 16 x 16 x 32: from 25 samples on, 32 x 32 x 64: 9, 64 x 64 x 64: 4).  Tables that are there
+// serve every field that is faster with them.
 // A capture on us takes what its warm-up call took: nothing is built then.  False: one transform per
 // sample, also where the memory is not to be had (it needs far less).
 bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     const wt_grid& g = c->grid;
     const int ncol = (int)c->cols.size();
-    if (nt < std::max(4, ncol * (g.Ny / 2) / 64) || !t64_takes(ncol)) return false;      // also when they exist: the same call, the same bits
-    if (c->t64_ready) return true;
+    if (!t64_takes(ncol)) return false;
+    const double t_own = nt * (12.0 + 5e-4 * g.Nx * g.Ny * (double)g.Nz), t_tab = 60.0 + t_own / 3.0;
+    if (c->t64_ready) return t_tab < t_own;
+    const double t_build = 400.0 + 1.5 * ncol * g.Nz * (double)g.Nx * g.Ny * g.Ny / 5.8e5;
+    if (nt < std::max(4, ncol * (g.Ny / 2) / 64) || t_build + 2.0 * t_tab > 2.0 * t_own) return false;
     if (capturing(us)) return false;
     std::vector<double> hux, hy(ncol);
     std::vector<int> hcu(ncol);
@@ -1188,33 +1196,38 @@ bool tables64(wt_ctx* c, int nt, cudaStream_t us) {
     return true;
 }
 
-// Buffers of a field of nt samples from the tables: pieces of about 1 GB of intermediates, smaller ones where
-// the memory is not to be had.  Samples per piece; 0 when not even one sample's are to be had.
-int tables64_piece(wt_ctx* c, int nt) {
-    if (c->t64_nt == nt) return c->t64_nb;       // as before (a capture allocates nothing)
+// Samples per piece of a field of nt samples from the tables: about 1 GB of intermediates, less where the
+// memory is not to be had; 0 when not even one sample's are.  The buffers grow only, and not under a
+// capture on us, so that the graph of a field stays valid.
+int tables64_piece(wt_ctx* c, int nt, cudaStream_t us) {
     const wt_grid& g = c->grid;
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const size_t per_t = t64_work(1, g.Nx, g.Ny, g.Nz) + 3 * npts * sizeof(double);
-    int nb = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
-    c->t64_nt = 0;
-    for (;; nb = nb / 2) {
-        nb = (nt + (nt + nb - 1) / nb - 1) / ((nt + nb - 1) / nb);          // even pieces
-        try {
-            c->Zt64.alloc((size_t)nb * c->cols.size() * g.Nz);
-            c->R64.alloc((size_t)3 * nb * npts);
-            c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
-            break;
-        } catch (const Error& e) {
-            c->Zt64.release();
-            c->R64.release();
-            c->ws64.release();
-            if (e.code != WT_ERR_OOM) throw;
-            if (nb == 1) return 0;
+    const int want = (int)std::min<size_t>(nt, std::max<size_t>(1, ((size_t)1 << 30) / per_t));
+    if (want > c->t64_nb && want > c->t64_tried && !capturing(us)) {
+        c->t64_nb = 0;
+        c->t64_tried = want;
+        for (int nb = want; nb > 0; nb /= 2) {
+            try {
+                c->Zt64.alloc((size_t)nb * c->cols.size() * g.Nz);
+                c->R64.alloc((size_t)3 * nb * npts);
+                c->ws64.alloc(t64_work(nb, g.Nx, g.Ny, g.Nz));
+                c->t64_nb = nb;
+                break;
+            } catch (const Error& e) {
+                c->Zt64.release();
+                c->R64.release();
+                c->ws64.release();
+                if (e.code != WT_ERR_OOM) throw;
+            }
         }
     }
-    c->t64_nt = nt;
-    c->t64_nb = nb;
-    return nb;
+    if (c->t64_nb == 0) {
+        c->t64_tried = 0;            // there may be memory the next time
+        return 0;
+    }
+    const int nb = std::min(want, c->t64_nb), pieces = (nt + nb - 1) / nb;
+    return (nt + pieces - 1) / pieces;                                   // even pieces
 }
 
 // FP64 plain path into out [nt][3][npts]: from the lateral tables, several time samples at a time
@@ -1223,7 +1236,7 @@ void extend64(wt_ctx* c, double* out, cudaStream_t s, int* launches) {
     const wt_grid& g = c->grid;
     const size_t npts = (size_t)g.Nx * g.Ny * g.Nz;
     const int nt = (int)c->times.size(), ncol = (int)c->cols.size();
-    if (const int nb = tables64(c, nt, s) ? tables64_piece(c, nt) : 0) {
+    if (const int nb = tables64(c, nt, s) ? tables64_piece(c, nt, s) : 0) {
         for (int t0 = 0; t0 < nt; t0 += nb) {
             const int b = std::min(nb, nt - t0);
             column_ztransform<double>(s, c->Qt.p + (size_t)t0 * c->ns, b, c->ns, c->ns, c->zcos.p, c->d_col_off.p, ncol,

@@ -9,7 +9,7 @@ from tests.gpu_common import device_tracks
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_t", [3, 12, 70])      # one transform per sample; from tables in one piece
+@pytest.mark.parametrize("n_t", [3, 12, 30, 70])      # one transform per sample; from tables in one piece
 def test_replay_after_other_calls(n_t):
     import torch
     import paper_2605_13987_gb300 as P

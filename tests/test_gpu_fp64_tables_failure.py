@@ -24,7 +24,7 @@ def fault(name):
 def test_failed_tables_are_not_used(name):
     import torch
     import paper_2605_13987_gb300 as P
-    w = W.tiny_cell(nx=16, nz=32, n_t=20, radius=0.5 * 55e-6 / 16)
+    w = W.tiny_cell(nx=16, nz=32, n_t=40, radius=0.5 * 55e-6 / 16)
     good = P.Sensor(w.grid, w.columns)
     good.fit()
     good.relax(w.times)
