@@ -1343,11 +1343,10 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
         if (!(t[i] >= 0.0) || !std::isfinite(t[i])) fail(WT_ERR_ARG, "sample times must be finite and >= 0");
     for (int i = 0; i < 3 * n; ++i)
         if (!std::isfinite(xyz[i])) fail(WT_ERR_NAN, "non-finite sample point");
-    // an error word of its own: the context's may still hold that of an extension under way
+    // an error word of its own (zero between calls): the context's may still hold that of an extension under way
     int* err = c->d_err.p + 2;
     int h_err = 0;
     CallMemory memory(err);
-    WT_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     TBuf<double> dt_, Q, Qt, Zc, T, Lat, pts, o;
     dt_.upload(t, nt, s);
     Q.alloc((size_t)ns * nt);
@@ -1396,9 +1395,13 @@ void do_sample(wt_ctx* c, const double* xyz, int n, const double* t, int nt, dou
                       c->pref, T.p, Zc.p, nt, F.p, G.p, Lat.p, o.p);
         hbuf.resize((size_t)nt * np * 3);
         o.download(hbuf.data(), hbuf.size(), s);
-        WT_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        if (memory.n_sm)                 // some product ran on the tensor cores
+            WT_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         WT_CUDA(cudaStreamSynchronize(s));
-        if (h_err) fail(WT_ERR_TIMEOUT, "device wait timed out in the point evaluation");
+        if (h_err) {
+            WT_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+            fail(WT_ERR_TIMEOUT, "device wait timed out in the point evaluation");
+        }
         for (int tt = 0; tt < nt; ++tt)
             std::memcpy(out + ((size_t)tt * n + p0) * 3, hbuf.data() + (size_t)tt * np * 3, sizeof(double) * np * 3);
     }
