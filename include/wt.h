@@ -246,7 +246,8 @@ wt_status wt_eq1(wt_ctx* ctx, const void* H, const wt_tracks* tracks, float* i, 
  * streams at once) race on it: order them on one stream.  Asynchronous on
  * cuda_stream; the call reads the relaxation's time samples there, and a
  * later wt_relax on the context waits for it (through an event recorded on
- * cuda_stream) before it replaces them. */
+ * cuda_stream) before it replaces them; launches of a graph captured from the
+ * call are ordered against wt_relax by the caller. */
 #define WT_EQ1_NOALLOC_MAX_OUT 16384
 wt_status wt_eq1_noalloc(wt_ctx* ctx, const float* H, const wt_tracks* tracks, float* i, void* cuda_stream);
 

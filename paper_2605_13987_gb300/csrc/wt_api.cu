@@ -2475,9 +2475,12 @@ wt_status wt_eq1_noalloc(wt_ctx* ctx, const float* H, const wt_tracks* tr, float
                            tr->q, (float)tr->charge, tr->n_tracks, tr->n_steps, tr->n_out, tr->dt, ctx->opts.v_w,
                            lag_samples_used(ctx->times, tr->dt, tr->n_out), i);
         // the call reads the relaxation's time samples on the caller's stream: a later wt_relax
-        // waits for this event before it rewrites them (the event was created by wt_relax)
-        WT_CUDA(cudaEventRecord(ctx->ev_noalloc, us));
-        ctx->noalloc_pending = true;
+        // waits for this event before it rewrites them (the event was created by wt_relax).  A captured call is
+        // ordered by whoever launches the graph: an event recorded under capture cannot be waited for
+        if (!capturing(us)) {
+            WT_CUDA(cudaEventRecord(ctx->ev_noalloc, us));
+            ctx->noalloc_pending = true;
+        }
     });
 }
 
